@@ -273,7 +273,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLow));
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             const int q_tiles = tile_b_active ? 2 : 1;
             mbar_arrive_expect_tx(q_full, q_tiles * L::kTileBytes);
             for (int t = 0; t < q_tiles; ++t)
@@ -326,7 +326,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
             // groups), which is slower than the alternation, where one tile's softmax runs under the
             // other tile's instructions. The token orders instruction issue only; no data depends on it.
             const int t = warp - 1;
-            if (lane == 0 && (t == 0 || tile_b_active)) {
+            if ((t == 0 || tile_b_active) && elect_one()) {
                 constexpr uint32_t idesc_s = idesc_bf16_f32(BQ, BKV, 0);
                 constexpr uint32_t idesc_o = idesc_bf16_f32(BQ, DH, 1);
                 // Shared-memory descriptors: (address >> 4) sits in the low 14 bits, so stepping through
@@ -438,7 +438,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         } else if (warp == 1) {
             // Head size 64: the groups are short, the token costs more than it saves, and one thread
             // serves both tiles in the fixed order A, B.
-            if (lane == 0) {
+            if (elect_one()) {
                 constexpr uint32_t idesc_s = idesc_bf16_f32(BQ, BKV, 0);
                 constexpr uint32_t idesc_o = idesc_bf16_f32(BQ, DH, 1);
                 // Shared-memory descriptors: (address >> 4) sits in the low 14 bits, so stepping through

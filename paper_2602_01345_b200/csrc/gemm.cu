@@ -217,7 +217,7 @@ gemm_bf16_tn(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__
     const uint32_t tmem_acc = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int issued = 0;
             for (int kb = 0; kb < num_kb; ++kb) {
                 const int s = kb % STAGES;
@@ -236,7 +236,7 @@ gemm_bf16_tn(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = idesc_bf16_f32(BM, BN, 0);
             bool ok = true;
             for (int kb = 0; kb < num_kb && ok; ++kb) {
@@ -529,7 +529,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             long it = 0;                         // k-blocks issued so far over all tiles of this pair
             bool ok = true;
             for (int local = 0; ok; ++local) {
@@ -561,7 +561,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             }
         }
     } else if (warp == 1) {
-        if (rank == 0 && lane == 0) {
+        if (rank == 0 && elect_one()) {
             // One elected thread of the leader CTA does nothing but wait and issue. Per 64-wide k-block
             // the tensor core works 512 clocks (four M=256, N=256, K=16 instructions); the thread spends
             // about 80 clocks per instruction, 50 on the commit and 65 on a wait that is already

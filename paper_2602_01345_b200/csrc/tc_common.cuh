@@ -13,6 +13,25 @@ constexpr unsigned long long kWaitLimitNs = 1000ull * 1000ull * 1000ull;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// True in one lane of a converged warp. Code that issues tcgen05.mma or TMA copies is guarded by this
+// and not by a lane number: those instructions take their operands from uniform registers, and only
+// behind elect.sync does the compiler know that a single thread is running and keep them there. Behind
+// `lane == 0` an instruction costs the issuing thread 45 clocks on an idle SM and 174 beside eight busy
+// warps (measured, 128x32x16 and 128x128x16 alike); behind elect.sync 128x128x16 issues every 64
+// to 66 clocks, which is what the tensor core needs to execute it, and 128x32x16 every 40 to 42.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t is_elected;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "elect.sync _|p, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(is_elected));
+    return is_elected != 0;
+}
+
 __device__ __forceinline__ unsigned long long global_ns()
 {
     unsigned long long t;
