@@ -3,7 +3,7 @@
 // One warp owns one row. The row is pulled from HBM exactly once and held packed in registers;
 // the warp takes the row maximum m, then one pass gives
 //   s = sum e^{z-m},  u = sum (z-m) e^{z-m},  H = ln s - u / s,
-// two logits per instruction (packed fp32). Rows of 2, 4 or 8 KiB (V = 4096 bf16 is 8 KiB) are
+// two logits per instruction (packed fp32). Rows of 2, 4, 8 or 16 KiB (V = 4096 is 8 KiB in bf16, 16 in fp32) are
 // staged through a shared-memory ring by bulk copies in a persistent kernel that also takes the
 // per-image means; other shapes use one-warp-per-row kernels and a separate mean kernel.
 #include "tc_common.cuh"
@@ -234,22 +234,32 @@ entropy_rows_reg(const void* __restrict__ logits, long rows, int V, long row_str
 }
 
 // ---- persistent kernel: rows staged through a shared-memory ring by bulk copies ----------------
-// One CTA per SM. A producer thread keeps the ring's slots (whole rows, 128 KB) in flight with
-// cp.async.bulk, one copy per row, completion counted on an mbarrier; sixteen consumer warps take
+// One CTA per SM. A producer thread keeps the ring's slots (whole rows) in flight with
+// cp.async.bulk, one copy per row, completion counted on an mbarrier; the consumer warps take
 // rows from the ring in turn, move the row into registers, hand the slot back at once and then do
 // the arithmetic. HBM sees one deep, steady stream per SM instead of waves of CTAs that load, then
 // compute. The per-segment means are completed by whichever CTA arrives last at a fixed-point
 // accumulator in global memory; integer addition commutes, so the result does not depend on the order.
-// Row i of a CTA goes to slot i % kSlots and to consumer warp i % 16; kSlots is a multiple of 16, so
-// every use of a slot is consumed by the same warp, in order. That matters: a parity wait for use
+// Row i of a CTA goes to slot i % kSlots and to consumer warp i % kConsumers; kSlots is a multiple of
+// kConsumers, so every use of a slot is consumed by the same warp, in order. That matters: a parity wait for use
 // n of a slot succeeds at once while use n-1 has not completed yet, and bulk copies may land out of
 // order (a copy that misses the TLB can trail later ones by microseconds), so a warp must never
 // poll a slot whose previous use some other warp has yet to see.
-constexpr int kRingConsumers = 16;
-constexpr int kRingProducers = 4;
-constexpr int kRingThreads = (kRingConsumers + 1) * 32;
 constexpr int kMaxMeanSegments = NOVA_MEAN_MAX_SEGMENTS;
-constexpr int kRingBytes = 128 * 1024;
+// Rows of 2 to 8 KiB: sixteen consumer warps on a 128 KiB ring, four producer lanes. Rows of 16 KiB
+// (V = 4096 in fp32): a lane holds 128 registers of its row, which leaves room for three warps per
+// scheduler, so eleven consumers with one slot each (176 KiB) and, at one row per 700 clocks, one producer. Eight
+// layers of 6400 such rows, with the selection after them, take 136 us (839 MB: 6.2 TB/s); as one-warp-per-row
+// and mean kernels, one pair of launches per layer, they took 248.
+template <int VEC>
+struct Ring {
+    static constexpr int kRowBytes = VEC * 512;
+    static constexpr int kConsumers = (VEC == 32) ? 11 : 16;
+    static constexpr int kProducers = (VEC == 32) ? 1 : 4;
+    static constexpr int kThreads = (kConsumers + 1) * 32;
+    static constexpr int kSlots = (VEC == 32) ? 11 : 128 * 1024 / kRowBytes;
+    static constexpr int kBytes = kSlots * kRowBytes;
+};
 
 // Bulk copy global -> shared of `bytes` (multiple of 16, both addresses 16-byte aligned).
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
@@ -266,7 +276,7 @@ struct LayerPtrs {
 };
 
 template <int VEC, bool BF16>
-__global__ void __launch_bounds__(kRingThreads, 1)
+__global__ void __launch_bounds__(Ring<VEC>::kThreads, 1)
 entropy_rows_ring(const LayerPtrs layers, long rows_per_layer, long rows, int V, long row_stride_bytes,
                   float* __restrict__ ent, float* __restrict__ mean, int seg_rows, int n_seg,
                   unsigned int* status, unsigned long long* __restrict__ accum, int fix_shift)
@@ -278,8 +288,8 @@ entropy_rows_ring(const LayerPtrs layers, long rows_per_layer, long rows, int V,
         return layers.p[l] + (long)((unsigned int)row - l * rpl) * row_stride_bytes;
     };
     using namespace tc;
-    constexpr int kRowBytes = VEC * 512;
-    constexpr int kSlots = kRingBytes / kRowBytes;
+    constexpr int kRowBytes = Ring<VEC>::kRowBytes, kSlots = Ring<VEC>::kSlots;
+    constexpr int kRingConsumers = Ring<VEC>::kConsumers, kRingProducers = Ring<VEC>::kProducers, kRingThreads = Ring<VEC>::kThreads;
     static_assert(kSlots % kRingConsumers == 0, "each slot must belong to one consumer warp");
     static_assert(kSlots % kRingProducers == 0, "each slot must belong to one producer lane");
     extern __shared__ uint8_t smem_raw[];
@@ -359,7 +369,7 @@ entropy_rows_ring(const LayerPtrs layers, long rows_per_layer, long rows, int V,
     if (!mean) return;
 
     // ---- means ---------------------------------------------------------------------------------
-    // A CTA's partial sum of a segment is added in a fixed order (a warp's rows in row order, the 16
+    // A CTA's partial sum of a segment is added in a fixed order (a warp's rows in row order, the
     // warps in warp order) and then joins the other CTAs' in ONE 64-bit atomic add per segment:
     //   bits 63..56  CTAs that have arrived      bits 55..46  how many of them had a non-finite sum
     //   bits 45..0   sum of the partial sums in fixed point (2^-fix_shift units)
@@ -442,8 +452,8 @@ template <int VEC, bool BF16>
 nova_status launch_ring(nova_ctx* ctx, const LayerPtrs& layers, long rows_per_layer, long rows, int V, long stride_bytes,
                         float* ent, float* mean, int N, int S, cudaStream_t st)
 {
-    constexpr int kSlots = kRingBytes / (VEC * 512);
-    const size_t smem = kRingBytes + 128 + 2 * sizeof(uint64_t) * kSlots + sizeof(float) * kRingConsumers * kMaxMeanSegments;
+    using R = Ring<VEC>;
+    const size_t smem = R::kBytes + 128 + 2 * sizeof(uint64_t) * R::kSlots + sizeof(float) * R::kConsumers * kMaxMeanSegments;
     static bool attr_done[64];
     if (ctx->device < 64 && !attr_done[ctx->device]) {
         NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(entropy_rows_ring<VEC, BF16>,
@@ -455,7 +465,7 @@ nova_status launch_ring(nova_ctx* ctx, const LayerPtrs& layers, long rows_per_la
     // has to stay below 2^46
     int fix_shift = 30;
     while (fix_shift > 0 && 24.0 * (double)N * exp2((double)fix_shift) >= 70368744177664.0 /* 2^46 */) --fix_shift;
-    entropy_rows_ring<VEC, BF16><<<grid, kRingThreads, smem, st>>>(
+    entropy_rows_ring<VEC, BF16><<<grid, R::kThreads, smem, st>>>(
         layers, rows_per_layer, rows, V, stride_bytes, ent, mean, N, S, ctx->dev_status,
         (unsigned long long*)(ctx->dev_status + NOVA_STATUS_WORDS), fix_shift);
     NOVA_CUDA_CHECK(ctx, cudaGetLastError());
@@ -489,7 +499,7 @@ static nova_status entropy_layers(nova_ctx* ctx, const void* const* layers, int 
     const int elt = (dt == NOVA_BF16) ? 2 : 4;
     const long row_bytes = (long)V * elt;
     const long segs = (long)n_layers * S;
-    if ((row_bytes == 2048 || row_bytes == 4096 || row_bytes == 8192) && rows >= 64 && rows <= 0x7fffffffL &&
+    if ((row_bytes == 2048 || row_bytes == 4096 || row_bytes == 8192 || (row_bytes == 16384 && dt == NOVA_F32)) && rows >= 64 && rows <= 0x7fffffffL &&
         n_layers <= kMaxEntropyLayers &&
         (!mean || (segs <= NOVA_MEAN_MAX_SEGMENTS && ctx->num_sms <= NOVA_MEAN_MAX_CTAS))) {
         // persistent ring kernel over the rows of all layers
@@ -504,6 +514,7 @@ static nova_status entropy_layers(nova_ctx* ctx, const void* const* layers, int 
                                          : launch_ring<4, false>(ctx, lp, rows_per_layer, rows, V, stride_bytes, ent, mean, N, sg, st);
         if (row_bytes == 4096) return bf ? launch_ring<8, true>(ctx, lp, rows_per_layer, rows, V, stride_bytes, ent, mean, N, sg, st)
                                          : launch_ring<8, false>(ctx, lp, rows_per_layer, rows, V, stride_bytes, ent, mean, N, sg, st);
+        if (row_bytes == 16384) return launch_ring<32, false>(ctx, lp, rows_per_layer, rows, V, stride_bytes, ent, mean, N, sg, st);
         return bf ? launch_ring<16, true>(ctx, lp, rows_per_layer, rows, V, stride_bytes, ent, mean, N, sg, st)
                   : launch_ring<16, false>(ctx, lp, rows_per_layer, rows, V, stride_bytes, ent, mean, N, sg, st);
     }

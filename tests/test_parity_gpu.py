@@ -79,6 +79,8 @@ def test_entropy_matches_oracle(ctx, S, N, V, dtype):
     (2, 700, 2048, torch.bfloat16),     # 4 KiB rows
     (1, 333, 1024, torch.bfloat16),     # 2 KiB rows
     (2, 200, 2048, torch.float32),      # 8 KiB rows of fp32
+    (3, 700, 4096, torch.float32),      # 16 KiB rows: eleven slots, reused
+    (1, 64, 4096, torch.float32),       # fewer rows than CTAs
     (4, 4096, 4096, torch.bfloat16),    # the benchmark's launch: batch 4 at 64 x 64 tokens
 ])
 def test_entropy_persistent_kernel_matches_oracle(ctx, S, N, V, dtype):
