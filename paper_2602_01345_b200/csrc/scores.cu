@@ -1,11 +1,7 @@
 // Alternative per-token selection scores of the paper's selection-metric ablation (the table that
 // compares entropy with an attention-based and an MSE-based criterion). Either score feeds the same
-// nova_select_topk as the entropy does. These are comparison criteria, not the method's hot path:
-// the kernels are straightforward (warp-per-row for the MSE score; warp-level matrix fragments for
-// the attention mass) and are not tuned beyond that.
-#include "common.cuh"
-
-#include <mma.h>
+// nova_select_topk as the entropy does.
+#include "tc_common.cuh"
 
 namespace {
 
@@ -72,171 +68,373 @@ score_mse_kernel(const uint4* __restrict__ x, const uint4* __restrict__ ref, int
 }
 
 // ---- attention mass ------------------------------------------------------------------------------
-// Two passes over S = q K^T / sqrt(dh) per (image, head), S tiles of 64 queries x 64 keys on
-// warp-level matrix fragments (bf16 in, fp32 out), one warp per 16 query rows:
-//   pass 1  row statistics: lse[b, h, q] = log2-domain log-sum-exp of row q over all keys
-//   pass 2  column sums over the scale's own keys: one CTA per 64 keys walks all heads and query
-//           tiles in a fixed order (deterministic, no atomics) and adds up 2^(s - lse).
-constexpr int kAmTile = 64;
-constexpr int kAmThreads = 128;
+// Two passes over S = q K^T / sqrt(dh) per (image, head), both as 128 x 128 tiles on the tensor cores:
+//   pass 1  rows: A = 128 queries, B = the key tiles (cache rows, then the scale's own keys);
+//           lse[b, h, q] = log2-domain log-sum-exp of row q over all keys
+//   pass 2  columns, transposed so that a thread's row is a key: A = 128 own keys, B = the query tiles of
+//           one head after the other; score[key] = sum of 2^(s - lse) over queries and heads
+// What bounds both is the special-function unit: one exponential per score, 16 per clock and SM, 44 us
+// for the 201 M scores of two images of 1024 tokens, 30 heads and 1216 prior keys. The rest is arranged
+// around keeping it busy: one thread per row of S reads its row from tensor memory 64 scores at a
+// time, two warpgroups take the tiles in turn, each with its own S buffer (256 columns of tensor memory),
+// and at head size 64 two CTAs share an SM. A row's work is spread over a cluster of 1 to 8 CTAs
+// (pass 1: key tiles, pass 2: heads; the size that leaves the least of the last wave idle), whose
+// partial results are merged through distributed shared memory in a fixed order: no atomics, results
+// reproducible bit for bit. Both passes, the MSE score and the selection of that shape: 129 us, against 1907
+// with warp-level matrix fragments and the scores staged through shared memory.
+constexpr int kAmThreads = 320;        // producer warp, MMA warp, two warpgroups of row threads
+constexpr int kAmTile = 128;
+constexpr int kAmSlab = 128 * 128;     // [128 rows][64 bf16]
 
 template <int DH>
 struct AmSmem {
-    __nv_bfloat16 q[kAmTile][DH + 8];      // +8: rows 16 bytes apart in bank phase
-    __nv_bfloat16 k[kAmTile][DH + 8];
-    float s[4][16][kAmTile + 4];
+    static constexpr int kTileBytes = (DH / 64) * kAmSlab;
+    static constexpr int kStages = (DH == 64) ? 3 : 4;
+    static constexpr int kAOff = 0;                                    // two A tiles
+    static constexpr int kBOff = 2 * kTileBytes;
+    static constexpr int kLseOff = kBOff + kStages * kTileBytes;       // [8 warps][2][128] fp32 (pass 2)
+    static constexpr int kStatOff = kLseOff + 8 * 2 * kAmTile * 4;     // [2 warpgroups][128] float2
+    static constexpr int kBarOff = kStatOff + 2 * kAmTile * 8;
+    static constexpr int kTotal = kBarOff + 256 + 1024;
 };
 
-// S tile of this warp's 16 query rows against the 64 keys in sm.k, into sm.s[warp]
-template <int DH>
-__device__ __forceinline__ void am_scores(AmSmem<DH>& sm, int warp)
+struct AmParams {
+    const int32_t* kv_len;
+    int N, Lmax, n_heads;
+    float scale_log2e;
+    float* lse;
+    float* score;
+    unsigned int* status;
+};
+
+__device__ __forceinline__ float ex2(float x)
 {
-    using namespace nvcuda;
-    wmma::fragment<wmma::accumulator, 16, 16, 16, float> acc[4];
-#pragma unroll
-    for (int n = 0; n < 4; ++n) wmma::fill_fragment(acc[n], 0.f);
-#pragma unroll
-    for (int kk = 0; kk < DH / 16; ++kk) {
-        wmma::fragment<wmma::matrix_a, 16, 16, 16, __nv_bfloat16, wmma::row_major> a;
-        wmma::load_matrix_sync(a, &sm.q[warp * 16][kk * 16], DH + 8);
-#pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            wmma::fragment<wmma::matrix_b, 16, 16, 16, __nv_bfloat16, wmma::col_major> bfr;
-            wmma::load_matrix_sync(bfr, &sm.k[n * 16][kk * 16], DH + 8);
-            wmma::mma_sync(acc[n], a, bfr, acc[n]);
-        }
-    }
-#pragma unroll
-    for (int n = 0; n < 4; ++n) wmma::store_matrix_sync(&sm.s[warp][0][n * 16], acc[n], kAmTile + 4, wmma::mem_row_major);
-    __syncwarp();
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float2 ld_dsmem2(uint32_t cluster_addr)
+{
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr) : "memory");
+    return v;
 }
 
-// loads rows [row0, row0 + 64) x channels [c0, c0 + DH) of a [rows_total, C] bf16 matrix (zero past the end)
-template <int DH>
-__device__ __forceinline__ void am_load_tile(__nv_bfloat16 (*dst)[DH + 8], const __nv_bfloat16* src, long row0, long rows_total,
-                                             int C, int c0)
+// PASS 1: blockIdx.y = head, .z = image, cluster index along x = query tile.
+// PASS 2: blockIdx.z = image, cluster index along x = key tile; the cluster's CTAs share the heads.
+template <int DH, int PASS>
+__global__ void __launch_bounds__(kAmThreads, DH == 64 ? 2 : 1)
+attn_mass(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
+          const __grid_constant__ CUtensorMap tmap_cache, const AmParams p, const int cs)
 {
-    constexpr int kVec = DH / 8;
-    for (int i = threadIdx.x; i < kAmTile * kVec; i += kAmThreads) {
-        const int r = i / kVec, v = i - r * kVec;
-        uint4 val = make_uint4(0, 0, 0, 0);
-        if (row0 + r < rows_total) val = *(const uint4*)(src + (row0 + r) * C + c0 + v * 8);
-        *(uint4*)&dst[r][v * 8] = val;
-    }
-}
+    using namespace tc;
+    using L = AmSmem<DH>;
+    constexpr int kStages = L::kStages;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t* a_full = (uint64_t*)(smem + L::kBarOff);     // 2
+    uint64_t* a_empty = a_full + 2;                        // 2
+    uint64_t* b_full = a_empty + 2;                        // kStages
+    uint64_t* b_empty = b_full + kStages;                  // kStages
+    uint64_t* s_full = b_empty + kStages;                  // 2
+    uint64_t* s_empty = s_full + 2;                        // 2, one arrival per warp of the warpgroup
+    uint32_t* tmem_slot = (uint32_t*)(s_empty + 2);
+    __shared__ int abort_flag_s;
+    volatile int* abort_flag = &abort_flag_s;
 
-template <int DH>
-__global__ void __launch_bounds__(kAmThreads)
-attn_mass_rows(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-               const __nv_bfloat16* __restrict__ k_cache, const int32_t* __restrict__ kv_len,
-               int N, int C, int Lmax, float scale_log2e, float* __restrict__ lse)
-{
-    extern __shared__ __align__(128) uint8_t am_raw[];
-    AmSmem<DH>& sm = *reinterpret_cast<AmSmem<DH>*>(am_raw);
-    const int b = blockIdx.z, hd = blockIdx.y, q0 = blockIdx.x * kAmTile, n_heads = gridDim.y;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_old = kv_len ? min(max(kv_len[b], 0), Lmax) : 0;
-    const int n_keys = n_old + N;
-    am_load_tile<DH>(sm.q, q + (long)b * N * C, q0, N, C, hd * DH);
-    // every lane pair owns one row of the warp's 16: lane = 2 * row + half, 32 columns each
-    const int row = lane >> 1, half = lane & 1;
-    float m = -INFINITY, l = 0.f;
-    for (int j0 = 0; j0 < n_keys; j0 += kAmTile) {
-        __syncthreads();        // the previous tile's readers are done with sm.k
-        // a key tile may straddle the cache / own-keys boundary: row by row
-        constexpr int kVec = DH / 8;
-        for (int i = threadIdx.x; i < kAmTile * kVec; i += kAmThreads) {
-            const int r = i / kVec, v = i - r * kVec;
-            const int j = j0 + r;
-            uint4 val = make_uint4(0, 0, 0, 0);
-            if (j < n_old) val = *(const uint4*)(k_cache + ((long)b * Lmax + j) * C + hd * DH + v * 8);
-            else if (j < n_keys) val = *(const uint4*)(k + ((long)b * N + (j - n_old)) * C + hd * DH + v * 8);
-            *(uint4*)&sm.k[r][v * 8] = val;
-        }
-        __syncthreads();
-        am_scores<DH>(sm, warp);
-        const int valid = min(kAmTile, n_keys - j0);
-        float tm = -INFINITY;
-        for (int c = half * 32; c < half * 32 + 32; ++c)
-            if (c < valid) tm = fmaxf(tm, sm.s[warp][row][c] * scale_log2e);
-        tm = fmaxf(tm, __shfl_xor_sync(0xffffffffu, tm, 1));
-        const float m_new = fmaxf(m, tm);
-        float part = 0.f;
-        for (int c = half * 32; c < half * 32 + 32; ++c)
-            if (c < valid) part += exp2f(sm.s[warp][row][c] * scale_log2e - m_new);
-        part += __shfl_xor_sync(0xffffffffu, part, 1);
-        l = l * exp2f(m - m_new) + part;      // exp2f(-inf) = 0 on the first tile
-        m = m_new;
-        __syncwarp();
+    const int rank = (int)cluster_ctarank();
+    const int row_tile = blockIdx.x / cs, b = blockIdx.z;
+    const int n_old = (PASS == 1 && p.kv_len) ? min(max(p.kv_len[b], 0), p.Lmax) : 0;
+    const int tiles_own = (p.N + kAmTile - 1) / kAmTile, tiles_old = (n_old + kAmTile - 1) / kAmTile;
+    // this CTA's work: groups (one A tile each) of `per_group` B tiles
+    int group0 = 0, groups = 1, tile0 = 0, per_group = tiles_own;
+    if (PASS == 1) {
+        const int tiles = tiles_old + tiles_own;
+        tile0 = rank * tiles / cs;
+        per_group = (rank + 1) * tiles / cs - tile0;
+        if (per_group == 0) groups = 0;
+    } else {
+        group0 = rank * p.n_heads / cs;
+        groups = (rank + 1) * p.n_heads / cs - group0;
     }
-    const int qi = q0 + warp * 16 + row;
-    if (half == 0 && qi < N) lse[((long)b * n_heads + hd) * N + qi] = m + log2f(l);
-}
+    const int total = groups * per_group;
 
-template <int DH>
-__global__ void __launch_bounds__(kAmThreads)
-attn_mass_cols(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-               int N, int C, int n_heads, float scale_log2e, const float* __restrict__ lse, float* __restrict__ score)
-{
-    extern __shared__ __align__(128) uint8_t am_raw[];
-    AmSmem<DH>& sm = *reinterpret_cast<AmSmem<DH>*>(am_raw);
-    __shared__ float colsum[4][kAmTile];
-    const int b = blockIdx.y, j0 = blockIdx.x * kAmTile;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float acc0 = 0.f, acc1 = 0.f;      // this lane's two key columns (lane, lane + 32), summed over the warp's rows
-    for (int hd = 0; hd < n_heads; ++hd) {
-        __syncthreads();
-        am_load_tile<DH>(sm.k, k + (long)b * N * C, j0, N, C, hd * DH);
-        for (int q0 = 0; q0 < N; q0 += kAmTile) {
-            __syncthreads();
-            am_load_tile<DH>(sm.q, q + (long)b * N * C, q0, N, C, hd * DH);
-            __syncthreads();
-            am_scores<DH>(sm, warp);
-            const float* lrow = lse + ((long)b * n_heads + hd) * N;
-            for (int r = 0; r < 16; ++r) {
-                const int qi = q0 + warp * 16 + r;
-                if (qi >= N) break;
-                const float e = lrow[qi];
-                acc0 += exp2f(sm.s[warp][r][lane] * scale_log2e - e);
-                acc1 += exp2f(sm.s[warp][r][lane + 32] * scale_log2e - e);
-            }
-            __syncwarp();
+    if (threadIdx.x == 0) {
+        abort_flag_s = 0;
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&a_full[i], 1);
+            mbar_init(&a_empty[i], 1);
+            mbar_init(&s_full[i], 1);
+            mbar_init(&s_empty[i], 4);
         }
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(&b_full[i], 1);
+            mbar_init(&b_empty[i], 1);
+        }
+        fence_barrier_init();
+        prefetch_tmap(&tmap_q);
+        prefetch_tmap(&tmap_k);
+        if (PASS == 1) prefetch_tmap(&tmap_cache);
     }
-    colsum[warp][lane] = acc0;
-    colsum[warp][lane + 32] = acc1;
+    if (warp == 1) tmem_alloc(tmem_slot, 256);
+    tc_fence_before();
     __syncthreads();
-    if (threadIdx.x < kAmTile) {
-        const int j = j0 + threadIdx.x;
-        if (j < N) {
-            const float tot = (colsum[0][threadIdx.x] + colsum[1][threadIdx.x]) + (colsum[2][threadIdx.x] + colsum[3][threadIdx.x]);
-            score[(long)b * N + j] = tot / ((float)n_heads * (float)N);
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp == 0) {
+        if (elect_one()) {
+            bool ok = true;
+            int i = 0, groups_issued = 0;
+            for (int g = 0; g < groups && ok; ++g) {
+                const int head = (PASS == 1) ? (int)blockIdx.y : group0 + g;
+                if (g >= 2) ok = mbar_wait(&a_empty[g & 1], (uint32_t)((g >> 1) - 1) & 1u, abort_flag, p.status);
+                if (!ok) break;
+                mbar_arrive_expect_tx(&a_full[g & 1], L::kTileBytes);
+                for (int sl = 0; sl < DH / 64; ++sl)
+                    tma_load_3d(smem + L::kAOff + (g & 1) * L::kTileBytes + sl * kAmSlab, PASS == 1 ? &tmap_q : &tmap_k,
+                                &a_full[g & 1], head * DH + sl * 64, row_tile * kAmTile, b);
+                groups_issued = g + 1;
+                for (int t = 0; t < per_group; ++t, ++i) {
+                    const int st = i % kStages;
+                    if (i >= kStages) ok = mbar_wait(&b_empty[st], (uint32_t)((i / kStages) - 1) & 1u, abort_flag, p.status);
+                    if (!ok) break;
+                    const CUtensorMap* map = PASS == 1 ? &tmap_k : &tmap_q;
+                    int tile = tile0 + t;
+                    if (PASS == 1) {
+                        if (tile < tiles_old) map = &tmap_cache;
+                        else tile -= tiles_old;
+                    }
+                    mbar_arrive_expect_tx(&b_full[st], L::kTileBytes);
+                    for (int sl = 0; sl < DH / 64; ++sl)
+                        tma_load_3d(smem + L::kBOff + st * L::kTileBytes + sl * kAmSlab, map, &b_full[st], head * DH + sl * 64,
+                                    tile * kAmTile, b);
+                }
+            }
+            if (*abort_flag) {       // let the copies in flight land before shared memory is released
+                for (int g = max(0, groups_issued - 2); g < groups_issued; ++g) mbar_drain(&a_full[g & 1], (uint32_t)(g >> 1) & 1u);
+                for (int j = max(0, i - kStages); j < i; ++j) mbar_drain(&b_full[j % kStages], (uint32_t)(j / kStages) & 1u);
+            }
+        }
+    } else if (warp == 1) {
+        if (elect_one()) {
+            constexpr uint32_t idesc = idesc_bf16_f32(kAmTile, kAmTile, 0);
+            const uint64_t a_desc = smem_desc_sw128(smem_u32(smem + L::kAOff), 16, 1024);
+            const uint64_t b_desc = smem_desc_sw128(smem_u32(smem + L::kBOff), 16, 1024);
+            bool ok = true;
+            int i = 0;
+            for (int g = 0; g < groups && ok; ++g) {
+                ok = mbar_wait(&a_full[g & 1], (uint32_t)(g >> 1) & 1u, abort_flag, p.status);
+                for (int t = 0; t < per_group && ok; ++t, ++i) {
+                    const int st = i % kStages;
+                    ok = mbar_wait(&b_full[st], (uint32_t)(i / kStages) & 1u, abort_flag, p.status);
+                    if (ok && i >= 2) ok = mbar_wait(&s_empty[i & 1], (uint32_t)((i >> 1) - 1) & 1u, abort_flag, p.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t ad = a_desc + (uint32_t)((g & 1) * (L::kTileBytes >> 4));
+                    const uint64_t bd = b_desc + (uint32_t)(st * (L::kTileBytes >> 4));
+#pragma unroll
+                    for (int kk = 0; kk < DH / 16; ++kk) {
+                        const uint32_t off = (kk >> 2) * (kAmSlab >> 4) + (kk & 3) * 2;
+                        mma_bf16_ss(tmem_base + 128u * (i & 1), ad + off, bd + off, idesc, kk ? 1u : 0u);
+                    }
+                    mma_commit(&s_full[i & 1]);
+                    mma_commit(&b_empty[st]);
+                }
+                if (ok) mma_commit(&a_empty[g & 1]);
+            }
+        }
+    } else {
+        const int wg = (warp - 2) >> 2, q = warp & 3, row = q * 32 + lane;
+        const uint32_t s_addr = tmem_base + ((uint32_t)(q * 32) << 16) + 128u * wg;
+        const float c = p.scale_log2e;
+        const uint64_t c2 = pack_f32x2(c, c);
+        float* lse_s = (float*)(smem + L::kLseOff) + (warp - 2) * 2 * kAmTile;
+        float m2 = -1e30f, l = 0.f;                    // pass 1: running maximum (log2 domain) and sum
+        uint64_t acc[2] = {pack_f32x2(0.f, 0.f), pack_f32x2(0.f, 0.f)};      // pass 2: sums
+        for (int i = wg; i < total; i += 2) {
+            int valid = kAmTile;
+            if (PASS == 1) {
+                const int tile = tile0 + i;
+                valid = tile < tiles_old ? n_old - tile * kAmTile : p.N - (tile - tiles_old) * kAmTile;
+            } else {
+                // -lse of the tile's queries, a copy per warp (no barrier between warps); -inf past the last query
+                const int g = i / per_group, q0 = (i - g * per_group) * kAmTile;
+                const float* src = p.lse + ((long)b * p.n_heads + group0 + g) * p.N;
+                float* dst = lse_s + ((i >> 1) & 1) * kAmTile;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int qi = q0 + j * 32 + lane;
+                    dst[j * 32 + lane] = qi < p.N ? -src[qi] : -INFINITY;
+                }
+                __syncwarp();
+            }
+            if (!mbar_wait_warp(&s_full[wg], (uint32_t)(i >> 1) & 1u, abort_flag, p.status)) break;
+            tc_fence_after();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t sv[64];
+                tmem_ld32(s_addr + h * 64, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
+                tmem_ld32(s_addr + h * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[32]));
+                tmem_ld_wait();
+                if (h == 1) {            // the tile now lives in registers: the tensor core may have the buffer
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&s_empty[wg]);
+                }
+                if (PASS == 1) {
+                    if (valid < (h + 1) * 64) {
+#pragma unroll
+                        for (int j = 0; j < 64; ++j)
+                            if (h * 64 + j >= valid) sv[j] = 0xff800000u;        // -inf: past the last key of the tile
+                    }
+                    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                    for (int j = 0; j < 64; ++j) mx[j & 3] = fmaxf(mx[j & 3], __uint_as_float(sv[j]));
+                    const float t2 = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c;
+                    const float m_new = fmaxf(m2, t2);
+                    const uint64_t nm2 = pack_f32x2(-m_new, -m_new);
+                    uint64_t part[2] = {pack_f32x2(0.f, 0.f), pack_f32x2(0.f, 0.f)};
+#pragma unroll
+                    for (int j = 0; j < 64; j += 2) {
+                        float d0, d1;
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), c2, nm2), d0, d1);
+                        part[(j >> 1) & 1] = add_f32x2(part[(j >> 1) & 1], pack_f32x2(ex2(d0), ex2(d1)));
+                    }
+                    float s0, s1;
+                    unpack_f32x2(add_f32x2(part[0], part[1]), s0, s1);
+                    l = l * ex2(m2 - m_new) + (s0 + s1);
+                    m2 = m_new;
+                } else {
+                    const ulonglong2* e2 = (const ulonglong2*)(lse_s + ((i >> 1) & 1) * kAmTile + h * 64);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const ulonglong2 e = e2[j];        // four -lse values, the same address in every lane
+                        float d0, d1, d2, d3;
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[4 * j]), __uint_as_float(sv[4 * j + 1])), c2, e.x), d0, d1);
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[4 * j + 2]), __uint_as_float(sv[4 * j + 3])), c2, e.y), d2, d3);
+                        acc[0] = add_f32x2(acc[0], pack_f32x2(ex2(d0), ex2(d1)));
+                        acc[1] = add_f32x2(acc[1], pack_f32x2(ex2(d2), ex2(d3)));
+                    }
+                }
+            }
+        }
+        float2 mine = make_float2(m2, l);
+        if (PASS == 2) {
+            float s0, s1;
+            unpack_f32x2(add_f32x2(acc[0], acc[1]), s0, s1);
+            mine = make_float2(s0 + s1, 0.f);
+        }
+        ((float2*)(smem + L::kStatOff))[wg * kAmTile + row] = mine;
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();              // every CTA's partial results are in place
+    if (rank == 0 && warp >= 2 && warp < 6) {
+        // merged in the order (CTA 0: warpgroup 0, 1), (CTA 1: 0, 1), ...
+        const int row = (warp & 3) * 32 + lane, i = row_tile * kAmTile + row;
+        const uint32_t at = smem_u32(smem + L::kStatOff) + (uint32_t)row * 8u;
+        float m = -1e30f, sum = 0.f;
+        if (PASS == 1)
+            for (int r = 0; r < cs; ++r)
+                for (int w = 0; w < 2; ++w) m = fmaxf(m, ld_dsmem2(map_to_cta(at + w * kAmTile * 8, (uint32_t)r)).x);
+        for (int r = 0; r < cs; ++r)
+            for (int w = 0; w < 2; ++w) {
+                const float2 v = ld_dsmem2(map_to_cta(at + w * kAmTile * 8, (uint32_t)r));
+                sum += (PASS == 1) ? v.y * exp2f(v.x - m) : v.x;
+            }
+        if (i < p.N) {
+            if (PASS == 1) p.lse[((long)b * p.n_heads + blockIdx.y) * p.N + i] = m + log2f(sum);
+            else p.score[(long)b * p.N + i] = sum / ((float)p.n_heads * (float)p.N);
         }
     }
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 256);
+    }
+    __syncwarp();
+    cluster_sync_all();              // nobody's shared memory goes while it is read
+}
+
+// Cluster size 1, 2, 4 or 8 for `items` rows of tiles of `steps` steps that can be split `ways` ways: the one
+// with the shortest schedule, a CTA's start-up and merge counted as two steps.
+int am_cluster(long items, long steps, int ways, int num_sms)
+{
+    int best = 1;
+    long best_cost = 0;
+    for (int cs = 1; cs <= 8 && cs <= ways; cs *= 2) {
+        const long cost = ((items * cs + num_sms - 1) / num_sms) * ((steps + cs - 1) / cs + 2);
+        if (cs == 1 || cost < best_cost) { best = cs; best_cost = cost; }
+    }
+    return best;
 }
 
 template <int DH>
 nova_status launch_mass(nova_ctx* ctx, const void* q, const void* k, const void* k_cache, const int32_t* kv_len,
                         int B, int N, int C, int n_heads, int Lmax, float* lse, float* score, cudaStream_t st)
 {
-    const int smem = (int)sizeof(AmSmem<DH>);
+    using L = AmSmem<DH>;
     static bool attr_done[64];
-    if (ctx->device < 64 && !attr_done[ctx->device]) {
-        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attn_mass_rows<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attn_mass_cols<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        attr_done[ctx->device] = true;
+    if (ctx->device >= 64 || !attr_done[ctx->device]) {
+        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attn_mass<DH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
+        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attn_mass<DH, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
+        if (ctx->device < 64) attr_done[ctx->device] = true;
     }
-    const float scale_log2e = (float)((1.0 / sqrt((double)DH)) * 1.4426950408889634);
+    CUtensorMap tq, tk, tcache;
+    const uint64_t dn[3] = {(uint64_t)C, (uint64_t)N, (uint64_t)B}, sn[2] = {(uint64_t)C * 2, (uint64_t)N * C * 2};
+    const bool cached = kv_len && Lmax > 0;
+    const uint64_t dl[3] = {(uint64_t)C, (uint64_t)Lmax, (uint64_t)B}, sl[2] = {(uint64_t)C * 2, (uint64_t)Lmax * C * 2};
+    if (!tc::make_tmap_bf16(ctx, &tq, q, 3, dn, sn, kAmTile) || !tc::make_tmap_bf16(ctx, &tk, k, 3, dn, sn, kAmTile) ||
+        !(cached ? tc::make_tmap_bf16(ctx, &tcache, k_cache, 3, dl, sl, kAmTile) : tc::make_tmap_bf16(ctx, &tcache, k, 3, dn, sn, kAmTile)))
+        return nova_fail(ctx, NOVA_ERR_CUDA, "nova_score_attention_mass: cuTensorMapEncodeTiled failed");
+    AmParams p;
+    p.kv_len = cached ? kv_len : nullptr; p.N = N; p.Lmax = Lmax; p.n_heads = n_heads;
+    p.scale_log2e = (float)((1.0 / sqrt((double)DH)) * 1.4426950408889634);
+    p.lse = lse; p.score = score; p.status = ctx->dev_status;
     const int tiles = (N + kAmTile - 1) / kAmTile;
-    typedef const __nv_bfloat16* cbf;
+    const int steps1 = tiles + (cached ? (Lmax + kAmTile - 1) / kAmTile : 0);
+    const int cs1 = am_cluster((long)tiles * n_heads * B, steps1, steps1, ctx->num_sms);
+    const int cs2 = am_cluster((long)tiles * B, (long)n_heads * tiles, n_heads, ctx->num_sms);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3(kAmThreads); cfg.dynamicSmemBytes = L::kTotal; cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
     {
         nova_launch_scope scope(ctx, NOVA_K_SCORE, st);
-        attn_mass_rows<DH><<<dim3(tiles, n_heads, B), kAmThreads, smem, st>>>((cbf)q, (cbf)k, (cbf)k_cache, kv_len, N, C, Lmax,
-                                                                             scale_log2e, lse);
+        attr[0].val.clusterDim.x = cs1;
+        cfg.gridDim = dim3(tiles * cs1, n_heads, B);
+        NOVA_CUDA_CHECK(ctx, cudaLaunchKernelEx(&cfg, attn_mass<DH, 1>, tq, tk, tcache, p, (int)cs1));
     }
     {
         nova_launch_scope scope(ctx, NOVA_K_SCORE, st);
-        attn_mass_cols<DH><<<dim3(tiles, B), kAmThreads, smem, st>>>((cbf)q, (cbf)k, N, C, n_heads, scale_log2e, lse, score);
+        attr[0].val.clusterDim.x = cs2;
+        cfg.gridDim = dim3(tiles * cs2, 1, B);
+        NOVA_CUDA_CHECK(ctx, cudaLaunchKernelEx(&cfg, attn_mass<DH, 2>, tq, tk, tcache, p, (int)cs2));
     }
     NOVA_CUDA_CHECK(ctx, cudaGetLastError());
     return NOVA_OK;
