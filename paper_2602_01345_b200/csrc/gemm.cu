@@ -1,18 +1,16 @@
 // out[M, N] = epilogue(A[M, K] * W[N, K]^T + bias) on the sm_100a tensor cores.
 //
-// Both operands are K-major bf16, so one TMA box of 64 K-elements (128 bytes, 128-byte
-// swizzle) per row feeds tcgen05.mma directly. One CTA computes one 128 x BN output tile:
-//   warp 0      TMA producer: fills a ring of kStages {A tile, W tile} buffers
-//   warp 1      allocates TMEM, issues tcgen05.mma (one elected thread), commits to mbarriers
-//   warps 2-5   epilogue: tcgen05.ld the fp32 accumulator (one row per thread), add bias,
-//               apply GELU / residual / QKV routing, store bf16
-// Large problems run on a second kernel, gemm_bf16_tn_pair: a persistent grid of CTA pairs
-// (clusters of two, tcgen05 cta_group::2), each pair computing 256 x BN tiles. Per tensor-core
-// instruction each CTA supplies only its 128 rows of A and BN/2 rows of W, which halves the
-// shared-memory and L2 traffic per flop of the single-CTA tile; the fp32 accumulator is double
-// buffered in tensor memory so that the epilogue of tile i overlaps the main loop of tile i+1, and
-// eight epilogue warps (two per tensor-memory lane quarter, alternate column chunks) keep the
-// epilogue shorter than the main loop even with GELU.
+// Both operands are K-major bf16, so one TMA box of 64 K-elements (128 bytes, 128-byte swizzle) per row
+// feeds tcgen05.mma directly. Two kernels, both of CTA pairs (tcgen05 cta_group::2: per instruction each
+// CTA supplies only half of the operand rows, which halves the shared-memory and L2 traffic per flop)
+// with the same warp roles:
+//   warp 0      TMA producer: fills a ring of {A tile, W tile} stages
+//   warp 1      allocates TMEM, issues tcgen05.mma (one elected thread of the leader CTA), commits to mbarriers
+//   warps 2-9   epilogue: the fp32 accumulator from tensor memory, bias, GELU / residual / QKV routing, bf16
+// gemm_bf16_tn_pair takes the larger problems: a persistent grid
+// whose accumulator is double buffered in tensor memory, so that the epilogue of tile i overlaps the main
+// loop of tile i+1, with two epilogue warps per tensor-memory lane quarter (alternate column chunks), which
+// keep the epilogue shorter than the main loop even with GELU. gemm_bf16_split takes the smaller ones.
 // Every mbarrier wait is bounded; on expiry the CTA records a timeout and tears down.
 #include "tc_common.cuh"
 
@@ -20,17 +18,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128;
 constexpr int BK = 64;
-constexpr int kThreads = 192;
-
-template <int BN, int STAGES>
-struct GemmSmem {
-    static constexpr int kABytes = BM * BK * 2;
-    static constexpr int kBBytes = BN * BK * 2;
-    static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kTotal = STAGES * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/;
-};
 
 __device__ __forceinline__ float gelu_tanh(float x)
 {
@@ -54,7 +42,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 struct GemmParams {
     const __nv_bfloat16* bias;
     int M, N, K;
-    int epilogue;
     __nv_bfloat16* out;
     const __nv_bfloat16* res;
     const int32_t* res_row;
@@ -92,212 +79,173 @@ __device__ __forceinline__ void advance_kv_len(const GemmParams& p)
 }
 
 
-// Epilogue of 32 consecutive accumulator columns [col0, col0 + 32) of output row `row`:
-// + bias, then GELU / residual / QKV routing, rounded to bf16 and stored with 128-bit stores.
-__device__ __forceinline__ void epilogue_chunk(const GemmParams& p, int row, int col0, const uint32_t (&acc)[32],
-                                               long res_base, long kv_base)
+// ---- epilogue: four consecutive features of eight rows per lane ---------------------------------------
+// Both kernels turn their accumulators round in shared memory so that the lanes of a warp hold
+// consecutive features of a few rows: every access to global memory then covers whole sectors of one
+// row, where the tensor-memory layout (one row per thread) would touch 32 rows with every instruction.
+// The eight rows of a lane are worked on together, without a branch between them: one after the other,
+// each row's chain of dependent instructions cost a warp about 400 clocks, and the epilogue of a 256 x 256
+// tile 8.4 us; so it takes 4.0, and a launch of 4096 x 2048 x 2048 27 us instead of 35.
+__device__ __forceinline__ void unpack_bf16x4(uint2 w, float (&v)[4])
 {
-    float v[32];
-    const uint4* bias4 = (const uint4*)(p.bias + col0);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint4 b = bias4[i];
-        const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            v[i * 8 + j * 2] = __uint_as_float(acc[i * 8 + j * 2]) + __uint_as_float(bw[j] << 16);
-            v[i * 8 + j * 2 + 1] = __uint_as_float(acc[i * 8 + j * 2 + 1]) + __uint_as_float(bw[j] & 0xffff0000u);
-        }
-    }
-    __nv_bfloat16* dst;
-    if (p.epilogue == NOVA_EPI_BIAS_GELU) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = gelu_tanh(v[i]);
-        dst = p.out + (long)row * p.N + col0;
-    } else if (p.epilogue == NOVA_EPI_BIAS_RES) {
-        if (p.gate) {
-            // per-image gate of the branch: out = residual + gate * (acc + bias)
-            const uint4* g4 = (const uint4*)(p.gate + (long)p.img_row[row] * p.N + col0);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint4 g = g4[i];
-                const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    v[i * 8 + j * 2] *= __uint_as_float(gw[j] << 16);
-                    v[i * 8 + j * 2 + 1] *= __uint_as_float(gw[j] & 0xffff0000u);
-                }
-            }
-        }
-        const uint4* r4 = (const uint4*)(p.res + res_base + col0);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint4 r = r4[i];
-            const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                v[i * 8 + j * 2] += __uint_as_float(rw[j] << 16);
-                v[i * 8 + j * 2 + 1] += __uint_as_float(rw[j] & 0xffff0000u);
-            }
-        }
-        const long orow = p.out_row ? (long)p.out_row[row] : (long)row;
-        dst = p.out + orow * p.N + col0;
-        if (p.diff_out) {
-            // second output: the stored (bf16-rounded) value minus diff_in's row, i.e. what a separate
-            // pass over the stored output would compute
-            const uint4* x4 = (const uint4*)(p.diff_in + orow * p.N + col0);
-            uint4* c4 = (uint4*)(p.diff_out + orow * p.N + col0);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint4 x = x4[i];
-                const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
-                uint32_t o[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t yb = pack_bf16(v[i * 8 + j * 2], v[i * 8 + j * 2 + 1]);
-                    o[j] = pack_bf16(__uint_as_float(yb << 16) - __uint_as_float(xw[j] << 16),
-                                     __uint_as_float(yb & 0xffff0000u) - __uint_as_float(xw[j] & 0xffff0000u));
-                }
-                c4[i] = make_uint4(o[0], o[1], o[2], o[3]);
-            }
-        }
-    } else {
-        // QKV routing: this 32-column chunk lies entirely in q, k or v (C % 32 == 0)
-        const int which = col0 / p.C, cc = col0 - which * p.C;
-        if (which == 0) dst = p.out + (long)row * p.C + cc;
-        else {
-            if (kv_base < 0) return;   // cache overflow: flagged when the row map was built
-            dst = (which == 1 ? p.k_cache : p.v_cache) + kv_base * p.C + cc;
-        }
-    }
-    uint4* d4 = (uint4*)dst;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        d4[i] = make_uint4(pack_bf16(v[i * 8], v[i * 8 + 1]), pack_bf16(v[i * 8 + 2], v[i * 8 + 3]),
-                           pack_bf16(v[i * 8 + 4], v[i * 8 + 5]), pack_bf16(v[i * 8 + 6], v[i * 8 + 7]));
+    v[0] = __uint_as_float(w.x << 16);
+    v[1] = __uint_as_float(w.x & 0xffff0000u);
+    v[2] = __uint_as_float(w.y << 16);
+    v[3] = __uint_as_float(w.y & 0xffff0000u);
 }
 
-template <int BN, int STAGES>
-__global__ void __launch_bounds__(kThreads)
-gemm_bf16_tn(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
-             const GemmParams p)
-{
-    using L = GemmSmem<BN, STAGES>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t* full_bar = (uint64_t*)(smem + STAGES * L::kStageBytes);
-    uint64_t* empty_bar = full_bar + STAGES;
-    uint64_t* acc_bar = empty_bar + STAGES;
-    uint32_t* tmem_slot = (uint32_t*)(acc_bar + 1);
-    __shared__ int abort_flag_s;
-    volatile int* abort_flag = &abort_flag_s;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int num_kb = p.K / BK;
-    const int M = true_rows(p);
-    if (blockIdx.x == 0 && blockIdx.y == 0) advance_kv_len(p);
-    if (m0 >= M) return;            // whole tile past the device-side row count (nothing allocated yet)
-
-    if (threadIdx.x == 0) {
-        abort_flag_s = 0;
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full_bar[s], 1);
-            mbar_init(&empty_bar[s], 1);
-        }
-        mbar_init(acc_bar, 1);
-        fence_barrier_init();
-        prefetch_tmap(&tmap_a);
-        prefetch_tmap(&tmap_w);
-    }
-    if (warp == 1) tmem_alloc(tmem_slot, BN);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_acc = *tmem_slot;
-
-    if (warp == 0) {
-        if (elect_one()) {
-            int issued = 0;
-            for (int kb = 0; kb < num_kb; ++kb) {
-                const int s = kb % STAGES;
-                if (kb >= STAGES && !mbar_wait(&empty_bar[s], ((kb / STAGES) - 1) & 1, abort_flag, p.status)) break;
-                uint8_t* a_dst = smem + s * L::kStageBytes;
-                uint8_t* b_dst = a_dst + L::kABytes;
-                mbar_arrive_expect_tx(&full_bar[s], L::kStageBytes);
-                tma_load_2d(a_dst, &tmap_a, &full_bar[s], kb * BK, m0);
-                tma_load_2d(b_dst, &tmap_w, &full_bar[s], kb * BK, n0);
-                issued = kb + 1;
-            }
-            if (*abort_flag) {
-                // let the copies already issued land before the CTA's shared memory is released
-                for (int kb = max(0, issued - STAGES); kb < issued; ++kb)
-                    mbar_drain(&full_bar[kb % STAGES], (kb / STAGES) & 1);
-            }
-        }
-    } else if (warp == 1) {
-        if (elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16_f32(BM, BN, 0);
-            bool ok = true;
-            for (int kb = 0; kb < num_kb && ok; ++kb) {
-                const int s = kb % STAGES;
-                ok = mbar_wait(&full_bar[s], (kb / STAGES) & 1, abort_flag, p.status);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t a_addr = smem_u32(smem + s * L::kStageBytes);
-                const uint32_t b_addr = a_addr + L::kABytes;
+// Rows row0 + STEP * i: where each reads its residual (in) and writes (out; -1: nothing to write).
+template <int EPI>
+struct EpiRows {
+    int in[8], out[8];
+    // rows past the last one (row_end) stand in for it when reading and are not written
+    template <int STEP>
+    __device__ __forceinline__ void load(const GemmParams& p, int row0, int row_end)
+    {
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk) {
-                    const uint64_t adesc = smem_desc_sw128(a_addr + kk * 32, 16, 1024);
-                    const uint64_t bdesc = smem_desc_sw128(b_addr + kk * 32, 16, 1024);
-                    mma_bf16_ss(tmem_acc, adesc, bdesc, idesc, (kb | kk) ? 1u : 0u);
-                }
-                mma_commit(&empty_bar[s]);   // frees the stage when these MMAs have read it
+        for (int i = 0; i < 8; ++i) {
+            const int row = min(row0 + STEP * i, row_end - 1);
+            in[i] = out[i] = row;
+            if (EPI == NOVA_EPI_BIAS_RES) {
+                if (p.res_row) in[i] = p.res_row[row];
+                if (p.out_row) out[i] = p.out_row[row];
             }
-            if (ok) mma_commit(acc_bar);     // accumulator complete
-        }
-    } else {
-        // epilogue: warp w may touch TMEM lanes 32*(w%4) .. +31
-        const int q = warp & 3;
-        const int row = m0 + q * 32 + lane;
-        if (mbar_wait_warp(acc_bar, 0, abort_flag, p.status)) {
-            tc_fence_after();
-            const bool row_ok = row < M;
-            long res_base = 0;
-            long kv_base = -1;
-            if (row_ok) {
-                if (p.epilogue == NOVA_EPI_BIAS_RES) res_base = (long)(p.res_row ? p.res_row[row] : row) * p.N;
-                if (p.epilogue == NOVA_EPI_QKV) kv_base = (long)p.kv_row[row];
-            }
-#pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
-                const int col0 = n0 + c * 32;
-                uint32_t acc[32];
-                tmem_ld32(tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32), acc);
-                tmem_ld_wait();
-                if (!row_ok || col0 >= p.N) continue;
-                epilogue_chunk(p, row, col0, acc, res_base, kv_base);
-            }
+            if (EPI == NOVA_EPI_QKV) out[i] = p.kv_row[row];      // -1: cache overflow, flagged when the row map was built
         }
     }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc(tmem_acc, BN);
+};
+// What the epilogue reads of four features of those rows, fetched before the accumulator is ready.
+template <int EPI>
+struct EpiData {
+    uint2 res[8];
+    __device__ __forceinline__ void fetch(const GemmParams& p, const EpiRows<EPI>& r, int col)
+    {
+        if (EPI != NOVA_EPI_BIAS_RES) return;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) res[i] = *(const uint2*)(p.res + (long)r.in[i] * p.N + col);
+    }
+};
+// v = accumulators; + bias, then GELU / residual / QKV routing, rounded to bf16. Features col .. col + 3 of
+// rows row0 + STEP * (FROM + i) < row_end, four of the eight at a time (registers).
+template <int EPI, int STEP, int FROM>
+__device__ __forceinline__ void epi_store(const GemmParams& p, int row0, int row_end, const EpiRows<EPI>& r, int col, uint2 bias,
+                                          const EpiData<EPI>& d, float (&v)[4][4])
+{
+    float t[4];
+    unpack_bf16x4(bias, t);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[i][j] += t[j];
+    uint2 y[4];
+    if (EPI == NOVA_EPI_BIAS_GELU) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[i][j] = gelu_tanh(v[i][j]);
+    }
+    if (EPI == NOVA_EPI_BIAS_RES) {
+        if (p.gate) {
+            // per-image gate of the branch: out = residual + gate * (acc + bias)
+            uint2 g[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                g[i] = *(const uint2*)(p.gate + (long)p.img_row[min(row0 + STEP * (FROM + i), row_end - 1)] * p.N + col);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                unpack_bf16x4(g[i], t);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[i][j] *= t[j];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            unpack_bf16x4(d.res[FROM + i], t);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[i][j] += t[j];
+        }
+    }
+    uint2 diff[4];
+    if (EPI == NOVA_EPI_BIAS_RES && p.diff_out) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) diff[i] = *(const uint2*)(p.diff_in + (long)r.out[FROM + i] * p.N + col);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) y[i] = make_uint2(pack_bf16(v[i][0], v[i][1]), pack_bf16(v[i][2], v[i][3]));
+    if (EPI == NOVA_EPI_QKV) {
+        const int which = col / p.C, cc = col - which * p.C;      // C % 4 == 0: the four lie in one of q, k, v
+        __nv_bfloat16* base = (which == 0 ? p.out : which == 1 ? p.k_cache : p.v_cache) + cc;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int row = row0 + STEP * (FROM + i), dst = which == 0 ? row : r.out[FROM + i];
+            if (row < row_end && dst >= 0) *(uint2*)(base + (long)dst * p.C) = y[i];
+        }
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (row0 + STEP * (FROM + i) < row_end) *(uint2*)(p.out + (long)r.out[FROM + i] * p.N + col) = y[i];
+    if (EPI == NOVA_EPI_BIAS_RES && p.diff_out) {
+        // second output: the stored (bf16-rounded) value minus diff_in's row, i.e. what a separate pass over
+        // the stored output would compute
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float s[4];
+            unpack_bf16x4(diff[i], t);
+            unpack_bf16x4(y[i], s);
+            if (row0 + STEP * (FROM + i) < row_end)
+                *(uint2*)(p.diff_out + (long)r.out[FROM + i] * p.N + col) =
+                    make_uint2(pack_bf16(s[0] - t[0], s[1] - t[1]), pack_bf16(s[2] - t[2], s[3] - t[3]));
+        }
     }
 }
 
 GemmParams make_params(nova_ctx* ctx, const nova_gemm_args& a)
 {
     GemmParams p;
-    p.bias = a.bias; p.M = a.M; p.N = a.N; p.K = a.K; p.epilogue = a.epilogue; p.out = a.out;
+    p.bias = a.bias; p.M = a.M; p.N = a.N; p.K = a.K; p.out = a.out;
     p.res = a.res; p.res_row = a.res_row; p.C = a.C; p.k_cache = a.k_cache; p.v_cache = a.v_cache;
     p.kv_row = a.kv_row; p.status = ctx->dev_status;
     p.adv_cu_keep = a.adv_cu_keep; p.adv_kv_len = a.adv_kv_len; p.adv_B = a.adv_B; p.adv_Lmax = a.adv_Lmax;
     p.ent = a.ent; p.m_dev = a.m_dev; p.gate = a.gate; p.img_row = a.img_row;
     p.out_row = a.out_row; p.diff_in = a.diff_in; p.diff_out = a.diff_out;
     return p;
+}
+
+// ---- which of the two kernels, and how ---------------------------------------------------------------
+// Clusters of 2 and of 4 CTAs that fit the device at the same time.
+struct SplitCaps {
+    int c[2];
+};
+struct SplitPlan {
+    int ls, nt;      // s = 1 << ls
+    bool takes;      // false: the problem is the pair kernel's
+};
+// The plan follows from the true M, N and K alone, on the host and in the kernel alike, so that a launch
+// whose row count only the device knows adds in the same order as one whose row count the host knows.
+// For each s, nt is the smallest token tile with which all tiles run at once; the cheaper s by estimated
+// clocks wins. The constants are fits to launches of 8 to 1600 tokens, 1024 to 8192 features and K from 1024
+// to 8192: a k-block takes its tensor time (2 nt clocks) or the 305 clocks at which a full ring of loads
+// comes in, exchange and epilogue take 40 clocks a token. A four-way split was within 3 % of the two-way
+// one or slower everywhere but at 256 x 1024 x 4096 (10.8 against 11.8 us).
+// Where K need not be split and the token tile would be wider than 192, and where one round of tiles is not
+// enough, the persistent kernel is the faster one (2250 x 1920 x 7680: 43.3 us against 46.3; with tiles
+// of 192 at 1600 x 2048 x 8192 it is 45.3 against 39.0).
+__host__ __device__ inline SplitPlan split_plan(int M, int N, int num_kb, const SplitCaps& caps)
+{
+    const int tiles_n = (N + 255) / 256;
+    SplitPlan best = {0, 256, false};
+    int best_cost = 0;
+    for (int ls = 0; ls < 2 && (1 << ls) <= num_kb; ++ls) {
+        const int tiles_t = caps.c[ls] / tiles_n;
+        if (tiles_t < 1) continue;
+        const int nt = ((M + tiles_t - 1) / tiles_t + 31) & ~31;
+        if (nt > (ls ? 256 : 192)) continue;
+        const int per_kb = 2 * nt > 305 ? 2 * nt : 305;
+        const int cost = ((num_kb + (1 << ls) - 1) >> ls) * per_kb + 40 * nt;
+        if (!best.takes || cost < best_cost) { best.ls = ls; best.nt = nt; best.takes = true; best_cost = cost; }
+    }
+    return best;
 }
 
 // ---- CTA-pair kernel ------------------------------------------------------------------------
@@ -309,7 +257,9 @@ struct PairSmem {
     static constexpr int kABytes = 128 * BK * 2;           // this CTA's 128 rows of A
     static constexpr int kBBytes = (BN / 2) * BK * 2;      // this CTA's half of the W rows
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kTotal = STAGES * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/;
+    static constexpr int kTurnOff = STAGES * kStageBytes;  // per epilogue warp: 32 rows x 32 fp32, for the turn-round
+    static constexpr int kBarOff = kTurnOff + 8 * 4096;
+    static constexpr int kTotal = kBarOff + 256 + 1024 /*alignment slack*/;
 };
 
 // Work list of one launch: entries [0, tiles_full) are whole 256 x BN tiles in column-major tile
@@ -465,21 +415,21 @@ struct EntropyState {
     }
 };
 
-// Role layout as in gemm_bf16_tn. Barriers (all in each CTA's shared memory at equal offsets):
+// Barriers (all in each CTA's shared memory at equal offsets):
 //   full[s]       leader's copy is used: one arrival (its own expect_tx) + the bytes of both CTAs
 //   empty[s]      each CTA's copy, signalled in both CTAs by the leader's tcgen05.commit
 //   acc_full[a]   each CTA's copy, same; a = accumulator buffer of tile parity
 //   acc_empty[a]  leader's copy: one arrival per epilogue warp of both CTAs (16)
-template <int BN, int STAGES>
+template <int BN, int STAGES, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                   const __grid_constant__ CUtensorMap tmap_w_half, const GemmParams p, const int span_host,
-                  const int tiles_full_host, const int num_tiles_host, const int group)
+                  const int tiles_full_host, const int num_tiles_host, const int group, const SplitCaps caps)
 {
     using L = PairSmem<BN, STAGES>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t* full_bar = (uint64_t*)(smem + STAGES * L::kStageBytes);
+    uint64_t* full_bar = (uint64_t*)(smem + L::kBarOff);
     uint64_t* empty_bar = full_bar + STAGES;
     uint64_t* acc_full = empty_bar + STAGES;     // 2
     uint64_t* acc_empty = acc_full + 2;          // 2
@@ -490,6 +440,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();     // 0 = leader
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
+    if (EPI != NOVA_EPI_ENTROPY && p.m_dev && split_plan(true_rows(p), p.N, p.K / BK, caps).takes) return;     // the split kernel's problem
     if (blockIdx.x == 0) advance_kv_len(p);
     const int num_kb = p.K / BK;
     // The work list is the host's, or, when only the device knows the row count, the same plan
@@ -609,9 +560,8 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         // state from chunk to chunk in one thread, so there the second warp of a quarter only
         // signals.)
         const int q = warp & 3;
-        const bool entropy_epi = (p.epilogue == NOVA_EPI_ENTROPY);
-        const int c_first = entropy_epi ? 0 : ((warp - 2) >> 2), c_step = entropy_epi ? 1 : 2;
-        const bool idle_warp = entropy_epi && warp >= 6;
+        const int c_first = (warp - 2) >> 2;
+        const bool idle_warp = (EPI == NOVA_EPI_ENTROPY) && warp >= 6;
         const uint32_t acc_empty_leader = map_to_cta(smem_u32(&acc_empty[0]), 0);
         int local = 0;
         bool ok = true;
@@ -622,32 +572,77 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             if (tile < 0) break;
             const int a = local & 1;
             const PairTile t = decode_tile<BN>(tile, span, tiles_full);
-            const int row = t.m0 + (int)rank * 128 + q * 32 + lane;
+            const int row0 = t.m0 + (int)rank * 128 + q * 32, row = row0 + lane;
             const int n0 = t.n0, n_chunks = t.bn / 32;
-            ok = mbar_wait_warp(&acc_full[a], (uint32_t)(local >> 1) & 1, abort_flag, p.status);
-            if (!ok) break;
-            tc_fence_after();
-            const bool row_ok = row < M;
-            long res_base = 0;
-            long kv_base = -1;
-            if (row_ok) {
-                if (p.epilogue == NOVA_EPI_BIAS_RES) res_base = (long)(p.res_row ? p.res_row[row] : row) * p.N;
-                if (p.epilogue == NOVA_EPI_QKV) kv_base = (long)p.kv_row[row];
-            }
             const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * BN);
+            if constexpr (EPI == NOVA_EPI_ENTROPY) {
+                ok = mbar_wait_warp(&acc_full[a], (uint32_t)(local >> 1) & 1, abort_flag, p.status);
+                if (!ok) break;
+                tc_fence_after();
 #pragma unroll 1
-            for (int c = c_first; c < n_chunks && !idle_warp; c += c_step) {
-                const int col0 = n0 + c * 32;
-                uint32_t acc[32];
-                tmem_ld32(t_addr + (uint32_t)(c * 32), acc);
-                tmem_ld_wait();
-                if (!row_ok || col0 >= p.N) continue;
-                if (p.epilogue == NOVA_EPI_ENTROPY) est.add_chunk(acc, p.bias ? p.bias + col0 : nullptr);
-                else epilogue_chunk(p, row, col0, acc, res_base, kv_base);
+                for (int c = 0; c < n_chunks && !idle_warp; ++c) {
+                    const int col0 = n0 + c * 32;
+                    uint32_t acc[32];
+                    tmem_ld32(t_addr + (uint32_t)(c * 32), acc);
+                    tmem_ld_wait();
+                    if (row < M && col0 < p.N) est.add_chunk(acc, p.bias ? p.bias + col0 : nullptr);
+                }
+            } else {
+                // After the turn-round this lane holds features 4 * (lane % 8) .. + 3 of a chunk's 32, of rows
+                // row0 + lane / 8 + 4 i. What the epilogue reads is fetched two chunks ahead, for the first two
+                // chunks before the accumulator is ready.
+                const int rows0 = row0 + (lane >> 3), col = n0 + c_first * 32 + (lane & 7) * 4;
+                constexpr int kChunks = BN / 64;        // of this warp: alternate ones of the tile's
+                EpiRows<EPI> er;
+                EpiData<EPI> ed[2];
+                uint2 bias[kChunks];
+                if (row0 < M) {
+                    er.template load<4>(p, rows0, M);
+#pragma unroll
+                    for (int c = 0; c < kChunks; ++c)
+                        if (2 * c + c_first < n_chunks && n0 + (2 * c + c_first) * 32 < p.N) {
+                            bias[c] = *(const uint2*)(p.bias + col + c * 64);
+                            if (c < 2) ed[c].fetch(p, er, col + c * 64);
+                        }
+                }
+                ok = mbar_wait_warp(&acc_full[a], (uint32_t)(local >> 1) & 1, abort_flag, p.status);
+                if (!ok) break;
+                tc_fence_after();
+                float* turn = (float*)(smem + L::kTurnOff + (warp - 2) * 4096);
+                if (row0 < M) {
+#pragma unroll
+                    for (int c = 0; c < kChunks; ++c) {
+                        const int ch = 2 * c + c_first;
+                        if (ch >= n_chunks || n0 + ch * 32 >= p.N) break;
+                        uint32_t acc[32];
+                        tmem_ld32(t_addr + (uint32_t)(ch * 32), acc);
+                        tmem_ld_wait();
+                        // 32 rows x 32 fp32, 16-byte pieces XOR-swizzled by the row: no bank conflicts either way
+                        __syncwarp();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            *(uint4*)(turn + lane * 32 + ((i ^ (lane & 7)) << 2)) =
+                                make_uint4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+                        __syncwarp();
+                        float v[4][4];
+                        auto take = [&](int from) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const int rr = (lane >> 3) + 4 * (from + i);
+                                *(float4*)v[i] = *(const float4*)(turn + rr * 32 + (((lane & 7) ^ (rr & 7)) << 2));
+                            }
+                        };
+                        take(0);
+                        epi_store<EPI, 4, 0>(p, rows0, M, er, col + c * 64, bias[c], ed[c & 1], v);
+                        take(4);
+                        epi_store<EPI, 4, 4>(p, rows0, M, er, col + c * 64, bias[c], ed[c & 1], v);
+                        if (c + 2 < kChunks && ch + 4 < n_chunks && n0 + (ch + 4) * 32 < p.N) ed[c & 1].fetch(p, er, col + (c + 2) * 64);
+                    }
+                }
             }
-            if (p.epilogue == NOVA_EPI_ENTROPY && !idle_warp && t.n0 + BN >= p.N) {
+            if (EPI == NOVA_EPI_ENTROPY && !idle_warp && t.n0 + BN >= p.N) {
                 // last column tile of this row block: the row's entropy is complete
-                if (row_ok) p.ent[row] = est.finish(p.status);
+                if (row < M) p.ent[row] = est.finish(p.status);
                 est.reset();
             }
             // this warp has read its part of the buffer: tell the leader's MMA thread
@@ -665,7 +660,13 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     }
 }
 
-template <int BN, int STAGES>
+SplitCaps split_caps(const nova_ctx* ctx)
+{
+    SplitCaps caps = {{ctx->split_clusters[0], ctx->split_clusters[1]}};
+    return caps;
+}
+
+template <int BN, int STAGES, int EPI>
 nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
 {
     using L = PairSmem<BN, STAGES>;
@@ -676,7 +677,7 @@ nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
     if (!make_tmap_bf16(ctx, &ta, a.A, 2, da, sa, 128) || !make_tmap_bf16(ctx, &tw, a.W, 2, dw, sw, BN / 2) ||
         !make_tmap_bf16(ctx, &tw_half, a.W, 2, dw, sw, BN / 4))
         return nova_fail(ctx, NOVA_ERR_CUDA, "gemm: cuTensorMapEncodeTiled failed");
-    auto kern = gemm_bf16_tn_pair<BN, STAGES>;
+    auto kern = gemm_bf16_tn_pair<BN, STAGES, EPI>;
     static bool attr_done[64];
     if (ctx->device < 64 && !attr_done[ctx->device]) {
         NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
@@ -685,7 +686,7 @@ nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
     GemmParams p = make_params(ctx, a);
     const int tiles_m = (a.M + kPairBM - 1) / kPairBM, tiles_n = (a.N + BN - 1) / BN;
     const int tiles = tiles_m * tiles_n;
-    const bool entropy = (a.epilogue == NOVA_EPI_ENTROPY);
+    constexpr bool entropy = (EPI == NOVA_EPI_ENTROPY);
     // the entropy epilogue hands whole row blocks to pairs; otherwise any tile goes to any pair
     const int pairs = min(entropy ? tiles_m : tiles, ctx->num_sms / 2);
     // a last partial wave that would occupy at most half of the pairs runs as half-width tiles
@@ -697,34 +698,300 @@ nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
         // sweep the smaller operand; the entropy epilogue needs the N-fastest order
         const int span = (entropy || (long)a.M >= (long)a.N) ? -tiles_n : tiles_m;
         kern<<<dim3(2 * pairs), kPairThreads, L::kTotal, st>>>(ta, tw, tw_half, p, span, tiles_full, entries,
-                                                           entropy ? tiles_n : 0);
+                                                           entropy ? tiles_n : 0, split_caps(ctx));
     }
     NOVA_CUDA_CHECK(ctx, cudaGetLastError());
     return NOVA_OK;
 }
 
-template <int BN, int STAGES>
-nova_status launch(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
+// ---- split-K kernel for problems that leave SM pairs idle ------------------------------------------
+// With few 256 x 256 tiles a GEMM is bound by latency and by how many SMs pull weights, not by the
+// tensor cores. Here the weights are the M operand: a pair of CTAs computes out^T[256 features, nt tokens], nt
+// a multiple of 32 up to 256, so that few tokens cost little padding, and K is split over s = 1 or 2
+// pairs of one cluster. Each pair sends every other one its share of the tokens of the fp32 partial tile
+// straight into that pair's shared memory (in the ring, which is idle by then) as [part][token][feature];
+// after a cluster barrier each CTA adds up the parts of its tokens, always in the order 0, 1, and
+// runs the epilogue on four consecutive features per lane, with the residual rows fetched before the
+// accumulator was ready. No global scratch, no atomics, nothing that depends on timing.
+// Measured in a graph over cold weights, against the kernel this replaced (one 128 x 128 tile per CTA, three
+// stages, no split): tokens x features x K = 256 x 1024 x 4096 11 us (26), 300 x 2048 x 8192 19 us (61),
+// 300 x 6144 x 2048 14 us (19). Launch, first load, exchange and epilogue are 5 to 7 us of each.
+constexpr int kSplitThreads = 320;     // producer warp, MMA warp, eight epilogue warps
+constexpr int kSplitRing = 192 * 1024;
+constexpr int kSplitSmem = kSplitRing + 1024 /*alignment slack*/ + 256 /*barriers*/;
+constexpr int kSplitMaxStages = 10;
+
+__device__ __forceinline__ void st_shared(uint32_t addr, uint32_t v)
 {
-    using L = GemmSmem<BN, STAGES>;
-    CUtensorMap ta, tw;
-    const uint64_t da[2] = {(uint64_t)a.K, (uint64_t)a.M}, sa[1] = {(uint64_t)a.K * 2};
-    const uint64_t dw[2] = {(uint64_t)a.K, (uint64_t)a.N}, sw[1] = {(uint64_t)a.K * 2};
-    if (!make_tmap_bf16(ctx, &ta, a.A, 2, da, sa, BM) || !make_tmap_bf16(ctx, &tw, a.W, 2, dw, sw, BN))
-        return nova_fail(ctx, NOVA_ERR_CUDA, "gemm: cuTensorMapEncodeTiled failed");
-    auto kern = gemm_bf16_tn<BN, STAGES>;
-    if (!ctx->attr_gemm) {
-        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
-        ctx->attr_gemm = true;
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(uint32_t cluster_addr, uint32_t v)
+{
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+// Barriers as in gemm_bf16_tn_pair (full: the pair leader's copy counts both CTAs' bytes; empty and
+// acc_full: signalled in both CTAs by the leader's commit). A unit of work is one output tile, run by s
+// consecutive pairs of a cluster of pc pairs. Every CTA passes the same cluster barriers whether or not
+// its pair has a unit, also after a failed wait.
+template <int EPI>
+__global__ void __launch_bounds__(kSplitThreads, 1)
+gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
+                const GemmParams p, const int pc, const int box, const SplitPlan plan_host, const SplitCaps caps)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int M = true_rows(p);
+    const int num_kb = p.K / BK;
+    const SplitPlan plan = p.m_dev ? split_plan(M, p.N, num_kb, caps) : plan_host;
+    if (!plan.takes) return;      // the other kernel's problem
+    if (blockIdx.x == 0) advance_kv_len(p);
+    if (M <= 0) return;
+    const int nt = plan.nt, s = 1 << plan.ls;
+    const int tiles_t = (M + nt - 1) / nt;
+    const int units = ((p.N + 255) / 256) * tiles_t;
+
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t* full_bar = (uint64_t*)(smem + kSplitRing);
+    uint64_t* empty_bar = full_bar + kSplitMaxStages;
+    uint64_t* acc_full = empty_bar + kSplitMaxStages;
+    uint32_t* tmem_slot = (uint32_t*)(acc_full + 1);
+    __shared__ int abort_flag_s;
+    volatile int* abort_flag = &abort_flag_s;
+
+    const uint32_t crank = cluster_ctarank();
+    const int r = (int)(crank & 1u), pi = (int)(crank >> 1);          // CTA of the pair, pair of the cluster
+    const uint32_t leader = crank & ~1u;
+    const int groups = pc >> plan.ls, group = pi >> plan.ls, part = pi & (s - 1);   // units of the cluster, mine, my share of K
+    const int num_clusters = gridDim.x / (2 * pc), cluster = blockIdx.x / (2 * pc);
+    const int kb0 = part * num_kb / s, kb1 = (part + 1) * num_kb / s;
+    const int stage_bytes = 16384 + nt * 64;
+    const int stages = min(kSplitMaxStages, kSplitRing / stage_bytes);
+    const int share = nt >> plan.ls;                                  // tokens whose sums this pair completes
+
+    if (threadIdx.x == 0) {
+        abort_flag_s = 0;
+        for (int i = 0; i < stages; ++i) {
+            mbar_init(&full_bar[i], 1);
+            mbar_init(&empty_bar[i], 1);
+        }
+        mbar_init(acc_full, 1);
+        fence_barrier_init();
+        prefetch_tmap(&tmap_w);
+        prefetch_tmap(&tmap_x);
     }
-    GemmParams p = make_params(ctx, a);
-    dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM);
+    if (warp == 1) tmem_alloc_pair(tmem_slot, 256);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    int it0 = 0;                 // k-blocks of the earlier units: position in the ring
+    uint32_t acc_parity = 0;
+    for (int c = cluster; c * groups < units; c += num_clusters, acc_parity ^= 1u, it0 += kb1 - kb0) {
+        const int unit = c * groups + group;
+        const bool active = unit < units;
+        const int f0 = (unit / tiles_t) * 256 + r * 128;              // this CTA's first feature
+        const int t0 = (unit % tiles_t) * nt;                         // the unit's first token
+        // epilogue of this thread: features col .. col + 3 of the tokens first, first + 8, ... < t_end
+        const int col = f0 + lane * 4;
+        const int first = t0 + part * share + warp - 2, t_end = min(t0 + (part + 1) * share, M);
+        EpiRows<EPI> er;
+        EpiData<EPI> ed;
+        uint2 bias = make_uint2(0, 0);
+        if (warp == 0) {
+            if (active && elect_one()) {
+                const uint32_t stage_tx = 2u * (uint32_t)stage_bytes;
+                int issued = it0, stage = it0 % stages;
+                uint32_t phase = (uint32_t)(it0 / stages) & 1u;
+                for (int kb = kb0; kb < kb1; ++kb) {
+                    if (issued >= stages && !mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, p.status)) break;
+                    uint8_t* w_dst = smem + stage * stage_bytes;
+                    uint8_t* x_dst = w_dst + 16384;
+                    if (r == 0) mbar_arrive_expect_tx(&full_bar[stage], stage_tx);
+                    const uint32_t bar = map_to_cta(smem_u32(&full_bar[stage]), leader);
+                    tma_load_2d_pair(w_dst, &tmap_w, bar, kb * BK, f0);
+                    for (int i = 0; i < nt / 2; i += box)
+                        tma_load_2d_pair(x_dst + i * 128, &tmap_x, bar, kb * BK, t0 + r * (nt / 2) + i);
+                    ++issued;
+                    if (++stage == stages) { stage = 0; phase ^= 1u; }
+                }
+                if (*abort_flag && r == 0)      // let the copies already issued land before anything reuses the ring
+                    for (int i = max(0, issued - stages); i < issued; ++i)
+                        mbar_drain(&full_bar[i % stages], (uint32_t)(i / stages) & 1u);
+            }
+        } else if (warp == 1) {
+            if (active && r == 0 && elect_one()) {
+                const uint32_t idesc = idesc_bf16_f32(256, nt, 0);
+                const uint64_t w_desc = smem_desc_sw128(smem_u32(smem), 16, 1024);
+                int stage = it0 % stages;
+                uint32_t phase = (uint32_t)(it0 / stages) & 1u;
+                bool ok = true;
+                for (int kb = kb0; kb < kb1; ++kb) {
+                    ok = mbar_wait(&full_bar[stage], phase, abort_flag, p.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t wd = w_desc + (uint32_t)stage * (uint32_t)(stage_bytes >> 4);
+                    const uint64_t xd = wd + (16384u >> 4);
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk)
+                        mma_bf16_ss_pair(tmem_base, wd + (uint32_t)(kk * 2), xd + (uint32_t)(kk * 2), idesc,
+                                         (kb != kb0 || kk) ? 1u : 0u);
+                    mma_commit_pair(&empty_bar[stage], (uint16_t)(3u << leader));
+                    if (++stage == stages) { stage = 0; phase ^= 1u; }
+                }
+                if (ok) mma_commit_pair(acc_full, (uint16_t)(3u << leader));
+            }
+        } else if (active) {
+            if (col < p.N && first < t_end) {
+                bias = *(const uint2*)(p.bias + col);
+                er.template load<8>(p, first, t_end);
+                ed.fetch(p, er, col);
+            }
+            if (mbar_wait_warp(acc_full, acc_parity, abort_flag, p.status)) tc_fence_after();
+        }
+        __syncwarp();
+        cluster_sync_all();          // every pair's main loop is over: the rings may be written
+        if (warp >= 2 && active) {
+            // token t of this CTA's 128 features (one per lane and tensor-memory lane quarter) to the pair that
+            // completes it; the store of a warp is 128 contiguous bytes
+            const int q = warp & 3;
+            const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+            const uint32_t slot = smem_u32(smem) + (uint32_t)(part * share * 512 + (q * 32 + lane) * 4);
+#pragma unroll 1
+            for (int ch = (warp - 2) >> 2; ch < nt / 32; ch += 2) {
+                uint32_t acc[32];
+                tmem_ld32(t_addr + (uint32_t)(ch * 32), acc);
+                tmem_ld_wait();
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {        // eight tokens always belong to one pair (share % 8 == 0)
+                    const int t = ch * 32 + g * 8, owner = t / share;
+                    const uint32_t off = (uint32_t)((t - owner * share) * 512);
+                    if (owner == part) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) st_shared(slot + off + (uint32_t)(i * 512), acc[g * 8 + i]);
+                    } else {
+                        const uint32_t dst = map_to_cta(slot, (uint32_t)(2 * ((group << plan.ls) + owner) + r)) + off;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) st_cluster(dst + (uint32_t)(i * 512), acc[g * 8 + i]);
+                    }
+                }
+            }
+            tc_fence_before();
+        }
+        __syncwarp();
+        cluster_sync_all();          // every part of this CTA's tokens has arrived
+        if (warp >= 2 && active && col < p.N) {
+            const float* parts = (const float*)smem + lane * 4 - (t0 + part * share) * 128;
+            for (int t = first; t < t_end; t += 64) {
+                float v[4][4];
+                auto take = [&](int from) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) *(float4*)v[i] = *(const float4*)(parts + (t + 8 * (from + i)) * 128);
+                    for (int j = 1; j < s; ++j) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float4 w = *(const float4*)(parts + (j * share + t + 8 * (from + i)) * 128);
+                            v[i][0] += w.x; v[i][1] += w.y; v[i][2] += w.z; v[i][3] += w.w;
+                        }
+                    }
+                };
+                take(0);
+                epi_store<EPI, 8, 0>(p, t, t_end, er, col, bias, ed, v);
+                if (t + 32 < t_end) {
+                    take(4);
+                    epi_store<EPI, 8, 4>(p, t, t_end, er, col, bias, ed, v);
+                }
+                if (t + 64 < t_end) {
+                    er.template load<8>(p, t + 64, t_end);
+                    ed.fetch(p, er, col);
+                }
+            }
+        }
+        fence_proxy_async_smem();    // the next unit's copies overwrite what was written and read here
+        __syncthreads();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();     // a peer's commit may still signal this CTA's barriers
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, 256);
+    }
+}
+
+// Once per context: shared memory opt-in of the split kernel and how many of its clusters fit the device.
+nova_status split_setup(nova_ctx* ctx)
+{
+    if (ctx->split_clusters[0]) return NOVA_OK;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3(kSplitThreads); cfg.dynamicSmemBytes = kSplitSmem; cfg.attrs = attr; cfg.numAttrs = 1;
+    NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(gemm_bf16_split<NOVA_EPI_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem));
+    NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(gemm_bf16_split<NOVA_EPI_BIAS_RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem));
+    NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(gemm_bf16_split<NOVA_EPI_BIAS_GELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem));
+    int n[2] = {0, 0};
+    for (int ls = 0; ls < 2; ++ls) {
+        attr[0].val.clusterDim.x = 2u << ls;
+        cfg.gridDim = dim3(2u << ls);
+        NOVA_CUDA_CHECK(ctx, cudaOccupancyMaxActiveClusters(&n[ls], gemm_bf16_split<NOVA_EPI_BIAS_RES>, &cfg));
+        if (n[ls] < 1) return nova_fail(ctx, NOVA_ERR_CUDA, "gemm: no cluster of the split kernel fits the device");
+    }
+    ctx->split_clusters[1] = n[1];
+    ctx->split_clusters[0] = n[0];
+    return NOVA_OK;
+}
+
+template <int EPI>
+nova_status launch_split(nova_ctx* ctx, const nova_gemm_args& a, const SplitPlan& plan, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3(kSplitThreads); cfg.dynamicSmemBytes = kSplitSmem; cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
+    const SplitCaps caps = split_caps(ctx);
+    const int tiles_n = (a.N + 255) / 256;
+    int pc, box, clusters;
+    if (a.m_dev) {
+        // only the device knows the row count: clusters for the wider split; unsplit tiles run two to a cluster
+        pc = a.K / BK >= 2 ? 2 : 1; box = 16; clusters = caps.c[pc - 1];
+    } else {
+        pc = 1 << plan.ls; box = plan.nt / 2; clusters = tiles_n * ((a.M + plan.nt - 1) / plan.nt);
+    }
+    CUtensorMap tw, tx;
+    const uint64_t dx[2] = {(uint64_t)a.K, (uint64_t)a.M}, sx[1] = {(uint64_t)a.K * 2};
+    const uint64_t dw[2] = {(uint64_t)a.K, (uint64_t)a.N}, sw[1] = {(uint64_t)a.K * 2};
+    if (!make_tmap_bf16(ctx, &tw, a.W, 2, dw, sw, 128) || !make_tmap_bf16(ctx, &tx, a.A, 2, dx, sx, (uint32_t)box))
+        return nova_fail(ctx, NOVA_ERR_CUDA, "gemm: cuTensorMapEncodeTiled failed");
+    const GemmParams p = make_params(ctx, a);
     {
         nova_launch_scope scope(ctx, a.cat, st);
-        kern<<<grid, kThreads, L::kTotal, st>>>(ta, tw, p);
+        attr[0].val.clusterDim.x = 2 * pc;
+        cfg.gridDim = dim3(clusters * 2 * pc);
+        NOVA_CUDA_CHECK(ctx, cudaLaunchKernelEx(&cfg, gemm_bf16_split<EPI>, tw, tx, p, pc, box, plan, caps));
     }
     NOVA_CUDA_CHECK(ctx, cudaGetLastError());
     return NOVA_OK;
+}
+
+template <int EPI>
+nova_status launch_gemm(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
+{
+    // When only the device knows the row count and the bound is past the split kernel's range, both kernels
+    // are launched and the one whose range the true count is not in returns at once.
+    const nova_status rc = split_setup(ctx);
+    if (rc != NOVA_OK) return rc;
+    const SplitPlan plan = split_plan(a.M, a.N, a.K / BK, split_caps(ctx));
+    if (plan.takes || a.m_dev) {
+        const nova_status rs = launch_split<EPI>(ctx, a, plan, st);
+        if (rs != NOVA_OK || plan.takes) return rs;
+    }
+    return launch_pair<256, 6, EPI>(ctx, a, st);
 }
 
 }  // namespace
@@ -733,13 +1000,9 @@ nova_status nova_launch_gemm(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_
 {
     if (a.M <= 0) return NOVA_OK;
     if (a.K % BK || a.N % 32 || a.K < BK) return nova_fail(ctx, NOVA_ERR_SHAPE, "gemm: K must be a multiple of 64 and N of 32");
-    // CTA pairs with 256 x 256 tiles once there is at least one tile per pair of SMs; below that the
-    // single-CTA 128 x 128 tiles spread a small problem over more SMs.
-    const long tiles_pair = (long)((a.M + 255) / 256) * ((a.N + 255) / 256);
-    if (a.epilogue == NOVA_EPI_ENTROPY) {
-        if (ctx->num_sms < 2) return nova_fail(ctx, NOVA_ERR_SHAPE, "gemm: the entropy epilogue needs the CTA-pair kernel");
-        return launch_pair<256, 6>(ctx, a, st);
-    }
-    if (tiles_pair >= ctx->num_sms / 2 && ctx->num_sms >= 2) return launch_pair<256, 6>(ctx, a, st);
-    return launch<128, 3>(ctx, a, st);
+    if (ctx->num_sms < 2) return nova_fail(ctx, NOVA_ERR_SHAPE, "gemm: needs at least two SMs");
+    if (a.epilogue == NOVA_EPI_ENTROPY) return launch_pair<256, 6, NOVA_EPI_ENTROPY>(ctx, a, st);
+    if (a.epilogue == NOVA_EPI_QKV) return launch_gemm<NOVA_EPI_QKV>(ctx, a, st);
+    if (a.epilogue == NOVA_EPI_BIAS_GELU) return launch_gemm<NOVA_EPI_BIAS_GELU>(ctx, a, st);
+    return launch_gemm<NOVA_EPI_BIAS_RES>(ctx, a, st);
 }

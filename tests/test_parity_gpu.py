@@ -669,6 +669,38 @@ def test_block_adaptive_layernorm_identity_equals_plain_block(ctx):
     assert ctx.device_status() == 0
 
 
+@pytest.mark.parametrize("C,heads,F,M", [
+    (320, 5, 960, 1),           # one row; 960 features are not whole 256-feature tiles
+    (256, 2, 2304, 33),         # two token tiles of 32, the second with one row
+    (1024, 16, 1088, 193),      # K split between two CTA pairs; odd rows, features past the last whole tile
+    (256, 2, 2304, 500),        # 72 tiles: more than the clusters of the device-count launch, which go round twice
+    (1024, 16, 4096, 1500),     # rows on both sides of the line between the two GEMM kernels
+])
+def test_block_gemm_tile_edges_host_and_device_count(ctx, C, heads, F, M):
+    """Kept counts at the edges of the GEMMs' token tiles, against the oracle, and the same call with the
+    count left on the device below a larger bound: keys, values and lengths are bit-identical."""
+    N, prior, seed = M + 37, 24, 61
+    _block_case(ctx, B=1, N=N, C=C, heads=heads, F=F, Lmax=prior + N, ks=[M], kv_lens=[prior], seed=seed,
+                rows=None if M < 600 else sorted({0, 31, 32, 255, 256, 1023, M - 1}))
+    wt = nova.BlockWeights(synth.block_weights(C, F, seed, DEV), 1e-6)
+    x = synth.activations(1, N, C, seed + 1, DEV)
+    k0, v0, _ = synth.kv_cache(1, prior + N, prior, C, seed + 2, DEV)
+    keep_idx, _, cu, _ = gpu_select(ctx, torch.rand((1, N), generator=torch.Generator().manual_seed(seed)).to(DEV), [M])
+    got = []
+    for bound in (M, N):
+        k, v, kv_len = k0.clone(), v0.clone(), torch.tensor([prior], dtype=torch.int32, device=DEV)
+        shape = nova.BlockShape(1, N, C, heads, F, prior + N, bound)
+        ctx.ensure_workspace(shape)
+        y = torch.zeros((bound, C), dtype=torch.bfloat16, device=DEV)
+        call = nova.nova_pruned_block_forward if bound == M else nova.nova_pruned_block_forward_device
+        call(ctx, wt, shape, x, keep_idx, cu, k, v, kv_len, True, y)
+        assert ctx.device_status() == 0
+        got.append((y[:M], k, v, kv_len))
+    for a, b in zip(got[0][1:], got[1][1:]):
+        assert torch.equal(a, b)
+    assert _rel_err(f32(got[1][0]), f32(got[0][0])) <= 2.0 ** -7       # attention may split its keys differently
+
+
 def test_block_without_append_leaves_kv_len(ctx):
     B, N, C, heads, F, Lmax = 1, 64, 128, 2, 256, 256
     wt = synth.block_weights(C, F, 1, DEV)
