@@ -176,6 +176,8 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     // reference maximum, sum) in scratch memory and draw a ticket; the one that draws the second
     // ticket finds the other's result complete, merges the two and writes the output. Nobody
     // waits for anybody.
+    pdl_launch_dependents();
+    pdl_wait();
     int units = 0;
     for (int i = 0; i < p.B; ++i) units += (p.cu_keep[i + 1] - p.cu_keep[i] + 2 * BQ - 1) / (2 * BQ);
     const int items = units * p.n_heads;
@@ -765,9 +767,8 @@ nova_status launch(nova_ctx* ctx, const nova_attn_args& a, cudaStream_t st)
     dim3 grid(((a.M + 2 * BQ - 1) / (2 * BQ) + a.B) * a.n_heads + ctx->num_sms / 2);
     {
         nova_launch_scope scope(ctx, NOVA_K_ATTENTION, st);
-        kern<<<grid, kThreads, L::kTotal, st>>>(tq, tk, tv, p);
+        NOVA_CUDA_CHECK(ctx, nova_launch_pdl(kern, grid, dim3(kThreads), L::kTotal, st, 0, tq, tk, tv, p));
     }
-    NOVA_CUDA_CHECK(ctx, cudaGetLastError());
     return NOVA_OK;
 }
 

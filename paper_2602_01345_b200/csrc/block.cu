@@ -59,6 +59,8 @@ layernorm_rows(const uint4* __restrict__ x, const uint4* __restrict__ gamma, con
                float eps, int M, const int32_t* __restrict__ m_dev, int vec_per_row, uint4* __restrict__ out,
                const RowMapArgs maps, const LnModArgs mod)
 {
+    pdl_launch_dependents();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int r = blockIdx.x * kLnWarps + (threadIdx.x >> 5);
     if (m_dev) M = min(M, *m_dev);      // the host knows only an upper bound
@@ -166,6 +168,8 @@ qk_transform_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k
                     const __nv_bfloat16* __restrict__ gain_q, const __nv_bfloat16* __restrict__ gain_k, float eps,
                     const float* __restrict__ rope_cos, const float* __restrict__ rope_sin)
 {
+    pdl_launch_dependents();
+    pdl_wait();
     constexpr int PER = DH / 32;          // 2 or 4 channels per lane
     const int lane = threadIdx.x & 31;
     const long wid = (long)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -262,9 +266,10 @@ static nova_status launch_ln(nova_ctx* ctx, const __nv_bfloat16* x, const RowMap
     const dim3 grid((M + kLnWarps - 1) / kLnWarps), block(kLnWarps * 32);
     RowMapArgs none;
     memset(&none, 0, sizeof(none));
+    cudaError_t le = cudaSuccess;
     nova_launch_scope scope(ctx, NOVA_K_LAYERNORM, st);
 #define NOVA_LN_LAUNCH(V, MAPS, MOD, MAPARG)                                                                     \
-    layernorm_rows<V, MAPS, MOD><<<grid, block, 0, st>>>((const uint4*)x, (const uint4*)g, (const uint4*)b, eps, M, m_dev, vec, (uint4*)out, MAPARG, mod)
+    le = nova_launch_pdl(layernorm_rows<V, MAPS, MOD>, grid, block, 0, st, 0, (const uint4*)x, (const uint4*)g, (const uint4*)b, eps, M, m_dev, vec, (uint4*)out, MAPARG, mod)
 #define NOVA_LN_CASE(V)                                                                                          \
     do {                                                                                                         \
         if (maps && modulated) NOVA_LN_LAUNCH(V, true, true, *maps);                                             \
@@ -281,7 +286,7 @@ static nova_status launch_ln(nova_ctx* ctx, const __nv_bfloat16* x, const RowMap
     else return nova_fail(ctx, NOVA_ERR_SHAPE, "layernorm: C > 8192");
 #undef NOVA_LN_LAUNCH
 #undef NOVA_LN_CASE
-    NOVA_CUDA_CHECK(ctx, cudaGetLastError());
+    NOVA_CUDA_CHECK(ctx, le);
     return NOVA_OK;
 }
 
@@ -381,16 +386,17 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
         const long warps = (long)M * s->n_heads;
         const unsigned blocks = (unsigned)((warps + 7) / 8);
         typedef const float* cfl;
+        cudaError_t qe;
         nova_launch_scope scope(ctx, NOVA_K_LAYERNORM, st);
         if (C / s->n_heads == 64)
-            qk_transform_kernel<64><<<blocks, 256, 0, st>>>(ws.q, (bf)k_cache, ws.kv_row, keep_idx, M, m_dev, C, s->n_heads,
+            qe = nova_launch_pdl(qk_transform_kernel<64>, dim3(blocks), dim3(256), 0, st, 0, ws.q, (bf)k_cache, ws.kv_row, keep_idx, M, m_dev, C, s->n_heads,
                                                           (cbf)ext->qk_gain_q, (cbf)ext->qk_gain_k, ext->qk_eps,
                                                           (cfl)ext->rope_cos, (cfl)ext->rope_sin);
         else
-            qk_transform_kernel<128><<<blocks, 256, 0, st>>>(ws.q, (bf)k_cache, ws.kv_row, keep_idx, M, m_dev, C, s->n_heads,
+            qe = nova_launch_pdl(qk_transform_kernel<128>, dim3(blocks), dim3(256), 0, st, 0, ws.q, (bf)k_cache, ws.kv_row, keep_idx, M, m_dev, C, s->n_heads,
                                                            (cbf)ext->qk_gain_q, (cbf)ext->qk_gain_k, ext->qk_eps,
                                                            (cfl)ext->rope_cos, (cfl)ext->rope_sin);
-        NOVA_CUDA_CHECK(ctx, cudaGetLastError());
+        NOVA_CUDA_CHECK(ctx, qe);
     }
     // o = softmax(q K^T / sqrt(dh)) V
     nova_attn_args a;

@@ -100,6 +100,34 @@ struct nova_launch_scope {
     }
 };
 
+// ---- programmatic dependent launch ---------------------------------------------------------------
+// The kernels of a block are launched with programmatic stream serialisation: each lets the next one start
+// as soon as all of its own CTAs have (pdl_launch_dependents, its first instruction), so that launch, barrier
+// and tensor-memory set-up and the next kernel's first CTAs overlap its tail. A kernel touches memory that
+// earlier launches write only after pdl_wait, which returns when the launch before it has completed with all its
+// writes visible; every CTA passes it, also those with nothing to do, so that completion stays transitive.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Launch with that attribute; cluster_x > 0 adds a cluster dimension (kernels without a compiled-in one).
+template <class... P, class... A>
+static inline cudaError_t nova_launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster_x, A... args)
+{
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (cluster_x > 0) {
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = cluster_x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+    }
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // One NVTX range per C-ABI call (a no-op unless a tool that listens to NVTX is attached).
 struct nova_api_range {
     explicit nova_api_range(const char* name) { nvtxRangePushA(name); }

@@ -440,8 +440,9 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();     // 0 = leader
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
+    pdl_launch_dependents();
+    if (p.m_dev) pdl_wait();        // the row count is an earlier launch's
     if (EPI != NOVA_EPI_ENTROPY && p.m_dev && split_plan(true_rows(p), p.N, p.K / BK, caps).takes) return;     // the split kernel's problem
-    if (blockIdx.x == 0) advance_kv_len(p);
     const int num_kb = p.K / BK;
     // The work list is the host's, or, when only the device knows the row count, the same plan
     // rebuilt here from that count (every thread computes the same values).
@@ -478,6 +479,8 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     cluster_sync_all();                          // both CTAs' barriers exist before either signals the other
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    if (!p.m_dev) pdl_wait();
+    if (blockIdx.x == 0) advance_kv_len(p);
 
     if (warp == 0) {
         if (elect_one()) {
@@ -697,10 +700,9 @@ nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
         nova_launch_scope scope(ctx, a.cat, st);
         // sweep the smaller operand; the entropy epilogue needs the N-fastest order
         const int span = (entropy || (long)a.M >= (long)a.N) ? -tiles_n : tiles_m;
-        kern<<<dim3(2 * pairs), kPairThreads, L::kTotal, st>>>(ta, tw, tw_half, p, span, tiles_full, entries,
-                                                           entropy ? tiles_n : 0, split_caps(ctx));
+        NOVA_CUDA_CHECK(ctx, nova_launch_pdl(kern, dim3(2 * pairs), dim3(kPairThreads), L::kTotal, st, 0, ta, tw, tw_half, p, span,
+                                             tiles_full, entries, entropy ? tiles_n : 0, split_caps(ctx)));
     }
-    NOVA_CUDA_CHECK(ctx, cudaGetLastError());
     return NOVA_OK;
 }
 
@@ -739,12 +741,16 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
                 const GemmParams p, const int pc, const int box, const SplitPlan plan_host, const SplitCaps caps)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_launch_dependents();
+    if (p.m_dev) pdl_wait();        // the row count is an earlier launch's
     const int M = true_rows(p);
     const int num_kb = p.K / BK;
     const SplitPlan plan = p.m_dev ? split_plan(M, p.N, num_kb, caps) : plan_host;
-    if (!plan.takes) return;      // the other kernel's problem
-    if (blockIdx.x == 0) advance_kv_len(p);
-    if (M <= 0) return;
+    if (!plan.takes) return;      // the other kernel's problem (only with a device-side count)
+    if (M <= 0) {
+        if (blockIdx.x == 0) advance_kv_len(p);
+        return;
+    }
     const int nt = plan.nt, s = 1 << plan.ls;
     const int tiles_t = (M + nt - 1) / nt;
     const int units = ((p.N + 255) / 256) * tiles_t;
@@ -785,6 +791,8 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    if (!p.m_dev) pdl_wait();
+    if (blockIdx.x == 0) advance_kv_len(p);
 
     int it0 = 0;                 // k-blocks of the earlier units: position in the ring
     uint32_t acc_parity = 0;
@@ -948,12 +956,6 @@ nova_status split_setup(nova_ctx* ctx)
 template <int EPI>
 nova_status launch_split(nova_ctx* ctx, const nova_gemm_args& a, const SplitPlan& plan, cudaStream_t st)
 {
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(kSplitThreads); cfg.dynamicSmemBytes = kSplitSmem; cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
     const SplitCaps caps = split_caps(ctx);
     const int tiles_n = (a.N + 255) / 256;
     int pc, box, clusters;
@@ -971,11 +973,9 @@ nova_status launch_split(nova_ctx* ctx, const nova_gemm_args& a, const SplitPlan
     const GemmParams p = make_params(ctx, a);
     {
         nova_launch_scope scope(ctx, a.cat, st);
-        attr[0].val.clusterDim.x = 2 * pc;
-        cfg.gridDim = dim3(clusters * 2 * pc);
-        NOVA_CUDA_CHECK(ctx, cudaLaunchKernelEx(&cfg, gemm_bf16_split<EPI>, tw, tx, p, pc, box, plan, caps));
+        NOVA_CUDA_CHECK(ctx, nova_launch_pdl(gemm_bf16_split<EPI>, dim3(clusters * 2 * pc), dim3(kSplitThreads), kSplitSmem, st, 2 * pc,
+                                             tw, tx, p, pc, box, plan, caps));
     }
-    NOVA_CUDA_CHECK(ctx, cudaGetLastError());
     return NOVA_OK;
 }
 

@@ -41,6 +41,8 @@ restore_kernel(const uint4* __restrict__ x_in, const uint4* __restrict__ y_kept,
                int hp, int wp, int h, int w, int vec_per_row, int B, int M, bool m_on_device, bool pruned_only,
                uint4* __restrict__ x_out, uint4* __restrict__ cache_out)
 {
+    pdl_launch_dependents();
+    pdl_wait();
     if (m_on_device) M = cu_keep[B];    // the kept count lives on the device
     const int lane = threadIdx.x & 31;
     // pruned_only: the kept rows were already written (by the block's last epilogue); work items
@@ -162,10 +164,9 @@ static nova_status restore(nova_ctx* ctx, const void* x_in, const void* y_kept,
     if (items == 0) return NOVA_OK;
     const unsigned blocks = (unsigned)((items + kWarpsPerBlock - 1) / kWarpsPerBlock);
     nova_launch_scope scope(ctx, NOVA_K_RESTORE, (cudaStream_t)stream);
-    restore_kernel<<<blocks, kWarpsPerBlock * 32, 0, (cudaStream_t)stream>>>(
-        (const uint4*)x_in, (const uint4*)y_kept, keep_idx, prune_idx, cu_keep, (const uint4*)cache_prev,
-        hp, wp, h, w, C / 8, B, M, m_on_device, pruned_only, (uint4*)x_out, (uint4*)cache_out);
-    NOVA_CUDA_CHECK(ctx, cudaGetLastError());
+    NOVA_CUDA_CHECK(ctx, nova_launch_pdl(
+        restore_kernel, dim3(blocks), dim3(kWarpsPerBlock * 32), 0, (cudaStream_t)stream, 0, (const uint4*)x_in, (const uint4*)y_kept, keep_idx, prune_idx, cu_keep, (const uint4*)cache_prev,
+        hp, wp, h, w, C / 8, B, M, m_on_device, pruned_only, (uint4*)x_out, (uint4*)cache_out));
     return NOVA_OK;
 }
 
