@@ -11,6 +11,7 @@
  *   nova_select_topk        text after Eq. 3 / Eq. 13: keep the highest-entropy tokens
  *   nova_pruned_block_forward   Eq. 14     the layer on the kept tokens only
  *   nova_restore_from_cache     Eq. 15-16  fill pruned rows from the residual cache
+ *   nova_pruned_scale_forward   all of these for the layers of a scale in one call
  *   nova_*_device               the same steps with the keep counts left on the device
  *
  * General rules
@@ -443,6 +444,53 @@ nova_status nova_pruned_layer_forward(nova_ctx* ctx, const nova_block_weights* w
                                       const int32_t* cu_keep, void* k_cache, void* v_cache, int32_t* kv_len,
                                       int append_kv, const void* cache_prev, int hp, int wp, int h, int w_tokens,
                                       void* x_out, void* cache_out, int m_on_device, void* stream);
+
+/* ---- a whole scale in one call ---------------------------------------------------------------- */
+/*
+ * (The paper fixes what is computed, not how the calls are packaged.) Layers first .. first + count - 1
+ * (0-based) of scale t: nova_scale_entropy_layers over their logits, one copy of the means to the host and
+ * one stream synchronisation, nova_keep_ratios_layers on the means of all layers so far,
+ * nova_select_topk_grouped, then nova_pruned_layer_forward layer by layer. Results are those of the single calls. A caller whose logits arrive piece by piece calls it
+ * for a few layers at a time, with x_in = where the previous call left its result: layer j (0-based) writes
+ * x_buf[j & 1], or the other buffer if its input lies there.
+ * With scale_logits the scale's own entropy map (Eq. 7) is taken first and its means complete column t - 1
+ * of hbar_scale; without, all t columns are the caller's.
+ * Host memory: every array of sl, hbar_scale [B, t], keep [L, B] (written), mean_host [L, B] and
+ * scale_mean_host [B] (written; page-locked memory makes the copies asynchronous). Device memory: the
+ * rest, laid out as for the single calls: ent [L, B, N], mean [L, B], keep_idx / prune_idx [L, B*N], cu_keep
+ * [L, B+1], scale_ent [B, N], scale_mean [B]. s->M is ignored; the workspace must hold the largest layer
+ * (B*N rows if nothing better is known). hp, wp: size of every cache_prev map. Errors as for the calls.
+ */
+typedef struct nova_scale_layers {
+    const nova_block_weights* const* weights;
+    const nova_block_modulation* const* modulation;   /* or NULL */
+    const void* const* logits;                        /* [B, N, V] per layer */
+    void* const* k_cache;
+    void* const* v_cache;
+    int32_t* const* kv_len;
+    const void* const* cache_prev;                    /* entries may be NULL where nothing is pruned */
+    void* const* cache_out;                           /* or NULL */
+    int hp, wp;
+} nova_scale_layers;
+
+typedef struct nova_scale_io {
+    const void* scale_logits;                         /* or NULL */
+    float *scale_ent, *scale_mean, *scale_mean_host;
+    nova_dtype logits_dtype;
+    int V;
+    int64_t row_stride;
+    float *ent, *mean, *mean_host;
+    float* hbar_scale;
+    int32_t* keep;
+    int32_t *keep_idx, *prune_idx, *cu_keep;
+    const void* x_in;
+    void* x_buf[2];
+    int h, w;
+} nova_scale_io;
+
+nova_status nova_pruned_scale_forward(nova_ctx* ctx, const nova_scale_layers* sl, const nova_scale_io* io,
+                                      const nova_block_shape* s, const nova_sched_params* p, int t,
+                                      int first, int count, int append_kv, void* stream);
 
 /* ---- the same steps driven from the device: no host value between the calls of a layer ----- */
 /*

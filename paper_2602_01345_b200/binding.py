@@ -597,3 +597,104 @@ def nova_pruned_block_forward_ext(ctx: Context, w: BlockWeights, modulation, ext
         ctx.handle, C.byref(w.c), C.byref(cm) if modulation else None, C.byref(ce), C.byref(c), _ptr(x_in), _ptr(keep_idx),
         _ptr(cu_keep), _ptr(k_cache), _ptr(v_cache), _ptr(kv_len), int(bool(append_kv)), _ptr(y_kept),
         int(bool(m_on_device)), _stream(stream)))
+
+
+# ---- a whole scale in one call -------------------------------------------------------------------------
+class _ScaleLayers(C.Structure):
+    _fields_ = [(n, _vp) for n in ("weights", "modulation", "logits", "k_cache", "v_cache", "kv_len", "cache_prev",
+                                   "cache_out")] + [("hp", _i), ("wp", _i)]
+
+
+class _ScaleIO(C.Structure):
+    _fields_ = ([(n, _vp) for n in ("scale_logits", "scale_ent", "scale_mean", "scale_mean_host")] +
+                [("logits_dtype", _i), ("V", _i), ("row_stride", _i64)] +
+                [(n, _vp) for n in ("ent", "mean", "mean_host", "hbar_scale", "keep", "keep_idx", "prune_idx",
+                                    "cu_keep", "x_in")] + [("x_buf", _vp * 2), ("h", _i), ("w", _i)])
+
+
+_lib.nova_pruned_scale_forward.argtypes = [_vp, C.POINTER(_ScaleLayers), C.POINTER(_ScaleIO), C.POINTER(_BlockShape),
+                                           C.POINTER(_SchedParams), _i, _i, _i, _i, _vp]
+_lib.nova_pruned_scale_forward.restype = _i
+
+
+def modulation_struct(modulation: dict, B: int, C_: int):
+    """The C struct of a modulation dict (names from MODULATION_NAMES to device bf16 [B, C] tensors)."""
+    ptrs = []
+    for n in MODULATION_NAMES:
+        t = modulation.get(n)
+        assert t is None or (t.dtype == torch.bfloat16 and t.shape == (B, C_))
+        ptrs.append(_ptr(t))
+    return _BlockModulation(*ptrs)
+
+
+class ScaleCall:
+    """Arguments of nova_pruned_scale_forward. The buffers given here are the caller's for as long as the
+    object lives; what a caller may exchange between passes goes through set_layers and set_logits, which
+    every pass calls anew."""
+
+    def __init__(self, ctx: Context, shape: BlockShape, h: int, w: int, L: int, ent, mean, mean_host, keep_idx, prune_idx, cu_keep,
+                 x_buf):
+        self.ctx, self.L = ctx, L
+        self.shape = shape._c()
+        self.keep = torch.empty((L, shape.B), dtype=torch.int32)
+        self._tables = [(_vp * L)() for _ in range(8)]
+        self.layers = _ScaleLayers()
+        self.io = _ScaleIO(ent=_ptr(ent), mean=_ptr(mean), mean_host=_ptr(mean_host), keep_idx=_ptr(keep_idx),
+                           prune_idx=_ptr(prune_idx), cu_keep=_ptr(cu_keep), keep=_ptr(self.keep), h=h, w=w)
+        self.io.x_buf[0], self.io.x_buf[1] = _ptr(x_buf[0]), _ptr(x_buf[1])
+        self._buffers = (ent, mean, mean_host, keep_idx, prune_idx, cu_keep, x_buf)
+
+    def set_layers(self, weights, modulation, k_caches, v_caches, kv_len, cache_prev, cache_out):
+        """weights: BlockWeights per layer; modulation: dict per layer or None; kv_len: [L, B] tensor or a
+        tensor [B] per layer; cache_prev: [B, hp, wp, C] per layer or None entries; cache_out per layer or None."""
+        B, Cc = self.shape.B, self.shape.C
+        mods = [modulation_struct(m, B, Cc) for m in modulation] if modulation else None
+        hp, wp = next(((c.shape[1], c.shape[2]) for c in cache_prev if c is not None), (0, 0))
+        tw, tm, _, tk, tv, tl, tp, to = self._tables
+        base, step = (_ptr(kv_len), 4 * B) if isinstance(kv_len, torch.Tensor) else (None, 0)
+        for j in range(self.L):
+            k, v, prev = k_caches[j], v_caches[j], cache_prev[j]
+            assert k.is_contiguous() and v.is_contiguous()
+            tw[j], tk[j], tv[j] = C.addressof(weights[j].c), k.data_ptr(), v.data_ptr()
+            tl[j] = base + j * step if base is not None else kv_len[j].data_ptr()
+            assert prev is None or (prev.shape[1] == hp and prev.shape[2] == wp and prev.is_contiguous())
+            tp[j] = prev.data_ptr() if prev is not None else None
+            if mods is not None:
+                tm[j] = C.addressof(mods[j])
+            if cache_out is not None:
+                to[j] = cache_out[j].data_ptr()
+        self._mods = mods
+        for name, table in zip(("weights", "modulation", "logits", "k_cache", "v_cache", "kv_len", "cache_prev", "cache_out"),
+                               (tw, tm if mods is not None else None, self._tables[2], tk, tv, tl, tp, to if cache_out is not None else None)):
+            setattr(self.layers, name, C.addressof(table) if table is not None else None)
+        self.layers.hp, self.layers.wp = hp, wp
+
+    def set_logits(self, layer_logits):
+        first = layer_logits[0]
+        S, N, V = first.shape
+        assert (S, N) == (self.shape.B, self.shape.N) and len(layer_logits) == self.L
+        stride, dtype = first.stride(), first.dtype
+        assert stride[2] == 1 and stride[0] == N * stride[1]
+        self.io.logits_dtype = {torch.bfloat16: NOVA_BF16, torch.float32: NOVA_F32}[dtype]
+        self.io.V, self.io.row_stride = V, stride[1]
+        table = self._tables[2]
+        for j, t in enumerate(layer_logits):
+            assert t.shape == first.shape and t.dtype == dtype and t.stride() == stride
+            table[j] = t.data_ptr()
+
+    def set_scale_logits(self, scale_logits, ent, mean, mean_host):
+        """The scale's own logits, of the layers' layout; hbar_scale's last column is then written by run."""
+        assert scale_logits.stride(2) == 1 and scale_logits.stride(1) == self.io.row_stride
+        self.io.scale_logits, self.io.scale_ent = scale_logits.data_ptr(), _ptr(ent)
+        self.io.scale_mean, self.io.scale_mean_host = _ptr(mean), _ptr(mean_host)
+        self._scale_buffers = (ent, mean, mean_host)
+
+    def run(self, sched: SchedParams, t: int, hbar_scale, x_in, first: int, count: int, append_kv: bool, stream=None):
+        assert hbar_scale.dtype == torch.float32 and not hbar_scale.is_cuda and hbar_scale.shape == (self.shape.B, t)
+        assert x_in.dtype == torch.bfloat16 and x_in.numel() == self.shape.B * self.shape.N * self.shape.C
+        io = self.io
+        io.hbar_scale, io.x_in = _ptr(hbar_scale), _ptr(x_in)
+        cs = sched._c()
+        self.ctx.check(_lib.nova_pruned_scale_forward(self.ctx.handle, C.byref(self.layers), C.byref(io), C.byref(self.shape),
+                                                      C.byref(cs), t, first, count, int(bool(append_kv)), _stream(stream)))
+        io.scale_logits = None

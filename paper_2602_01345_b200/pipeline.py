@@ -18,7 +18,7 @@ from . import binding as nv
 class PrunedScaleRunner:
     """Buffers and launch sequence for one pruned scale of an L-layer model.
 
-    weights:     list of L dicts of bf16 device tensors (see BlockWeights)
+    weights:     list of L dicts of bf16 device tensors, or of L BlockWeights made from them
     k_caches / v_caches: lists of L tensors [B, Lmax, C]; kv_len: int32 tensor [L, B]
     cache_prev:  list of L tensors [B, hp, wp, C] (previous scale's residual cache per layer)
     """
@@ -28,35 +28,44 @@ class PrunedScaleRunner:
                  modulation=None, fused_restore: bool = False):
         """modulation: optional list of L dicts of per-image [B, C] bf16 tensors (adaptive LayerNorm
         of the class-conditional backbones, see nova_pruned_block_forward_adaln).
-        fused_restore: run each layer as one nova_pruned_layer_forward call (the block's last GEMM
-        scatters the kept rows into x_out / cache_out, the restore pass touches pruned rows only)
-        instead of nova_pruned_block_forward + nova_restore_from_cache; same results."""
+        fused_restore: with a layer_hook or select_ent, run each layer as one nova_pruned_layer_forward call instead of
+        nova_pruned_block_forward + nova_restore_from_cache. The results are bit-identical; otherwise
+        the whole scale is one nova_pruned_scale_forward call either way."""
         self.ctx = ctx
         self.fused_restore = fused_restore
         self.modulation = modulation
         self.L = len(weights)
         self.B, self.h, self.w, self.N = B, h, w, h * w
-        self.C = weights[0]["w_o"].shape[0]
-        self.F = weights[0]["w_fc1"].shape[0]
+        tensors = weights[0].tensors if isinstance(weights[0], nv.BlockWeights) else weights[0]
+        self.C, self.F = tensors["w_o"].shape[0], tensors["w_fc1"].shape[0]
+        dev = self.dev = tensors["w_o"].device
         self.n_heads, self.Lmax = n_heads, Lmax
-        self.weights = [nv.BlockWeights(wt, eps) for wt in weights]
+        self.weights = [wt if isinstance(wt, nv.BlockWeights) else nv.BlockWeights(wt, eps) for wt in weights]
         self.k_caches, self.v_caches, self.kv_len = k_caches, v_caches, kv_len
         self.cache_prev = cache_prev
-        dev = weights[0]["w_o"].device
-        self.dev = dev
-        N, Cc = self.N, self.C
-        self.ent = torch.empty((self.L, B, N), dtype=torch.float32, device=dev)
-        self.mean = torch.empty((self.L, B), dtype=torch.float32, device=dev)
-        self.mean_host = torch.empty((self.L, B), dtype=torch.float32).pin_memory()
-        self.keep_idx = torch.empty((self.L, B * N), dtype=torch.int32, device=dev)      # one list per layer
-        self.prune_idx = torch.empty((self.L, B * N), dtype=torch.int32, device=dev)
-        self.cu_keep = torch.empty((self.L, B + 1), dtype=torch.int32, device=dev)
-        self.y_kept = torch.empty((B * N, Cc), dtype=torch.bfloat16, device=dev)
+        N, Cc, L = self.N, self.C, self.L
+        self.ent = torch.empty((L, B, N), dtype=torch.float32, device=dev)
+        self.mean = torch.empty((L, B), dtype=torch.float32, device=dev)
+        self.mean_host = torch.empty((L, B), dtype=torch.float32, pin_memory=True)
+        self.keep_idx = torch.empty((L, B * N), dtype=torch.int32, device=dev)      # one list per layer
+        self.prune_idx = torch.empty((L, B * N), dtype=torch.int32, device=dev)
+        self.cu_keep = torch.empty((L, B + 1), dtype=torch.int32, device=dev)
+        self._y_kept = None
         self.x_buf = [torch.empty((B, N, Cc), dtype=torch.bfloat16, device=dev) for _ in range(2)]
-        self.cache_out = ([torch.empty((B, N, Cc), dtype=torch.bfloat16, device=dev) for _ in range(self.L)]
+        self.cache_out = (list(torch.empty((L, B, N, Cc), dtype=torch.bfloat16, device=dev).unbind(0))
                           if keep_cache_out else None)
-        ctx.ensure_workspace(nv.BlockShape(B, N, Cc, n_heads, self.F, Lmax, B * N))
+        shape = nv.BlockShape(B, N, Cc, n_heads, self.F, Lmax, B * N)
+        ctx.ensure_workspace(shape)
+        self.call = nv.ScaleCall(ctx, shape, h, w, L, self.ent, self.mean, self.mean_host, self.keep_idx, self.prune_idx,
+                                 self.cu_keep, self.x_buf)
         self.last_keep = None
+
+    @property
+    def y_kept(self):
+        """Compacted block output of the layer-by-layer path (allocated when first asked for)."""
+        if self._y_kept is None:
+            self._y_kept = torch.empty((self.B * self.N, self.C), dtype=torch.bfloat16, device=self.dev)
+        return self._y_kept
 
     def run_scale(self, x_in, layer_logits, sched: nv.SchedParams, t: int, hbar_scale, append_kv: bool = True,
                   stream=None, logits_ready=None, select_ent=None, layer_hook=None):
@@ -71,69 +80,74 @@ class PrunedScaleRunner:
         layer_hook: optional callable(stage, j, info) called with stage "before" / "after" around layer
         j's launches (info: dict of the tensors involved); for tests that compare layer by layer.
         """
-        ctx, B, N = self.ctx, self.B, self.N
         st = stream if stream is not None else torch.cuda.current_stream()
-        # The layers' logits are inputs of the scale, not results of its layers, so the entropy maps
-        # of a whole group of layers are taken first, in one launch, and their means cross to the host
-        # in one copy: one synchronisation per group decides the keep counts of all its layers, and one
-        # more launch selects for all of them. With resident logits the group is the whole scale; while
-        # logits are still being uploaded a small group lets the blocks of the first layers run under
-        # the uploads of the later ones.
+        if layer_hook is not None or select_ent is not None:
+            return self._run_layer_by_layer(x_in, layer_logits, sched, t, hbar_scale, append_kv, st, logits_ready, select_ent,
+                                            layer_hook)
+        # The layers' logits are inputs of the scale, not results of its layers: the entropy maps of a whole
+        # group of layers are taken in one launch, their means cross to the host in one copy, one
+        # synchronisation decides the keep counts of all its layers and one launch selects for them; all of
+        # it and the layers themselves are one native call. With resident logits the group is the whole
+        # scale; while logits are still being uploaded a small group lets the blocks of the first layers
+        # run under the uploads of the later ones.
         group = self.L if logits_ready is None else min(self.L, 4)
-        hbar_layer = torch.zeros((B, self.L), dtype=torch.float32)
-        keeps = []
+        hbar_scale = hbar_scale.to("cpu", torch.float32).contiguous()
+        self.call.set_layers(self.weights, self.modulation, self.k_caches, self.v_caches, self.kv_len, self.cache_prev, self.cache_out)
+        self.call.set_logits(layer_logits)
         x = x_in
         for g0 in range(0, self.L, group):
             g1 = min(self.L, g0 + group)
             if logits_ready is not None:
                 for j in range(g0, g1):
                     st.wait_event(logits_ready[j])
-            nv.nova_scale_entropy_layers(ctx, layer_logits[g0:g1], self.ent[g0:g1], self.mean[g0:g1], stream=st)
-            self.mean_host[g0:g1].copy_(self.mean[g0:g1], non_blocking=True)
-            st.synchronize()
-            hbar_layer[:, g0:g1] = self.mean_host[g0:g1].t()
-            keep_all = nv.nova_keep_ratios_layers(sched, t, N, hbar_scale, hbar_layer[:, :g1])["keep"]
-            if select_ent is None:
-                nv.nova_select_topk_grouped(ctx, self.ent[g0:g1], keep_all[g0:g1], self.keep_idx[g0:g1],
-                                            self.prune_idx[g0:g1], self.cu_keep[g0:g1], None, stream=st)
+            self.call.run(sched, t, hbar_scale, x, g0, g1 - g0, append_kv, st)
             for j in range(g0, g1):
-                keep = keep_all[j]
-                M = int(keep.sum())
-                keeps.append(keep)
-                keep_idx, prune_idx, cu_keep = self.keep_idx[j, :M], self.prune_idx[j, : B * N - M], self.cu_keep[j]
-                if select_ent is not None:
-                    nv.nova_select_topk(ctx, select_ent, keep, keep_idx, prune_idx, cu_keep, None, stream=st)
-                shape = nv.BlockShape(B, N, self.C, self.n_heads, self.F, self.Lmax, M)
-                x_out = self.x_buf[j & 1] if x is not self.x_buf[j & 1] else self.x_buf[(j + 1) & 1]
-                cache_out = self.cache_out[j] if self.cache_out is not None else None
-                if layer_hook is not None:
-                    info = dict(x_in=x, x_out=x_out, cache_out=cache_out, keep=keep, keep_idx=keep_idx, prune_idx=prune_idx,
-                                cu_keep=cu_keep, k_cache=self.k_caches[j], v_cache=self.v_caches[j], kv_len=self.kv_len[j],
-                                cache_prev=self.cache_prev[j], ent=self.ent[j], stream=st)
-                    layer_hook("before", j, info)
-                if self.fused_restore:
-                    nv.nova_pruned_layer_forward(ctx, self.weights[j], self.modulation[j] if self.modulation else None,
-                                                 shape, x, keep_idx, prune_idx, cu_keep, self.k_caches[j],
-                                                 self.v_caches[j], self.kv_len[j], append_kv, self.cache_prev[j],
-                                                 self.h, self.w, x_out, cache_out, stream=st)
-                    if layer_hook is not None:
-                        layer_hook("after", j, info)
-                    x = x_out
-                    continue
-                if self.modulation is None:
-                    nv.nova_pruned_block_forward(ctx, self.weights[j], shape, x, keep_idx, cu_keep,
-                                                 self.k_caches[j], self.v_caches[j], self.kv_len[j], append_kv,
-                                                 self.y_kept[:M], stream=st)
-                else:
-                    nv.nova_pruned_block_forward_adaln(ctx, self.weights[j], self.modulation[j], shape, x,
-                                                       keep_idx, cu_keep, self.k_caches[j],
-                                                       self.v_caches[j], self.kv_len[j], append_kv, self.y_kept[:M],
-                                                       stream=st)
-                nv.nova_restore_from_cache(ctx, x, self.y_kept[:M], keep_idx, prune_idx,
-                                           cu_keep, self.cache_prev[j], self.h, self.w, x_out, cache_out, stream=st)
-                if layer_hook is not None:
-                    layer_hook("after", j, info)
-                x = x_out
+                x = self.x_buf[(j & 1) ^ (x.data_ptr() == self.x_buf[j & 1].data_ptr())]
+        self.last_keep = list(self.call.keep.clone().unbind(0))
+        return x, self.last_keep
+
+    def _run_layer_by_layer(self, x_in, layer_logits, sched, t, hbar_scale, append_kv, st, logits_ready, select_ent, layer_hook):
+        """The same scale call by call, as one nova_pruned_layer_forward (fused_restore) or block + restore
+        per layer, with the hook, if there is one, around every layer."""
+        ctx, B, N, L = self.ctx, self.B, self.N, self.L
+        if logits_ready is not None:
+            for e in logits_ready:
+                st.wait_event(e)
+        nv.nova_scale_entropy_layers(ctx, layer_logits, self.ent, self.mean, stream=st)
+        self.mean_host.copy_(self.mean, non_blocking=True)
+        st.synchronize()
+        keeps = list(nv.nova_keep_ratios_layers(sched, t, N, hbar_scale, self.mean_host.t())["keep"].unbind(0))
+        if select_ent is None:
+            nv.nova_select_topk_grouped(ctx, self.ent, torch.stack(keeps), self.keep_idx, self.prune_idx, self.cu_keep, None, stream=st)
+        x = x_in
+        for j in range(L):
+            keep = keeps[j]
+            M = int(keep.sum())
+            keep_idx, prune_idx, cu_keep = self.keep_idx[j, :M], self.prune_idx[j, : B * N - M], self.cu_keep[j]
+            if select_ent is not None:
+                nv.nova_select_topk(ctx, select_ent, keep, keep_idx, prune_idx, cu_keep, None, stream=st)
+            shape = nv.BlockShape(B, N, self.C, self.n_heads, self.F, self.Lmax, M)
+            x_out = self.x_buf[(j & 1) ^ (x.data_ptr() == self.x_buf[j & 1].data_ptr())]
+            cache_out = self.cache_out[j] if self.cache_out is not None else None
+            info = dict(x_in=x, x_out=x_out, cache_out=cache_out, keep=keep, keep_idx=keep_idx, prune_idx=prune_idx,
+                        cu_keep=cu_keep, k_cache=self.k_caches[j], v_cache=self.v_caches[j], kv_len=self.kv_len[j],
+                        cache_prev=self.cache_prev[j], ent=self.ent[j], stream=st)
+            if layer_hook is not None:
+                layer_hook("before", j, info)
+            mod = self.modulation[j] if self.modulation else None
+            if self.fused_restore:
+                nv.nova_pruned_layer_forward(ctx, self.weights[j], mod, shape, x, keep_idx, prune_idx, cu_keep, self.k_caches[j],
+                                             self.v_caches[j], self.kv_len[j], append_kv, self.cache_prev[j],
+                                             self.h, self.w, x_out, cache_out, stream=st)
+            else:
+                y = self.y_kept[:M]
+                nv.nova_pruned_block_forward_adaln(ctx, self.weights[j], mod, shape, x, keep_idx, cu_keep, self.k_caches[j],
+                                                   self.v_caches[j], self.kv_len[j], append_kv, y, stream=st)
+                nv.nova_restore_from_cache(ctx, x, y, keep_idx, prune_idx, cu_keep, self.cache_prev[j], self.h, self.w, x_out,
+                                           cache_out, stream=st)
+            if layer_hook is not None:
+                layer_hook("after", j, info)
+            x = x_out
         self.last_keep = keeps
         return x, keeps
 
@@ -161,8 +175,9 @@ class MultiScaleRunner:
         self.C = weights[0]["w_o"].shape[0]
         self.Lmax = sum(s * s for s in self.scales)
         dev = weights[0]["w_o"].device
-        self.k_caches = [torch.zeros((B, self.Lmax, self.C), dtype=torch.bfloat16, device=dev) for _ in range(self.L)]
-        self.v_caches = [torch.zeros((B, self.Lmax, self.C), dtype=torch.bfloat16, device=dev) for _ in range(self.L)]
+        self.block_weights = [nv.BlockWeights(wt, eps) for wt in weights]
+        kv = torch.zeros((2 * self.L, B, self.Lmax, self.C), dtype=torch.bfloat16, device=dev).unbind(0)
+        self.k_caches, self.v_caches = list(kv[: self.L]), list(kv[self.L:])
         self.kv_len = torch.zeros((self.L, B), dtype=torch.int32, device=dev)
         self.res_cache = [None] * self.L          # previous scale's residual cache per layer, [B, h, w, C]
         self.hbar_scale = torch.zeros((B, 0), dtype=torch.float32)
@@ -193,13 +208,21 @@ class MultiScaleRunner:
             return x_out, runner.keep, runner
         ent = torch.empty((B, N), dtype=torch.float32, device=x_in.device)
         mean = torch.empty((B,), dtype=torch.float32, device=x_in.device)
-        nv.nova_scale_entropy(self.ctx, scale_logits, ent, mean, stream=st)
-        self.hbar_scale = torch.cat([self.hbar_scale, mean.cpu().view(B, 1)], dim=1)
-        runner = PrunedScaleRunner(self.ctx, self.weights, self.n_heads, B, side, side, self.Lmax, self.k_caches,
+        runner = PrunedScaleRunner(self.ctx, self.block_weights, self.n_heads, B, side, side, self.Lmax, self.k_caches,
                                    self.v_caches, self.kv_len, self.res_cache, eps=self.eps,
                                    fused_restore=self.fused_restore)
-        x_out, keeps = runner.run_scale(x_in, layer_logits, sched, t, self.hbar_scale.contiguous(), stream=st,
-                                        layer_hook=layer_hook)
+        same_layout = layer_hook is None and scale_logits.dtype == layer_logits[0].dtype and \
+            scale_logits.shape == layer_logits[0].shape and scale_logits.stride() == layer_logits[0].stride()
+        if same_layout:
+            # the scale's own map in the same native call: its means complete the history there
+            hbar = torch.cat([self.hbar_scale, torch.zeros((B, 1))], dim=1).contiguous()
+            runner.call.set_logits(layer_logits)
+            runner.call.set_scale_logits(scale_logits, ent, mean, torch.empty((B,), dtype=torch.float32, pin_memory=True))
+        else:
+            nv.nova_scale_entropy(self.ctx, scale_logits, ent, mean, stream=st)
+            hbar = torch.cat([self.hbar_scale, mean.cpu().view(B, 1)], dim=1).contiguous()
+        self.hbar_scale = hbar
+        x_out, keeps = runner.run_scale(x_in, layer_logits, sched, t, hbar, stream=st, layer_hook=layer_hook)
         self.res_cache = [c.view(B, side, side, self.C) for c in runner.cache_out]
         return x_out, keeps, runner
 

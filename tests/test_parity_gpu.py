@@ -1208,6 +1208,45 @@ def test_runners_with_modulation_agree_and_match_oracle(ctx):
     assert _rel_err(f32(host.x_buf[0]), w_x1) <= BLOCK_TOL
 
 
+@pytest.mark.parametrize("L,grouped,modulated", [(1, False, False), (3, False, True), (6, True, False)])
+def test_scale_in_one_call_equals_layer_by_layer(ctx, L, grouped, modulated):
+    """A scale as one native call (also for a few layers at a time, while logits arrive) gives what the single
+    calls give bit for bit: outputs, residual caches, appended keys, lengths, index lists, keep counts."""
+    from paper_2602_01345_b200 import pipeline
+    B, h, w, C, heads, V, prior, t = 2, 9, 7, 256, 4, 1024, 40, 8
+    N = h * w
+    weights = [synth.block_weights(C, 512, 100 + j, DEV) for j in range(L)]
+    prev = [synth.residual_cache(B, 5, 4, C, 70 + j, DEV) for j in range(L)]
+    mods = [_modulation(B, C, 900 + j) for j in range(L)] if modulated else None
+    x_in = synth.activations(B, N, C, 7, DEV)
+    a = synth.smooth_temperature_field(B, h, w, 5, device=DEV)
+    logits = [synth.logits_from_temperature(a * (1 + 0.1 * j), V, 20 + j) for j in range(L)]
+    hbar = torch.linspace(2.0, 7.0, t).repeat(B, 1).contiguous()
+    sched = nova.SchedParams(force_act_scale=t)
+    ready = None
+    if grouped:
+        ready = [torch.cuda.Event() for _ in range(L)]
+        for e in ready:
+            e.record()
+    got = []
+    for hook in (None, lambda stage, j, info: None):
+        ks, vs = [], []
+        for j in range(L):
+            k, v, _ = synth.kv_cache(B, prior + N, prior, C, 50 + 2 * j, DEV)
+            ks.append(k)
+            vs.append(v)
+        kv_len = torch.full((L, B), prior, dtype=torch.int32, device=DEV)
+        r = pipeline.PrunedScaleRunner(ctx, weights, heads, B, h, w, prior + N, ks, vs, kv_len, prev, modulation=mods)
+        x_out, keeps = r.run_scale(x_in, logits, sched, t, hbar, logits_ready=ready, layer_hook=hook)
+        assert ctx.device_status() == 0
+        M = [int(k.sum()) for k in keeps]
+        assert min(M) < B * N
+        got.append([x_out.clone(), torch.stack(keeps), kv_len, r.cu_keep, *ks, *vs, *[c.clone() for c in r.cache_out],
+                    *[r.keep_idx[j, :M[j]] for j in range(L)], *[r.prune_idx[j, :B * N - M[j]] for j in range(L)]])
+    for p, q in zip(*got):
+        assert torch.equal(p, q)
+
+
 def test_selection_on_one_scale_map_gives_nested_sets(ctx):
     """The other reading of how layers get their entropy map: one map per scale, selected on by every
     layer with that layer's keep count. Kept sets of layers with fewer kept tokens are subsets of
