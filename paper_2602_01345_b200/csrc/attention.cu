@@ -1,75 +1,88 @@
 // Attention of the kept queries over [prior-scale K/V cache ++ kept tokens' own K/V]
 // (no mask), on the sm_100a tensor cores.
 //
-// One CTA = 256 query rows (two 128-row tiles A and B) of one image and one head, streaming
-// over 128-key tiles of K and V:
-//   warp 0        TMA producer: Q tiles once, then a ring of K tiles and a ring of V tiles
-//   warps 2-3     idle (they fill the producer/issuer warpgroup, which gives up registers)
-//   warp 1        tcgen05.mma issuer. Per key tile j:  O_A += P_A V_j ; S_A = Q_A K_{j+1}^T ;
-//                 O_B += P_B V_j ; S_B = Q_B K_{j+1}^T.  S and O are fp32 in tensor memory and
-//                 O accumulates there across all key tiles.
-//   warps 4-7     softmax of tile A, one query row per thread: read the row of S from tensor
-//   warps 8-11    memory once, probabilities P = 2^((s - m) * scale) packed to bf16 and stored
-//   (tile B)      back into tensor memory over the S columns, from where the next MMA takes them
-//                 as its A operand. While one tile's softmax runs, the tensor core works on the
-//                 other tile.
-// Probabilities are taken against a reference maximum m fixed at the row's first key tile: bf16
-// and fp32 share their exponent range, so a reference that is not the running maximum costs no
-// precision, and it cancels in the final division by l. Only a score about 2^40 above the
-// reference (seen as a huge row sum) raises it, with O and l rescaled in tensor memory; the row
-// maximum is therefore not computed on the way. K tiles are K-major operands; V tiles are
-// the MN-major B operand, i.e. V is consumed exactly as it lies in the cache ([keys, dh]).
-// MMAs issued by one thread execute in issue order, which orders "P_A read by O_A += P_A V" before
-// "S_A overwritten by the next Q_A K^T" and "O complete" before the next S of the same tile.
-// When the grid's last wave would be less than half full, each of its work items is shared by
-// two CTAs that take half of the key tiles each and merge their partial results (see below).
+// A persistent CTA takes 128 query rows of one image and one head at a time and streams over 128-key tiles
+// of K and V; at head size 128 two CTAs form a pair (cta_group::2) on 256 rows and each brings in half of
+// every tile, because a CTA alone would need 1280 clocks of shared-memory bandwidth per 128 x 128 tile where
+// the tensor core needs 1024. Sixteen warps:
+//   warp 0        TMA producer: Q (two buffers) and a ring of stages {K of a tile, V of the tile three before it}
+//   warp 1        tcgen05.mma issuer (the pair's leader issues for both): O += P_u V_u, then S_{u+3}
+//   warps 4-7     epilogue: O / l to bf16, or a partial result, while the next rows are under way
+//   warps 8-15    softmax, two warpgroups that take the key tiles in turn, one query row per thread: the row of
+//                 S from tensor memory to registers, P = 2^((s - m) * scale) packed to bf16 and stored over the
+//                 S columns, from where O += P V takes it as its A operand
+// Tensor memory holds O and three S buffers, so S runs up to three tiles ahead of O += P V, across the
+// boundary between two work items: neither the latency of a softmax nor its hand-overs are on the tensor
+// core's path as long as a tile's softmax takes less than two tiles of tensor work. (With both 128-row tiles
+// of 256 rows in one CTA there was room for one S buffer each, and S, softmax and P V of a tile followed one
+// another: 3285 clocks per key tile for 2048 clocks of tensor work.)
+// Probabilities are taken against a reference maximum m, the row's maximum over the last 32 keys of its first
+// key tile: bf16 and fp32 share their exponent range, so a reference that is not the running maximum costs no
+// precision, and it cancels in the final division by l. Only a score about 2^80 above the reference (seen as a huge row
+// sum) could get near the end of that range; work items in which one appears are run once more at the
+// end, with a first pass over the keys that finds the rows' true maxima.
+// K tiles are K-major operands; V tiles are the MN-major B operand, i.e. V is consumed exactly as it lies in
+// the cache ([keys, dh]). The last key tile ends at the last key and overlaps the one before it (its repeated
+// columns are masked; rows before the first key read as zeros), so no row past the end is ever loaded.
+// MMAs issued by one thread execute in issue order, which orders "P_u read by O += P_u V" before "its
+// buffer overwritten by S_{u+3}".
+// When the last round of work items would fill at most half of the CTAs (pairs), each of its items is shared
+// by two that take half of the key tiles each and merge their partial results (see below).
 // Every mbarrier wait is bounded.
+// What bounds it: at many keys power (head size 128 runs at 1.6 to 1.7 GHz) and the exponentials: 1340 clocks per
+// key tile of 256 rows for 1024 of tensor work, 1050 without exponentials. In the smallest calls the chain of
+// table, loads, S, softmax, O. Measured against the kernel before it (two tiles of one item in a CTA), us:
+// 3277 rows x 29414 keys, 16 heads x 128: 684 -> 572; 4 x 2048 x 8473: 510 -> 416; 1024 x 7449: 86 -> 52;
+// 300 x 821: 22.8 -> 12.5; 4 x 563 x 1779, 30 heads x 64: 80 -> 55; 2 x 128 x 552, 16 x 64: 11.8 -> 9.2.
 #include "tc_common.cuh"
 
 namespace {
 
 using namespace tc;
 
-constexpr int BQ = 128;        // query rows per tile (two tiles per CTA)
+constexpr int BQ = 128;        // query rows per CTA
 constexpr int BKV = 128;       // keys per tile
-constexpr int kThreads = 384;     // warpgroup 0: producer + MMA issuer (+2 idle warps); 1, 2: softmax of tile A, B
-// setmaxnreg.inc waits until the registers are there, and nothing bounds that wait: the split must
-// leave slack in the 64 K register file (128 * 64 + 256 * 216 = 63488; a split that used all
-// 65536 never got its registers and the kernel hung).
-constexpr int kRegsLow = 64, kRegsHigh = 216;
-static_assert(128 * kRegsLow + 256 * kRegsHigh <= 65536 - 2048, "keep slack for setmaxnreg.inc");
+constexpr int kBufs = 3;       // S buffers in tensor memory
+constexpr int kThreads = 512;  // warpgroups: producer + issuer (+2 idle warps), epilogue, softmax 0, softmax 1
 constexpr int kSlabBytes = 128 * 128;   // [128 rows][64 bf16]
 // A row's sum of probabilities over one key tile at or above this (or NaN) means a score about
-// 2^40 above the row's reference maximum: the reference is raised and O, l rescaled. Far below
-// anything that could overflow fp32 in l or O, far above anything ordinary data reaches.
-constexpr float kHugeSum = 1.0995116e12f;   // 2^40
+// 2^80 above the row's reference maximum. Far below anything that could overflow fp32 in l or O
+// (sums over 2^16 keys, values up to 2^20), far above anything ordinary data reaches.
+constexpr float kHugeSum = 1.2089258e24f;   // 2^80
+// Passes whose row sums and references are kept. A warpgroup that reaches pass i has done its last tile before
+// that, tile t >= i - 2 if passes are single tiles; S of it was issued after O += P V of tile t - kBufs, which
+// waited for the epilogue of the pass before that tile's: passes up to i - kBufs - 3 are done with their slots.
+constexpr int kSlots = kBufs + 3;
 
 template <int DH>
-struct AttnSmem {
-    // K_{j+1} is last read by S = Q K_{j+1}^T in step j, V_j by O += P V_j in the same step, one
-    // softmax after V_j's own scores, so the two rings have different depths and one release (after
-    // the step's last instruction) serves both; head size 128 fills the 227 KB with two Q tiles,
-    // three K stages and two V stages.
-    static constexpr int kKStages = (DH == 64) ? 4 : 3;
-    static constexpr int kVStages = (DH == 64) ? 4 : 2;
-    static constexpr int kSlabs = DH / 64;
-    static constexpr int kTileBytes = kSlabs * kSlabBytes;      // one 128-row Q, K or V tile
-    static constexpr int kQOff = 0;
-    static constexpr int kKOff = 2 * kTileBytes;
-    static constexpr int kVOff = kKOff + kKStages * kTileBytes;
-    static constexpr int kBarOff = kVOff + kVStages * kTileBytes;
+struct AttnCfg {
+    static constexpr bool kPair = (DH == 128);
+    static constexpr int kCtas = kPair ? 2 : 1;
+    static constexpr int kRows = kCtas * BQ;                    // query rows of one work item
+    static constexpr int kKRows = BKV / kCtas;                  // rows of K per CTA (all of dh)
+    static constexpr int kVCols = DH / kCtas;                   // columns of V per CTA (all keys)
+    static constexpr int kQBytes = BQ * DH * 2;
+    static constexpr int kTileBytes = kKRows * DH * 2;          // K and V alike (BKV * kVCols * 2)
+    static constexpr int kStages = kPair ? 4 : 5;               // stage: K of a tile and V of the tile kBufs before it
+    static constexpr int kStageOff = 2 * kQBytes;
+    static constexpr int kLOff = kStageOff + kStages * 2 * kTileBytes;  // [kSlots][2][128] row sums of the two warpgroups
+    static constexpr int kMOff = kLOff + kSlots * 2 * BQ * 4;           // [kSlots][128] reference maxima
+    static constexpr int kAOff = kMOff + kSlots * BQ * 4;               // [2][128] maxima of a maximum pass
+    static constexpr int kTabOff = kAOff + 2 * BQ * 4;                  // [kTable] passes
+    static constexpr int kBarOff = kTabOff + 64 * 44;
     static constexpr int kTotal = kBarOff + 512 + 1024;
+    static_assert(kVCols == 64, "a V stage is one 128-byte-wide slab");
 };
 
 struct AttnParams {
     const int32_t* cu_keep;
     const int32_t* kv_len;
     __nv_bfloat16* o;
-    int B, C, Lmax, n_heads, num_sms;
+    int B, C, Lmax, n_heads, slots;      // slots: CTAs (pairs) that run at the same time
     int own_keys;          // 1: keys = cache rows followed by this call's k_b rows; 0: cache rows only (cross-attention)
     float scale_log2e;     // (1 / sqrt(dh)) * log2(e)
-    // key-split of a last partial wave: per split item two partial results [2][256 rows][DH + 4]
-    // fp32 (unnormalised O row, reference maximum, sum) and a ticket counter; part == NULL: no split
+    // key-split of a last partial round: per split item two partial results [2][kRows][DH + 4] fp32
+    // (unnormalised O row, reference maximum, sum) and a ticket counter per CTA; part == NULL: no split
     float* part;
     unsigned int* tickets;
     int part_slots;
@@ -134,13 +147,14 @@ __device__ __forceinline__ float fmax3(float a, float b, float c)
 // saturate (it evaluates 16 exponentials per clock per SM against 128 multiply-adds). With
 // t = x + 1.5 * 2^23 rounded toward -inf, the low bits of t hold j = floor(x) and f = x - j lies in
 // [0, 1); 2^f comes from a cubic fitted to 9.2e-5 relative error (far below the bf16 rounding the
-// probabilities get next) and j is added to the exponent field as an integer. x is clamped at
-// -126 so that the exponent cannot wrap; a masked (-inf) score therefore yields 2^-126, not 0.
+// probabilities get next) and j is added to the exponent field as an integer. x is clamped to
+// [-126, 126] so that the exponent cannot wrap; a masked (-inf) score therefore yields 2^-126, not 0,
+// and one far above the reference a value that the overflow check sees.
 __device__ __forceinline__ void exp2_poly_x2(uint64_t x2, float& p0, float& p1)
 {
     float x0, x1;
     unpack_f32x2(x2, x0, x1);
-    const uint64_t xc = pack_f32x2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+    const uint64_t xc = pack_f32x2(fminf(fmaxf(x0, -126.f), 126.f), fminf(fmaxf(x1, -126.f), 126.f));
     const uint64_t magic = pack_f32x2(12582912.f, 12582912.f);
     const uint64_t t = add_rm_f32x2(xc, magic);
     const uint64_t f = sub_f32x2(xc, sub_f32x2(t, magic));
@@ -155,416 +169,603 @@ __device__ __forceinline__ void exp2_poly_x2(uint64_t x2, float& p0, float& p1)
     p1 = __uint_as_float(__float_as_uint(q1) + (__float_as_uint(t1) << 23));
 }
 
+// One pass over the keys of a work item. Work items are (head, query block), blocks fastest so that CTAs
+// running together share K/V in L2. All items of an image cost the same, so when the last round of them would
+// occupy at most half of the slots, each of its items becomes two passes, one per half of the keys. Both leave
+// their unnormalised result (O row, reference maximum, sum) in scratch memory and draw a ticket; the one that
+// draws the second ticket finds the other's result complete, merges the two and writes the output. Nobody
+// waits for anybody.
+// The passes of a CTA (pair) are laid out in shared memory, kTable at a time: the roles read what they need of
+// them instead of each carrying the whole state in its few registers.
+constexpr int kTable = 64;
+// Publishing and merging a partial result takes as long as about five key tiles, which halving fewer than twelve
+// would not win back.
+constexpr int kSplitTiles = 12;
+struct Pass {
+    int x;               // first column of the head
+    int b, q_begin, rows_valid;
+    int n;               // key tiles of this pass; 0: nothing to do (but zeros to write if `empty`)
+    int first;           // first key of the first tile
+    int last;            // first key of the last tile (it ends at the image's last key if the pass does)
+    int masked;          // columns of the last tile that repeat keys of the tile before, or precede key 0
+    int half;            // -1, or which half of a split item, + 2 * its slot
+    int empty;
+    int over;            // past the last pass of the launch
+};
+
+// cu, len: cu_keep and kv_len, or copies of them in shared memory.
+template <int DH>
+__device__ __forceinline__ Pass make_pass(const AttnParams& p, const int32_t* cu, const int32_t* len, int entry)
+{
+    constexpr int kRows = AttnCfg<DH>::kRows;
+    Pass r;
+    r.n = 0;
+    r.empty = 0;
+    r.over = 0;
+    int units = 0;
+    for (int i = 0; i < p.B; ++i) units += (cu[i + 1] - cu[i] + kRows - 1) / kRows;
+    const int items = units * p.n_heads, rem = items % p.slots;
+    const bool split = p.part && rem > 0 && 2 * rem <= p.slots && rem <= p.part_slots;
+    const int whole = split ? items - rem : items;
+    if (entry >= whole + 2 * (items - whole)) {
+        r.over = 1;
+        return r;
+    }
+    int item = entry, khalf = -1, slot = 0;
+    if (item >= whole) {
+        slot = (item - whole) >> 1;
+        khalf = (item - whole) & 1;
+        item = whole + slot;
+    }
+    const int head = item / units;
+    int block = item - head * units, k_b = 0;
+    r.x = head * DH;
+    for (r.b = 0; r.b < p.B; ++r.b) {
+        const int c0 = cu[r.b];
+        k_b = cu[r.b + 1] - c0;
+        const int blocks = (k_b + kRows - 1) / kRows;
+        if (block < blocks) { r.q_begin = c0 + block * kRows; break; }
+        block -= blocks;
+    }
+    r.rows_valid = min(kRows, k_b - block * kRows);
+    const int n_keys = min(max(len[r.b], 0) + (p.own_keys ? k_b : 0), p.Lmax);
+    const int tiles = (n_keys + BKV - 1) / BKV;
+    if (khalf >= 0 && tiles < kSplitTiles) {      // too few key tiles to share: the first half takes them all
+        if (khalf == 1) return r;
+        khalf = -1;
+    }
+    const int t0 = khalf == 1 ? (tiles + 1) / 2 : 0, t1 = khalf == 0 ? (tiles + 1) / 2 : tiles;
+    r.n = t1 - t0;
+    r.empty = r.n == 0;
+    r.first = t0 * BKV;
+    r.last = t1 == tiles ? n_keys - BKV : (t1 - 1) * BKV;
+    r.masked = t1 == tiles ? tiles * BKV - n_keys : 0;
+    r.half = khalf < 0 ? -1 : khalf + 2 * slot;
+    return r;
+}
+
 template <int DH>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                  const __grid_constant__ CUtensorMap tmap_v, const AttnParams p)
 {
-    using L = AttnSmem<DH>;
-    constexpr int kSlabs = L::kSlabs;
-    constexpr int kKStages = L::kKStages, kVStages = L::kVStages;
-    constexpr int kIssuers = (DH == 128) ? 2 : 1;     // threads that issue tcgen05.mma (see the issuer code below)
+    using L = AttnCfg<DH>;
+    constexpr bool kPair = L::kPair;
+    constexpr int kStages = L::kStages;
+    // Tensor memory: O (fp32, DH columns) at column 0, S buffer i (fp32) at 128 + 128 i; P (bf16 pairs) over the
+    // first 64 columns of its S buffer.
     constexpr uint32_t kTmemCols = 512;
-    // S tile t (fp32) sits at column 128*t; its first 64 columns are reused for P (bf16 pairs).
-    // O tile t (fp32, DH columns) sits at column 256 + 128*t.
-
-    // ---- which (image, 256-row query block, head) is this CTA? ----------------------------
-    // Work items are (head, query block), blocks fastest so that CTAs running together share K/V
-    // in L2. All items cost the same, so a grid of T items runs in ceil(T / SMs) waves and the last
-    // wave may be nearly empty: when it would fill at most half of the SMs, each of its items is
-    // run by two CTAs, one per half of the keys. Both leave their unnormalised result (O row,
-    // reference maximum, sum) in scratch memory and draw a ticket; the one that draws the second
-    // ticket finds the other's result complete, merges the two and writes the output. Nobody
-    // waits for anybody.
-    pdl_launch_dependents();
-    pdl_wait();
-    int units = 0;
-    for (int i = 0; i < p.B; ++i) units += (p.cu_keep[i + 1] - p.cu_keep[i] + 2 * BQ - 1) / (2 * BQ);
-    const int items = units * p.n_heads;
-    const int rem = items % p.num_sms;
-    const bool split = p.part && rem > 0 && 2 * rem <= p.num_sms && rem <= p.part_slots;
-    const int whole_items = split ? items - rem : items;
-    int item = blockIdx.x, khalf = -1, tail_slot = 0;
-    if (item >= whole_items) {
-        const int h = item - whole_items;
-        item = whole_items + (h >> 1);
-        khalf = h & 1;
-        tail_slot = h >> 1;
-    }
-    if (item >= items) return;
-    const int head = item / units;
-    int slot = item - head * units, b = 0, k_b = 0, q_begin = 0;
-    for (b = 0; b < p.B; ++b) {
-        const int c0 = p.cu_keep[b];
-        k_b = p.cu_keep[b + 1] - c0;
-        const int blocks = (k_b + 2 * BQ - 1) / (2 * BQ);
-        if (slot < blocks) { q_begin = c0 + slot * 2 * BQ; break; }
-        slot -= blocks;
-    }
-    const int rows_valid = min(2 * BQ, k_b - slot * 2 * BQ);
-    const bool tile_b_active = rows_valid > BQ;
-    const int n_keys = min(max(p.kv_len[b], 0) + (p.own_keys ? k_b : 0), p.Lmax);
-    const int n_tiles_all = (n_keys + BKV - 1) / BKV;
-    if (khalf >= 0 && n_tiles_all < 4) {      // too few key tiles to share: the first CTA takes them all
-        if (khalf == 1) return;
-        khalf = -1;
-    }
-    if (n_keys == 0) {
-        // nothing to attend to (cross-attention with no condition tokens): the output rows are zero
-        for (int i = threadIdx.x; i < rows_valid * (DH / 8); i += kThreads) {
-            const int r = i / (DH / 8), v = i - r * (DH / 8);
-            *(uint4*)(p.o + (long)(q_begin + r) * p.C + head * DH + v * 8) = make_uint4(0, 0, 0, 0);
-        }
-        return;
-    }
-    // this CTA's key tiles are jt0 .. jt0 + n_tiles - 1; loops below count j from 0
-    int jt0 = 0, n_tiles = n_tiles_all;
-    if (khalf == 0) n_tiles = (n_tiles_all + 1) / 2;
-    if (khalf == 1) { jt0 = (n_tiles_all + 1) / 2; n_tiles = n_tiles_all - jt0; }
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    // Barriers; at head size 128 those marked * are used in the leader's shared memory and count both CTAs, and
+    // commits signal the others in both.
     uint64_t* bars = (uint64_t*)(smem + L::kBarOff);
-    uint64_t* q_full = bars;                          // 1
-    uint64_t* k_full = bars + 1;                      // kKStages
-    uint64_t* k_empty = k_full + kKStages;            // kKStages
-    uint64_t* v_full = k_empty + kKStages;            // kVStages
-    uint64_t* s_full = v_full + kVStages;             // 2 (tile A, tile B)
-    uint64_t* p_full = s_full + 2;                    // 2, one arrival per softmax warp
-    uint64_t* o_done = p_full + 2;                    // 1, one arrival per issuing thread
-    uint64_t* turn = o_done + 1;                      // 2 counters (not barriers): turns granted to the issuing thread of tile t
-    uint32_t* tmem_slot = (uint32_t*)(turn + 2);
+    uint64_t* q_full = bars;                          // 2 *
+    uint64_t* q_empty = q_full + 2;                   // 2
+    uint64_t* kv_full = q_empty + 2;                  // kStages *
+    uint64_t* kv_empty = kv_full + kStages;           // kStages: everything that reads a stage is done
+    uint64_t* s_full = kv_empty + kStages;            // kBufs: S of a tile is there
+    uint64_t* p_full = s_full + kBufs;                // kBufs *, one arrival per warp of the tile's warpgroup
+    uint64_t* o_full = p_full + kBufs;                // 1
+    uint64_t* o_empty = o_full + 1;                   // 1 *, one arrival per epilogue warp
+    uint64_t* m_full = o_empty + 1;                   // kSlots, one arrival per warp of the first tile's warpgroup
+    uint64_t* l_full = m_full + kSlots;               // kSlots, one arrival per softmax warp
+    uint32_t* tmem_slot = (uint32_t*)(l_full + kSlots);
     __shared__ int abort_flag_s;
     __shared__ int ticket_s;
+    __shared__ unsigned long long redo_s;             // passes of the round in which a row sum was huge in this CTA
+    __shared__ unsigned long long redo_peer_s;        // the same of the pair's other CTA, written by it
+    constexpr int kCuCopy = 64;
+    __shared__ int32_t cu_s[kCuCopy], len_s[kCuCopy];
     volatile int* abort_flag = &abort_flag_s;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = kPair ? cluster_ctarank() : 0u;
+    const int me = kPair ? blockIdx.x >> 1 : blockIdx.x, stride = kPair ? gridDim.x >> 1 : gridDim.x;
 
     if (threadIdx.x == 0) {
         abort_flag_s = 0;
-        mbar_init(q_full, 1);
-        // a K or V stage is free once the issuing thread of every active query tile has committed
-        const int n_issuers = (kIssuers == 2 && tile_b_active) ? 2 : 1;
-        for (int s = 0; s < kKStages; ++s) {
-            mbar_init(&k_full[s], 1);
-            mbar_init(&k_empty[s], n_issuers);
-        }
-        for (int s = 0; s < kVStages; ++s) mbar_init(&v_full[s], 1);
-        for (int t = 0; t < 2; ++t) {
-            mbar_init(&s_full[t], 1);
-            mbar_init(&p_full[t], 4);
-            turn[t] = 0;                              // a plain counter, not a barrier
-        }
-        mbar_init(o_done, n_issuers);
+        redo_s = 0;
+        for (int i = 0; i < 2; ++i) { mbar_init(&q_full[i], 1); mbar_init(&q_empty[i], 1); }
+        for (int i = 0; i < kStages; ++i) { mbar_init(&kv_full[i], 1); mbar_init(&kv_empty[i], 1); }
+        for (int i = 0; i < kBufs; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 4 * L::kCtas); }
+        mbar_init(o_full, 1);
+        mbar_init(o_empty, 4 * L::kCtas);
+        for (int i = 0; i < kSlots; ++i) { mbar_init(&m_full[i], 4); mbar_init(&l_full[i], 8); }
         fence_barrier_init();
         prefetch_tmap(&tmap_q);
         prefetch_tmap(&tmap_k);
         prefetch_tmap(&tmap_v);
     }
-    if (warp == 1) tmem_alloc(tmem_slot, kTmemCols);
+    if (warp == 1) {
+        if constexpr (kPair) tmem_alloc_pair(tmem_slot, kTmemCols);
+        else tmem_alloc(tmem_slot, kTmemCols);
+    }
     tc_fence_before();
     __syncthreads();
+    if constexpr (kPair) cluster_sync_all();         // both CTAs' barriers exist before either signals the other
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
 
-    uint8_t* q_smem = smem + L::kQOff;
-
-    // The softmax warps hold a whole 128-column row of S in registers; the producer and the MMA
-    // issuer need few. Each warpgroup resizes its share of the register file accordingly (the
-    // resize must dominate all of the role's code, hence the nesting).
-    if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLow));
-    if (warp == 0) {
-        if (elect_one()) {
-            const int q_tiles = tile_b_active ? 2 : 1;
-            mbar_arrive_expect_tx(q_full, q_tiles * L::kTileBytes);
-            for (int t = 0; t < q_tiles; ++t)
-                for (int sl = 0; sl < kSlabs; ++sl)
-                    tma_load_2d(q_smem + t * L::kTileBytes + sl * kSlabBytes, &tmap_q, q_full,
-                                head * DH + sl * 64, q_begin + t * BQ);
-            // order of issue = order in which the slots come free: K_j, V_j, K_{j+1}, ...
-            int k_issued = 0, v_issued = 0;
-            for (int j = 0; j < n_tiles; ++j) {
-                const int ks = j % kKStages, vs = j % kVStages;
-                if (j >= kKStages && !mbar_wait(&k_empty[ks], ((j / kKStages) - 1) & 1, abort_flag, p.status)) break;
-                uint8_t* k_dst = smem + L::kKOff + ks * L::kTileBytes;
-                mbar_arrive_expect_tx(&k_full[ks], L::kTileBytes);
-                for (int sl = 0; sl < kSlabs; ++sl)
-                    tma_load_3d(k_dst + sl * kSlabBytes, &tmap_k, &k_full[ks], head * DH + sl * 64, (jt0 + j) * BKV, b);
-                k_issued = j + 1;
-                // The slot of V_j held V_{j-kVStages}, whose last reader is step j-kVStages. That step ends with
-                // S = Q K_{j-kVStages+1}^T, and the commit that releases that K tile (k_empty) follows every
-                // instruction of the step, O += P V included: it releases the V tile as well. (The K slot is
-                // not released again before K_{j-kVStages+1+kKStages} has been loaded, which comes after
-                // this wait since kKStages + 1 > kVStages: the phase waited for cannot be overtaken twice.)
-                static_assert(kKStages + 1 > kVStages, "the K release that stands for the V release must not be overtaken");
-                if (j >= kVStages) {
-                    const int kj = j - kVStages + 1;
-                    if (!mbar_wait(&k_empty[kj % kKStages], (kj / kKStages) & 1, abort_flag, p.status)) break;
-                }
-                uint8_t* v_dst = smem + L::kVOff + vs * L::kTileBytes;
-                mbar_arrive_expect_tx(&v_full[vs], L::kTileBytes);
-                for (int sl = 0; sl < kSlabs; ++sl)
-                    tma_load_3d(v_dst + sl * kSlabBytes, &tmap_v, &v_full[vs], head * DH + sl * 64, (jt0 + j) * BKV, b);
-                v_issued = j + 1;
-            }
-            if (*abort_flag) {
-                mbar_drain(q_full, 0);
-                for (int j = max(0, k_issued - kKStages); j < k_issued; ++j) mbar_drain(&k_full[j % kKStages], (j / kKStages) & 1);
-                for (int j = max(0, v_issued - kVStages); j < v_issued; ++j) mbar_drain(&v_full[j % kVStages], (j / kVStages) & 1);
-            }
+    auto commit = [&](uint64_t* bar) {
+        if constexpr (kPair) mma_commit_pair(bar, 3);
+        else mma_commit(bar);
+    };
+    // arrival of one warp at a barrier of the leader
+    auto arrive_leader = [&](uint64_t* bar) {
+        if (kPair && rank != 0) mbar_arrive_cluster(map_to_cta(smem_u32(bar), 0));
+        else mbar_arrive(bar);
+    };
+    Pass* table = (Pass*)(smem + L::kTabOff);
+    static_assert(kTable * sizeof(Pass) <= 64 * 44, "pass table");
+    // Rounds: up to kTable passes, then, if a row sum in any of them was huge (in either CTA of the pair), those
+    // passes once more with a maximum pass before each; then the next kTable. begin_round lays out the table if
+    // there are passes left; end_of_round gives the passes to run again.
+    auto begin_round = [&](int base) -> bool {
+        if (base > 0 && table[kTable - 1].over) return false;
+        const bool copy = p.B < kCuCopy;
+        if (base == 0 && copy) {
+            if (threadIdx.x <= p.B) cu_s[threadIdx.x] = p.cu_keep[threadIdx.x];
+            else if (threadIdx.x >= 128 && threadIdx.x < 128 + p.B) len_s[threadIdx.x - 128] = p.kv_len[threadIdx.x - 128];
         }
-    } else if (warp == 1 || warp == 2) {
-        // tcgen05.mma issuers. Per key tile j and query tile t one elected thread issues
-        //     O_t += P_t V_j ; S_t = Q_t K_{j+1}^T          (16 instructions at head size 128)
-        // Issuing costs a thread about 80 clocks per instruction in this kernel (more than the 64 an
-        // instruction executes in) and a satisfied barrier wait 65 to 180.
-        if constexpr (kIssuers == 2) {
-            // Head size 128: one thread serving both tiles was itself the limit (its waits and loop
-            // bookkeeping sat between the two tiles' instruction groups), so each tile has its own thread
-            // (warp 1 for tile A, warp 2 for tile B) and all of that happens while the other thread
-            // issues. The two pass a token so that the groups still alternate A, B, A, B: left to
-            // themselves the tiles drift into phase (both softmaxes at once, then both instruction
-            // groups), which is slower than the alternation, where one tile's softmax runs under the
-            // other tile's instructions. The token orders instruction issue only; no data depends on it.
-            const int t = warp - 1;
-            if ((t == 0 || tile_b_active) && elect_one()) {
-                constexpr uint32_t idesc_s = idesc_bf16_f32(BQ, BKV, 0);
-                constexpr uint32_t idesc_o = idesc_bf16_f32(BQ, DH, 1);
-                // Shared-memory descriptors: (address >> 4) sits in the low 14 bits, so stepping through
-                // a tile or to another stage is an integer add.
-                constexpr uint32_t kTileStep = L::kTileBytes >> 4;
-                const uint64_t q_desc = smem_desc_sw128(smem_u32(q_smem), 16, 1024) + (uint32_t)t * kTileStep;
-                const uint64_t k_desc = smem_desc_sw128(smem_u32(smem + L::kKOff), 16, 1024);
-                const uint64_t v_desc = smem_desc_sw128(smem_u32(smem + L::kVOff), kSlabBytes, 1024);
-                const uint32_t s_tmem = tmem_base + 128u * t, o_tmem = tmem_base + 256u + 128u * t;
-                const bool paired = tile_b_active;
-                uint32_t turn_par = 0;
-                // S_t = Q_t K^T with K in stage ks
-                auto issue_s = [&](int ks) {
-                    const uint64_t kd = k_desc + (uint32_t)ks * kTileStep;
-#pragma unroll
-                    for (int kk = 0; kk < DH / 16; ++kk) {
-                        constexpr uint32_t kSlabStep = kSlabBytes >> 4;
-                        const uint32_t off = (kk >> 2) * kSlabStep + (kk & 3) * 2;    // 32 bytes per 16 k
-                        mma_bf16_ss(s_tmem, q_desc + off, kd + off, idesc_s, kk ? 1u : 0u);
+        __syncthreads();
+        if (threadIdx.x < kTable) table[threadIdx.x] = make_pass<DH>(p, copy ? cu_s : p.cu_keep, copy ? len_s : p.kv_len, me + (base + threadIdx.x) * stride);
+        if (threadIdx.x == 0) redo_s = 0;
+        __syncthreads();
+        return true;
+    };
+    auto end_of_round = [&]() -> unsigned long long {
+        __syncwarp();
+        __syncthreads();
+        unsigned long long mask = *(volatile unsigned long long*)&redo_s;
+        if constexpr (kPair) {
+            if (threadIdx.x == 0)
+                asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(map_to_cta(smem_u32(&redo_peer_s), rank ^ 1u)), "l"(mask) : "memory");
+            __syncwarp();
+            cluster_sync_all();
+            mask |= *(volatile unsigned long long*)&redo_peer_s;
+        }
+        return mask;
+    };
+    // next pass to run from index i on (of those in `only`, if that is not 0), kTable if none is left
+    auto next_pass = [&](int i, unsigned long long only) -> int {
+        for (; i < kTable; ++i) {
+            if (table[i].over) return kTable;
+            if (table[i].n > 0 && (!only || ((only >> i) & 1ull))) break;
+        }
+        return i;
+    };
+
+    if (warp < 4) {
+        int st = 0, qb = 0;                            // ring positions
+        uint32_t spar = 0, qpar = 0;                   // and their phase parities
+        int units = 0, qcount = 0;                     // loaded so far (producer)
+        int sbuf = 0, pbuf = 0;                        // S buffer of the next S, of the next P (issuer)
+        uint32_t ppar = 0, opar = 1;
+        bool o_used = false;
+        for (int base = 0; begin_round(base); base += kTable) {
+            unsigned long long only = 0;
+            do {
+                // S runs kBufs tiles ahead of O += P V, across the passes: two cursors over the table
+                int si = next_pass(0, only), s_n = si < kTable ? table[si].n : 0, s_left = s_n, s_passes = only ? 2 : 1;
+                auto s_step = [&]() -> bool {          // past one S tile; true at the end of a pass
+                    if (--s_left) return false;
+                    if (--s_passes == 0) {
+                        si = next_pass(si + 1, only);
+                        s_passes = only ? 2 : 1;
                     }
-                    mma_commit(&s_full[t]);
-                };
-                // O_t (+)= P_t V with V in stage vs; P_t sits in the first 64 columns of S_t, two keys per column
-                auto issue_pv = [&](int vs, bool first) {
-                    const uint64_t vd = v_desc + (uint32_t)vs * kTileStep;
-#pragma unroll
-                    for (int kk = 0; kk < BKV / 16; ++kk)
-                        mma_bf16_ts(o_tmem, s_tmem + kk * 8, vd + (uint32_t)(kk * 128), idesc_o, (first && kk == 0) ? 0u : 1u);
-                };
-                // the token: wait for this tile's turn, hand the turn to the other tile once this tile's
-                // instructions are issued (they execute in the order in which they were issued)
-                // (a counter in shared memory polled with plain loads: the waiting thread has nothing else to
-                // do, and a load comes back several times faster than a suspended barrier wait wakes up)
-                volatile uint32_t* turn_ctr = (volatile uint32_t*)turn;      // [2], zeroed with the barriers
-                auto take_turn = [&]() {
-                    if (!paired) return true;
-                    ++turn_par;                                   // number of the turn this thread waits for
-                    if (turn_ctr[t * 2] >= turn_par) return true;
-                    const unsigned long long t0 = global_ns();
-                    uint32_t spins = 0;
-                    while (turn_ctr[t * 2] < turn_par) {
-                        if ((++spins & 255u) == 0) {
-                            if (*abort_flag) return false;
-                            unsigned long long limit = *(volatile const unsigned long long*)(p.status + NOVA_WAIT_LIMIT_WORD);
-                            if (limit == 0) limit = kWaitLimitNs;
-                            if (global_ns() - t0 > limit) {
-                                *abort_flag = 1;
-                                atomicOr(p.status, NOVA_DEV_TIMEOUT);
-                                return false;
-                            }
-                        }
-                    }
+                    s_n = s_left = si < kTable ? table[si].n : 0;
                     return true;
                 };
-                uint32_t passed = 0;
-                auto pass_turn = [&]() {
-                    if (!paired) return;
-                    turn_ctr[(t ^ 1) * 2] = ++passed;      // no fence: the token orders issue in time, no data hangs on it
-                };
-                bool ok = mbar_wait(q_full, 0, abort_flag, p.status);
-                if (ok) ok = mbar_wait(&k_full[0], 0, abort_flag, p.status);
-                if (ok && t == 1) ok = take_turn();          // tile A goes first
-                if (ok) {
-                    tc_fence_after();
-                    issue_s(0);
-                    mma_commit(&k_empty[0]);
-                    pass_turn();
-                }
-                // ring positions and phase parities, stepped without divisions
-                int vs = 0, ks_next = (kKStages > 1) ? 1 : 0;
-                uint32_t v_par = 0, k_par_next = (kKStages > 1) ? 0u : 1u;
-                for (int j = 0; j < n_tiles && ok; ++j) {
-                    const bool more = j + 1 < n_tiles;
-                    // V_j and K_{j+1} have usually landed long ago; P is what a step waits for
-                    ok = mbar_wait(&v_full[vs], v_par, abort_flag, p.status);
-                    if (ok && more) ok = mbar_wait(&k_full[ks_next], k_par_next, abort_flag, p.status);
-                    if (ok && !mbar_test_wait(&p_full[t], j & 1)) {
-                        // polled without suspending: this thread has nothing else to do
-                        const unsigned long long t0 = global_ns();
-                        uint32_t spins = 0;
-                        while (!mbar_test_wait(&p_full[t], j & 1)) {
-                            if ((++spins & 255u) == 0) {
-                                if (*abort_flag) { ok = false; break; }
-                                unsigned long long limit = *(volatile const unsigned long long*)(p.status + NOVA_WAIT_LIMIT_WORD);
-                                if (limit == 0) limit = kWaitLimitNs;
-                                if (global_ns() - t0 > limit) {
-                                    *abort_flag = 1;
-                                    atomicOr(p.status, NOVA_DEV_TIMEOUT);
-                                    ok = false;
-                                    break;
+                if (warp == 0) {
+                    if (elect_one()) {
+                        bool ok = true;
+                        // one stage: V of tile vj of pass vi (vi < 0: none) and K of the next S tile, if there is one
+                        auto load_stage = [&](int vi, int vj) {
+                            if (s_left == 0 && vi < 0) return;
+                            // (the stage's last use is waited for by its own barrier, which cannot complete twice
+                            // before the next fill; S's barriers go on without the producer and could)
+                            if (units >= kStages && !mbar_wait(&kv_empty[st], spar ^ 1u, abort_flag, p.status)) { ok = false; return; }
+                            const bool has_k = s_left > 0;
+                            if (has_k && s_left == s_n) {
+                                if (qcount >= 2 && !mbar_wait(&q_empty[qb], qpar ^ 1u, abort_flag, p.status)) { ok = false; return; }
+                                if (rank == 0) mbar_arrive_expect_tx(&q_full[qb], L::kCtas * L::kQBytes);
+#pragma unroll
+                                for (int sl = 0; sl < DH / 64; ++sl) {
+                                    uint8_t* dst = smem + qb * L::kQBytes + sl * kSlabBytes;
+                                    const int row = table[si].q_begin + (int)rank * BQ;
+                                    if constexpr (kPair) tma_load_2d_pair(dst, &tmap_q, map_to_cta(smem_u32(&q_full[qb]), 0), table[si].x + sl * 64, row);
+                                    else tma_load_2d(dst, &tmap_q, &q_full[qb], table[si].x + sl * 64, row);
+                                }
+                                ++qcount;
+                                if (++qb == 2) { qb = 0; qpar ^= 1u; }
+                            }
+                            uint8_t* dst = smem + L::kStageOff + st * 2 * L::kTileBytes;
+                            if (rank == 0)
+                                mbar_arrive_expect_tx(&kv_full[st], (uint32_t)((has_k ? L::kCtas * L::kTileBytes : 0) + (vi >= 0 ? L::kCtas * L::kTileBytes : 0)));
+                            const uint32_t bar = kPair ? map_to_cta(smem_u32(&kv_full[st]), 0) : 0u;
+                            if (vi >= 0) {
+                                const int y = vj == table[vi].n - 1 ? table[vi].last : table[vi].first + vj * BKV;
+                                if constexpr (kPair) tma_load_3d_pair(dst + L::kTileBytes, &tmap_v, bar, table[vi].x + (int)rank * L::kVCols, y, table[vi].b);
+                                else tma_load_3d(dst + L::kTileBytes, &tmap_v, &kv_full[st], table[vi].x, y, table[vi].b);
+                            }
+                            if (has_k) {
+                                const int j = s_n - s_left;
+                                const int y = (s_left == 1 ? table[si].last : table[si].first + j * BKV) + (int)rank * L::kKRows;
+#pragma unroll
+                                for (int sl = 0; sl < DH / 64; ++sl) {
+                                    if constexpr (kPair) tma_load_3d_pair(dst + sl * L::kKRows * 128, &tmap_k, bar, table[si].x + sl * 64, y, table[si].b);
+                                    else tma_load_3d(dst + sl * L::kKRows * 128, &tmap_k, &kv_full[st], table[si].x + sl * 64, y, table[si].b);
+                                }
+                                s_step();
+                            }
+                            ++units;
+                            if (++st == kStages) { st = 0; spar ^= 1u; }
+                        };
+                        for (int i = 0; i < kBufs && ok; ++i) load_stage(-1, 0);
+                        for (int i = next_pass(0, only); i < kTable && ok; i = next_pass(i + 1, only)) {
+                            const int n = table[i].n;
+                            for (int pass = only ? 0 : 1; pass < 2; ++pass)        // 0: maximum pass (K only)
+                                for (int j = 0; j < n && ok; ++j) load_stage(pass ? i : -1, j);
+                        }
+                        // A round ends with every copy landed and every use of a stage or of Q done.
+                        for (int i = max(0, units - kStages); i < units && ok; ++i)
+                            ok = mbar_wait(&kv_empty[i % kStages], (uint32_t)(i / kStages) & 1u, abort_flag, p.status);
+                        for (int i = max(0, qcount - 2); i < qcount && ok; ++i)
+                            ok = mbar_wait(&q_empty[i & 1], (uint32_t)(i >> 1) & 1u, abort_flag, p.status);
+                        if (!ok || *abort_flag) {       // what is in flight gets some time to finish before memory is released
+                            if (rank == 0) {
+                                for (int i = max(0, qcount - 2); i < qcount; ++i) mbar_drain(&q_full[i & 1], (uint32_t)(i >> 1) & 1u);
+                                for (int i = max(0, units - kStages); i < units; ++i) mbar_drain(&kv_full[i % kStages], (uint32_t)(i / kStages) & 1u);
+                            }
+                            for (int i = max(0, units - kStages); i < units; ++i) mbar_drain(&kv_empty[i % kStages], (uint32_t)(i / kStages) & 1u);
+                        }
+                    }
+                } else if (warp == 1) {
+                    if (rank == 0 && elect_one()) {
+                        constexpr uint32_t idesc_s = idesc_bf16_f32(L::kRows, BKV, 0);
+                        constexpr uint32_t idesc_o = idesc_bf16_f32(L::kRows, DH, 1);
+                        // Shared-memory descriptors: (address >> 4) sits in the low 14 bits, so stepping through
+                        // a tile or to another stage is an integer add.
+                        const uint64_t q_desc = smem_desc_sw128(smem_u32(smem), 16, 1024);
+                        const uint64_t k_desc = smem_desc_sw128(smem_u32(smem + L::kStageOff), 16, 1024);
+                        const uint64_t v_desc = smem_desc_sw128(smem_u32(smem + L::kStageOff + L::kTileBytes), kSlabBytes, 1024);
+                        bool ok = true, new_q = true;
+                        // S of the next tile, whichever pass it belongs to, with K in stage `from`.
+                        auto issue_s = [&](int from) {
+                            if (new_q) {
+                                ok = mbar_wait(&q_full[qb], qpar, abort_flag, p.status);
+                                if (!ok) return;
+                                tc_fence_after();
+                            }
+                            const uint64_t qd = q_desc + (uint32_t)(qb * (L::kQBytes >> 4));
+                            const uint64_t kd = k_desc + (uint32_t)(from * (2 * L::kTileBytes >> 4));
+                            const uint32_t s_tmem = tmem_base + 128u + BKV * (uint32_t)sbuf;
+#pragma unroll
+                            for (int kk = 0; kk < DH / 16; ++kk) {
+                                const uint32_t qo = (kk >> 2) * (kSlabBytes >> 4) + (kk & 3) * 2;         // 32 bytes per 16 k
+                                const uint32_t ko = (kk >> 2) * (L::kKRows * 128 >> 4) + (kk & 3) * 2;
+                                if constexpr (kPair) mma_bf16_ss_pair(s_tmem, qd + qo, kd + ko, idesc_s, kk ? 1u : 0u);
+                                else mma_bf16_ss(s_tmem, qd + qo, kd + ko, idesc_s, kk ? 1u : 0u);
+                            }
+                            commit(&s_full[sbuf]);
+                            if (++sbuf == kBufs) sbuf = 0;
+                            new_q = s_step();
+                            if (new_q) {
+                                commit(&q_empty[qb]);
+                                if (++qb == 2) { qb = 0; qpar ^= 1u; }
+                            }
+                        };
+                        auto take_stage = [&]() -> int {
+                            ok = mbar_wait(&kv_full[st], spar, abort_flag, p.status);
+                            tc_fence_after();
+                            const int at = st;
+                            if (++st == kStages) { st = 0; spar ^= 1u; }
+                            return at;
+                        };
+                        for (int i = 0; i < kBufs && ok && s_left; ++i) {
+                            const int at = take_stage();
+                            if (!ok) break;
+                            issue_s(at);
+                            commit(&kv_empty[at]);
+                        }
+                        for (int i = next_pass(0, only); i < kTable && ok; i = next_pass(i + 1, only)) {
+                            const int n = table[i].n;
+                            for (int pass = only ? 0 : 1; pass < 2 && ok; ++pass) {
+                                for (int j = 0; j < n && ok; ++j) {
+                                    int at = -1;
+                                    if (pass || s_left) at = take_stage();
+                                    if (ok && pass && j == 0) {
+                                        if (o_used) ok = mbar_wait(o_empty, opar, abort_flag, p.status);
+                                        o_used = true;
+                                        opar ^= 1u;
+                                    }
+                                    if (ok) ok = mbar_wait(&p_full[pbuf], ppar, abort_flag, p.status);
+                                    if (!ok) break;
+                                    tc_fence_after();
+                                    if (pass) {
+                                        const uint64_t vd = v_desc + (uint32_t)(at * (2 * L::kTileBytes >> 4));
+                                        const uint32_t p_tmem = tmem_base + 128u + BKV * (uint32_t)pbuf;
+#pragma unroll
+                                        for (int kk = 0; kk < BKV / 16; ++kk) {
+                                            const uint32_t acc = kk ? 1u : (j ? 1u : 0u);
+                                            if constexpr (kPair) mma_bf16_ts_pair(tmem_base, p_tmem + kk * 8, vd + (uint32_t)(kk * 128), idesc_o, acc);
+                                            else mma_bf16_ts(tmem_base, p_tmem + kk * 8, vd + (uint32_t)(kk * 128), idesc_o, acc);
+                                        }
+                                        if (j == n - 1) commit(o_full);
+                                    }
+                                    if (++pbuf == kBufs) { pbuf = 0; ppar ^= 1u; }
+                                    if (s_left) issue_s(at);
+                                    if (at >= 0) commit(&kv_empty[at]);
                                 }
                             }
                         }
                     }
-                    if (ok) ok = take_turn();
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_pv(vs, j == 0);
-                    if (more) {
-                        issue_s(ks_next);
-                        mma_commit(&k_empty[ks_next]);              // this tile no longer reads K_{j+1}, nor V_j
-                    }
-                    pass_turn();
-                    if (++vs == kVStages) { vs = 0; v_par ^= 1u; }
-                    if (++ks_next == kKStages) { ks_next = 0; k_par_next ^= 1u; }
                 }
-                if (ok) mma_commit(o_done);
-            }
-        } else if (warp == 1) {
-            // Head size 64: the groups are short, the token costs more than it saves, and one thread
-            // serves both tiles in the fixed order A, B.
-            if (elect_one()) {
-                constexpr uint32_t idesc_s = idesc_bf16_f32(BQ, BKV, 0);
-                constexpr uint32_t idesc_o = idesc_bf16_f32(BQ, DH, 1);
-                // Shared-memory descriptors: (address >> 4) sits in the low 14 bits, so stepping through
-                // a tile or to another stage is an integer add.
-                constexpr uint32_t kTileStep = L::kTileBytes >> 4;
-                const uint64_t q_desc = smem_desc_sw128(smem_u32(q_smem), 16, 1024);
-                const uint64_t k_desc = smem_desc_sw128(smem_u32(smem + L::kKOff), 16, 1024);
-                const uint64_t v_desc = smem_desc_sw128(smem_u32(smem + L::kVOff), kSlabBytes, 1024);
-                const int n_q = tile_b_active ? 2 : 1;
-                // S_t = Q_t K^T with K in stage ks
-                auto issue_s = [&](int t, int ks) {
-                    const uint64_t qd = q_desc + (uint32_t)t * kTileStep;
-                    const uint64_t kd = k_desc + (uint32_t)ks * kTileStep;
-#pragma unroll
-                    for (int kk = 0; kk < DH / 16; ++kk) {
-                        constexpr uint32_t kSlabStep = kSlabBytes >> 4;
-                        const uint32_t off = (kk >> 2) * kSlabStep + (kk & 3) * 2;    // 32 bytes per 16 k
-                        mma_bf16_ss(tmem_base + 128u * t, qd + off, kd + off, idesc_s, kk ? 1u : 0u);
-                    }
-                    mma_commit(&s_full[t]);
-                };
-                // O_t (+)= P_t V with V in stage vs; P_t sits in the first 64 columns of S_t, two keys per column
-                auto issue_pv = [&](int t, int vs, bool first) {
-                    const uint64_t vd = v_desc + (uint32_t)vs * kTileStep;
-#pragma unroll
-                    for (int kk = 0; kk < BKV / 16; ++kk)
-                        mma_bf16_ts(tmem_base + 256u + 128u * t, tmem_base + 128u * t + kk * 8, vd + (uint32_t)(kk * 128),
-                                    idesc_o, (first && kk == 0) ? 0u : 1u);
-                };
-                bool ok = mbar_wait(q_full, 0, abort_flag, p.status);
-                if (ok) ok = mbar_wait(&k_full[0], 0, abort_flag, p.status);
-                if (ok) {
-                    tc_fence_after();
-                    for (int t = 0; t < n_q; ++t) issue_s(t, 0);
-                    mma_commit(&k_empty[0]);
+                const unsigned long long again = end_of_round();
+                if (only || !again) break;
+                only = again;
+            } while (true);
+        }
+    } else if (warp < 8) {
+        // ---- epilogue -------------------------------------------------------------------------------
+        const int q = warp & 3, row = q * 32 + lane;              // row within the CTA's 128 = tensor-memory lane
+        const int grow = (int)rank * BQ + row;                    // row within the work item
+        const uint32_t o_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+        const float* l_s = (const float*)(smem + L::kLOff);
+        const float* m_s = (const float*)(smem + L::kMOff);
+        int np = 0;                                               // passes with an O so far
+        for (int base = 0; begin_round(base); base += kTable) {
+            unsigned long long only = 0;
+            for (int i = 0; i < kTable && !table[i].over; ++i)
+                if (table[i].empty && grow < table[i].rows_valid) {
+                    // nothing to attend to: the output rows are zero
+                    __nv_bfloat16* dst_row = p.o + (long)(table[i].q_begin + grow) * p.C + table[i].x;
+                    for (int v = 0; v < DH / 8; ++v) *(uint4*)(dst_row + v * 8) = make_uint4(0, 0, 0, 0);
                 }
-                // ring positions and phase parities, stepped without divisions
-                int vs = 0, ks_next = (kKStages > 1) ? 1 : 0;
-                uint32_t v_par = 0, k_par_next = (kKStages > 1) ? 0u : 1u;
-                for (int j = 0; j < n_tiles && ok; ++j) {
-                    const bool more = j + 1 < n_tiles;
-                    // V_j and K_{j+1} have usually landed long ago; P is what a step waits for
-                    ok = mbar_wait(&v_full[vs], v_par, abort_flag, p.status);
-                    if (ok && more) ok = mbar_wait(&k_full[ks_next], k_par_next, abort_flag, p.status);
-                    for (int t = 0; t < n_q && ok; ++t) {
-                        ok = mbar_wait(&p_full[t], j & 1, abort_flag, p.status);
-                        if (!ok) break;
-                        tc_fence_after();
-                        issue_pv(t, vs, j == 0);
-                        if (more) {
-                            issue_s(t, ks_next);
-                            if (t == n_q - 1) mma_commit(&k_empty[ks_next]);        // K_{j+1} and V_j have no reader left
+            do {
+                for (int i = next_pass(0, only); i < kTable; i = next_pass(i + 1, only), ++np) {
+                    const int half = table[i].half, rows_valid = table[i].rows_valid;
+                    __nv_bfloat16* dst_row = p.o + (long)(table[i].q_begin + grow) * p.C + table[i].x;
+                    const int slot = np % kSlots;
+                    // (after a failed wait everybody goes on with garbage to the end: the status word says so)
+                    bool ok = mbar_wait_warp(&l_full[slot], (uint32_t)(np / kSlots) & 1u, abort_flag, p.status);
+                    const float l_run = l_s[(slot * 2 + 0) * BQ + row] + l_s[(slot * 2 + 1) * BQ + row];
+                    const float m_ref = m_s[slot * BQ + row];
+                    // The first time, a pass that will be run again is left alone; the second time, one that
+                    // only the other CTA of the pair asked for.
+                    const bool huge = (*(volatile unsigned long long*)&redo_s >> i) & 1ull;
+                    const bool act = only ? huge : !huge;
+                    ok = mbar_wait_warp(o_full, (uint32_t)np & 1u, abort_flag, p.status) && ok;
+                    tc_fence_after();
+                    // The next kernel is let in at the last pass. A trigger at the start puts its first CTAs on the SMs
+                    // this grid leaves free, long before the others find room, and it ends later for it: a 16-layer
+                    // 256x256 generation took 9750 us with the trigger at the start, 9600 after the table, 9667 at
+                    // the end, 9518 to 9534 here or at the first pass.
+                    if (next_pass(i + 1, only) == kTable) pdl_launch_dependents();
+                    if (act && half < 0) {
+                        const float inv = 1.f / l_run;
+#pragma unroll 1
+                        for (int cch = 0; cch < DH / 32; ++cch) {
+                            uint32_t ov[32];
+                            tmem_ld32(o_addr + cch * 32, ov);
+                            tmem_ld_wait();
+                            if (ok && grow < rows_valid) {
+                                uint4* dst = (uint4*)(dst_row + cch * 32);
+#pragma unroll
+                                for (int g = 0; g < 4; ++g)
+                                    dst[g] = make_uint4(
+                                        pack_bf16(__uint_as_float(ov[g * 8]) * inv, __uint_as_float(ov[g * 8 + 1]) * inv),
+                                        pack_bf16(__uint_as_float(ov[g * 8 + 2]) * inv, __uint_as_float(ov[g * 8 + 3]) * inv),
+                                        pack_bf16(__uint_as_float(ov[g * 8 + 4]) * inv, __uint_as_float(ov[g * 8 + 5]) * inv),
+                                        pack_bf16(__uint_as_float(ov[g * 8 + 6]) * inv, __uint_as_float(ov[g * 8 + 7]) * inv));
+                            }
+                        }
+                    } else if (act) {
+                        const int khalf = half & 1, tail_slot = half >> 1;
+                        const float c = p.scale_log2e;
+                        // ---- half of the keys: publish the partial result, then merge if the other is there. The two
+                        // CTAs of a pair do so independently, each for its rows.
+                        // [DH columns, then reference and sum][rows]: a warp's accesses are 128 contiguous bytes
+                        float* mine = p.part + (size_t)(tail_slot * 2 + khalf) * (DH + 4) * L::kRows + grow;
+                        const float* other = p.part + (size_t)(tail_slot * 2 + (khalf ^ 1)) * (DH + 4) * L::kRows + grow;
+                        unsigned int* ticket = p.tickets + tail_slot * L::kCtas + rank;
+#pragma unroll 1
+                        for (int cch = 0; cch < DH / 32; ++cch) {
+                            uint32_t ov[32];
+                            tmem_ld32(o_addr + cch * 32, ov);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int g = 0; g < 32; ++g) mine[(cch * 32 + g) * L::kRows] = __uint_as_float(ov[g]);
+                        }
+                        mine[DH * L::kRows] = m_ref;
+                        mine[(DH + 1) * L::kRows] = l_run;
+                        __threadfence();
+                        asm volatile("bar.sync 1, 128;" ::: "memory");
+                        if (threadIdx.x == 128) {
+                            const unsigned int t = atomicAdd(ticket, 1u);
+                            if (t == 1u) *ticket = 0;          // ready for the next launch
+                            ticket_s = (int)t;
+                        }
+                        asm volatile("bar.sync 1, 128;" ::: "memory");
+                        if (ok && ticket_s == 1) {
+                            // the other fenced its partial result before it drew ticket 0
+                            // The merge is written in terms of (half 0, half 1), not (mine, other), with every
+                            // rounding spelled out: either may be the one that merges, and the output must
+                            // not depend on which.
+                            const float m_o = __ldcg(other + DH * L::kRows), l_o = __ldcg(other + (DH + 1) * L::kRows);
+                            const float m_new = fmaxf(m_ref, m_o);
+                            const float a_me = ex2((m_ref - m_new) * c), a_o = ex2((m_o - m_new) * c);
+                            const bool first = (khalf == 0);
+                            const float a0 = first ? a_me : a_o, a1 = first ? a_o : a_me;
+                            const float l0 = first ? l_run : l_o, l1 = first ? l_o : l_run;
+                            const float inv = 1.f / __fmaf_rn(l0, a0, __fmul_rn(l1, a1));
+                            const float w0 = a0 * inv, w1 = a1 * inv;
+                            const float w_me = first ? w0 : w1, w_o = first ? w1 : w0;
+                            auto mix = [&](uint32_t mine_bits, float theirs) {
+                                const float v = __uint_as_float(mine_bits);
+                                // half 0's term is the multiply-add operand, half 1's the rounded product
+                                return first ? __fmaf_rn(v, w_me, __fmul_rn(theirs, w_o))
+                                             : __fmaf_rn(theirs, w_o, __fmul_rn(v, w_me));
+                            };
+#pragma unroll 1
+                            for (int cch = 0; cch < DH / 32; ++cch) {
+                                uint32_t ov[32];
+                                tmem_ld32(o_addr + cch * 32, ov);
+                                tmem_ld_wait();
+                                float th[32];
+#pragma unroll
+                                for (int g = 0; g < 32; ++g) th[g] = __ldcg(other + (cch * 32 + g) * L::kRows);
+                                if (grow < rows_valid) {
+                                    uint4* dst = (uint4*)(dst_row + cch * 32);
+#pragma unroll
+                                    for (int g = 0; g < 4; ++g)
+                                        dst[g] = make_uint4(
+                                            pack_bf16(mix(ov[g * 8], th[g * 8]), mix(ov[g * 8 + 1], th[g * 8 + 1])),
+                                            pack_bf16(mix(ov[g * 8 + 2], th[g * 8 + 2]), mix(ov[g * 8 + 3], th[g * 8 + 3])),
+                                            pack_bf16(mix(ov[g * 8 + 4], th[g * 8 + 4]), mix(ov[g * 8 + 5], th[g * 8 + 5])),
+                                            pack_bf16(mix(ov[g * 8 + 6], th[g * 8 + 6]), mix(ov[g * 8 + 7], th[g * 8 + 7])));
+                                }
+                            }
                         }
                     }
-                    if (++vs == kVStages) { vs = 0; v_par ^= 1u; }
-                    if (++ks_next == kKStages) { ks_next = 0; k_par_next ^= 1u; }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) arrive_leader(o_empty);
                 }
-                if (ok) mma_commit(o_done);
-            }
+                const unsigned long long again = end_of_round();
+                if (only || !again) break;
+                only = again;
+            } while (true);
         }
-    }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsHigh));
-        const int t = (warp >= 8) ? 1 : 0;            // which query tile this warpgroup owns
-        if (t == 0 || tile_b_active) {
-            const int q = warp & 3;
-            const int row = q * 32 + lane;               // row within the tile = TMEM lane
-            const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-            const uint32_t s_addr = tmem_base + lane_off + 128u * t;
-            const uint32_t o_addr = tmem_base + lane_off + 256u + 128u * t;
-            const float c = p.scale_log2e;
-            // Polynomial share of the exponentials (pairs out of every four pairs of scores). The
-            // special-function unit delivers one exponential per 8 clocks and scheduler; the polynomial
-            // costs a scheduler about as much in issue slots, so it does not replace that unit, it only
-            // works beside it: a quarter of the scores on the polynomial measured best at both head sizes
-            // (6.9 clocks per score and scheduler against 7.5 at a half and 8.2 with none).
-            constexpr int kPolyPairs = 1;
-            // The reference maximum starts at a finite floor, not -inf: (-inf) - (-inf) must not appear.
-            float m_ref = -1e30f, l_run = 0.f;
-            bool ok = true;
-            for (int j = 0; j < n_tiles && ok; ++j) {
-                ok = mbar_wait_warp(&s_full[t], j & 1, abort_flag, p.status);
-                if (!ok) break;
-                tc_fence_after();
-                const int cols_valid = n_keys - (jt0 + j) * BKV;      // >= 1; < BKV only on a ragged last tile
-                // the whole row of S (128 scores) into registers with one round trip to tensor memory
-                uint32_t sv[128];
+        // ---- softmax ------------------------------------------------------------------------------------
+        const int wg = (warp - 8) >> 2, q = warp & 3, row = q * 32 + lane;
+        const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+        const float c = p.scale_log2e;
+        float* l_s = (float*)(smem + L::kLOff) + wg * BQ + row;
+        float* m_s = (float*)(smem + L::kMOff) + row;
+        float* a_s = (float*)(smem + L::kAOff) + row;
+        // Polynomial share of the exponentials (pairs out of every four pairs of scores). The
+        // special-function unit delivers one exponential per 8 clocks and scheduler; the polynomial
+        // costs a scheduler about as much in issue slots, so it does not replace that unit, it only
+        // works beside it: a quarter of the scores on the polynomial measured best at both head sizes
+        // (6.9 clocks per score and scheduler against 7.5 at a half and 8.2 with none).
+        constexpr int kPolyPairs = 1;
+        int np = 0;                            // ordinary passes so far
+        int mine = wg;                         // tiles until this warpgroup's next one
+        int buf = wg;                          // S buffer of that tile: every other one, of three
+        uint32_t par = 0;                      // and its phase parity
+        for (int base = 0; begin_round(base); base += kTable) {
+            unsigned long long only = 0;
+            do {
+            for (int i = next_pass(0, only); i < kTable; i = next_pass(i + 1, only)) {
+            const int n = table[i].n, masked = table[i].masked;
+            float m_true = -1e30f;             // the row's maximum over all keys, from a maximum pass
+            for (int pass = only ? 0 : 1; pass < 2; ++pass) {
+                const int slot = np % kSlots;
+                // The reference maximum starts at a finite floor, not -inf: (-inf) - (-inf) must not appear.
+                float m_ref = -1e30f, l_run = 0.f, m_run = -1e30f;
+                bool huge = false;
+                // tiles alternate between the warpgroups, also across passes
+                int j = mine;
+                for (; j < n; j += 2) {
+                    const uint32_t s_addr = tmem_base + lane_off + 128u + BKV * (uint32_t)buf;
+                    mbar_wait_warp(&s_full[buf], par, abort_flag, p.status);
+                    tc_fence_after();
+                    uint64_t* done = &p_full[buf];
+                    if (buf == 0) buf = 2;                       // two tiles on
+                    else { --buf; par ^= 1u; }
+                    // The row is taken 32 scores at a time, in loops that are not unrolled: the code of a whole
+                    // row is 16 KB, and fetching it costs a launch's first tile 6 us. The latency of the
+                    // tensor-memory reads hides behind the other warpgroup.
+                    const int skip = j == n - 1 ? masked : 0;       // columns that do not count
+                    auto load = [&](int ch, uint32_t (&sv)[32]) {
+                        tmem_ld32(s_addr + ch * 32, sv);
+                        tmem_ld_wait();
+                        if (skip > ch * 32) {
 #pragma unroll
-                for (int cch = 0; cch < 4; ++cch)
-                    tmem_ld32(s_addr + cch * 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[cch * 32]));
-                tmem_ld_wait();
-                if (cols_valid < BKV) {
+                            for (int e = 0; e < 32; ++e)
+                                if (ch * 32 + e < skip) sv[e] = 0xff800000u;   // -inf: a key of the tile before, or none
+                        }
+                    };
+                    if (pass == 0 || (j == 0 && !only)) {
+                        // (the reference: over the tile's last 32 columns, which always hold a key, is enough)
+                        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 1
+                        for (int ch = pass ? 3 : 0; ch < 4; ++ch) {
+                            uint32_t sv[32];
+                            load(ch, sv);
 #pragma unroll
-                    for (int i = 0; i < 128; ++i)
-                        if (i >= cols_valid) sv[i] = 0xff800000u;   // -inf: key past the end
-                }
-                auto row_max = [&]() {
-                    float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                    for (int i = 0; i < 128; i += 8) {
-#pragma unroll
-                        for (int a = 0; a < 4; ++a)
-                            mx4[a] = fmax3(mx4[a], __uint_as_float(sv[i + 2 * a]), __uint_as_float(sv[i + 2 * a + 1]));
+                            for (int e = 0; e < 32; e += 2) mx[(e >> 1) & 3] = fmax3(mx[(e >> 1) & 3], __uint_as_float(sv[e]), __uint_as_float(sv[e + 1]));
+                        }
+                        m_run = fmaxf(m_run, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])));
                     }
-                    return fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-                };
-                if (j == 0) m_ref = fmaxf(m_ref, row_max());      // the row's reference: its maximum over the first key tile
-                // p = 2^(s*c - m*c), 32 scores at a time: 16 registers of bf16 pairs each, written over the
-                // first columns of S as they are ready. Returns the sum of the 128 probabilities.
-                auto exponentials = [&](bool store) {
+                    if (pass == 0) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) arrive_leader(done);
+                        continue;
+                    }
+                    if (j == 0) {
+                        // the row's reference, for both warpgroups and the epilogue
+                        m_ref = only ? m_true : m_run;
+                        m_s[slot * BQ] = m_ref;
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&m_full[slot]);
+                    } else if (j == 1) {
+                        mbar_wait_warp(&m_full[slot], (uint32_t)(np / kSlots) & 1u, abort_flag, p.status);
+                        m_ref = m_s[slot * BQ];
+                    }
+                    // p = 2^(s*c - m*c): 16 registers of bf16 pairs per chunk, written over columns of S that have
+                    // been read
                     const uint64_t c2 = pack_f32x2(c, c);
                     const uint64_t nm2 = pack_f32x2(-m_ref * c, -m_ref * c);
                     uint64_t lsum_a = pack_f32x2(0.f, 0.f), lsum_b = lsum_a;
+                    // (chunks of which no column counts take zeros and no arithmetic: three of four in the smallest calls,
+                    // 7.1 -> 6.3 us for eight images with one kept token each)
+                    int ch = 0;
+#pragma unroll 1
+                    for (; (ch + 1) * 32 <= skip; ++ch) {
+                        uint32_t zero[16];
 #pragma unroll
-                    for (int cch = 0; cch < 4; ++cch) {
-                        uint32_t pk[16];
+                        for (int e = 0; e < 16; ++e) zero[e] = 0u;
+                        tmem_st16(s_addr + ch * 16, zero);
+                    }
+#pragma unroll 1
+                    for (; ch < 4; ++ch) {
+                        uint32_t sv[32], pk[16];
+                        load(ch, sv);
 #pragma unroll
                         for (int g = 0; g < 4; ++g) {
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int i = cch * 32 + 8 * g + 2 * q;
+                            for (int e = 0; e < 4; ++e) {
+                                const int i = 8 * g + 2 * e;
                                 const uint64_t y = fma_f32x2(pack_f32x2(__uint_as_float(sv[i]), __uint_as_float(sv[i + 1])), c2, nm2);
                                 float p0, p1;
-                                if (q < kPolyPairs) {
+                                if (e < kPolyPairs) {
                                     exp2_poly_x2(y, p0, p1);
                                 } else {
                                     float y0, y1;
@@ -572,202 +773,92 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                                     p0 = ex2(y0);
                                     p1 = ex2(y1);
                                 }
-                                if (q & 1) lsum_b = add_f32x2(lsum_b, pack_f32x2(p0, p1));
+                                if (e & 1) lsum_b = add_f32x2(lsum_b, pack_f32x2(p0, p1));
                                 else lsum_a = add_f32x2(lsum_a, pack_f32x2(p0, p1));
-                                pk[4 * g + q] = pack_bf16(p0, p1);
+                                pk[4 * g + e] = pack_bf16(p0, p1);
                             }
                         }
-                        if (store) tmem_st16(s_addr + cch * 16, pk);
+                        tmem_st16(s_addr + ch * 16, pk);
                     }
                     float s0, s1, s2, s3;
                     unpack_f32x2(lsum_a, s0, s1);
                     unpack_f32x2(lsum_b, s2, s3);
-                    return (s0 + s2) + (s1 + s3);
-                };
-                float lsum = exponentials(true);
-                if (j > 0 && __any_sync(0xffffffffu, !(lsum < kHugeSum))) {
-                    // a score far above the reference: raise it, rescale what has been accumulated
-                    // (the tile's previous O += P V is complete: its S could not have been written
-                    // otherwise) and take the tile's probabilities again
-                    const float m_new = fmaxf(m_ref, row_max());
-                    const float alpha = ex2((m_ref - m_new) * c);
+                    const float lsum = (s0 + s2) + (s1 + s3);
+                    huge |= !(lsum < kHugeSum);
+                    l_run += lsum;
                     tmem_st_wait();
-#pragma unroll
-                    for (int cch = 0; cch < DH / 32; ++cch) {
-                        uint32_t ov[32];
-                        tmem_ld32(o_addr + cch * 32, ov);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
-                        tmem_st32(o_addr + cch * 32, ov);
-                    }
-                    l_run *= alpha;
-                    m_ref = m_new;
-                    lsum = exponentials(true);
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) arrive_leader(done);
                 }
-                l_run += lsum;
-                tmem_st_wait();
-                if ((t == 0 || kIssuers == 2) && cols_valid < BKV) {
-                    // ragged last tile: rows of V past the last key may hold anything (even NaN);
-                    // zero them so that 0 * garbage cannot poison the accumulator. With one issuing
-                    // thread tile A's O += P V is issued before tile B's, so tile A's softmax warps do it
-                    // for both; with a thread per tile each tile's warps do it before their own hand-over
-                    // (zeros written over zeros are harmless)
-                    const int s = j % kVStages;
-                    ok = mbar_wait_warp(&v_full[s], (j / kVStages) & 1, abort_flag, p.status);
-                    if (!ok) break;
-                    if (row >= cols_valid) {
-                        uint8_t* v_row = smem + L::kVOff + s * L::kTileBytes + row * 128;
-#pragma unroll
-                        for (int sl = 0; sl < kSlabs; ++sl)
-#pragma unroll
-                            for (int g = 0; g < 8; ++g) *(uint4*)(v_row + sl * kSlabBytes + g * 16) = make_uint4(0, 0, 0, 0);
-                    }
-                    fence_proxy_async_smem();
+                mine = j - n;
+                if (pass == 0) {
+                    a_s[wg * BQ] = m_run;
+                    asm volatile("bar.sync 2, 256;" ::: "memory");
+                    m_true = fmaxf(a_s[0], a_s[BQ]);
+                    asm volatile("bar.sync 2, 256;" ::: "memory");
+                    continue;
                 }
-                tc_fence_before();
+                l_s[slot * 2 * BQ] = l_run;
+                if (!only && __any_sync(0xffffffffu, huge) && lane == 0) atomicOr(&redo_s, 1ull << i);
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&p_full[t]);
+                if (lane == 0) mbar_arrive(&l_full[slot]);
+                ++np;
             }
-            if (ok) ok = mbar_wait_warp(o_done, 0, abort_flag, p.status);
-            const int grow = t * BQ + row;
-            __nv_bfloat16* dst_row = p.o + (long)(q_begin + grow) * p.C + head * DH;
-            if (ok && khalf < 0) {
-                tc_fence_after();
-                const float inv = 1.f / l_run;
-#pragma unroll
-                for (int cch = 0; cch < DH / 32; ++cch) {
-                    uint32_t ov[32];
-                    tmem_ld32(o_addr + cch * 32, ov);
-                    tmem_ld_wait();
-                    if (grow < rows_valid) {
-                        uint4* dst = (uint4*)(dst_row + cch * 32);
-#pragma unroll
-                        for (int g = 0; g < 4; ++g)
-                            dst[g] = make_uint4(
-                                pack_bf16(__uint_as_float(ov[g * 8]) * inv, __uint_as_float(ov[g * 8 + 1]) * inv),
-                                pack_bf16(__uint_as_float(ov[g * 8 + 2]) * inv, __uint_as_float(ov[g * 8 + 3]) * inv),
-                                pack_bf16(__uint_as_float(ov[g * 8 + 4]) * inv, __uint_as_float(ov[g * 8 + 5]) * inv),
-                                pack_bf16(__uint_as_float(ov[g * 8 + 6]) * inv, __uint_as_float(ov[g * 8 + 7]) * inv));
-                    }
-                }
-            } else if (khalf >= 0) {
-                // ---- half of the keys: publish the partial result, then merge if the other is there
-                // (all softmax threads of the CTA take part, also after a failed wait, so that the
-                // named barrier below is complete; a failed CTA publishes nothing useful and the
-                // status word says so)
-                constexpr int kStride = DH + 4;
-                float* mine = p.part + ((size_t)(tail_slot * 2 + khalf) * (2 * BQ) + grow) * kStride;
-                const float* other = p.part + ((size_t)(tail_slot * 2 + (khalf ^ 1)) * (2 * BQ) + grow) * kStride;
-                if (ok) {
-                    tc_fence_after();
-#pragma unroll
-                    for (int cch = 0; cch < DH / 32; ++cch) {
-                        uint32_t ov[32];
-                        tmem_ld32(o_addr + cch * 32, ov);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int g = 0; g < 8; ++g)
-                            *(uint4*)(mine + cch * 32 + g * 4) = make_uint4(ov[g * 4], ov[g * 4 + 1], ov[g * 4 + 2], ov[g * 4 + 3]);
-                    }
-                    mine[DH] = m_ref;
-                    mine[DH + 1] = l_run;
-                }
-                __threadfence();
-                const int n_soft = tile_b_active ? 256 : 128;
-                asm volatile("bar.sync 1, %0;" ::"r"(n_soft) : "memory");
-                if (threadIdx.x == 128) {
-                    const unsigned int ticket = atomicAdd(&p.tickets[tail_slot], 1u);
-                    if (ticket == 1u) p.tickets[tail_slot] = 0;          // ready for the next launch
-                    ticket_s = (int)ticket;
-                }
-                asm volatile("bar.sync 1, %0;" ::"r"(n_soft) : "memory");
-                if (ok && ticket_s == 1) {
-                    // the other CTA fenced its partial result before it drew ticket 0
-                    // The merge is written in terms of (half 0, half 1), not (mine, other), with every
-                    // rounding spelled out: either CTA may be the one that merges, and the output must
-                    // not depend on which.
-                    const float m_o = __ldcg(other + DH), l_o = __ldcg(other + DH + 1);
-                    const float m_new = fmaxf(m_ref, m_o);
-                    const float a_me = ex2((m_ref - m_new) * c), a_o = ex2((m_o - m_new) * c);
-                    const bool first = (khalf == 0);
-                    const float a0 = first ? a_me : a_o, a1 = first ? a_o : a_me;
-                    const float l0 = first ? l_run : l_o, l1 = first ? l_o : l_run;
-                    const float inv = 1.f / __fmaf_rn(l0, a0, __fmul_rn(l1, a1));
-                    const float w0 = a0 * inv, w1 = a1 * inv;
-                    const float w_me = first ? w0 : w1, w_o = first ? w1 : w0;
-                    auto mix = [&](uint32_t mine_bits, float theirs) {
-                        const float me = __uint_as_float(mine_bits);
-                        // half 0's term is the multiply-add operand, half 1's the rounded product
-                        return first ? __fmaf_rn(me, w_me, __fmul_rn(theirs, w_o))
-                                     : __fmaf_rn(theirs, w_o, __fmul_rn(me, w_me));
-                    };
-#pragma unroll
-                    for (int cch = 0; cch < DH / 32; ++cch) {
-                        uint32_t ov[32];
-                        tmem_ld32(o_addr + cch * 32, ov);
-                        tmem_ld_wait();
-                        if (grow < rows_valid) {
-                            uint4* dst = (uint4*)(dst_row + cch * 32);
-#pragma unroll
-                            for (int g = 0; g < 4; ++g) {
-                                const float4 o0 = __ldcg((const float4*)(other + cch * 32 + g * 8));
-                                const float4 o1 = __ldcg((const float4*)(other + cch * 32 + g * 8 + 4));
-                                dst[g] = make_uint4(
-                                    pack_bf16(mix(ov[g * 8], o0.x), mix(ov[g * 8 + 1], o0.y)),
-                                    pack_bf16(mix(ov[g * 8 + 2], o0.z), mix(ov[g * 8 + 3], o0.w)),
-                                    pack_bf16(mix(ov[g * 8 + 4], o1.x), mix(ov[g * 8 + 5], o1.y)),
-                                    pack_bf16(mix(ov[g * 8 + 6], o1.z), mix(ov[g * 8 + 7], o1.w)));
-                            }
-                        }
-                    }
-                }
             }
+            const unsigned long long again = end_of_round();
+            if (only || !again) break;
+            only = again;
+            } while (true);
         }
     }
+    // (the last end_of_round saw everybody's work done: nobody signals this CTA any more)
     tc_fence_before();
+    __syncwarp();
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, kTmemCols);
+        if constexpr (kPair) tmem_dealloc_pair(tmem_base, kTmemCols);
+        else tmem_dealloc(tmem_base, kTmemCols);
     }
 }
 
 template <int DH>
 nova_status launch(nova_ctx* ctx, const nova_attn_args& a, cudaStream_t st)
 {
-    using L = AttnSmem<DH>;
+    using L = AttnCfg<DH>;
     CUtensorMap tq, tk, tv;
     const uint64_t dq[2] = {(uint64_t)a.C, (uint64_t)a.M}, sq[1] = {(uint64_t)a.C * 2};
     const uint64_t dk[3] = {(uint64_t)a.C, (uint64_t)a.Lmax, (uint64_t)a.B};
     const uint64_t sk[2] = {(uint64_t)a.C * 2, (uint64_t)a.Lmax * a.C * 2};
-    if (!make_tmap_bf16(ctx, &tq, a.q, 2, dq, sq, BQ) || !make_tmap_bf16(ctx, &tk, a.k_cache, 3, dk, sk, BKV) ||
+    if (!make_tmap_bf16(ctx, &tq, a.q, 2, dq, sq, BQ) || !make_tmap_bf16(ctx, &tk, a.k_cache, 3, dk, sk, L::kKRows) ||
         !make_tmap_bf16(ctx, &tv, a.v_cache, 3, dk, sk, BKV))
         return nova_fail(ctx, NOVA_ERR_CUDA, "attention: cuTensorMapEncodeTiled failed");
-    auto kern = attention_kernel<DH>;
-    if (!ctx->attr_attn) {   // both head sizes opt in once per context
-        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<64>::kTotal));
-        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<128>::kTotal));
+    if (!ctx->attr_attn) {   // both head sizes once per context
+        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64>::kTotal));
+        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128>::kTotal));
         ctx->attr_attn = true;
     }
     AttnParams p;
     p.cu_keep = a.cu_keep; p.kv_len = a.kv_len; p.o = a.o; p.B = a.B; p.C = a.C; p.Lmax = a.Lmax;
     p.scale_log2e = (float)((1.0 / sqrt((double)DH)) * 1.4426950408889634);
     p.status = ctx->dev_status;
-    p.n_heads = a.n_heads; p.num_sms = ctx->num_sms;
+    p.n_heads = a.n_heads; p.slots = ctx->num_sms / L::kCtas;
     p.own_keys = a.cache_only ? 0 : 1;
-    // scratch for a key-split last wave: [slots][2][256][DH + 4] fp32; tickets live in the context's
+    // scratch for a key-split last round: [slots][2][kRows][DH + 4] fp32; tickets live in the context's
     // status allocation (zero at creation, reset by the CTA that draws the second ticket)
-    const size_t slot_bytes = (size_t)2 * 2 * BQ * (DH + 4) * sizeof(float);
-    p.part = (float*)a.scratch;
-    p.part_slots = a.scratch ? (int)min((size_t)NOVA_ATTN_TICKETS, a.scratch_bytes / slot_bytes) : 0;
+    const size_t slot_bytes = (size_t)2 * L::kRows * (DH + 4) * sizeof(float);
+    const bool can_split = a.scratch && (a.Lmax + BKV - 1) / BKV >= kSplitTiles;
+    p.part = can_split ? (float*)a.scratch : nullptr;
+    p.part_slots = can_split ? (int)min((size_t)(NOVA_ATTN_TICKETS / L::kCtas), a.scratch_bytes / slot_bytes) : 0;
     p.tickets = ctx->dev_status + NOVA_ATTN_TICKET_WORD0;
-    // upper bound of the work items (the kept counts per image live on the device) plus the CTAs a
-    // split last wave adds; CTAs past the end return at once
-    dim3 grid(((a.M + 2 * BQ - 1) / (2 * BQ) + a.B) * a.n_heads + ctx->num_sms / 2);
+    // One CTA (pair) per SM (two), or fewer if there cannot be as much work: upper bound of the work items (the
+    // kept counts per image live on the device), each split in two at most.
+    const long items = (((long)a.M + (long)a.B * (L::kRows - 1)) / L::kRows) * a.n_heads;
+    const int ctas = (int)min((long)p.slots, (can_split ? 2 : 1) * items) * L::kCtas;
     {
         nova_launch_scope scope(ctx, NOVA_K_ATTENTION, st);
-        NOVA_CUDA_CHECK(ctx, nova_launch_pdl(kern, grid, dim3(kThreads), L::kTotal, st, 0, tq, tk, tv, p));
+        NOVA_CUDA_CHECK(ctx, nova_launch_pdl(attention_kernel<DH>, dim3(ctas), dim3(kThreads), L::kTotal, st, L::kPair ? 2 : 0, tq, tk, tv, p));
     }
     return NOVA_OK;
 }

@@ -69,13 +69,14 @@ def attn_metric(y, y_ref, x_rows):
 
 
 def attention_case(ctx, B, N, C, heads, F, Lmax, ks, kv_lens, seed, rows=None, q_gain=1.0, q_zero=False,
-                   k_profile=None, dead_keys=None, half_keys_check=True, label=""):
+                   k_profile=None, dead_keys=None, live_keys=None, half_keys_check=True, label=""):
     """Runs the block on the GPU and the oracle on the same bytes; returns the attention-branch
     error. k_profile: per-key gains [max kv_len] applied to the prior K cache. dead_keys: indices of
     prior keys that every query scores about 100 nats below the rest (query bias 16 on the first
-    channel of each head, that channel of those keys set to -72 at head size 128 / -50 at 64)."""
+    channel of each head, that channel of those keys set to -72 at head size 128 / -50 at 64). live_keys:
+    (indices, value): the same with that channel set to a positive value."""
     dh = C // heads
-    wt = probe_weights(C, F, seed, q_gain=q_gain, q_zero=q_zero, q_bias=16.0 if dead_keys is not None else None,
+    wt = probe_weights(C, F, seed, q_gain=q_gain, q_zero=q_zero, q_bias=None if dead_keys is None and live_keys is None else 16.0,
                        heads=heads)
     x = (synth.activations(B, N, C, seed + 1, DEV).float() * X_SCALE).to(torch.bfloat16)
     k_cache, v_cache, _ = synth.kv_cache(B, Lmax, max(max(kv_lens), 1), C, seed + 2, DEV)
@@ -87,6 +88,10 @@ def attention_case(ctx, B, N, C, heads, F, Lmax, ks, kv_lens, seed, rows=None, q
         dk = torch.as_tensor(np.asarray(dead_keys), device=DEV)
         for c0 in range(0, C, dh):
             k_cache[:, dk, c0] = -72.0 if dh == 128 else -50.0
+    if live_keys is not None:
+        lk = torch.as_tensor(np.asarray(live_keys[0]), device=DEV)
+        for c0 in range(0, C, dh):
+            k_cache[:, lk, c0] = live_keys[1]
     for b, n in enumerate(kv_lens):          # rows past each image's length must never be used
         k_cache[b, n:] = float("nan")
         v_cache[b, n:] = float("nan")
@@ -264,6 +269,32 @@ def test_attention_rising_maximum_in_key_split_items(ctx):
     the merge weights of the low half underflow towards zero."""
     attention_case(ctx, B=1, N=600, C=256, heads=2, F=2048, Lmax=1024, ks=[300], kv_lens=[517], seed=53,
                    k_profile=_step_profile(517, at=384, hi=8.0), label="rising maximum, key-split items")
+
+
+@pytest.mark.parametrize("C,heads,value", [(256, 2, 50.0), (256, 2, 72.0), (128, 2, 40.0), (128, 2, 50.0)])
+@pytest.mark.parametrize("B", [1, 40])
+def test_attention_score_beyond_what_the_reference_carries(ctx, C, heads, value, B):
+    """Keys in the second half of the prior ones score about 16 value / sqrt(dh) nats (2^100 to 2^150) above
+    every key of the first tile, more than can be carried against a reference from there: the work items
+    concerned are run again with the rows' true maxima. One image: every item is shared by two CTAs (pairs);
+    forty: whole items, several per CTA, in which only every other image has such keys. The offset is one channel
+    that these keys have in common, so it cancels among them exactly, the query's bf16 rounding (2^-9 of a score
+    of 100 nats) included; what is left are ordinary scores, and the block tolerance holds as it does there."""
+    ks = [300 if b == 0 else 3 + b % 5 for b in range(B)]
+    attention_case(ctx, B=B, N=300, C=C, heads=heads, F=128, Lmax=1900, ks=ks,
+                   kv_lens=[1500 if b % 2 == 0 else 700 - b for b in range(B)], seed=97, q_gain=2.0,
+                   live_keys=(np.arange(750, 1500), value), rows=None if B == 1 else list(range(0, sum(ks), 7)),
+                   label=f"far above the reference, channel {value}, batch {B}")
+
+
+@pytest.mark.parametrize("C,heads", [(2048, 16), (1024, 16)])
+def test_attention_more_passes_than_the_table_holds(ctx, C, heads):
+    """More images than the CTAs' copy of the index offsets holds and more than 64 work items per CTA (pair):
+    the pass table is laid out several times."""
+    B = 310 if heads * 310 // (74 if C // heads == 128 else 148) >= 64 else 640
+    ks = [1 + (b % 3 == 0) for b in range(B)]
+    attention_case(ctx, B=B, N=2, C=C, heads=heads, F=64, Lmax=16, ks=ks, kv_lens=[b % 12 for b in range(B)], seed=103, q_gain=4.0,
+                   rows=list(range(0, sum(ks), 17)) + [sum(ks) - 1], half_keys_check=False, label=f"many images, head size {C // heads}")
 
 
 @pytest.mark.parametrize("C,heads", [(256, 2), (128, 2)])
