@@ -102,10 +102,13 @@ struct nova_launch_scope {
 
 // ---- programmatic dependent launch ---------------------------------------------------------------
 // The kernels of a block are launched with programmatic stream serialisation: each lets the next one start
-// as soon as all of its own CTAs have (pdl_launch_dependents, its first instruction), so that launch, barrier
-// and tensor-memory set-up and the next kernel's first CTAs overlap its tail. A kernel touches memory that
-// earlier launches write only after pdl_wait, which returns when the launch before it has completed with all its
-// writes visible; every CTA passes it, also those with nothing to do, so that completion stays transitive.
+// once all of its own CTAs have called pdl_launch_dependents or ended, so that launch, barrier and tensor-memory
+// set-up and the next kernel's first CTAs overlap its tail. The short kernels (LayerNorm, restore) call it first
+// thing, or the launch of the next would not be hidden (after their wait: a 16-layer generation 9540 -> 9730 us);
+// the GEMMs and the attention near their end. A kernel touches memory that earlier launches write only after
+// pdl_wait, which returns when the launch before it has completed with all its writes visible; every CTA passes
+// it, also those with nothing to do, so that completion stays transitive. That goes for weights too: a kernel
+// may start while one two launches back, of the caller's, is still writing them.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

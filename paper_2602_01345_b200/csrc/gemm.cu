@@ -440,7 +440,6 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();     // 0 = leader
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
-    pdl_launch_dependents();
     if (p.m_dev) pdl_wait();        // the row count is an earlier launch's
     if (EPI != NOVA_EPI_ENTROPY && p.m_dev && split_plan(true_rows(p), p.N, p.K / BK, caps).takes) return;     // the split kernel's problem
     const int num_kb = p.K / BK;
@@ -611,6 +610,8 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 ok = mbar_wait_warp(&acc_full[a], (uint32_t)(local >> 1) & 1, abort_flag, p.status);
                 if (!ok) break;
                 tc_fence_after();
+                // the next kernel is let in at the last tile (measured at the split kernel's trigger)
+                if (pair_entry(local + 1, pair, num_pairs, num_tiles, group) < 0) pdl_launch_dependents();
                 float* turn = (float*)(smem + L::kTurnOff + (warp - 2) * 4096);
                 if (row0 < M) {
 #pragma unroll
@@ -741,7 +742,6 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
                 const GemmParams p, const int pc, const int box, const SplitPlan plan_host, const SplitCaps caps)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    pdl_launch_dependents();
     if (p.m_dev) pdl_wait();        // the row count is an earlier launch's
     const int M = true_rows(p);
     const int num_kb = p.K / BK;
@@ -860,6 +860,11 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
         }
         __syncwarp();
         cluster_sync_all();          // every pair's main loop is over: the rings may be written
+        // The next kernel is let in when the last main loop is over: with the trigger at the start its first CTAs sat
+        // on the SMs this grid leaves free, and it ended later. With the same in the kernel for many tiles, us: a
+        // 16-layer 256x256 generation 9565 -> 9380 (9358 with the trigger right after the wait, but there the calls
+        // below gained less), 20x20 scale of one image 3148 -> 3097, last 64x64 scale 6775 -> 6665.
+        if ((c + num_clusters) * groups >= units) pdl_launch_dependents();
         if (warp >= 2 && active) {
             // token t of this CTA's 128 features (one per lane and tensor-memory lane quarter) to the pair that
             // completes it; the store of a warp is 128 contiguous bytes
