@@ -243,6 +243,40 @@ def test_attention_single_key_returns_its_value(ctx):
     assert err <= BLOCK_TOL
 
 
+@pytest.mark.parametrize("C,heads,key", [(256, 2, 26.0), (256, 4, 20.125)])
+@pytest.mark.parametrize("at", [0, 43, 88, 120])
+def test_attention_dominant_keys_of_the_first_tile_have_probability_one(ctx, C, heads, key, at):
+    """Eight keys of the first key tile score alike and about 2^53 to 2^58 above the others. Against the tile's
+    maximum their probability is 1, exact in bf16, wherever in the tile they lie, so the output is the mean of their
+    values, (1 + 5/8 2^-7) or (1 + 3/8 2^-7), rounded to bf16. (Against the maximum of the others it would be
+    a power of two times a mantissa that bf16 holds only to 1.6e-3, more than the 2^-10 from either mean to the
+    next rounding boundary.)"""
+    B, N, F, Lmax, dh, ks, kv_lens = 2, 40, 256, 512, C // heads, [40, 3], [300, 128]
+    wt = probe_weights(C, F, 73, q_zero=True, q_bias=16.0, heads=heads)
+    x = (synth.activations(B, N, C, 74, DEV).float() * 2.0 ** -20).to(torch.bfloat16)       # far below the output's rounding
+    k_cache, v_cache, _ = synth.kv_cache(B, Lmax, max(kv_lens), C, 75, DEV)
+    k_cache[:, :, 0:C:dh] = 0.0
+    k_cache[:, at:at + 8, 0:C:dh] = key
+    v_cache[:, at:at + 8] = 1.0
+    v_cache[:, at:at + 5, 0::2] += 2.0 ** -7
+    v_cache[:, at:at + 3, 1::2] += 2.0 ** -7
+    ent = torch.rand((B, N), generator=torch.Generator(device="cpu").manual_seed(7)).to(DEV)
+    M = sum(ks)
+    keep_idx = torch.empty(M, dtype=torch.int32, device=DEV)
+    prune_idx = torch.empty(B * N - M, dtype=torch.int32, device=DEV)
+    cu = torch.empty(B + 1, dtype=torch.int32, device=DEV)
+    nova.nova_select_topk(ctx, ent, torch.tensor(ks, dtype=torch.int32), keep_idx, prune_idx, cu, None)
+    shape = nova.BlockShape(B, N, C, heads, F, Lmax, M)
+    ctx.ensure_workspace(shape)
+    y = torch.empty((M, C), dtype=torch.bfloat16, device=DEV)
+    nova.nova_pruned_block_forward(ctx, nova.BlockWeights(wt, 1e-6), shape, x, keep_idx, cu, k_cache, v_cache,
+                                   torch.tensor(kv_lens, dtype=torch.int32, device=DEV), True, y)
+    assert ctx.device_status() == 0
+    want = np.ones((M, C), np.float32)
+    want[:, 0::2] += 2.0 ** -7
+    assert np.array_equal(f32(y), want)
+
+
 # ----------------------------------------------------------------- peaked rows: rescale, clamp, merge
 def _step_profile(n, lo=0.25, hi=4.0, at=None):
     at = n // 2 if at is None else at
