@@ -801,6 +801,9 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                     continue;
                 }
                 l_s[slot * 2 * BQ] = l_run;
+                // (only rows of this item may ask: those past its last one are the next image's, or whatever the
+                // buffer held, and must not decide how the others are rounded)
+                huge = huge && (int)rank * BQ + row < table[i].rows_valid;
                 if (!only && __any_sync(0xffffffffu, huge) && lane == 0) atomicOr(&redo_s, 1ull << i);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&l_full[slot]);

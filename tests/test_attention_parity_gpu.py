@@ -341,6 +341,73 @@ def test_attention_keys_with_vanishing_probability(ctx, C, heads):
                    q_gain=2.0, dead_keys=dead, label=f"vanishing probabilities, head size {C // heads}")
 
 
+@pytest.mark.parametrize("C,heads", [(256, 2), (256, 4)])
+@pytest.mark.parametrize("kv_len,Lmax", [(700, 1000), (1500, 1800)])
+def test_attention_of_an_image_does_not_depend_on_the_next_images_queries(ctx, C, heads, kv_len, Lmax):
+    """The last query block of an image also holds the next image's first rows, which score against the wrong
+    image's keys and are not written. Here only the second image's queries meet a channel that half of the first
+    image's keys carry, 85 nats and more above the others: the first image's output is the same bit for bit as
+    with ordinary queries there, in whole work items (700 keys) and in items shared by two (1500)."""
+    B, N, F, dh, seed, probe = 2, 200, 256, C // heads, 131, 17
+    ks = [100, 60]
+    wt = probe_weights(C, F, seed, q_gain=2.0)
+    wt["ln1_b"][probe] = 0.0
+    wt["w_qkv"][0:C:dh] = 0.0                    # the first channel of every head's query is 4 LayerNorm(x)[probe]
+    wt["w_qkv"][0:C:dh, probe] = 4.0
+    wt["b_qkv"][0:C:dh] = 0.0
+    k_cache, v_cache, _ = synth.kv_cache(B, Lmax, kv_len, C, seed + 2, DEV)
+    k_cache[0, kv_len // 2:kv_len, 0:C:dh] = 60.0
+    x = synth.activations(B, N, C, seed + 1, DEV)
+    rest = torch.arange(C, device=DEV) != probe
+    x[:, :, probe] = x[:, :, rest].float().mean(-1).to(torch.bfloat16)      # LayerNorm leaves next to nothing of it
+    ent = torch.rand((B, N), generator=torch.Generator(device="cpu").manual_seed(seed)).to(DEV)
+    M = sum(ks)
+    keep_idx = torch.empty(M, dtype=torch.int32, device=DEV)
+    prune_idx = torch.empty(B * N - M, dtype=torch.int32, device=DEV)
+    cu = torch.empty(B + 1, dtype=torch.int32, device=DEV)
+    nova.nova_select_topk(ctx, ent, torch.tensor(ks, dtype=torch.int32), keep_idx, prune_idx, cu, None)
+    shape = nova.BlockShape(B, N, C, heads, F, Lmax, M)
+    ctx.ensure_workspace(shape)
+    got = []
+    for extreme in (False, True):
+        if extreme:
+            x[1, :, probe] = 64.0
+        y = torch.full((M, C), float("nan"), dtype=torch.bfloat16, device=DEV)
+        nova.nova_pruned_block_forward(ctx, nova.BlockWeights(wt, 1e-6), shape, x, keep_idx, cu, k_cache.clone(),
+                                       v_cache.clone(), torch.full((B,), kv_len, dtype=torch.int32, device=DEV), True, y)
+        assert ctx.device_status() == 0 and torch.isfinite(y.float()).all()
+        got.append(y)
+    assert torch.equal(got[0][:ks[0]], got[1][:ks[0]])
+    assert not torch.equal(got[0][ks[0]:], got[1][ks[0]:])
+
+
+@pytest.mark.parametrize("C,heads", [(256, 2), (256, 4)])
+@pytest.mark.parametrize("M", [1, 127, 257])
+def test_device_count_does_not_depend_on_what_the_workspace_holds(ctx, C, heads, M):
+    """With the kept count on the device the launches are sized by a bound, and query rows between the count and
+    the bound are whatever the workspace held: NaN there and zeros there give the same bits."""
+    B, N, F, Lmax, kv_len, seed = 1, 300, 256, 1100, 700, 137
+    wt = nova.BlockWeights(probe_weights(C, F, seed, q_gain=4.0), 1e-6)
+    x = synth.activations(B, N, C, seed + 1, DEV)
+    k_cache, v_cache, _ = synth.kv_cache(B, Lmax, kv_len, C, seed + 2, DEV)
+    ent = torch.rand((B, N), generator=torch.Generator(device="cpu").manual_seed(seed)).to(DEV)
+    keep_idx = torch.zeros(N, dtype=torch.int32, device=DEV)
+    prune_idx = torch.empty(N - M, dtype=torch.int32, device=DEV)
+    cu = torch.empty(B + 1, dtype=torch.int32, device=DEV)
+    nova.nova_select_topk(ctx, ent, torch.tensor([M], dtype=torch.int32), keep_idx[:M], prune_idx, cu, None)
+    shape = nova.BlockShape(B, N, C, heads, F, Lmax, N)
+    got = []
+    for bits in (0, 0x7fc0):          # bf16 zero, bf16 NaN
+        ws = torch.full((nova.nova_block_workspace_bytes(shape) // 2 + 128,), bits, dtype=torch.int16, device=DEV)
+        ctx.set_workspace(ws.view(torch.uint8))
+        y = torch.zeros((N, C), dtype=torch.bfloat16, device=DEV)
+        nova.nova_pruned_block_forward_device(ctx, wt, shape, x, keep_idx, cu, k_cache.clone(), v_cache.clone(),
+                                              torch.full((B,), kv_len, dtype=torch.int32, device=DEV), True, y)
+        assert ctx.device_status() == 0 and torch.isfinite(y.float()).all()
+        got.append(y)
+    assert torch.equal(got[0], got[1])
+
+
 # ------------------------------------------------- block variants: rotary embedding, QK norm, cross-attention
 def _rope_tables(h, w, dh, seed):
     """Axial 2-D rotary tables for an h x w token grid: the first half of a head's channel pairs turns
