@@ -9,7 +9,7 @@
 //   warp 1        tcgen05.mma issuer (the pair's leader issues for both): O += P_u V_u, then S_{u+3}
 //   warps 4-7     epilogue: O / l to bf16, or a partial result, while the next rows are under way
 //   warps 8-15    softmax, two warpgroups that take the key tiles in turn, one query row per thread: the row of
-//                 S from tensor memory to registers, P = 2^((s - m) * scale) packed to bf16 and stored over the
+//                 S from tensor memory to registers, P = 2^((s - m) * scale - 48) packed to bf16 and stored over the
 //                 S columns, from where O += P V takes it as its A operand
 // Tensor memory holds O and three S buffers, so S runs up to three tiles ahead of O += P V, across the
 // boundary between two work items: neither the latency of a softmax nor its hand-overs are on the tensor
@@ -20,9 +20,12 @@
 // share their exponent range, so a reference that is not the running maximum costs no precision, and it cancels
 // in the final division by l. (The whole tile's, not that of some of its keys: a key that holds most of a row's
 // weight then has probability 1 where it lies in that tile, which bf16 holds exactly. Over the last 32 keys alone the
-// attention's error against 64 bits was 2.76e-3 instead of 2.47e-3 for peaked rows over 217 keys.) Only a score about
-// 2^80 above the reference (seen as a huge row sum) could get near the end of that range; work items in which one
-// appears are run once more at the end, with a first pass over the keys that finds the rows' true maxima.
+// attention's error against 64 bits was 2.76e-3 instead of 2.47e-3 for peaked rows over 217 keys.) They are scaled
+// by 2^-kHeadroom, exactly, because what follows can be far above the first tile and never far below what matters.
+// Only a score about 2^128 (88 nats) above the reference, seen as a huge row sum, could get near the end of the
+// range; work items in which one appears are run once more at the end, with a first pass over the keys that finds the
+// rows' true maxima. A launch in which that happens to all items takes 2.6 times as long (4 x 2048 rows x 8473 keys, 16
+// heads x 128: 428 -> 1110 us).
 // K tiles are K-major operands; V tiles are the MN-major B operand, i.e. V is consumed exactly as it lies in
 // the cache ([keys, dh]). The last key tile ends at the last key and overlaps the one before it (its repeated
 // columns are masked; rows before the first key read as zeros), so no row past the end is ever loaded.
@@ -47,9 +50,11 @@ constexpr int BKV = 128;       // keys per tile
 constexpr int kBufs = 3;       // S buffers in tensor memory
 constexpr int kThreads = 512;  // warpgroups: producer + issuer (+2 idle warps), epilogue, softmax 0, softmax 1
 constexpr int kSlabBytes = 128 * 128;   // [128 rows][64 bf16]
-// A row's sum of probabilities over one key tile at or above this (or NaN) means a score about
-// 2^80 above the row's reference maximum. Far below anything that could overflow fp32 in l or O
-// (sums over 2^16 keys, values up to 2^20), far above anything ordinary data reaches.
+// The probability of a score equal to the reference is 2^-kHeadroom. A row's sum of probabilities over one key tile at
+// or above kHugeSum (or NaN) means a score about 2^(80 + kHeadroom) above the reference. That is far below
+// anything that could overflow fp32 in l or O (sums over 2^16 keys, values up to 2^20), and at the other end
+// probabilities down to 2^-78 of the reference's, and O of values down to 2^-54, keep all their bits.
+constexpr float kHeadroom = 48.f;
 constexpr float kHugeSum = 1.2089258e24f;   // 2^80
 // Passes whose row sums and references are kept. A warpgroup that reaches pass i has done its last tile before
 // that, tile t >= i - 2 if passes are single tiles; S of it was issued after O += P V of tile t - kBufs, which
@@ -740,10 +745,10 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
                         mbar_wait_warp(&m_full[slot], (uint32_t)(np / kSlots) & 1u, abort_flag, p.status);
                         m_ref = m_s[slot * BQ];
                     }
-                    // p = 2^(s*c - m*c): 16 registers of bf16 pairs per chunk, written over columns of S that have
+                    // p = 2^(s*c - m*c - kHeadroom): 16 registers of bf16 pairs per chunk, written over columns of S that have
                     // been read
                     const uint64_t c2 = pack_f32x2(c, c);
-                    const uint64_t nm2 = pack_f32x2(-m_ref * c, -m_ref * c);
+                    const uint64_t nm2 = pack_f32x2(fmaf(-m_ref, c, -kHeadroom), fmaf(-m_ref, c, -kHeadroom));
                     uint64_t lsum_a = pack_f32x2(0.f, 0.f), lsum_b = lsum_a;
                     // (chunks of which no column counts take zeros and no arithmetic: three of four in the smallest calls,
                     // 7.1 -> 6.3 us for eight images with one kept token each)

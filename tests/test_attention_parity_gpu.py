@@ -408,6 +408,51 @@ def test_device_count_does_not_depend_on_what_the_workspace_holds(ctx, C, heads,
     assert torch.equal(got[0], got[1])
 
 
+@pytest.mark.parametrize("C,heads", [(256, 2), (256, 4)])
+@pytest.mark.parametrize("nats", [60.0, 84.0])
+@pytest.mark.parametrize("kv_len,Lmax", [(700, 1000), (1500, 1800)])
+def test_attention_wide_row_leaves_the_other_rows_of_its_item_alone(ctx, C, heads, nats, kv_len, Lmax):
+    """One row scores the second half of the prior keys 60 or 84 nats (2^86, 2^121) above its first key tile; the
+    other rows do not see the channel that does it, because their query is exactly zero there. Both are within what is
+    carried against the first tile's maximum (2^128): the work item is not run again with other references, and
+    the other rows' outputs are the same bit for bit as without that channel."""
+    N, F, dh, seed, M, hot = 200, 256, C // heads, 151, 110, 90
+    p0, p1 = 17, 101
+    wt = probe_weights(C, F, seed, q_gain=2.0)
+    wt["ln1_g"][[p0, p1]] = 1.0
+    wt["ln1_b"][[p0, p1]] = 0.0
+    wt["w_qkv"][0:C:dh] = 0.0                    # a head's first query channel: 4 (LayerNorm(x)[p0] - LayerNorm(x)[p1])
+    wt["w_qkv"][0:C:dh, p0] = 4.0
+    wt["w_qkv"][0:C:dh, p1] = -4.0
+    wt["b_qkv"][0:C:dh] = 0.0
+    k_cache, v_cache, _ = synth.kv_cache(1, Lmax, kv_len, C, seed + 2, DEV)
+    k_cache[:, :, 0:C:dh] = 0.0
+    x = synth.activations(1, N, C, seed + 1, DEV)
+    x[:, :, p1] = x[:, :, p0]
+    ent = torch.rand((1, N), generator=torch.Generator(device="cpu").manual_seed(seed)).to(DEV)
+    keep_idx = torch.empty(M, dtype=torch.int32, device=DEV)
+    prune_idx = torch.empty(N - M, dtype=torch.int32, device=DEV)
+    cu = torch.empty(2, dtype=torch.int32, device=DEV)
+    nova.nova_select_topk(ctx, ent, torch.tensor([M], dtype=torch.int32), keep_idx, prune_idx, cu, None)
+    token = int(keep_idx[hot])
+    x[0, token, p0], x[0, token, p1] = 64.0, -64.0
+    h = torch.nn.functional.layer_norm(x[0, token].float(), (C,), eps=1e-6)
+    q0 = 4.0 * float(h[p0] - h[p1])
+    shape = nova.BlockShape(1, N, C, heads, F, Lmax, M)
+    ctx.ensure_workspace(shape)
+    got = []
+    for value in (0.0, nats * dh ** 0.5 / q0):
+        k = k_cache.clone()
+        k[:, kv_len // 2:kv_len, 0:C:dh] = value
+        y = torch.full((M, C), float("nan"), dtype=torch.bfloat16, device=DEV)
+        nova.nova_pruned_block_forward(ctx, nova.BlockWeights(wt, 1e-6), shape, x, keep_idx, cu, k, v_cache.clone(),
+                                       torch.tensor([kv_len], dtype=torch.int32, device=DEV), True, y)
+        assert ctx.device_status() == 0 and torch.isfinite(y.float()).all()
+        got.append(y)
+    same = (got[0] == got[1]).all(dim=1)
+    assert not same[hot] and int(same.sum()) == M - 1
+
+
 # ------------------------------------------------- block variants: rotary embedding, QK norm, cross-attention
 def _rope_tables(h, w, dh, seed):
     """Axial 2-D rotary tables for an h x w token grid: the first half of a head's channel pairs turns
