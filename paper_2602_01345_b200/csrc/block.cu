@@ -36,10 +36,10 @@ struct LnModArgs {
 // variance and the normalisation, so x is read once and out written once.
 constexpr int kLnWarps = 8;
 
-__device__ __forceinline__ uint4 ld_nc_stream(const uint4* p)
+__device__ __forceinline__ uint4 ld_stream(const uint4* p)
 {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
@@ -55,9 +55,8 @@ __device__ __forceinline__ float warp_sum(float v)
 // waves of load-then-compute and sat at 0.41 of the HBM peak.
 template <int VEC, bool MAPS, bool MOD>
 __global__ void __launch_bounds__(kLnWarps * 32, 3)
-layernorm_rows(const uint4* __restrict__ x, const uint4* __restrict__ gamma, const uint4* __restrict__ beta,
-               float eps, int M, const int32_t* __restrict__ m_dev, int vec_per_row, uint4* __restrict__ out,
-               const RowMapArgs maps, const LnModArgs mod)
+layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps, int M, const int32_t* m_dev, int vec_per_row,
+               uint4* __restrict__ out, const RowMapArgs maps, const LnModArgs mod)
 {
     pdl_launch_dependents();
     // Gain and bias are needed last and come from HBM (each layer has its own): brought to L2 while the launch before
@@ -105,7 +104,7 @@ layernorm_rows(const uint4* __restrict__ x, const uint4* __restrict__ gamma, con
 #pragma unroll
     for (int i = 0; i < VEC; ++i) {
         const int c = i * 32 + lane;
-        raw[i] = (c < vec_per_row) ? ld_nc_stream(xr + c) : make_uint4(0, 0, 0, 0);
+        raw[i] = (c < vec_per_row) ? ld_stream(xr + c) : make_uint4(0, 0, 0, 0);
     }
     float sum0 = 0.f, sum1 = 0.f;
 #pragma unroll
@@ -171,10 +170,10 @@ layernorm_rows(const uint4* __restrict__ x, const uint4* __restrict__ gamma, con
 // consecutive channels, i.e. whole pairs.
 template <int DH>
 __global__ void __launch_bounds__(256)
-qk_transform_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k_cache, const int32_t* __restrict__ kv_row,
-                    const int32_t* __restrict__ keep_idx, int M, const int32_t* __restrict__ m_dev, int C, int n_heads,
-                    const __nv_bfloat16* __restrict__ gain_q, const __nv_bfloat16* __restrict__ gain_k, float eps,
-                    const float* __restrict__ rope_cos, const float* __restrict__ rope_sin)
+qk_transform_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k_cache, const int32_t* kv_row,
+                    const int32_t* keep_idx, int M, const int32_t* m_dev, int C, int n_heads,
+                    const __nv_bfloat16* gain_q, const __nv_bfloat16* gain_k, float eps,
+                    const float* rope_cos, const float* rope_sin)
 {
     pdl_launch_dependents();
     pdl_wait();

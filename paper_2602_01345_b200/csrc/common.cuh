@@ -108,7 +108,9 @@ struct nova_launch_scope {
 // the GEMMs and the attention near their end. A kernel touches memory that earlier launches write only after
 // pdl_wait, which returns when the launch before it has completed with all its writes visible; every CTA passes
 // it, also those with nothing to do, so that completion stays transitive. That goes for weights too: a kernel
-// may start while one two launches back, of the caller's, is still writing them.
+// may start while one two launches back, of the caller's, is still writing them. For the same reason these kernels
+// read with ordinary loads only: ld.global.nc, also as the compiler makes it of a `const T* __restrict__` parameter, is
+// for memory that nobody writes while the kernel lives, and the wait does not order it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -12,10 +12,10 @@ namespace {
 
 constexpr int kWarpsPerBlock = 8;
 
-__device__ __forceinline__ uint4 ld_nc(const uint4* p)
+__device__ __forceinline__ uint4 ld_stream(const uint4* p)
 {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
@@ -35,9 +35,8 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi)
 }
 
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
-restore_kernel(const uint4* __restrict__ x_in, const uint4* __restrict__ y_kept,
-               const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ prune_idx,
-               const int32_t* __restrict__ cu_keep, const uint4* __restrict__ cache_prev,
+restore_kernel(const uint4* x_in, const uint4* y_kept, const int32_t* keep_idx, const int32_t* prune_idx,
+               const int32_t* cu_keep, const uint4* cache_prev,
                int hp, int wp, int h, int w, int vec_per_row, int B, int M, bool m_on_device, bool pruned_only,
                uint4* __restrict__ x_out, uint4* __restrict__ cache_out)
 {
@@ -63,10 +62,10 @@ restore_kernel(const uint4* __restrict__ x_in, const uint4* __restrict__ y_kept,
         const uint4* ysrc = y_kept + r * vec_per_row;
         const uint4* xsrc = x_in + row * vec_per_row;
         for (int v = lane; v < vec_per_row; v += 32) {
-            const uint4 yv = ld_nc(ysrc + v);
+            const uint4 yv = ld_stream(ysrc + v);
             st_cs(x_out + row * vec_per_row + v, yv);
             if (cache_out) {
-                const uint4 xv = ld_nc(xsrc + v);
+                const uint4 xv = ld_stream(xsrc + v);
                 const uint32_t yw[4] = {yv.x, yv.y, yv.z, yv.w}, xw[4] = {xv.x, xv.y, xv.z, xv.w};
                 uint32_t o[4];
 #pragma unroll
@@ -106,7 +105,7 @@ restore_kernel(const uint4* __restrict__ x_in, const uint4* __restrict__ y_kept,
     const uint4* c11 = cache_prev + (((long)b * hp + y1) * wp + x1) * vec_per_row;
     const long row = (long)b * N + i;
     for (int v = lane; v < vec_per_row; v += 32) {
-        const uint4 xv = ld_nc(x_in + row * vec_per_row + v);
+        const uint4 xv = ld_stream(x_in + row * vec_per_row + v);
         const uint4 a = c00[v], bq = c01[v], c = c10[v], d = c11[v];
         const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
         const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {bq.x, bq.y, bq.z, bq.w};

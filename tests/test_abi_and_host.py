@@ -121,3 +121,21 @@ def test_keep_ratios_worked_example_and_errors():
         nova.nova_keep_ratios(nova.SchedParams(tau=0.0), 8, 1, 256, torch.from_numpy(hs[:, :8]))
     with pytest.raises(nova.NovaError):
         nova.nova_keep_ratios(nova.SchedParams(t_est=1), 8, 1, 256, torch.from_numpy(hs[:, :8]))
+
+
+def test_overlapping_kernels_use_no_non_coherent_loads():
+    """Kernels launched with programmatic stream serialisation live while the launch before them still writes.
+    ld.global.nc (which a `const T* __restrict__` parameter or __ldg lets the compiler use) is only for memory that nobody writes
+    during the kernel's life, and griddepcontrol.wait does not order it."""
+    csrc = os.path.join(ROOT, "paper_2602_01345_b200", "csrc")
+    seen = set()
+    for name in sorted(os.listdir(csrc)):
+        text = re.sub(r"//[^\n]*|__(launch_bounds|cluster_dims)__\([^()]*\)", "", open(os.path.join(csrc, name)).read())
+        if "nova_launch_pdl(" not in text or name == "common.cuh":
+            continue
+        assert "ld.global.nc" not in text and "__ldg" not in text, name
+        for m in re.finditer(r"__global__[^;{]*?(\w+)\(([^{;]*)\)\s*\{", text):
+            if "pdl_wait();" in text[m.end():]:
+                assert not re.search(r"const\s+[\w ]+\*\s*__restrict__", m.group(2)), (name, m.group(1))
+                seen.add(m.group(1))
+    assert {"layernorm_rows", "qk_transform_kernel", "restore_kernel", "gemm_bf16_tn_pair", "gemm_bf16_split", "attention_kernel"} <= seen
