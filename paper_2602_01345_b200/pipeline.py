@@ -87,10 +87,8 @@ class PrunedScaleRunner:
         # The layers' logits are inputs of the scale, not results of its layers: the entropy maps of a whole
         # group of layers are taken in one launch, their means cross to the host in one copy, one
         # synchronisation decides the keep counts of all its layers and one launch selects for them; all of
-        # it and the layers themselves are one native call. With resident logits the group is the whole
-        # scale; while logits are still being uploaded a small group lets the blocks of the first layers
-        # run under the uploads of the later ones.
-        group = self.L if logits_ready is None else min(self.L, 4)
+        # it and the layers themselves are one native call.
+        group = self._group(logits_ready)
         hbar_scale = hbar_scale.to("cpu", torch.float32).contiguous()
         self.call.set_layers(self.weights, self.modulation, self.k_caches, self.v_caches, self.kv_len, self.cache_prev, self.cache_out)
         self.call.set_logits(layer_logits)
@@ -106,48 +104,58 @@ class PrunedScaleRunner:
         self.last_keep = list(self.call.keep.clone().unbind(0))
         return x, self.last_keep
 
+    def _group(self, logits_ready) -> int:
+        """Layers whose keep counts are decided together. With resident logits the whole scale; while logits are
+        still being uploaded a few, so that the blocks of the first layers run under the uploads of the later ones."""
+        return self.L if logits_ready is None else min(self.L, 4)
+
     def _run_layer_by_layer(self, x_in, layer_logits, sched, t, hbar_scale, append_kv, st, logits_ready, select_ent, layer_hook):
         """The same scale call by call, as one nova_pruned_layer_forward (fused_restore) or block + restore
         per layer, with the hook, if there is one, around every layer."""
         ctx, B, N, L = self.ctx, self.B, self.N, self.L
-        if logits_ready is not None:
-            for e in logits_ready:
-                st.wait_event(e)
-        nv.nova_scale_entropy_layers(ctx, layer_logits, self.ent, self.mean, stream=st)
-        self.mean_host.copy_(self.mean, non_blocking=True)
-        st.synchronize()
-        keeps = list(nv.nova_keep_ratios_layers(sched, t, N, hbar_scale, self.mean_host.t())["keep"].unbind(0))
-        if select_ent is None:
-            nv.nova_select_topk_grouped(ctx, self.ent, torch.stack(keeps), self.keep_idx, self.prune_idx, self.cu_keep, None, stream=st)
+        group = self._group(logits_ready)
+        keeps = []
         x = x_in
-        for j in range(L):
-            keep = keeps[j]
-            M = int(keep.sum())
-            keep_idx, prune_idx, cu_keep = self.keep_idx[j, :M], self.prune_idx[j, : B * N - M], self.cu_keep[j]
-            if select_ent is not None:
-                nv.nova_select_topk(ctx, select_ent, keep, keep_idx, prune_idx, cu_keep, None, stream=st)
-            shape = nv.BlockShape(B, N, self.C, self.n_heads, self.F, self.Lmax, M)
-            x_out = self.x_buf[(j & 1) ^ (x.data_ptr() == self.x_buf[j & 1].data_ptr())]
-            cache_out = self.cache_out[j] if self.cache_out is not None else None
-            info = dict(x_in=x, x_out=x_out, cache_out=cache_out, keep=keep, keep_idx=keep_idx, prune_idx=prune_idx,
-                        cu_keep=cu_keep, k_cache=self.k_caches[j], v_cache=self.v_caches[j], kv_len=self.kv_len[j],
-                        cache_prev=self.cache_prev[j], ent=self.ent[j], stream=st)
-            if layer_hook is not None:
-                layer_hook("before", j, info)
-            mod = self.modulation[j] if self.modulation else None
-            if self.fused_restore:
-                nv.nova_pruned_layer_forward(ctx, self.weights[j], mod, shape, x, keep_idx, prune_idx, cu_keep, self.k_caches[j],
-                                             self.v_caches[j], self.kv_len[j], append_kv, self.cache_prev[j],
-                                             self.h, self.w, x_out, cache_out, stream=st)
-            else:
-                y = self.y_kept[:M]
-                nv.nova_pruned_block_forward_adaln(ctx, self.weights[j], mod, shape, x, keep_idx, cu_keep, self.k_caches[j],
-                                                   self.v_caches[j], self.kv_len[j], append_kv, y, stream=st)
-                nv.nova_restore_from_cache(ctx, x, y, keep_idx, prune_idx, cu_keep, self.cache_prev[j], self.h, self.w, x_out,
-                                           cache_out, stream=st)
-            if layer_hook is not None:
-                layer_hook("after", j, info)
-            x = x_out
+        for g0 in range(0, L, group):
+            g1 = min(L, g0 + group)
+            if logits_ready is not None:
+                for e in logits_ready[g0:g1]:
+                    st.wait_event(e)
+            nv.nova_scale_entropy_layers(ctx, layer_logits[g0:g1], self.ent[g0:g1], self.mean[g0:g1], stream=st)
+            self.mean_host[g0:g1].copy_(self.mean[g0:g1], non_blocking=True)
+            st.synchronize()
+            keeps += nv.nova_keep_ratios_layers(sched, t, N, hbar_scale, self.mean_host[:g1].t())["keep"][g0:].unbind(0)
+            if select_ent is None:
+                nv.nova_select_topk_grouped(ctx, self.ent[g0:g1], torch.stack(keeps[g0:]), self.keep_idx[g0:g1],
+                                            self.prune_idx[g0:g1], self.cu_keep[g0:g1], None, stream=st)
+            for j in range(g0, g1):
+                keep = keeps[j]
+                M = int(keep.sum())
+                keep_idx, prune_idx, cu_keep = self.keep_idx[j, :M], self.prune_idx[j, : B * N - M], self.cu_keep[j]
+                if select_ent is not None:
+                    nv.nova_select_topk(ctx, select_ent, keep, keep_idx, prune_idx, cu_keep, None, stream=st)
+                shape = nv.BlockShape(B, N, self.C, self.n_heads, self.F, self.Lmax, M)
+                x_out = self.x_buf[(j & 1) ^ (x.data_ptr() == self.x_buf[j & 1].data_ptr())]
+                cache_out = self.cache_out[j] if self.cache_out is not None else None
+                info = dict(x_in=x, x_out=x_out, cache_out=cache_out, keep=keep, keep_idx=keep_idx, prune_idx=prune_idx,
+                            cu_keep=cu_keep, k_cache=self.k_caches[j], v_cache=self.v_caches[j], kv_len=self.kv_len[j],
+                            cache_prev=self.cache_prev[j], ent=self.ent[j], stream=st)
+                if layer_hook is not None:
+                    layer_hook("before", j, info)
+                mod = self.modulation[j] if self.modulation else None
+                if self.fused_restore:
+                    nv.nova_pruned_layer_forward(ctx, self.weights[j], mod, shape, x, keep_idx, prune_idx, cu_keep, self.k_caches[j],
+                                                 self.v_caches[j], self.kv_len[j], append_kv, self.cache_prev[j],
+                                                 self.h, self.w, x_out, cache_out, stream=st)
+                else:
+                    y = self.y_kept[:M]
+                    nv.nova_pruned_block_forward_adaln(ctx, self.weights[j], mod, shape, x, keep_idx, cu_keep, self.k_caches[j],
+                                                       self.v_caches[j], self.kv_len[j], append_kv, y, stream=st)
+                    nv.nova_restore_from_cache(ctx, x, y, keep_idx, prune_idx, cu_keep, self.cache_prev[j], self.h, self.w, x_out,
+                                               cache_out, stream=st)
+                if layer_hook is not None:
+                    layer_hook("after", j, info)
+                x = x_out
         self.last_keep = keeps
         return x, keeps
 

@@ -1247,6 +1247,54 @@ def test_scale_in_one_call_equals_layer_by_layer(ctx, L, grouped, modulated):
         assert torch.equal(p, q)
 
 
+def _small_scale(ctx, L, B=2, h=9, w=7, C=256, heads=4, V=1024, prior=40, **kw):
+    """A scale of L small layers over 40 prior keys: (runner, x_in, logits, history of 8 scales)."""
+    from paper_2602_01345_b200 import pipeline
+    N, t = h * w, 8
+    ks, vs = zip(*[synth.kv_cache(B, prior + N, prior, C, 50 + 2 * j, DEV)[:2] for j in range(L)])
+    args = dict(weights=[synth.block_weights(C, 512, 100 + j, DEV) for j in range(L)], n_heads=heads, B=B, h=h, w=w, Lmax=prior + N,
+                k_caches=list(ks), v_caches=list(vs), kv_len=torch.full((L, B), prior, dtype=torch.int32, device=DEV),
+                cache_prev=[synth.residual_cache(B, 5, 4, C, 70 + j, DEV) for j in range(L)])
+    a = synth.smooth_temperature_field(B, h, w, 5, device=DEV)
+    logits = [synth.logits_from_temperature(a * (1 + 0.1 * j), V, 20 + j) for j in range(L)]
+    return (pipeline.PrunedScaleRunner(ctx, **{**args, **kw}), synth.activations(B, N, C, 7, DEV), logits,
+            torch.linspace(2.0, 7.0, t).repeat(B, 1).contiguous())
+
+
+@pytest.mark.parametrize("form", ["native", "hook", "select_ent"])
+def test_layers_run_under_the_upload_of_later_layers(ctx, form):
+    """With logits_ready no form waits for the last layers' logits before it has issued the first layers."""
+    from paper_2602_01345_b200 import pipeline
+    runner, x_in, logits, hbar = _small_scale(ctx, L=6)
+    sched = nova.SchedParams(force_act_scale=8)
+    want, _ = runner.run_scale(x_in, logits, sched, 8, hbar, append_kv=False)
+    want = want.clone()
+    ready = [torch.cuda.Event() for _ in logits]
+    for e in ready:
+        e.record()
+    launches, waited = [], []
+
+    class Stream(torch.cuda.Stream):
+        def wait_event(self, event):
+            if event in ready:
+                waited.append(ready.index(event))
+                launches.append(pipeline.launch_count(ctx))
+            super().wait_event(event)
+
+    stream = Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    kw = {"hook": dict(layer_hook=lambda stage, j, info: None), "native": {},
+          "select_ent": dict(select_ent=runner.ent[0].clone())}[form]
+    torch.cuda.synchronize()
+    got, _ = runner.run_scale(x_in, logits, sched, 8, hbar, append_kv=False, stream=stream, logits_ready=ready, **kw)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0 and waited == list(range(6))
+    per_layer = 8                       # LayerNorm, QKV, attention, projection, LayerNorm, FC1, FC2, restore
+    assert launches[4] - launches[3] >= 4 * per_layer
+    if form != "select_ent":
+        assert torch.equal(got, want)
+
+
 def test_selection_on_one_scale_map_gives_nested_sets(ctx):
     """The other reading of how layers get their entropy map: one map per scale, selected on by every
     layer with that layer's keep count. Kept sets of layers with fewer kept tokens are subsets of
