@@ -122,7 +122,8 @@ class PrunedScaleRunner:
                 for e in logits_ready[g0:g1]:
                     st.wait_event(e)
             nv.nova_scale_entropy_layers(ctx, layer_logits[g0:g1], self.ent[g0:g1], self.mean[g0:g1], stream=st)
-            self.mean_host[g0:g1].copy_(self.mean[g0:g1], non_blocking=True)
+            with torch.cuda.stream(st):
+                self.mean_host[g0:g1].copy_(self.mean[g0:g1], non_blocking=True)
             st.synchronize()
             keeps += nv.nova_keep_ratios_layers(sched, t, N, hbar_scale, self.mean_host[:g1].t())["keep"][g0:].unbind(0)
             if select_ent is None:
@@ -228,7 +229,8 @@ class MultiScaleRunner:
             runner.call.set_scale_logits(scale_logits, ent, mean, torch.empty((B,), dtype=torch.float32, pin_memory=True))
         else:
             nv.nova_scale_entropy(self.ctx, scale_logits, ent, mean, stream=st)
-            hbar = torch.cat([self.hbar_scale, mean.cpu().view(B, 1)], dim=1).contiguous()
+            with torch.cuda.stream(st):
+                hbar = torch.cat([self.hbar_scale, mean.cpu().view(B, 1)], dim=1).contiguous()
         self.hbar_scale = hbar
         x_out, keeps = runner.run_scale(x_in, layer_logits, sched, t, hbar, stream=st, layer_hook=layer_hook)
         self.res_cache = [c.view(B, side, side, self.C) for c in runner.cache_out]

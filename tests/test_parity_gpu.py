@@ -1295,6 +1295,50 @@ def test_layers_run_under_the_upload_of_later_layers(ctx, form):
         assert torch.equal(got, want)
 
 
+def test_hook_form_takes_its_keep_counts_from_the_stream_it_runs_on(ctx):
+    """On a stream that is still busy the means have to be read behind the entropy maps, not at once from the
+    current stream: the keep counts equal the native form's, which follow the means of this call."""
+    runner, x_in, logits, hbar = _small_scale(ctx, L=3)
+    sched = nova.SchedParams(force_act_scale=8)
+    _, want = runner.run_scale(x_in, logits, sched, 8, hbar, append_kv=False)
+    runner.mean_host.fill_(1.0)
+    runner.mean.copy_(torch.tensor([1.0, 3.0, 0.5], device=DEV).view(3, 1).expand(3, 2))
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        torch.cuda._sleep(20_000_000)                # about 10 ms
+    _, keeps = runner.run_scale(x_in, logits, sched, 8, hbar, append_kv=False, stream=stream,
+                                layer_hook=lambda stage, j, info: None)
+    torch.cuda.synchronize()
+    assert torch.equal(torch.stack(keeps), torch.stack(want))
+
+
+def test_generation_history_is_read_from_the_stream_it_runs_on(ctx):
+    """The same for the scale's own mean entropy, which MultiScaleRunner appends to its history."""
+    from paper_2602_01345_b200 import pipeline
+    weights = [synth.block_weights(256, 512, 100, DEV)]
+    a = synth.smooth_temperature_field(2, 4, 4, 5, device=DEV)
+    logits = synth.logits_from_temperature(a, 1024, 20)
+    x_in = synth.activations(2, 16, 256, 7, DEV)
+    history = []
+    for busy in (False, True):
+        gen = pipeline.MultiScaleRunner(ctx, weights, 4, 2, (4,))
+        stream = torch.cuda.Stream()
+        stale = [torch.full((2,), 99.0, device=DEV) for _ in range(8)]       # what freshly allocated means will hold
+        torch.cuda.synchronize()
+        del stale
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(20_000_000 if busy else 1)
+        if not busy:
+            torch.cuda.synchronize()
+        gen.run_scale(1, x_in, logits, [logits], nova.SchedParams(), stream=stream, layer_hook=lambda stage, j, info: None)
+        torch.cuda.synchronize()
+        history.append(gen.hbar_scale)
+    _, mean = gpu_entropy(ctx, logits)
+    for h in history:
+        assert torch.equal(h[:, 0], mean.cpu())
+
+
 def test_selection_on_one_scale_map_gives_nested_sets(ctx):
     """The other reading of how layers get their entropy map: one map per scale, selected on by every
     layer with that layer's keep count. Kept sets of layers with fewer kept tokens are subsets of
