@@ -690,11 +690,13 @@ class ScaleCall:
         self._scale_buffers = (ent, mean, mean_host)
 
     def run(self, sched: SchedParams, t: int, hbar_scale, x_in, first: int, count: int, append_kv: bool, stream=None):
-        assert hbar_scale.dtype == torch.float32 and not hbar_scale.is_cuda and hbar_scale.shape == (self.shape.B, t)
-        assert x_in.dtype == torch.bfloat16 and x_in.numel() == self.shape.B * self.shape.N * self.shape.C
         io = self.io
-        io.hbar_scale, io.x_in = _ptr(hbar_scale), _ptr(x_in)
-        cs = sched._c()
-        self.ctx.check(_lib.nova_pruned_scale_forward(self.ctx.handle, C.byref(self.layers), C.byref(io), C.byref(self.shape),
-                                                      C.byref(cs), t, first, count, int(bool(append_kv)), _stream(stream)))
-        io.scale_logits = None
+        try:
+            assert hbar_scale.dtype == torch.float32 and not hbar_scale.is_cuda and hbar_scale.shape == (self.shape.B, t)
+            assert x_in.dtype == torch.bfloat16 and x_in.numel() == self.shape.B * self.shape.N * self.shape.C
+            io.hbar_scale, io.x_in = _ptr(hbar_scale), _ptr(x_in)
+            cs = sched._c()
+            self.ctx.check(_lib.nova_pruned_scale_forward(self.ctx.handle, C.byref(self.layers), C.byref(io), C.byref(self.shape),
+                                                          C.byref(cs), t, first, count, int(bool(append_kv)), _stream(stream)))
+        finally:
+            io.scale_logits = None      # of this pass only, whether or not it went through

@@ -6,6 +6,7 @@ import os
 import re
 
 import numpy as np
+import pytest
 import torch
 
 import oracle
@@ -139,3 +140,36 @@ def test_overlapping_kernels_use_no_non_coherent_loads():
                 assert not re.search(r"const\s+[\w ]+\*\s*__restrict__", m.group(2)), (name, m.group(1))
                 seen.add(m.group(1))
     assert {"layernorm_rows", "qk_transform_kernel", "restore_kernel", "gemm_bf16_tn_pair", "gemm_bf16_split", "attention_kernel"} <= seen
+
+
+def _scale_call(B=2, N=6, C=64, L=3):
+    """A ScaleCall on host memory without a context: its tables can be looked at, and every native call is refused."""
+    from paper_2602_01345_b200 import binding as nv
+
+    class NoContext:
+        handle = None
+
+        def check(self, status):
+            if status:
+                raise nova.NovaError(status, "refused")
+
+    z = lambda *s, dtype=torch.float32: torch.zeros(s, dtype=dtype)  # noqa: E731
+    i32, bf16 = torch.int32, torch.bfloat16
+    call = nv.ScaleCall(NoContext(), nova.BlockShape(B, N, C, 1, 64, 32, B * N), 2, 3, L, z(L, B, N), z(L, B), z(L, B), z(L, B * N, dtype=i32),
+                        z(L, B * N, dtype=i32), z(L, B + 1, dtype=i32), [z(B, N, C, dtype=bf16) for _ in range(2)])
+    weights = [type("W", (), {"c": nv._BlockWeights()}) for _ in range(L)]
+    caches = [z(B, 32, C, dtype=bf16) for _ in range(L)]
+    layers = dict(weights=weights, modulation=None, k_caches=caches, v_caches=caches, kv_len=z(L, B, dtype=i32),
+                  cache_prev=[z(B, 2, 2, C, dtype=bf16) for _ in range(L)], cache_out=None)
+    return call, layers
+
+
+def test_scale_call_forgets_the_scale_logits_of_a_pass_that_failed():
+    call, layers = _scale_call()
+    call.set_layers(**layers)
+    logits = torch.zeros((2, 6, 32), dtype=torch.bfloat16)
+    call.set_logits([logits] * 3)
+    call.set_scale_logits(logits, torch.zeros(2, 6), torch.zeros(2), torch.zeros(2))
+    with pytest.raises(nova.NovaError):
+        call.run(nova.SchedParams(), 1, torch.zeros(2, 1), torch.zeros((2, 6, 64), dtype=torch.bfloat16), 0, 3, True, stream=0)
+    assert call.io.scale_logits is None
