@@ -645,24 +645,28 @@ class ScaleCall:
         self._buffers = (ent, mean, mean_host, keep_idx, prune_idx, cu_keep, x_buf)
 
     def set_layers(self, weights, modulation, k_caches, v_caches, kv_len, cache_prev, cache_out):
-        """weights: BlockWeights per layer; modulation: dict per layer or None; kv_len: [L, B] tensor or a
-        tensor [B] per layer; cache_prev: [B, hp, wp, C] per layer or None entries; cache_out per layer or None."""
+        """weights: BlockWeights per layer; modulation: dict per layer or None; kv_len: int32 [L, B] tensor or a
+        tensor [B] per layer, each layer's lengths next to each other; cache_prev: [B, hp, wp, C] per layer or None entries; cache_out per layer or None."""
         B, Cc = self.shape.B, self.shape.C
         mods = [modulation_struct(m, B, Cc) for m in modulation] if modulation else None
         hp, wp = next(((c.shape[1], c.shape[2]) for c in cache_prev if c is not None), (0, 0))
         tw, tm, _, tk, tv, tl, tp, to = self._tables
-        base, step = (_ptr(kv_len), 4 * B) if isinstance(kv_len, torch.Tensor) else (None, 0)
+        whole = isinstance(kv_len, torch.Tensor) and kv_len.is_contiguous() and kv_len.dtype == torch.int32 and kv_len.shape[1:] == (B,)
+        base, step = (kv_len.data_ptr(), 4 * B) if whole else (None, 0)
         for j in range(self.L):
             k, v, prev = k_caches[j], v_caches[j], cache_prev[j]
-            assert k.is_contiguous() and v.is_contiguous()
-            tw[j], tk[j], tv[j] = C.addressof(weights[j].c), k.data_ptr(), v.data_ptr()
-            tl[j] = base + j * step if base is not None else kv_len[j].data_ptr()
-            assert prev is None or (prev.shape[1] == hp and prev.shape[2] == wp and prev.is_contiguous())
-            tp[j] = prev.data_ptr() if prev is not None else None
+            tw[j], tk[j], tv[j] = C.addressof(weights[j].c), _ptr(k), _ptr(v)
+            if whole:
+                tl[j] = base + j * step
+            else:
+                assert kv_len[j].dtype == torch.int32 and kv_len[j].numel() >= B
+                tl[j] = _ptr(kv_len[j])
+            assert prev is None or (prev.shape[1] == hp and prev.shape[2] == wp)
+            tp[j] = _ptr(prev)
             if mods is not None:
                 tm[j] = C.addressof(mods[j])
             if cache_out is not None:
-                to[j] = cache_out[j].data_ptr()
+                to[j] = _ptr(cache_out[j])
         self._mods = mods
         for name, table in zip(("weights", "modulation", "logits", "k_cache", "v_cache", "kv_len", "cache_prev", "cache_out"),
                                (tw, tm if mods is not None else None, self._tables[2], tk, tv, tl, tp, to if cache_out is not None else None)):

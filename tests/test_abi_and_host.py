@@ -173,3 +173,28 @@ def test_scale_call_forgets_the_scale_logits_of_a_pass_that_failed():
     with pytest.raises(nova.NovaError):
         call.run(nova.SchedParams(), 1, torch.zeros(2, 1), torch.zeros((2, 6, 64), dtype=torch.bfloat16), 0, 3, True, stream=0)
     assert call.io.scale_logits is None
+
+
+def test_scale_call_takes_only_lengths_that_lie_together():
+    """kv_len: a whole [L, B] tensor, rows of a wider one, or a tensor per layer; never strided views, whose
+    neighbours would be read and advanced instead, and never 64-bit lengths."""
+    call, layers = _scale_call()
+    L, B, i32 = 3, 2, torch.int32
+    table = call._tables[5]
+    for good in (torch.zeros((L, B), dtype=i32), torch.zeros((L + 1, B), dtype=i32), torch.zeros((L, B + 2), dtype=i32)[:, :B],
+                 list(torch.zeros((L, B), dtype=i32).unbind(0)), torch.zeros((2 * L, B), dtype=i32)[::2]):
+        call.set_layers(**{**layers, "kv_len": good})
+        assert [table[j] for j in range(L)] == [good[j].data_ptr() for j in range(L)]
+    for bad in (torch.zeros((B, L), dtype=i32).t(), list(torch.zeros((B, L), dtype=i32).unbind(1)),
+                torch.zeros((L, B), dtype=torch.int64), torch.zeros((L, 1), dtype=i32)):
+        with pytest.raises(AssertionError):
+            call.set_layers(**{**layers, "kv_len": bad})
+
+
+def test_scale_call_takes_only_contiguous_caches():
+    call, layers = _scale_call()
+    for name in ("k_caches", "v_caches", "cache_prev", "cache_out"):
+        wide = torch.zeros((3, 2, 2, 2, 128), dtype=torch.bfloat16)
+        views = [t[..., :64] if name.startswith("cache") else t.flatten(1, 2)[..., :64] for t in wide]
+        with pytest.raises(AssertionError):
+            call.set_layers(**{**layers, name: views})
