@@ -463,7 +463,7 @@ nova_status nova_pruned_layer_forward(nova_ctx* ctx, const nova_block_weights* w
  */
 typedef struct nova_scale_layers {
     const nova_block_weights* const* weights;
-    const nova_block_modulation* const* modulation;   /* or NULL */
+    const nova_block_modulation* const* modulation;   /* or NULL; entries may be NULL */
     const void* const* logits;                        /* [B, N, V] per layer */
     void* const* k_cache;
     void* const* v_cache;

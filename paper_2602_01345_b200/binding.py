@@ -645,10 +645,10 @@ class ScaleCall:
         self._buffers = (ent, mean, mean_host, keep_idx, prune_idx, cu_keep, x_buf)
 
     def set_layers(self, weights, modulation, k_caches, v_caches, kv_len, cache_prev, cache_out):
-        """weights: BlockWeights per layer; modulation: dict per layer or None; kv_len: int32 [L, B] tensor or a
+        """weights: BlockWeights per layer; modulation: dict or None per layer, or None; kv_len: int32 [L, B] tensor or a
         tensor [B] per layer, each layer's lengths next to each other; cache_prev: [B, hp, wp, C] per layer or None entries; cache_out per layer or None."""
         B, Cc = self.shape.B, self.shape.C
-        mods = [modulation_struct(m, B, Cc) for m in modulation] if modulation else None
+        mods = [modulation_struct(m, B, Cc) if m else None for m in modulation] if modulation else None
         hp, wp = next(((c.shape[1], c.shape[2]) for c in cache_prev if c is not None), (0, 0))
         tw, tm, _, tk, tv, tl, tp, to = self._tables
         whole = isinstance(kv_len, torch.Tensor) and kv_len.is_contiguous() and kv_len.dtype == torch.int32 and kv_len.shape[1:] == (B,)
@@ -664,7 +664,7 @@ class ScaleCall:
             assert prev is None or (prev.shape[1] == hp and prev.shape[2] == wp)
             tp[j] = _ptr(prev)
             if mods is not None:
-                tm[j] = C.addressof(mods[j])
+                tm[j] = C.addressof(mods[j]) if mods[j] is not None else None
             if cache_out is not None:
                 to[j] = _ptr(cache_out[j])
         self._mods = mods

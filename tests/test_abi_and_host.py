@@ -198,3 +198,12 @@ def test_scale_call_takes_only_contiguous_caches():
         views = [t[..., :64] if name.startswith("cache") else t.flatten(1, 2)[..., :64] for t in wide]
         with pytest.raises(AssertionError):
             call.set_layers(**{**layers, name: views})
+
+
+def test_scale_call_takes_layers_without_modulation_among_others():
+    call, layers = _scale_call()
+    shift = {"shift1": torch.zeros((2, 64), dtype=torch.bfloat16)}
+    call.set_layers(**{**layers, "modulation": [shift, None, {}]})
+    assert [bool(p) for p in call._tables[1]] == [True, False, False]
+    call.set_layers(**{**layers, "modulation": [None, shift, shift]})
+    assert [bool(p) for p in call._tables[1]] == [False, True, True]
