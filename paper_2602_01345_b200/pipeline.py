@@ -81,7 +81,8 @@ class PrunedScaleRunner:
         j's launches (info: dict of the tensors involved); for tests that compare layer by layer.
         """
         st = stream if stream is not None else torch.cuda.current_stream()
-        if layer_hook is not None or select_ent is not None:
+        # (the native call takes one size for all residual caches)
+        if layer_hook is not None or select_ent is not None or len({c.shape[1:3] for c in self.cache_prev if c is not None}) > 1:
             return self._run_layer_by_layer(x_in, layer_logits, sched, t, hbar_scale, append_kv, st, logits_ready, select_ent,
                                             layer_hook)
         # The layers' logits are inputs of the scale, not results of its layers: the entropy maps of a whole

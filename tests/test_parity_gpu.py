@@ -1339,6 +1339,24 @@ def test_generation_history_is_read_from_the_stream_it_runs_on(ctx):
         assert torch.equal(h[:, 0], mean.cpu())
 
 
+def _forms_agree(ctx, x_in, logits, hbar, **kw):
+    """A scale without and with a hook, from the same state: outputs, residual caches and keep counts agree."""
+    got = []
+    for hook in (None, lambda stage, j, info: None):
+        runner = _small_scale(ctx, **kw)[0]
+        x_out, keeps = runner.run_scale(x_in, logits, nova.SchedParams(force_act_scale=8), 8, hbar, layer_hook=hook)
+        assert ctx.device_status() == 0 and int(keeps[0].sum()) < x_in.shape[0] * x_in.shape[1]
+        got.append([x_out.clone(), torch.stack(keeps), *runner.cache_out])
+    for p, q in zip(*got):
+        assert torch.equal(p, q)
+
+
+def test_residual_caches_of_different_sizes(ctx):
+    """Every layer's residual cache may have a size of its own."""
+    _, x_in, logits, hbar = _small_scale(ctx, L=3)
+    _forms_agree(ctx, x_in, logits, hbar, L=3, cache_prev=[synth.residual_cache(2, s, s + 1, 256, 70 + s, DEV) for s in (3, 5, 4)])
+
+
 def test_selection_on_one_scale_map_gives_nested_sets(ctx):
     """The other reading of how layers get their entropy map: one map per scale, selected on by every
     layer with that layer's keep count. Kept sets of layers with fewer kept tokens are subsets of
