@@ -674,6 +674,8 @@ class ScaleCall:
         self.layers.hp, self.layers.wp = hp, wp
 
     def set_logits(self, layer_logits):
+        """layer_logits: the layers' logits [B, N, V], all of one layout; what follows the L-th is not looked at."""
+        layer_logits = layer_logits[: self.L]
         first = layer_logits[0]
         S, N, V = first.shape
         assert (S, N) == (self.shape.B, self.shape.N) and len(layer_logits) == self.L

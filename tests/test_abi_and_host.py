@@ -207,3 +207,13 @@ def test_scale_call_takes_layers_without_modulation_among_others():
     assert [bool(p) for p in call._tables[1]] == [True, False, False]
     call.set_layers(**{**layers, "modulation": [None, shift, shift]})
     assert [bool(p) for p in call._tables[1]] == [False, True, True]
+
+
+def test_scale_call_ignores_logits_past_its_last_layer():
+    call, _ = _scale_call()
+    logits = torch.zeros((5, 2, 6, 32), dtype=torch.bfloat16)
+    for given in (logits, list(logits), [*logits[:3], None]):
+        call.set_logits(given)
+        assert [call._tables[2][j] for j in range(3)] == [logits[j].data_ptr() for j in range(3)]
+    with pytest.raises(AssertionError):
+        call.set_logits(logits[:2])
