@@ -1357,6 +1357,16 @@ def test_residual_caches_of_different_sizes(ctx):
     _forms_agree(ctx, x_in, logits, hbar, L=3, cache_prev=[synth.residual_cache(2, s, s + 1, 256, 70 + s, DEV) for s in (3, 5, 4)])
 
 
+@pytest.mark.parametrize("first,count", [(0, -1), (-1, 2), (1, 2 ** 31 - 1), (2 ** 31 - 1, 1)])
+def test_scale_call_refuses_a_bad_layer_range(ctx, first, count):
+    runner, x_in, logits, hbar = _small_scale(ctx, L=2)
+    runner.call.set_layers(runner.weights, None, runner.k_caches, runner.v_caches, runner.kv_len, runner.cache_prev, None)
+    runner.call.set_logits(logits)
+    with pytest.raises(nova.NovaError) as ei:
+        runner.call.run(nova.SchedParams(), 8, hbar, x_in, first, count, False)
+    assert ei.value.status == 1
+
+
 def test_selection_on_one_scale_map_gives_nested_sets(ctx):
     """The other reading of how layers get their entropy map: one map per scale, selected on by every
     layer with that layer's keep count. Kept sets of layers with fewer kept tokens are subsets of
