@@ -646,32 +646,44 @@ class ScaleCall:
 
     def set_layers(self, weights, modulation, k_caches, v_caches, kv_len, cache_prev, cache_out):
         """weights: BlockWeights per layer; modulation: dict or None per layer, or None; kv_len: int32 [L, B] tensor or a
-        tensor [B] per layer, each layer's lengths next to each other; cache_prev: [B, hp, wp, C] per layer or None entries; cache_out per layer or None."""
+        tensor [B] per layer, each layer's lengths next to each other; cache_prev: [B, hp, wp, C] per layer or None
+        entries; cache_out per layer or None. Returns whether all of cache_prev has one size, which run needs."""
         B, Cc = self.shape.B, self.shape.C
         mods = [modulation_struct(m, B, Cc) if m else None for m in modulation] if modulation else None
         hp, wp = next(((c.shape[1], c.shape[2]) for c in cache_prev if c is not None), (0, 0))
         tw, tm, _, tk, tv, tl, tp, to = self._tables
         whole = isinstance(kv_len, torch.Tensor) and kv_len.is_contiguous() and kv_len.dtype == torch.int32 and kv_len.shape[1:] == (B,)
         base, step = (kv_len.data_ptr(), 4 * B) if whole else (None, 0)
+        one_size = True
         for j in range(self.L):
             k, v, prev = k_caches[j], v_caches[j], cache_prev[j]
-            tw[j], tk[j], tv[j] = C.addressof(weights[j].c), _ptr(k), _ptr(v)
+            assert k.is_contiguous() and v.is_contiguous()
+            tw[j], tk[j], tv[j] = C.addressof(weights[j].c), k.data_ptr(), v.data_ptr()
             if whole:
                 tl[j] = base + j * step
             else:
-                assert kv_len[j].dtype == torch.int32 and kv_len[j].numel() >= B
-                tl[j] = _ptr(kv_len[j])
-            assert prev is None or (prev.shape[1] == hp and prev.shape[2] == wp)
-            tp[j] = _ptr(prev)
+                n = kv_len[j]
+                assert n.dtype == torch.int32 and n.is_contiguous() and n.numel() >= B
+                tl[j] = n.data_ptr()
+            if prev is None:
+                tp[j] = None
+            else:
+                assert prev.is_contiguous()
+                _, ph, pw, _ = prev.shape
+                one_size = one_size and ph == hp and pw == wp
+                tp[j] = prev.data_ptr()
             if mods is not None:
                 tm[j] = C.addressof(mods[j]) if mods[j] is not None else None
             if cache_out is not None:
-                to[j] = _ptr(cache_out[j])
+                assert cache_out[j].is_contiguous()
+                to[j] = cache_out[j].data_ptr()
         self._mods = mods
         for name, table in zip(("weights", "modulation", "logits", "k_cache", "v_cache", "kv_len", "cache_prev", "cache_out"),
                                (tw, tm if mods is not None else None, self._tables[2], tk, tv, tl, tp, to if cache_out is not None else None)):
             setattr(self.layers, name, C.addressof(table) if table is not None else None)
         self.layers.hp, self.layers.wp = hp, wp
+        self._one_size = one_size
+        return one_size
 
     def set_logits(self, layer_logits):
         """layer_logits: the layers' logits [B, N, V], all of one layout; what follows the L-th is not looked at."""
@@ -698,6 +710,7 @@ class ScaleCall:
     def run(self, sched: SchedParams, t: int, hbar_scale, x_in, first: int, count: int, append_kv: bool, stream=None):
         io = self.io
         try:
+            assert self._one_size, "the native call takes one size for all residual caches"
             assert hbar_scale.dtype == torch.float32 and not hbar_scale.is_cuda and hbar_scale.shape == (self.shape.B, t)
             assert x_in.dtype == torch.bfloat16 and x_in.numel() == self.shape.B * self.shape.N * self.shape.C
             io.hbar_scale, io.x_in = _ptr(hbar_scale), _ptr(x_in)

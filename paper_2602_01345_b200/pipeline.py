@@ -81,8 +81,8 @@ class PrunedScaleRunner:
         j's launches (info: dict of the tensors involved); for tests that compare layer by layer.
         """
         st = stream if stream is not None else torch.cuda.current_stream()
-        # (the native call takes one size for all residual caches)
-        if layer_hook is not None or select_ent is not None or len({c.shape[1:3] for c in self.cache_prev if c is not None}) > 1:
+        if layer_hook is not None or select_ent is not None or not self.call.set_layers(
+                self.weights, self.modulation, self.k_caches, self.v_caches, self.kv_len, self.cache_prev, self.cache_out):
             return self._run_layer_by_layer(x_in, layer_logits, sched, t, hbar_scale, append_kv, st, logits_ready, select_ent,
                                             layer_hook)
         # The layers' logits are inputs of the scale, not results of its layers: the entropy maps of a whole
@@ -91,7 +91,6 @@ class PrunedScaleRunner:
         # it and the layers themselves are one native call.
         group = self._group(logits_ready)
         hbar_scale = hbar_scale.to("cpu", torch.float32).contiguous()
-        self.call.set_layers(self.weights, self.modulation, self.k_caches, self.v_caches, self.kv_len, self.cache_prev, self.cache_out)
         self.call.set_logits(layer_logits)
         x = x_in
         for g0 in range(0, self.L, group):
