@@ -100,6 +100,10 @@ nova_status nova_debug_wait_probe(nova_ctx* ctx, void* stream);
  * Both cost host synchronisations: not for timed runs. Independently of debug mode every launching
  * call opens an NVTX range named after itself (no cost unless a tool listens). */
 nova_status nova_set_debug(nova_ctx* ctx, int on);
+/* How a GEMM of M rows, N features and K runs on a device with num_sms SMs (host arithmetic, no device): returns 1 for the
+ * kernel that may split K, with the parts of K and the rows of its token tile, 0 for the one that does not. The order of
+ * the sums, and so the results to the last bit, follow from these four numbers and nothing else. */
+int nova_debug_gemm_plan(int num_sms, int M, int N, int K, int* k_parts, int* token_tile);
 
 /* ---- measurement (no counterpart in the paper) --------------------------------- */
 /* Kernels launched by this context since nova_create. */

@@ -213,15 +213,24 @@ GemmParams make_params(nova_ctx* ctx, const nova_gemm_args& a)
 }
 
 // ---- which of the two kernels, and how ---------------------------------------------------------------
-// Clusters of 2 and of 4 CTAs that fit the device at the same time.
+// Clusters of 2 and of 4 CTAs that the plan counts on running at the same time. They follow from the SM count and not
+// from what the driver says fits: that depends on how the SMs left on a chip are spread over its eight GPCs, and with it
+// would the plan, the order of the sums and the last bits of the results. Clusters of 4 are taken to lose two SMs in every
+// GPC: 33 on 148 SMs, which is also what the driver said there. On a chip that holds fewer, a few tiles
+// would run after the others; no cluster waits for another.
 struct SplitCaps {
     int c[2];
 };
+inline SplitCaps split_caps(int num_sms)
+{
+    SplitCaps caps = {{num_sms / 2, num_sms > 20 ? (num_sms - 16) / 4 : 1}};
+    return caps;
+}
 struct SplitPlan {
     int ls, nt;      // s = 1 << ls
     bool takes;      // false: the problem is the pair kernel's
 };
-// The plan follows from the true M, N and K alone, on the host and in the kernel alike, so that a launch
+// The plan follows from the true M, N, K and the SM count alone, on the host and in the kernel alike, so that a launch
 // whose row count only the device knows adds in the same order as one whose row count the host knows.
 // For each s, nt is the smallest token tile with which all tiles run at once; the cheaper s by estimated
 // clocks wins. The constants are fits to launches of 8 to 1600 tokens, 1024 to 8192 features and K from 1024
@@ -664,12 +673,6 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     }
 }
 
-SplitCaps split_caps(const nova_ctx* ctx)
-{
-    SplitCaps caps = {{ctx->split_clusters[0], ctx->split_clusters[1]}};
-    return caps;
-}
-
 template <int BN, int STAGES, int EPI>
 nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
 {
@@ -702,7 +705,7 @@ nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
         // sweep the smaller operand; the entropy epilogue needs the N-fastest order
         const int span = (entropy || (long)a.M >= (long)a.N) ? -tiles_n : tiles_m;
         NOVA_CUDA_CHECK(ctx, nova_launch_pdl(kern, dim3(2 * pairs), dim3(kPairThreads), L::kTotal, st, 0, ta, tw, tw_half, p, span,
-                                             tiles_full, entries, entropy ? tiles_n : 0, split_caps(ctx)));
+                                             tiles_full, entries, entropy ? tiles_n : 0, split_caps(ctx->num_sms)));
     }
     return NOVA_OK;
 }
@@ -933,10 +936,10 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     }
 }
 
-// Once per context: shared memory opt-in of the split kernel and how many of its clusters fit the device.
+// Once per context: shared memory opt-in of the split kernel; its clusters have to fit the device at all.
 nova_status split_setup(nova_ctx* ctx)
 {
-    if (ctx->split_clusters[0]) return NOVA_OK;
+    if (ctx->attr_split) return NOVA_OK;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cudaLaunchAttribute attr[1];
@@ -946,22 +949,21 @@ nova_status split_setup(nova_ctx* ctx)
     NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(gemm_bf16_split<NOVA_EPI_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem));
     NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(gemm_bf16_split<NOVA_EPI_BIAS_RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem));
     NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(gemm_bf16_split<NOVA_EPI_BIAS_GELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem));
-    int n[2] = {0, 0};
     for (int ls = 0; ls < 2; ++ls) {
         attr[0].val.clusterDim.x = 2u << ls;
         cfg.gridDim = dim3(2u << ls);
-        NOVA_CUDA_CHECK(ctx, cudaOccupancyMaxActiveClusters(&n[ls], gemm_bf16_split<NOVA_EPI_BIAS_RES>, &cfg));
-        if (n[ls] < 1) return nova_fail(ctx, NOVA_ERR_CUDA, "gemm: no cluster of the split kernel fits the device");
+        int n = 0;
+        NOVA_CUDA_CHECK(ctx, cudaOccupancyMaxActiveClusters(&n, gemm_bf16_split<NOVA_EPI_BIAS_RES>, &cfg));
+        if (n < 1) return nova_fail(ctx, NOVA_ERR_CUDA, "gemm: no cluster of the split kernel fits the device");
     }
-    ctx->split_clusters[1] = n[1];
-    ctx->split_clusters[0] = n[0];
+    ctx->attr_split = true;
     return NOVA_OK;
 }
 
 template <int EPI>
 nova_status launch_split(nova_ctx* ctx, const nova_gemm_args& a, const SplitPlan& plan, cudaStream_t st)
 {
-    const SplitCaps caps = split_caps(ctx);
+    const SplitCaps caps = split_caps(ctx->num_sms);
     const int tiles_n = (a.N + 255) / 256;
     int pc, box, clusters;
     if (a.m_dev) {
@@ -991,7 +993,7 @@ nova_status launch_gemm(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
     // are launched and the one whose range the true count is not in returns at once.
     const nova_status rc = split_setup(ctx);
     if (rc != NOVA_OK) return rc;
-    const SplitPlan plan = split_plan(a.M, a.N, a.K / BK, split_caps(ctx));
+    const SplitPlan plan = split_plan(a.M, a.N, a.K / BK, split_caps(ctx->num_sms));
     if (plan.takes || a.m_dev) {
         const nova_status rs = launch_split<EPI>(ctx, a, plan, st);
         if (rs != NOVA_OK || plan.takes) return rs;
@@ -1000,6 +1002,14 @@ nova_status launch_gemm(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
 }
 
 }  // namespace
+
+extern "C" int nova_debug_gemm_plan(int num_sms, int M, int N, int K, int* k_parts, int* token_tile)
+{
+    const SplitPlan plan = split_plan(M, N, K / BK, split_caps(num_sms));
+    *k_parts = 1 << plan.ls;
+    *token_tile = plan.nt;
+    return plan.takes ? 1 : 0;
+}
 
 nova_status nova_launch_gemm(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
 {

@@ -217,3 +217,32 @@ def test_scale_call_ignores_logits_past_its_last_layer():
         assert [call._tables[2][j] for j in range(3)] == [logits[j].data_ptr() for j in range(3)]
     with pytest.raises(AssertionError):
         call.set_logits(logits[:2])
+
+
+def _gemm_plan(num_sms, M, N, K):
+    lib = ctypes.CDLL(nova.lib_path())
+    parts, tile = ctypes.c_int(), ctypes.c_int()
+    takes = lib.nova_debug_gemm_plan(num_sms, M, N, K, ctypes.byref(parts), ctypes.byref(tile))
+    return bool(takes), parts.value, tile.value
+
+
+def test_gemm_plan_follows_from_the_sizes_and_the_sm_count():
+    """The plan needs no device and is the one measured on 148 SMs; its token tiles all run at once on the
+    clusters it counts on (two SMs lost per GPC and cluster of four), and past the first row count that the split
+    kernel leaves to the other one it takes none."""
+    assert _gemm_plan(148, 256, 1024, 4096) == (True, 2, 32)
+    assert _gemm_plan(148, 300, 2048, 8192) == (True, 2, 96)
+    assert _gemm_plan(148, 300, 6144, 2048) == (True, 1, 128)
+    assert _gemm_plan(148, 1600, 2048, 8192)[0] and not _gemm_plan(148, 2250, 1920, 7680)[0]
+    assert not _gemm_plan(148, 8192, 2048, 2048)[0]
+    for num_sms in (2, 18, 64, 132, 148, 160):
+        for N, K in ((1024, 1024), (1920, 7680), (6144, 2048), (64, 64), (320, 320)):
+            taken = True
+            for M in (*range(1, 400, 7), *range(400, 3000, 61)):
+                takes, parts, tile = _gemm_plan(num_sms, M, N, K)
+                assert taken or not takes
+                taken = takes
+                if takes:
+                    assert parts in (1, 2) and parts <= K // 64 and tile % 32 == 0 and 32 <= tile <= 256
+                    clusters = num_sms // 2 if parts == 1 else max(1, (num_sms - 16) // 4)
+                    assert -(-N // 256) * -(-M // tile) <= clusters
