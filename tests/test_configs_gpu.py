@@ -225,3 +225,65 @@ def test_large_shapes_keep_sweep_through_the_runner(cfg, B, keep):
     assert _bf16_ulp_ok(gx, wx) and _bf16_ulp_ok(gc, wc)
     assert kv_len.cpu().tolist() == [[P + k_want] * B] * L
     ctx.close()
+
+
+def _equal_state(a, b):
+    return all(torch.equal(p, q) for p, q in zip(a, b, strict=True))
+
+
+@pytest.mark.parametrize("cfg,spatial", [("c2_var_d16_256", False), ("c3_var_d30_512", True)])
+def test_generation_in_one_call_per_scale_equals_layer_by_layer(cfg, spatial):
+    """The generations above, which a hook drives layer by layer, against the form without a hook (a native call
+    per scale) at full depth: after every scale the outputs, keep counts, histories, residual caches, K/V caches and their lengths are the
+    same bit for bit."""
+    ms = synth.CONFIGS[cfg]
+    B, L, C, seed = ms.B, ms.L, ms.C, 11
+    ctx = nova.Context(0)
+    weights = [synth.block_weights(C, ms.F, 1000 * seed + j, DEV) for j in range(L)]
+    gens = [pipeline.MultiScaleRunner(ctx, weights, ms.heads, B, ms.scales) for _ in range(2)]
+    a_env, _ = synth.scale_envelope_temperatures(B, len(ms.scales), seed=seed)
+    beta = synth.layer_inverse_temperatures(L, seed)
+    pruned = 0
+    for t, side in enumerate(ms.scales, 1):
+        N = side * side
+        a = a_env[:, t - 1].view(B, 1).expand(B, N).contiguous().to(DEV)
+        if spatial and side >= 3:
+            a = a * synth.smooth_temperature_field(B, side, side, seed * 31 + t, a_lo=0.6, a_hi=1.4, device=DEV)
+        x_in = synth.activations(B, N, C, 200 * seed + t, DEV)
+        scale_logits = synth.logits_from_temperature(a, synth.V_CODEBOOK, 300 * seed + t)
+        layer_logits = [synth.logits_from_temperature(a * float(beta[j]), synth.V_CODEBOOK, 400 * seed + 40 * t + j) for j in range(L)]
+        state = []
+        for gen, hook in zip(gens, (None, lambda stage, j, info: None)):
+            x_out, keeps, _ = gen.run_scale(t, x_in, scale_logits, layer_logits, nova.SchedParams(), layer_hook=hook)
+            assert ctx.device_status() == 0
+            state.append([x_out, torch.stack(keeps), gen.hbar_scale, gen.kv_len, *gen.res_cache, *gen.k_caches, *gen.v_caches])
+        assert _equal_state(*state), t
+        pruned += int(torch.stack(keeps).sum()) < L * B * N
+    assert pruned
+    ctx.close()
+
+
+@pytest.mark.parametrize("cfg,B,keep", [("c4_1024", 4, 0.5), ("c5_2048", 1, 0.2)])
+def test_large_scale_in_one_call_equals_layer_by_layer(cfg, B, keep):
+    """The same for the last 1024x1024 scale of four images and the last 2048x2048 scale, two layers."""
+    ms = synth.CONFIGS[cfg]
+    L, t, side, C = 2, len(ms.scales), ms.scales[-1], ms.C
+    N, P, Lmax = side * side, ms.prior_tokens(t), ms.total_tokens
+    ctx = nova.Context(0)
+    weights = [synth.block_weights(C, ms.F, 70 + j, DEV) for j in range(L)]
+    cache_prev = [synth.residual_cache(B, ms.scales[-2], ms.scales[-2], C, 90 + j, DEV) for j in range(L)]
+    a = synth.smooth_temperature_field(B, side, side, 7, device=DEV)
+    logits = [synth.logits_from_temperature(a * (1.0 + 0.1 * j), synth.V_CODEBOOK, 100 + j) for j in range(L)]
+    x_in = synth.activations(B, N, C, 110, DEV)
+    sched = nova.SchedParams(force_act_scale=t, force_keep_ratio=keep)
+    hbar = torch.linspace(2.0, 7.0, t).repeat(B, 1).contiguous()
+    state = []
+    for hook in (None, lambda stage, j, info: None):
+        ks, vs = zip(*[synth.kv_cache(B, Lmax, P, C, 80 + 2 * j, DEV)[:2] for j in range(L)])
+        kv_len = torch.full((L, B), P, dtype=torch.int32, device=DEV)
+        runner = pipeline.PrunedScaleRunner(ctx, weights, ms.heads, B, side, side, Lmax, list(ks), list(vs), kv_len, cache_prev)
+        x_out, keeps = runner.run_scale(x_in, logits, sched, t, hbar, layer_hook=hook)
+        assert ctx.device_status() == 0
+        state.append([x_out.clone(), torch.stack(keeps), kv_len, *runner.cache_out, *ks, *vs])
+    assert _equal_state(*state)
+    ctx.close()

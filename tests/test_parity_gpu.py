@@ -678,7 +678,8 @@ def test_block_adaptive_layernorm_identity_equals_plain_block(ctx):
 ])
 def test_block_gemm_tile_edges_host_and_device_count(ctx, C, heads, F, M):
     """Kept counts at the edges of the GEMMs' token tiles, against the oracle, and the same call with the
-    count left on the device below a larger bound: keys, values and lengths are bit-identical."""
+    count left on the device below a larger bound: keys, values and lengths are bit-identical, and so is the output
+    (projection, FC1 and FC2) where there are too few keys for attention to split its work by its scratch."""
     N, prior, seed = M + 37, 24, 61
     _block_case(ctx, B=1, N=N, C=C, heads=heads, F=F, Lmax=prior + N, ks=[M], kv_lens=[prior], seed=seed,
                 rows=None if M < 600 else sorted({0, 31, 32, 255, 256, 1023, M - 1}))
@@ -698,7 +699,10 @@ def test_block_gemm_tile_edges_host_and_device_count(ctx, C, heads, F, M):
         got.append((y[:M], k, v, kv_len))
     for a, b in zip(got[0][1:], got[1][1:]):
         assert torch.equal(a, b)
-    assert _rel_err(f32(got[1][0]), f32(got[0][0])) <= 2.0 ** -7       # attention may split its keys differently
+    if (prior + N + 127) // 128 < 12:
+        assert torch.equal(got[0][0], got[1][0])
+    else:               # the bound decides how much scratch attention has, and with it whether it splits its keys
+        assert _rel_err(f32(got[1][0]), f32(got[0][0])) <= 2.0 ** -7
 
 
 def test_block_without_append_leaves_kv_len(ctx):
