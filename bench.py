@@ -75,9 +75,6 @@ def parse_args():
     ap.add_argument("--keep", type=float, default=0.5)
     ap.add_argument("--scale", type=int, default=None, help="1-based scale index (default: last)")
     ap.add_argument("--layers", type=int, default=None, help="override the number of layers (small profiling cases)")
-    ap.add_argument("--two-call-layers", action="store_true",
-                    help="time nova_pruned_block_forward + nova_restore_from_cache per layer instead of the one "
-                         "nova_pruned_layer_forward call (the other form is timed after the timed region either way)")
     ap.add_argument("--all-configs", action="store_true",
                     help="one JSON line per stated configuration (the five workloads; the 1024 shape at keep ratios "
                          "0.25 / 0.5 / 0.75 and batch 1 / 4), device-resident timing only")
@@ -231,10 +228,9 @@ def run_ours(args):
 
     ctx = nova.Context(local)
     st = build_state(wd, dev)
-    fused = not args.two_call_layers
     runner = pipeline.PrunedScaleRunner(ctx, st["weights"], ms.heads, B, wd["h"], wd["w"], wd["Lmax"],
                                         st["k_caches"], st["v_caches"], st["kv_len"], st["cache_prev"],
-                                        fused_restore=fused)
+                                        fused_restore=True)
     sched = nova.SchedParams(force_act_scale=wd["t"], force_keep_ratio=wd["keep"])
     hbar_scale = torch.linspace(2.0, 7.0, wd["t"]).repeat(B, 1).contiguous()
     stream = torch.cuda.current_stream()
@@ -334,13 +330,11 @@ def run_ours(args):
     rows = B * N
     # HBM-bound passes: algorithmic bytes of all launches of a step over their summed event time.
     # entropy: per token V * 2 bytes read + 4 written; select: per token a 4-byte key read and a 4-byte
-    # index written; restore: kept row = y and x_in read, x_out and cache_out written (4 rows; when the
-    # block's last GEMM writes the kept rows itself, restore touches the pruned rows only), pruned row =
-    # x_in read, x_out and cache_out written (3 rows), plus the low-resolution cache once.
+    # index written; restore: pruned row = x_in read, x_out and cache_out written (3 rows), plus the
+    # low-resolution cache once (the kept rows are written by the block's last GEMM).
     ent_bytes_step = ms.L * rows * (synth.V_CODEBOOK * 2 + 4)
     sel_bytes_step = ms.L * rows * 8
-    kept_rows_in_restore = 0 if fused else M
-    restore_bytes = (kept_rows_in_restore * 4 + (rows - M) * 3) * ms.C * 2 + B * wd["hp"] * wd["wp"] * ms.C * 2
+    restore_bytes = (rows - M) * 3 * ms.C * 2 + B * wd["hp"] * wd["wp"] * ms.C * 2
     for key, step_bytes in (("entropy_rows", ent_bytes_step), ("select_topk", sel_bytes_step),
                             ("restore", restore_bytes * ms.L)):
         if prof.get(key, (0, 0))[1]:
@@ -361,31 +355,32 @@ def run_ours(args):
         us = b0.elapsed_time(b1) * 1e3 / 3
         key = "gbs_back_to_back" if with_mean else "gbs_back_to_back_no_mean"
         kernels["entropy_rows"][key] = round(ent_bytes_step / us / 1e3, 1)
-    # Both forms of a layer (one nova_pruned_layer_forward call, or block + restore as two calls) on the
-    # same inputs, timed alike: no per-kernel event brackets here, which cost the timed region above two
-    # event records per launch.
-    other = pipeline.PrunedScaleRunner(ctx, st["weights"], ms.heads, B, wd["h"], wd["w"], wd["Lmax"], st["k_caches"],
-                                       st["v_caches"], st["kv_len"], st["cache_prev"], fused_restore=not fused)
+    # The timed region issues the whole scale as one nova_pruned_scale_forward call. The same scale layer by layer
+    # from Python (a hook makes the runner do that), with one nova_pruned_layer_forward call or with block + restore
+    # per layer, on the same inputs, all three timed alike: no per-kernel event brackets here, which cost the
+    # timed region two event records per launch.
+    two_calls = pipeline.PrunedScaleRunner(ctx, st["weights"], ms.heads, B, wd["h"], wd["w"], wd["Lmax"], st["k_caches"],
+                                           st["v_caches"], st["kv_len"], st["cache_prev"], fused_restore=False)
     form_ms, form_out = {}, {}
-    for name, rn in (("timed", runner), ("other", other)):
+    for name, rn, hook in (("whole_scale", runner, None), ("one_call", runner, lambda stage, j, info: None),
+                           ("two_calls", two_calls, lambda stage, j, info: None)):
         for it in range(2 + args.steps):
             if it == 2:
                 torch.cuda.synchronize()
                 b0.record(stream)
             st["kv_len"].copy_(st["kv_len0"])
-            # the hook makes the runner issue its layers call by call, in its own form
-            form_out[name], _ = rn.run_scale(st["x_in"], st["logits"], sched, wd["t"], hbar_scale, stream=stream,
-                                             layer_hook=lambda stage, j, info: None)
+            got, _ = rn.run_scale(st["x_in"], st["logits"], sched, wd["t"], hbar_scale, stream=stream, layer_hook=hook)
         b1.record(stream)
         torch.cuda.synchronize()
         form_ms[name] = b0.elapsed_time(b1) / args.steps
-    layer_forms = {"timed": "one call per layer (nova_pruned_layer_forward)" if fused else
-                            "two calls per layer (nova_pruned_block_forward + nova_restore_from_cache)",
-                   "ms_per_step_one_call": round(form_ms["timed" if fused else "other"], 4),
-                   "ms_per_step_two_calls": round(form_ms["other" if fused else "timed"], 4),
-                   "note": "both without the per-kernel event brackets of the timed region",
-                   "same_result": bool(torch.equal(form_out["timed"], form_out["other"]))}
-    del other
+        form_out[name] = got.clone()
+    layer_forms = {"timed": "one call per scale (nova_pruned_scale_forward)",
+                   "ms_per_step_whole_scale": round(form_ms["whole_scale"], 4),
+                   "ms_per_step_one_call": round(form_ms["one_call"], 4),
+                   "ms_per_step_two_calls": round(form_ms["two_calls"], 4),
+                   "note": "all without the per-kernel event brackets of the timed region",
+                   "same_result": all(bool(torch.equal(form_out["whole_scale"], y)) for y in form_out.values())}
+    del two_calls, form_out
     head_entropy = device_schedule = None
     if not args.no_next:
         # Entropy fused with the codebook head (the step before the path: hidden states -> entropy, the
@@ -413,7 +408,7 @@ def run_ours(args):
         drun = pipeline.DeviceScaleRunner(ctx, st["weights"], ms.heads, B, wd["h"], wd["w"], wd["Lmax"], st["k_caches"],
                                           st["v_caches"], st["kv_len"], st["cache_prev"], sched, wd["t"], hist_dev,
                                           synth.V_CODEBOOK, x_in=st["x_in"], layer_logits=st["logits"], scale_entropy=False,
-                                          fused_restore=fused)
+                                          fused_restore=True)
         st["kv_len"].copy_(st["kv_len0"])
         l0 = pipeline.launch_count(ctx)
         drun.capture()
