@@ -454,9 +454,9 @@ nova_status nova_pruned_layer_forward(nova_ctx* ctx, const nova_block_weights* w
  * (The paper fixes what is computed, not how the calls are packaged.) Layers first .. first + count - 1
  * (0-based) of scale t: nova_scale_entropy_layers over their logits, one copy of the means to the host and
  * one stream synchronisation, nova_keep_ratios_layers on the means of all layers so far,
- * nova_select_topk_grouped, then nova_pruned_layer_forward layer by layer. Results are those of the single calls. A caller whose logits arrive piece by piece calls it
- * for a few layers at a time, with x_in = where the previous call left its result: layer j (0-based) writes
- * x_buf[j & 1], or the other buffer if its input lies there.
+ * nova_select_topk_grouped, then nova_pruned_layer_forward layer by layer. Results are those of the single
+ * calls. A caller whose logits arrive piece by piece calls it for a few layers at a time, with x_in = where the
+ * previous call left its result: layer j (0-based) writes x_buf[j & 1], or the other buffer if its input lies there.
  * With scale_logits the scale's own entropy map (Eq. 7) is taken first and its means complete column t - 1
  * of hbar_scale; without, all t columns are the caller's.
  * Host memory: every array of sl, hbar_scale [B, t], keep [L, B] (written), mean_host [L, B] and

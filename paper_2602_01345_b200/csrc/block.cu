@@ -61,8 +61,8 @@ layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps,
     pdl_launch_dependents();
     // Gain and bias are needed last and come from HBM (each layer has its own): brought to L2 while the launch before
     // this one ends. A prefetch hands nothing to this kernel, so whoever still writes them does no harm. With few
-    // rows the launch is a chain of latencies, of which this takes one off: a 16-layer 256x256 generation 9366 ->
-    // 9255 us, a 20x20 scale of one image 3098 -> 3056.
+    // rows the launch is a chain of latencies, of which this takes one off: a 16-layer 256x256 generation 9412 ->
+    // 9316 us, a 20x20 scale of one image 3097 -> 3058.
     for (int c = threadIdx.x * 8; c < vec_per_row; c += kLnWarps * 32 * 8) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(gamma + c));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(beta + c));

@@ -865,8 +865,8 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
         cluster_sync_all();          // every pair's main loop is over: the rings may be written
         // The next kernel is let in when the last main loop is over: with the trigger at the start its first CTAs sat
         // on the SMs this grid leaves free, and it ended later. With the same in the kernel for many tiles, us: a
-        // 16-layer 256x256 generation 9565 -> 9380 (9358 with the trigger right after the wait, but there the calls
-        // below gained less), 20x20 scale of one image 3148 -> 3097, last 64x64 scale 6775 -> 6665.
+        // 16-layer 256x256 generation 9489 -> 9292, 20x20 scale of one image 3140 -> 3097, last 64x64 scale in a
+        // graph 6905 -> 6858. (Right after the wait the generation gains as much and the others less.)
         if ((c + num_clusters) * groups >= units) pdl_launch_dependents();
         if (warp >= 2 && active) {
             // token t of this CTA's 128 features (one per lane and tensor-memory lane quarter) to the pair that
