@@ -10,7 +10,7 @@ namespace {
 // src_row[r] = b*N + keep_idx[r]            row of x_in feeding compacted row r
 // kv_row[r]  = b*Lmax + kv_len[b] + (r - cu_keep[b])   cache row receiving r's k and v
 //              (-1 and a SHAPE flag if the image's cache would overflow)
-// Both are produced by the first LayerNorm (one warp per compacted row) on its way: it needs
+// Both are produced by the first LayerNorm on its way: it needs
 // src_row to gather its input anyway.
 struct RowMapArgs {
     const int32_t* keep_idx;
@@ -32,9 +32,19 @@ struct LnModArgs {
 };
 
 // ---- LayerNorm ----------------------------------------------------------------------------
-// One warp per row; the row (C <= 32*8*VEC bf16) stays in registers between the mean, the
+// Two warps per row, and eight blocks of them per SM that go through the rows in turn, each loading its next row
+// before it works on the present one. The row (C <= 64 * 8 * VEC bf16) stays in registers between the mean, the
 // variance and the normalisation, so x is read once and out written once.
-constexpr int kLnWarps = 8;
+// What bounds it: HBM and L2 at many rows; at few the chain list -> row -> two reductions -> store, so a thread
+// has little to do and all its loads go out first, gain and bias too. With one warp per row and eight rows per block the
+// code was four times as long and gain and bias were a load of their own at the end of the chain; back to back over warm
+// inputs, us: 300 rows x 2048 4.4 -> 2.4, 1024 x 2048 5.2 -> 3.3, 1600 x 2048 5.3 -> 4.2, 2252 x 1920 5.4 -> 4.7, 8192 x 2048
+// 12.5 -> 12.3 (5.5 TB/s), 256 x 1024 3.1 -> 2.3. With a block for each row 2.4, 3.7, 4.0, 5.0, 12.5 and 2.3, but a launch sized by
+// a bound paid for its empty blocks (1024 rows of 4096: 6.4, now 3.5). Six blocks per SM: 4.0, 4.5, 6.1, 15.9 from 1024 x 2048 on.
+// (Four warps per row: 3.0, 4.6, 4.6, 5.6, 14.9 and 2.0. The warps per row must not depend on the row count, which a
+// device-driven launch does not know, or the sums of the two forms would differ in their last bits.)
+constexpr int kLnThreads = 64;
+constexpr int kLnBlocksPerSm = 8;
 
 __device__ __forceinline__ uint4 ld_stream(const uint4* p)
 {
@@ -51,114 +61,151 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
-// Three resident blocks per SM (80 registers): with two (94 registers) a launch of 1024 blocks ran 3.5
-// waves of load-then-compute and sat at 0.41 of the HBM peak.
+// Sum over the block's two warps, in warp order. Two slots in turn: all have read one when they meet at the other's barrier.
+__device__ __forceinline__ float row_sum(float v, float* slot)
+{
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = v;
+    __syncthreads();
+    return slot[0] + slot[1];
+}
+
 template <int VEC, bool MAPS, bool MOD>
-__global__ void __launch_bounds__(kLnWarps * 32, 3)
+__global__ void __launch_bounds__(kLnThreads, kLnBlocksPerSm)
 layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps, int M, const int32_t* m_dev, int vec_per_row,
                uint4* __restrict__ out, const RowMapArgs maps, const LnModArgs mod)
 {
+    constexpr bool kAhead = VEC <= 4;      // wider rows have no registers for the next one, nor for gain and bias
+    __shared__ float part[4];
     pdl_launch_dependents();
-    // Gain and bias are needed last and come from HBM (each layer has its own): brought to L2 while the launch before
-    // this one ends. A prefetch hands nothing to this kernel, so whoever still writes them does no harm. With few
+    const int tid = threadIdx.x;
+    // Gain and bias come from HBM (each layer has its own): brought to L2 while the launch before this one ends. A
+    // prefetch hands nothing to this kernel, so whoever still writes them does no harm. With few
     // rows the launch is a chain of latencies, of which this takes one off: a 16-layer 256x256 generation 9412 ->
     // 9316 us, a 20x20 scale of one image 3097 -> 3058.
-    for (int c = threadIdx.x * 8; c < vec_per_row; c += kLnWarps * 32 * 8) {
+    for (int c = tid * 8; c < vec_per_row; c += kLnThreads * 8) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(gamma + c));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(beta + c));
     }
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    const int r = blockIdx.x * kLnWarps + (threadIdx.x >> 5);
     if (m_dev) M = min(M, *m_dev);      // the host knows only an upper bound
-    if (r >= M) return;
-    long src = r;
-    int img = 0;
-    if (MOD && !MAPS) img = mod.img_row[r];
-    if (MAPS) {
-        // image of compacted row r: largest b with cu_keep[b] <= r
-        int lo = 0, hi = maps.B;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (maps.cu_keep[mid] <= r) lo = mid; else hi = mid;
+    // row r of the launch: its row of x and its image
+    auto locate = [&](int r, long& src, int& img) {
+        src = r;
+        img = MOD && !MAPS ? mod.img_row[r] : 0;
+        if (MAPS) {
+            const int token = maps.keep_idx[r];
+            int lo = 0, hi = maps.B;        // largest b with cu_keep[b] <= r
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (maps.cu_keep[mid] <= r) lo = mid; else hi = mid;
+            }
+            src = (long)lo * maps.N + token;
+            img = lo;
         }
-        const int b = lo, c0 = maps.cu_keep[b];
-        src = (long)b * maps.N + maps.keep_idx[r];
-        img = b;
-        if (lane == 0) {
+    };
+    auto load = [&](long src, uint4 (&d)[VEC]) {
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            const int c = i * kLnThreads + tid;
+            d[i] = (c < vec_per_row) ? ld_stream(x + src * vec_per_row + c) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    int r = blockIdx.x;
+    if (r >= M) return;
+    long src, src_next = 0;
+    int img, img_next = 0;
+    uint4 raw[VEC], next[VEC], g[VEC], bt[VEC];
+    locate(r, src, img);
+    load(src, raw);
+    if (kAhead) {
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            const int c = i * kLnThreads + tid;
+            if (c < vec_per_row) { g[i] = gamma[c]; bt[i] = beta[c]; }
+        }
+    }
+    const float n = (float)(vec_per_row * 8);
+    while (true) {
+        const int r_next = r + (int)gridDim.x;
+        if (r_next < M) {
+            locate(r_next, src_next, img_next);
+            if (kAhead) load(src_next, next);
+        }
+        if (MAPS && tid == 0) {
+            const int c0 = maps.cu_keep[img], k_b = maps.cu_keep[img + 1] - c0, len = maps.kv_len[img];
             maps.src_row[r] = (int32_t)src;
-            maps.img_row[r] = b;
-            const int k_b = maps.cu_keep[b + 1] - c0, len = maps.kv_len[b];
+            maps.img_row[r] = img;
             if (len + k_b > maps.Lmax) {
                 maps.kv_row[r] = -1;
                 atomicOr(maps.status, NOVA_DEV_SHAPE);
             } else {
-                maps.kv_row[r] = b * maps.Lmax + len + (r - c0);
+                maps.kv_row[r] = img * maps.Lmax + len + (r - c0);
             }
         }
-    }
-    const uint4* xr = x + src * vec_per_row;
-    // The row is read once (streaming loads, all issued before the first use) and stays in
-    // registers for the three sweeps: sum, squared deviations, normalise.
-    uint4 raw[VEC];
+        float sum0 = 0.f, sum1 = 0.f;
 #pragma unroll
-    for (int i = 0; i < VEC; ++i) {
-        const int c = i * 32 + lane;
-        raw[i] = (c < vec_per_row) ? ld_stream(xr + c) : make_uint4(0, 0, 0, 0);
-    }
-    float sum0 = 0.f, sum1 = 0.f;
-#pragma unroll
-    for (int i = 0; i < VEC; ++i) {
-        const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            sum0 += __uint_as_float(w[q] << 16);
-            sum1 += __uint_as_float(w[q] & 0xffff0000u);
-        }
-    }
-    const float n = (float)(vec_per_row * 8);
-    const float mean = warp_sum(sum0 + sum1) / n;
-    float sq0 = 0.f, sq1 = 0.f;
-#pragma unroll
-    for (int i = 0; i < VEC; ++i) {
-        if (i * 32 + lane < vec_per_row) {
+        for (int i = 0; i < VEC; ++i) {
             const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float d0 = __uint_as_float(w[q] << 16) - mean, d1 = __uint_as_float(w[q] & 0xffff0000u) - mean;
-                sq0 = fmaf(d0, d0, sq0);
-                sq1 = fmaf(d1, d1, sq1);
+                sum0 += __uint_as_float(w[q] << 16);
+                sum1 += __uint_as_float(w[q] & 0xffff0000u);
             }
         }
-    }
-    const float rstd = rsqrtf(warp_sum(sq0 + sq1) / n + eps);
-    const float shift = -mean * rstd;
+        const float mean = row_sum(sum0 + sum1, part) / n;
+        float sq0 = 0.f, sq1 = 0.f;
 #pragma unroll
-    for (int i = 0; i < VEC; ++i) {
-        const int c = i * 32 + lane;
-        if (c < vec_per_row) {
-            const uint4 g = gamma[c], bt = beta[c];
-            const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
-            const uint32_t gw[4] = {g.x, g.y, g.z, g.w}, bw[4] = {bt.x, bt.y, bt.z, bt.w};
-            uint32_t o[4];
-            uint32_t sc[4] = {0, 0, 0, 0}, sh[4] = {0, 0, 0, 0};        // bf16 zeros: no modulation
-            if (MOD && mod.scale) { const uint4 t = mod.scale[(long)img * vec_per_row + c]; sc[0] = t.x; sc[1] = t.y; sc[2] = t.z; sc[3] = t.w; }
-            if (MOD && mod.shift) { const uint4 t = mod.shift[(long)img * vec_per_row + c]; sh[0] = t.x; sh[1] = t.y; sh[2] = t.z; sh[3] = t.w; }
+        for (int i = 0; i < VEC; ++i) {
+            if (i * kLnThreads + tid < vec_per_row) {
+                const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                // (x - mean) * rstd = x * rstd + shift
-                const float n0 = fmaf(__uint_as_float(w[q] << 16), rstd, shift);
-                const float n1 = fmaf(__uint_as_float(w[q] & 0xffff0000u), rstd, shift);
-                float y0 = fmaf(n0, __uint_as_float(gw[q] << 16), __uint_as_float(bw[q] << 16));
-                float y1 = fmaf(n1, __uint_as_float(gw[q] & 0xffff0000u), __uint_as_float(bw[q] & 0xffff0000u));
-                if (MOD) {
-                    y0 = fmaf(y0, 1.f + __uint_as_float(sc[q] << 16), __uint_as_float(sh[q] << 16));
-                    y1 = fmaf(y1, 1.f + __uint_as_float(sc[q] & 0xffff0000u), __uint_as_float(sh[q] & 0xffff0000u));
+                for (int q = 0; q < 4; ++q) {
+                    const float d0 = __uint_as_float(w[q] << 16) - mean, d1 = __uint_as_float(w[q] & 0xffff0000u) - mean;
+                    sq0 = fmaf(d0, d0, sq0);
+                    sq1 = fmaf(d1, d1, sq1);
                 }
-                __nv_bfloat162 t = __floats2bfloat162_rn(y0, y1);
-                o[q] = *reinterpret_cast<uint32_t*>(&t);
             }
-            out[(long)r * vec_per_row + c] = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+        const float rstd = rsqrtf(row_sum(sq0 + sq1, part + 2) / n + eps);
+        const float shift = -mean * rstd;
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            const int c = i * kLnThreads + tid;
+            if (c < vec_per_row) {
+                if (!kAhead) { g[i] = gamma[c]; bt[i] = beta[c]; }
+                const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+                const uint32_t gw[4] = {g[i].x, g[i].y, g[i].z, g[i].w}, bw[4] = {bt[i].x, bt[i].y, bt[i].z, bt[i].w};
+                uint32_t o[4];
+                uint32_t sc[4] = {0, 0, 0, 0}, sh[4] = {0, 0, 0, 0};        // bf16 zeros: no modulation
+                if (MOD && mod.scale) { const uint4 t = mod.scale[(long)img * vec_per_row + c]; sc[0] = t.x; sc[1] = t.y; sc[2] = t.z; sc[3] = t.w; }
+                if (MOD && mod.shift) { const uint4 t = mod.shift[(long)img * vec_per_row + c]; sh[0] = t.x; sh[1] = t.y; sh[2] = t.z; sh[3] = t.w; }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    // (x - mean) * rstd = x * rstd + shift
+                    const float n0 = fmaf(__uint_as_float(w[q] << 16), rstd, shift);
+                    const float n1 = fmaf(__uint_as_float(w[q] & 0xffff0000u), rstd, shift);
+                    float y0 = fmaf(n0, __uint_as_float(gw[q] << 16), __uint_as_float(bw[q] << 16));
+                    float y1 = fmaf(n1, __uint_as_float(gw[q] & 0xffff0000u), __uint_as_float(bw[q] & 0xffff0000u));
+                    if (MOD) {
+                        y0 = fmaf(y0, 1.f + __uint_as_float(sc[q] << 16), __uint_as_float(sh[q] << 16));
+                        y1 = fmaf(y1, 1.f + __uint_as_float(sc[q] & 0xffff0000u), __uint_as_float(sh[q] & 0xffff0000u));
+                    }
+                    __nv_bfloat162 t = __floats2bfloat162_rn(y0, y1);
+                    o[q] = *reinterpret_cast<uint32_t*>(&t);
+                }
+                out[(long)r * vec_per_row + c] = make_uint4(o[0], o[1], o[2], o[3]);
+            }
+        }
+        if (r_next >= M) return;
+        r = r_next;
+        src = src_next;
+        img = img_next;
+        if (kAhead) {
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) raw[i] = next[i];
+        } else {
+            load(src, raw);
         }
     }
 }
@@ -269,8 +316,8 @@ static nova_status launch_ln(nova_ctx* ctx, const __nv_bfloat16* x, const RowMap
 {
     if (M <= 0) return NOVA_OK;
     const int vec = C / 8;
-    const int per_lane = (vec + 31) / 32;
-    const dim3 grid((M + kLnWarps - 1) / kLnWarps), block(kLnWarps * 32);
+    const int per_lane = (vec + kLnThreads - 1) / kLnThreads;
+    const dim3 grid(min(M, ctx->num_sms * kLnBlocksPerSm)), block(kLnThreads);
     RowMapArgs none;
     memset(&none, 0, sizeof(none));
     cudaError_t le = cudaSuccess;
@@ -286,10 +333,10 @@ static nova_status launch_ln(nova_ctx* ctx, const __nv_bfloat16* x, const RowMap
     } while (0)
     const bool modulated = mod.scale || mod.shift;
     if (per_lane <= 2) NOVA_LN_CASE(2);
+    else if (per_lane <= 3) NOVA_LN_CASE(3);
     else if (per_lane <= 4) NOVA_LN_CASE(4);
     else if (per_lane <= 8) NOVA_LN_CASE(8);
     else if (per_lane <= 16) NOVA_LN_CASE(16);
-    else if (per_lane <= 32) NOVA_LN_CASE(32);
     else return nova_fail(ctx, NOVA_ERR_SHAPE, "layernorm: C > 8192");
 #undef NOVA_LN_LAUNCH
 #undef NOVA_LN_CASE

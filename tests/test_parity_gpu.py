@@ -705,6 +705,15 @@ def test_block_gemm_tile_edges_host_and_device_count(ctx, C, heads, F, M):
         assert _rel_err(f32(got[1][0]), f32(got[0][0])) <= 2.0 ** -7
 
 
+@pytest.mark.parametrize("C,heads,ks", [(64, 1, [3, 0]), (192, 3, [1, 2]), (576, 9, [5, 7]), (1088, 17, [2, 3]), (1600, 25, [3, 1]),
+                                        (2112, 33, [1, 2]), (128, 2, [700, 695])])
+def test_block_layernorm_widths_and_rows_per_block(ctx, C, heads, ks):
+    """LayerNorm's widths: one to five 128-bit pieces per thread, the last of them shared by only some threads, and more
+    rows than blocks, so that a block goes on to a second row (of the other image)."""
+    N = max(max(ks), 8)
+    _block_case(ctx, B=2, N=N, C=C, heads=heads, F=64, Lmax=N + 8, ks=ks, kv_lens=[5, 8], seed=C)
+
+
 def test_block_without_append_leaves_kv_len(ctx):
     B, N, C, heads, F, Lmax = 1, 64, 128, 2, 256, 256
     wt = synth.block_weights(C, F, 1, DEV)
