@@ -233,6 +233,7 @@ struct nova_gemm_args {
     const int32_t* adv_cu_keep;
     int32_t* adv_kv_len;
     int adv_B, adv_Lmax;
+    bool early_trigger;         // the next launch may start as soon as this one has passed its wait (it works beside it)
 };
 
 nova_status nova_launch_gemm(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st);
@@ -252,8 +253,9 @@ struct nova_attn_args {
 
 nova_status nova_launch_attention(nova_ctx* ctx, const nova_attn_args& a, cudaStream_t st);
 
-// Eq. 16 for the pruned rows only (restore.cu); the kept rows were written by the block's last epilogue.
+// Eq. 16 for the pruned rows only (restore.cu); the kept rows are written by the block's last epilogue. wait_last: start
+// before the launch before it has ended (which must neither write what this reads nor read what this writes).
 nova_status nova_restore_pruned_rows(nova_ctx* ctx, const void* x_in, const int32_t* prune_idx,
                                      const int32_t* cu_keep, const void* cache_prev,
                                      int hp, int wp, int h, int w, int C, int B, int M, bool m_on_device,
-                                     void* x_out, void* cache_out, void* stream);
+                                     void* x_out, void* cache_out, void* stream, bool wait_last);

@@ -60,6 +60,7 @@ struct GemmParams {
     const int32_t* out_row;
     const __nv_bfloat16* diff_in;
     __nv_bfloat16* diff_out;
+    int early_trigger;
 };
 
 // Rows of this launch: p.M, or the device-side count when the host only knows an upper bound.
@@ -208,7 +209,7 @@ GemmParams make_params(nova_ctx* ctx, const nova_gemm_args& a)
     p.kv_row = a.kv_row; p.status = ctx->dev_status;
     p.adv_cu_keep = a.adv_cu_keep; p.adv_kv_len = a.adv_kv_len; p.adv_B = a.adv_B; p.adv_Lmax = a.adv_Lmax;
     p.ent = a.ent; p.m_dev = a.m_dev; p.gate = a.gate; p.img_row = a.img_row;
-    p.out_row = a.out_row; p.diff_in = a.diff_in; p.diff_out = a.diff_out;
+    p.out_row = a.out_row; p.diff_in = a.diff_in; p.diff_out = a.diff_out; p.early_trigger = a.early_trigger;
     return p;
 }
 
@@ -488,6 +489,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     if (!p.m_dev) pdl_wait();
+    if (p.early_trigger) pdl_launch_dependents();
     if (blockIdx.x == 0) advance_kv_len(p);
 
     if (warp == 0) {
@@ -795,6 +797,7 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     if (!p.m_dev) pdl_wait();
+    if (p.early_trigger) pdl_launch_dependents();
     if (blockIdx.x == 0) advance_kv_len(p);
 
     int it0 = 0;                 // k-blocks of the earlier units: position in the ring
