@@ -37,7 +37,7 @@ nova_status nova_create(nova_ctx** out, int device)
     ctx->workspace_bytes = 0;
     ctx->encode_tiled = nullptr;
     ctx->num_sms = 0;
-    ctx->attr_select = ctx->attr_attn = ctx->attr_split = false;
+    ctx->attr_attn = ctx->attr_split = false;
     ctx->err[0] = 0;
     ctx->launches = 0;
     ctx->profiling = false;

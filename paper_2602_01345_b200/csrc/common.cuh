@@ -48,7 +48,7 @@ struct nova_ctx {
     size_t workspace_bytes;
     void* encode_tiled;         // cuTensorMapEncodeTiled, resolved through the runtime
     int num_sms;
-    bool attr_select, attr_attn, attr_split;   // dynamic shared memory opt-in done on this device
+    bool attr_attn, attr_split;   // dynamic shared memory opt-in done on this device
     unsigned long long wait_limit_ns;   // mirrored in the status block (0 = default)
     bool debug;                 // debug mode: index lists validated before use, every launch synchronised
     bool debug_failed;          // a launch failed in debug mode (message in err); reported by nova_device_status

@@ -286,6 +286,26 @@ def test_select_edge_counts_and_many_segments(ctx):
     assert np.array_equal(prune_idx.cpu().numpy(), w_prune)
 
 
+@pytest.mark.parametrize("N", [512, 513, 1025, 2049, 4097, 8193, 16384])
+@pytest.mark.parametrize("values", ["low_bits", "few", "one", "all_bits"])
+def test_select_digits_and_ties(ctx, N, values):
+    """Keys that share all but their last bits, few distinct values (bins that never get small), one value, and keys that
+    differ in every bit (three digits), with counts at the ends, inside a tie and in the middle."""
+    g = torch.Generator(device="cpu").manual_seed(N)
+    if values == "low_bits":
+        ent = (torch.randint(0, 3000, (6, N), generator=g, dtype=torch.int32) + 0x40e00000).view(torch.float32)
+    elif values == "few":
+        ent = torch.randint(0, 3, (6, N), generator=g).float() * 1.75
+    elif values == "one":
+        ent = torch.full((6, N), 3.25)
+    else:
+        ent = torch.randn((6, N), generator=g) * 10.0 ** torch.randint(-30, 30, (6, N), generator=g).float()
+    ks = [0, 1, N // 3, N // 2, N - 1, N]
+    keep_idx, prune_idx, cu, pos = gpu_select(ctx, ent.to(DEV), ks)
+    for got, want in zip((keep_idx, prune_idx, cu, pos), oracle.select_topk(ent.numpy(), ks)):
+        assert np.array_equal(got.cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("G,S,N", [(3, 4, 1000), (32, 4, 4096), (70, 4, 300), (2, 1, 16384)])
 @pytest.mark.parametrize("counts_on_device", [False, True])
 def test_select_all_layers_in_one_call(ctx, G, S, N, counts_on_device):
