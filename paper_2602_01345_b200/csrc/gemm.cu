@@ -897,12 +897,13 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
             if (mbar_wait_warp(acc_full, acc_parity, abort_flag, p.status)) tc_fence_after();
         }
         __syncwarp();
-        cluster_sync_all();          // every pair's main loop is over: the rings may be written
+        // Every pair's main loop is over: the rings may be written. (Unsplit, a CTA writes only its own, which acc_full gave free.)
+        if (s > 1) cluster_sync_all();
         // The next kernel is let in when the last main loop is over: with the trigger at the start its first CTAs sat
         // on the SMs this grid leaves free, and it ended later. With the same in the kernel for many tiles, us: a
         // 16-layer 256x256 generation 9489 -> 9292, 20x20 scale of one image 3140 -> 3097, last 64x64 scale in a
         // graph 6905 -> 6858. (Right after the wait the generation gains as much and the others less.)
-        if ((c + num_clusters) * groups >= units) pdl_launch_dependents();
+        if (warp >= 2 && (c + num_clusters) * groups >= units) pdl_launch_dependents();
         if (warp >= 2 && active) {
             // token t of this CTA's 128 features (one per lane and tensor-memory lane quarter) to the pair that
             // completes it; the store of a warp is 128 contiguous bytes
@@ -916,7 +917,7 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
                 tmem_ld_wait();
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {        // eight tokens always belong to one pair (share % 8 == 0)
-                    const int t = ch * 32 + g * 8, owner = t / share;
+                    const int t = ch * 32 + g * 8, owner = t >= share;          // (two parts at most)
                     const uint32_t off = (uint32_t)((t - owner * share) * 512);
                     if (owner == part) {
 #pragma unroll
@@ -931,7 +932,8 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
             tc_fence_before();
         }
         __syncwarp();
-        cluster_sync_all();          // every part of this CTA's tokens has arrived
+        if (s > 1) cluster_sync_all();          // every part of this CTA's tokens has arrived
+        else if (warp >= 2) asm volatile("bar.sync 1, 256;" ::: "memory");
         if (warp >= 2 && active && col < p.N) {
             const float* parts = (const float*)smem + lane * 4 - (t0 + part * share) * 128;
             for (int t = first; t < t_end; t += 64) {
