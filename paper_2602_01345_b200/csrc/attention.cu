@@ -314,6 +314,26 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     if constexpr (kPair) cluster_sync_all();         // both CTAs' barriers exist before either signals the other
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+
+    // The passes of a CTA are laid out in shared memory, kTable at a time.
+    Pass* table = (Pass*)(smem + L::kTabOff);
+    static_assert(kTable * sizeof(Pass) <= 64 * 44, "pass table");
+    const bool copy = p.B < kCuCopy;
+    auto lay_out = [&](int base) {
+        if (base == 0 && copy) {
+            if (threadIdx.x <= p.B) cu_s[threadIdx.x] = p.cu_keep[threadIdx.x];
+            else if (threadIdx.x >= 128 && threadIdx.x < 128 + p.B) len_s[threadIdx.x - 128] = p.kv_len[threadIdx.x - 128];
+        }
+        __syncthreads();
+        if (threadIdx.x < kTable) table[threadIdx.x] = make_pass<DH>(p, copy ? cu_s : p.cu_keep, copy ? len_s : p.kv_len, me + (base + threadIdx.x) * stride);
+        if (threadIdx.x == 0) redo_s = 0;
+        __syncthreads();
+    };
+    // The first of them before the wait. What it reads, kept counts and cache lengths, was complete before the GEMM ahead of
+    // this launch (or ahead of the query/key transform) passed its own wait, and that GEMM has let this launch in only after
+    // it. Laid out behind the wait it was 1.5 us of each launch: 20x20 scale of one image, 32 layers, 2622 -> 2590 us, 16-layer
+    // 256x256 generation 8713 -> 8645, 512x512 scale 8796 -> 8744.
+    lay_out(0);
     pdl_wait();
 
     auto commit = [&](uint64_t* bar) {
@@ -325,22 +345,13 @@ attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         if (kPair && rank != 0) mbar_arrive_cluster(map_to_cta(smem_u32(bar), 0));
         else mbar_arrive(bar);
     };
-    Pass* table = (Pass*)(smem + L::kTabOff);
-    static_assert(kTable * sizeof(Pass) <= 64 * 44, "pass table");
     // Rounds: up to kTable passes, then, if a row sum in any of them was huge (in either CTA of the pair), those
     // passes once more with a maximum pass before each; then the next kTable. begin_round lays out the table if
     // there are passes left; end_of_round gives the passes to run again.
     auto begin_round = [&](int base) -> bool {
-        if (base > 0 && table[kTable - 1].over) return false;
-        const bool copy = p.B < kCuCopy;
-        if (base == 0 && copy) {
-            if (threadIdx.x <= p.B) cu_s[threadIdx.x] = p.cu_keep[threadIdx.x];
-            else if (threadIdx.x >= 128 && threadIdx.x < 128 + p.B) len_s[threadIdx.x - 128] = p.kv_len[threadIdx.x - 128];
-        }
-        __syncthreads();
-        if (threadIdx.x < kTable) table[threadIdx.x] = make_pass<DH>(p, copy ? cu_s : p.cu_keep, copy ? len_s : p.kv_len, me + (base + threadIdx.x) * stride);
-        if (threadIdx.x == 0) redo_s = 0;
-        __syncthreads();
+        if (base == 0) return true;
+        if (table[kTable - 1].over) return false;
+        lay_out(base);
         return true;
     };
     auto end_of_round = [&]() -> unsigned long long {
