@@ -436,6 +436,8 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
     nova_gemm_args g;
     memset(&g, 0, sizeof(g));
     g.A = ws.h; g.W = (cbf)w->w_qkv; g.bias = (cbf)w->b_qkv; g.M = M; g.m_dev = m_dev; g.N = 3 * C; g.K = C;
+    // (count_settled only for the GEMMs after this one: LN1 lets this one in before its own wait, and the kernel that writes
+    // the counts may be the one before LN1)
     g.epilogue = NOVA_EPI_QKV; g.cat = NOVA_K_GEMM_QKV; g.out = ws.q; g.C = C; g.k_cache = (bf)k_cache; g.v_cache = (bf)v_cache; g.kv_row = ws.kv_row;
     rc = nova_launch_gemm(ctx, g, st);
     if (rc) return rc;
@@ -471,6 +473,7 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
     memset(&g, 0, sizeof(g));
     g.A = ws.o; g.W = (cbf)w->w_o; g.bias = (cbf)w->b_o; g.M = M; g.m_dev = m_dev; g.N = C; g.K = C;
     g.epilogue = NOVA_EPI_BIAS_RES; g.cat = NOVA_K_GEMM_PROJ; g.out = ws.x1; g.res = (cbf)x_in; g.res_row = ws.src_row;
+    g.count_settled = true;
     g.gate = (cbf)md.gate1; g.img_row = ws.img_row;
     rc = nova_launch_gemm(ctx, g, st);
     if (rc) return rc;
@@ -484,6 +487,7 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
         memset(&g, 0, sizeof(g));
         g.A = ws.h; g.W = (cbf)ext->w_q2; g.bias = (cbf)ext->b_q2; g.M = M; g.m_dev = m_dev; g.N = C; g.K = C;
         g.epilogue = NOVA_EPI_QKV; g.cat = NOVA_K_GEMM_QKV; g.out = ws.q; g.C = C; g.kv_row = ws.kv_row;   // all columns are q
+        g.count_settled = true;
         rc = nova_launch_gemm(ctx, g, st);
         if (rc) return rc;
         nova_attn_args ca;
@@ -496,6 +500,7 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
         memset(&g, 0, sizeof(g));
         g.A = ws.o; g.W = (cbf)ext->w_o2; g.bias = (cbf)ext->b_o2; g.M = M; g.m_dev = m_dev; g.N = C; g.K = C;
         g.epilogue = NOVA_EPI_BIAS_RES; g.cat = NOVA_K_GEMM_PROJ; g.out = ws.x1; g.res = ws.x1; g.res_row = nullptr;   // in place
+        g.count_settled = true;
         rc = nova_launch_gemm(ctx, g, st);
         if (rc) return rc;
     }
@@ -519,6 +524,7 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
     memset(&g, 0, sizeof(g));
     g.A = ws.h; g.W = (cbf)w->w_fc1; g.bias = (cbf)w->b_fc1; g.M = M; g.m_dev = m_dev; g.N = F; g.K = C;
     g.epilogue = NOVA_EPI_BIAS_GELU; g.cat = NOVA_K_GEMM_FC1; g.out = ws.f;
+    g.count_settled = true;
     g.early_trigger = beside;
     rc = nova_launch_gemm(ctx, g, st);
     if (rc) return rc;
@@ -530,6 +536,7 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
     memset(&g, 0, sizeof(g));
     g.A = ws.f; g.W = (cbf)w->w_fc2; g.bias = (cbf)w->b_fc2; g.M = M; g.m_dev = m_dev; g.N = C; g.K = F;
     g.epilogue = NOVA_EPI_BIAS_RES; g.cat = NOVA_K_GEMM_FC2; g.out = (bf)y_kept; g.res = ws.x1; g.res_row = nullptr;
+    g.count_settled = true;
     g.gate = (cbf)md.gate2; g.img_row = ws.img_row;
     if (scatter) {
         // kept row r is token src_row[r] of the map: x_out[token] = y, cache_out[token] = y - x_in[token]

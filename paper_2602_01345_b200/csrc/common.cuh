@@ -233,6 +233,8 @@ struct nova_gemm_args {
     const int32_t* adv_cu_keep;
     int32_t* adv_kv_len;
     int adv_B, adv_Lmax;
+    // with m_dev: the launch that wrote the count had ended before the launch before this one could let this one in
+    bool count_settled;
     bool early_trigger;         // the next launch may start as soon as this one has passed its wait (it works beside it)
 };
 
