@@ -52,13 +52,13 @@ nova_status nova_create(nova_ctx** out, int device)
     const bool have_prev = (cudaGetDevice(&prev) == cudaSuccess);
     auto restore_device = [&]() { if (have_prev && prev != device) cudaSetDevice(prev); };
     if (cudaSetDevice(device) != cudaSuccess ||
-        cudaMalloc(&ctx->dev_status, NOVA_STATUS_BYTES) != cudaSuccess ||
+        cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaMalloc(&ctx->dev_status, NOVA_STATUS_BYTES + NOVA_PART_BYTES(ctx->num_sms)) != cudaSuccess ||
         cudaMemset(ctx->dev_status, 0, NOVA_STATUS_BYTES) != cudaSuccess) {
         delete ctx;
         restore_device();
         return NOVA_ERR_CUDA;
     }
-    cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
     cudaDriverEntryPointQueryResult qres;
     void* fn = nullptr;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess ||

@@ -20,14 +20,20 @@
 
 // Layout of the context's one device allocation: NOVA_STATUS_WORDS 32-bit words (word 0 = status
 // flags, a block of tickets for key-split attention items), then one 64-bit accumulator per segment
-// for the entropy means (NOVA_MEAN_MAX_SEGMENTS of them). All of it is zero between launches.
+// for the entropy means (NOVA_MEAN_MAX_SEGMENTS of them), then tickets of rows shared by CTAs. All of it is zero between launches.
 #define NOVA_STATUS_WORDS 128
 #define NOVA_WAIT_LIMIT_WORD 2        // words 2-3: limit of a device-side wait in ns (0 = the default of one second)
 #define NOVA_ATTN_TICKET_WORD0 16     // words 16 .. 16 + NOVA_ATTN_TICKETS - 1: tickets of key-split attention items
 #define NOVA_ATTN_TICKETS 96
 #define NOVA_MEAN_MAX_CTAS 192        // the accumulator's arrival count has 8 bits
 #define NOVA_MEAN_MAX_SEGMENTS 256
-#define NOVA_STATUS_BYTES (NOVA_STATUS_WORDS * 4 + NOVA_MEAN_MAX_SEGMENTS * 8)
+#define NOVA_TICKETS 512              // of rows that several CTAs of the head or of the attention-mass kernel share, by CTA
+#define NOVA_STATUS_BYTES (NOVA_STATUS_WORDS * 4 + NOVA_MEAN_MAX_SEGMENTS * 8 + NOVA_TICKETS * 4)
+// Behind it: partial results of such rows. Head: [pair][first or last of its row blocks][m, s, u][256 rows] fp32; attention mass:
+// [CTA, up to two per SM][first or last of its rows][128 rows] float2.
+#define NOVA_HEAD_SLOT_FLOATS (3 * 256)
+#define NOVA_PART_BYTES(num_sms) ((size_t)(num_sms) * 2 * 2 * 128 * 8)
+static_assert(2 * 2 * 128 * 8 >= NOVA_HEAD_SLOT_FLOATS * 4, "two slots for every pair");
 
 // Kernel categories for the launch counter and the optional per-kernel event timing.
 enum nova_kernel_cat {

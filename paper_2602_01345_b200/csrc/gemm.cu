@@ -54,6 +54,8 @@ struct GemmParams {
     int32_t* adv_kv_len;
     int adv_B, adv_Lmax;
     float* ent;
+    float* head_part;
+    unsigned int* head_tickets;
     const int32_t* m_dev;
     const __nv_bfloat16* gate;
     const int32_t* img_row;
@@ -229,6 +231,8 @@ GemmParams make_params(nova_ctx* ctx, const nova_gemm_args& a)
     p.res = a.res; p.res_row = a.res_row; p.C = a.C; p.k_cache = a.k_cache; p.v_cache = a.v_cache;
     p.kv_row = a.kv_row; p.status = ctx->dev_status;
     p.adv_cu_keep = a.adv_cu_keep; p.adv_kv_len = a.adv_kv_len; p.adv_B = a.adv_B; p.adv_Lmax = a.adv_Lmax;
+    p.head_tickets = ctx->dev_status + NOVA_STATUS_WORDS + NOVA_MEAN_MAX_SEGMENTS * 2;
+    p.head_part = (float*)(p.head_tickets + NOVA_TICKETS);
     p.ent = a.ent; p.m_dev = a.m_dev; p.gate = a.gate; p.img_row = a.img_row;
     p.out_row = a.out_row; p.diff_in = a.diff_in; p.diff_out = a.diff_out; p.early_trigger = a.early_trigger;
     p.count_settled = a.count_settled;
@@ -325,14 +329,26 @@ __device__ __forceinline__ PairTile decode_tile(int entry, int span, int tiles_f
 }
 
 // Entry of the work list that pair `pair` handles as its `local`-th tile, or -1 past the end.
-// group == 0: entries pair, pair + num_pairs, ... (any tile to any pair). group > 0 (entropy
-// epilogue, group = tiles along N, N-fastest order): a pair takes whole row blocks, all their `group`
-// column tiles in turn, so that the epilogue threads can carry a row's softmax state across them.
+// group == 0: entries pair, pair + num_pairs, ... (any tile to any pair). Otherwise (entropy epilogue, |group| = tiles along N,
+// N-fastest order) the epilogue threads carry a row's softmax state along its row block, and a pair takes
+//   group > 0  whole row blocks, all their column tiles in turn;
+//   group < 0  as many consecutive tiles as any other, or one less. A row block that lies in the ranges of several pairs is
+//              merged by the one that finishes its part last (EntropyState::publish).
+// Ranges where they take at most five sixths of the rounds: 16384 rows of 2048 against 4096 codes, 64 blocks on 74 pairs, take
+// 178 us as whole blocks, in 16 rounds in which all pairs read the same column tile, and 188 us as ranges of 14 tiles.
+// Fewer rows, us as whole blocks -> as ranges: 130 rows 150 -> 24, 4096 151 -> 54, 8192 152 -> 85, 12288 155 -> 129.
+__device__ __forceinline__ int range_start(int pair, int num_pairs, int num_tiles) { return (int)((long)pair * num_tiles / num_pairs); }
+__device__ __forceinline__ int range_owner(int tile, int num_pairs, int num_tiles)
+{
+    return (int)(((long)(tile + 1) * num_pairs - 1) / num_tiles);
+}
 __device__ __forceinline__ int pair_entry(int local, int pair, int num_pairs, int num_tiles, int group)
 {
-    int e;
-    if (group == 0) e = pair + local * num_pairs;
-    else e = (pair + (local / group) * num_pairs) * group + local % group;
+    if (group < 0) {
+        const int e = range_start(pair, num_pairs, num_tiles) + local;
+        return e < range_start(pair + 1, num_pairs, num_tiles) ? e : -1;
+    }
+    const int e = group == 0 ? pair + local * num_pairs : (pair + (local / group) * num_pairs) * group + local % group;
     return e < num_tiles ? e : -1;
 }
 
@@ -429,6 +445,37 @@ struct EntropyState {
             u2 = fma_f32x2(d2, e2, u2);
         }
     }
+    // A part of a row, for the pair that merges: slot of [m, s, u][256 rows] at the row.
+    __device__ __forceinline__ void publish(float* slot) const
+    {
+        float s_lo, s_hi, u_lo, u_hi;
+        unpack_f32x2(s2, s_lo, s_hi);
+        unpack_f32x2(u2, u_lo, u_hi);
+        __stcg(slot, m);
+        __stcg(slot + 256, s_lo + s_hi);
+        __stcg(slot + 512, u_lo + u_hi);
+    }
+    // One more part. (A part without a finite maximum is not finite itself, and stays so in the result.)
+    __device__ __forceinline__ void merge(const float* slot, bool first)
+    {
+        constexpr float kLog2e = 1.4426950408889634f;
+        const float m_p = __ldcg(slot), s_p = __ldcg(slot + 256), u_p = __ldcg(slot + 512);
+        if (first) {
+            m = m_p;
+            s2 = pack_f32x2(s_p, 0.f);
+            u2 = pack_f32x2(u_p, 0.f);
+            return;
+        }
+        float s, u, zero;
+        unpack_f32x2(s2, s, zero);
+        unpack_f32x2(u2, u, zero);
+        const float top = fmaxf(m, m_p), d = (m - top) * kLog2e, d_p = (m_p - top) * kLog2e, f = ex2_approx(d), f_p = ex2_approx(d_p);
+        u = (u + d * s) * f + (u_p + d_p * s_p) * f_p;
+        s = s * f + s_p * f_p;
+        m = top;
+        s2 = pack_f32x2(s, 0.f);
+        u2 = pack_f32x2(u, 0.f);
+    }
     // H = ln s - u/s (u in log2 units); non-finite inputs give NaN and flag the status word
     __device__ __forceinline__ float finish(unsigned int* status) const
     {
@@ -466,7 +513,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     uint64_t* acc_full = empty_bar + STAGES;     // 2
     uint64_t* acc_empty = acc_full + 2;          // 2
     uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
-    __shared__ int abort_flag_s;
+    __shared__ int abort_flag_s, head_ticket_s;
     volatile int* abort_flag = &abort_flag_s;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -690,9 +737,34 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                     bias = bias_next;
                 }
             }
-            if (EPI == NOVA_EPI_ENTROPY && !idle_warp && t.n0 + BN >= p.N) {
-                // last column tile of this row block: the row's entropy is complete
-                if (row < M) p.ent[row] = est.finish(p.status);
+            if (EPI == NOVA_EPI_ENTROPY && !idle_warp && (t.n0 + BN >= p.N || pair_entry(local + 1, pair, num_pairs, num_tiles, group) < 0)) {
+                // this pair's last column tile of the row block
+                bool mine = true;
+                const int block0 = group < 0 ? tile - tile % -group : 0, first = range_owner(block0, num_pairs, num_tiles);
+                const int last = range_owner(block0 - group - 1, num_pairs, num_tiles);
+                if (group < 0 && first != last) {
+                    // a pair's parts: of its first row block, and of another that is its last
+                    auto slot = [&](int of) {
+                        const int which = range_start(of, num_pairs, num_tiles) < block0 ? 1 : 0;
+                        return p.head_part + (size_t)(of * 2 + which) * NOVA_HEAD_SLOT_FLOATS + rank * 128 + q * 32 + lane;
+                    };
+                    est.publish(slot(pair));
+                    __threadfence();
+                    asm volatile("bar.sync 1, 128;" ::: "memory");
+                    if (warp == 2 && lane == 0) {
+                        unsigned int* ticket = p.head_tickets + first * 2 + rank;
+                        const unsigned int drawn = atomicAdd(ticket, 1u);
+                        if ((int)drawn == last - first) *ticket = 0;       // ready for the next launch
+                        head_ticket_s = (int)drawn;
+                        __threadfence();
+                    }
+                    asm volatile("bar.sync 1, 128;" ::: "memory");
+                    mine = head_ticket_s == last - first;                 // everybody else has published
+                    if (mine) {
+                        for (int of = first; of <= last; ++of) est.merge(slot(of), of == first);      // in this order, whoever does it
+                    }
+                }
+                if (mine && row < M) p.ent[row] = est.finish(p.status);
                 est.reset();
             }
             // this warp has read its part of the buffer: tell the leader's MMA thread
@@ -731,8 +803,9 @@ nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
     const int tiles_m = (a.M + kPairBM - 1) / kPairBM, tiles_n = (a.N + BN - 1) / BN;
     const int tiles = tiles_m * tiles_n;
     constexpr bool entropy = (EPI == NOVA_EPI_ENTROPY);
-    // the entropy epilogue hands whole row blocks to pairs; otherwise any tile goes to any pair
-    const int pairs = min(entropy ? tiles_m : tiles, ctx->num_sms / 2);
+    const int all_pairs = min(ctx->num_sms / 2, NOVA_TICKETS / 2), block_pairs = min(tiles_m, all_pairs);
+    const bool ranges = entropy && 6 * ((tiles + all_pairs - 1) / all_pairs) <= 5 * ((tiles_m + block_pairs - 1) / block_pairs) * tiles_n;
+    const int pairs = entropy && !ranges ? block_pairs : min(tiles, all_pairs);
     // a last partial wave that would occupy at most half of the pairs runs as half-width tiles
     const int rem = tiles % pairs;
     const int tiles_full = (!entropy && rem > 0 && 2 * rem <= pairs) ? tiles - rem : tiles;
@@ -742,7 +815,7 @@ nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
         // sweep the smaller operand; the entropy epilogue needs the N-fastest order
         const int span = (entropy || (long)a.M >= (long)a.N) ? -tiles_n : tiles_m;
         NOVA_CUDA_CHECK(ctx, nova_launch_pdl(kern, dim3(2 * pairs), dim3(kPairThreads), L::kTotal, st, 0, ta, tw, tw_half, p, span,
-                                             tiles_full, entries, entropy ? tiles_n : 0, split_caps(ctx->num_sms)));
+                                             tiles_full, entries, !entropy ? 0 : ranges ? -tiles_n : tiles_n, split_caps(ctx->num_sms)));
     }
     return NOVA_OK;
 }

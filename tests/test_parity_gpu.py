@@ -227,6 +227,19 @@ def test_head_entropy_matches_oracle(ctx, S, N, C, V, bias):
     _head_case(ctx, S, N, C, V, seed=31, bias=bias)
 
 
+@pytest.mark.parametrize("S,N,V", [(1, 130, 4096), (3, 1000, 1024), (5, 700, 2080)])
+def test_head_entropy_row_blocks_shared_by_cta_pairs(ctx, S, N, V):
+    """Row blocks whose column tiles several CTA pairs share (16 pairs one block; blocks that lie across two ranges): against
+    the oracle, and the same bits whichever pair merges."""
+    _head_case(ctx, S, N, 64, V, seed=41)
+    x, w = synth.activations(S, N, 64, 41, DEV), synth.randn_bf16((V, 64), 42, DEV, std=0.4)
+    got = [torch.empty((S, N), dtype=torch.float32, device=DEV) for _ in range(6)]
+    for ent in got:
+        nova.nova_head_entropy(ctx, x, w, None, ent, None)
+    assert ctx.device_status() == 0
+    assert all(torch.equal(got[0], ent) for ent in got[1:])
+
+
 def test_head_entropy_full_size_sampled_rows(ctx):
     """Batch 4 at 64 x 64 tokens, width 2048, V = 4096 (the benchmark's launch): sampled rows."""
     rows = np.array([0, 127, 128, 255, 256, 4095, 4096, 8191, 12287, 12288, 16383])
