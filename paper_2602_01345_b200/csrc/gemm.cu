@@ -672,7 +672,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             } else {
                 // After the turn-round this lane holds features 4 * (lane % 8) .. + 3 of a chunk's 32, of rows
                 // row0 + lane / 8 + 4 i. What the epilogue reads of the first chunk is fetched before the accumulator is
-                // ready, of the next one while this one is worked on; all of it is brought to L2 before. With a residual the
+                // ready, of the next one while this one is worked on; in a pair's last tile all of it is brought to L2 before. With a residual the
                 // loop is not unrolled: a launch whose pairs have one tile each runs this code once. After the last MMA of
                 // 2252 rows x 1920 features, gated, it takes 6.4 us (7 before, unrolled and with the gate's row looked up and loaded
                 // in turn), 8.7 with a second output (13, its other operand loaded where it was used): latency of what is
@@ -683,7 +683,8 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 EpiRows<EPI> er;
                 EpiData<EPI> ed;
                 uint2 bias = make_uint2(0, 0);
-                if (EPI == NOVA_EPI_BIAS_RES && chunks > 0) {
+                const bool last_tile = pair_entry(local + 1, pair, num_pairs, num_tiles, group) < 0;
+                if (EPI == NOVA_EPI_BIAS_RES && last_tile && chunks > 0) {
                     // the tile's part of this lane's row, of the residual (first warp of the quarter) or of diff_in
                     const int at = min(row, M - 1), in = p.res_row ? p.res_row[at] : at, out = p.out_row ? p.out_row[at] : at;
                     const __nv_bfloat16* src = c_first == 0 ? p.res + (long)in * p.N : p.diff_out ? p.diff_in + (long)out * p.N : nullptr;
@@ -699,7 +700,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 if (!ok) break;
                 tc_fence_after();
                 // the next kernel is let in at the last tile (measured at the split kernel's trigger)
-                if (pair_entry(local + 1, pair, num_pairs, num_tiles, group) < 0) pdl_launch_dependents();
+                if (last_tile) pdl_launch_dependents();
                 float* turn = (float*)(smem + L::kTurnOff + (warp - 2) * 4096);
 #pragma unroll (EPI == NOVA_EPI_BIAS_RES ? 1 : BN / 64)
                 for (int c = 0; c < BN / 64; ++c, col += 64) {
