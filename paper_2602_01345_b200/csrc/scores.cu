@@ -77,10 +77,11 @@ score_mse_kernel(const uint4* __restrict__ x, const uint4* __restrict__ ref, int
 // for the 201 M scores of two images of 1024 tokens, 30 heads and 1216 prior keys. The rest is arranged
 // around keeping it busy: one thread per row of S reads its row from tensor memory 64 scores at a
 // time, two warpgroups take the tiles in turn, each with its own S buffer (256 columns of tensor memory),
-// and at head size 64 two CTAs share an SM. A row's work is spread over a cluster of 1 to 8 CTAs
+// and at head size 64 two CTAs share an SM. In small calls a row's work is spread over a cluster of 1 to 8 CTAs
 // (pass 1: key tiles, pass 2: heads; the size that leaves the least of the last wave idle), whose
-// partial results are merged through distributed shared memory in a fixed order: no atomics, results
-// reproducible bit for bit. Both passes, the MSE score and the selection of that shape: 129 us, against 1907
+// partial results are merged through distributed shared memory in a fixed order; in large ones, where a quarter of the time
+// went into starting and merging those and another into the last wave, the launch's tiles are divided evenly (attn_mass_ranges).
+// Either way results are reproducible bit for bit. Both passes of that shape: 105 us in clusters, 87 in ranges, 1876
 // with warp-level matrix fragments and the scores staged through shared memory.
 constexpr int kAmThreads = 320;        // producer warp, MMA warp, two warpgroups of row threads
 constexpr int kAmTile = 128;
@@ -93,8 +94,8 @@ struct AmSmem {
     static constexpr int kAOff = 0;                                    // two A tiles
     static constexpr int kBOff = 2 * kTileBytes;
     static constexpr int kLseOff = kBOff + kStages * kTileBytes;       // [8 warps][2][128] fp32 (pass 2)
-    static constexpr int kStatOff = kLseOff + 8 * 2 * kAmTile * 4;     // [2 warpgroups][128] float2
-    static constexpr int kBarOff = kStatOff + 2 * kAmTile * 8;
+    static constexpr int kStatOff = kLseOff + 8 * 2 * kAmTile * 4;     // [2 in turn][2 warpgroups][128] float2
+    static constexpr int kBarOff = kStatOff + 2 * 2 * kAmTile * 8;
     static constexpr int kTotal = kBarOff + 256 + 1024;
 };
 
@@ -102,8 +103,11 @@ struct AmParams {
     const int32_t* kv_len;
     int N, Lmax, n_heads;
     float scale_log2e;
+    int B;
     float* lse;
     float* score;
+    float2* part;                // [CTA][first or last of its rows][128]
+    unsigned int* tickets;       // one per CTA: of the row that starts in its range and does not end there
     unsigned int* status;
 };
 
@@ -140,6 +144,79 @@ __device__ __forceinline__ float2 ld_dsmem2(uint32_t cluster_addr)
     float2 v;
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr) : "memory");
     return v;
+}
+
+// State of one row of S across its tiles, and one tile: the thread's row of S from tensor memory, 64 scores at a time, then the
+// buffer is released. Pass 1: `valid` columns count. Pass 2: neg_lse holds -lse of the tile's columns.
+struct AmRow {
+    float c, m2, l;              // score scale in the log2 domain; pass 1: running maximum (log2 domain) and sum
+    uint64_t c2, acc[2];         // pass 2: sums
+    __device__ __forceinline__ void reset()
+    {
+        m2 = -1e30f;
+        l = 0.f;
+        acc[0] = acc[1] = pack_f32x2(0.f, 0.f);
+    }
+    // what is left of the row: (maximum, sum), or (0, sum)
+    template <int PASS>
+    __device__ __forceinline__ float2 result() const
+    {
+        if (PASS == 1) return make_float2(m2, l);
+        float s0, s1;
+        unpack_f32x2(add_f32x2(acc[0], acc[1]), s0, s1);
+        return make_float2(0.f, s0 + s1);
+    }
+};
+template <int PASS>
+__device__ __forceinline__ void am_tile(AmRow& s, uint32_t s_addr, uint64_t* s_empty, int lane, int valid, const float* neg_lse)
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t sv[64];
+        tc::tmem_ld32(s_addr + h * 64, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
+        tc::tmem_ld32(s_addr + h * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[32]));
+        tc::tmem_ld_wait();
+        if (h == 1) {            // the tile now lives in registers: the tensor core may have the buffer
+            tc::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(s_empty);
+        }
+        if (PASS == 1) {
+            if (valid < (h + 1) * 64) {
+#pragma unroll
+                for (int j = 0; j < 64; ++j)
+                    if (h * 64 + j >= valid) sv[j] = 0xff800000u;        // -inf: past the last key of the tile
+            }
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int j = 0; j < 64; ++j) mx[j & 3] = fmaxf(mx[j & 3], __uint_as_float(sv[j]));
+            const float t2 = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * s.c;
+            const float m_new = fmaxf(s.m2, t2);
+            const uint64_t nm2 = pack_f32x2(-m_new, -m_new);
+            uint64_t part[2] = {pack_f32x2(0.f, 0.f), pack_f32x2(0.f, 0.f)};
+#pragma unroll
+            for (int j = 0; j < 64; j += 2) {
+                float d0, d1;
+                unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), s.c2, nm2), d0, d1);
+                part[(j >> 1) & 1] = add_f32x2(part[(j >> 1) & 1], pack_f32x2(ex2(d0), ex2(d1)));
+            }
+            float s0, s1;
+            unpack_f32x2(add_f32x2(part[0], part[1]), s0, s1);
+            s.l = s.l * ex2(s.m2 - m_new) + (s0 + s1);
+            s.m2 = m_new;
+        } else {
+            const ulonglong2* e2 = (const ulonglong2*)(neg_lse + h * 64);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const ulonglong2 e = e2[j];        // four -lse values, the same address in every lane
+                float d0, d1, d2, d3;
+                unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[4 * j]), __uint_as_float(sv[4 * j + 1])), s.c2, e.x), d0, d1);
+                unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[4 * j + 2]), __uint_as_float(sv[4 * j + 3])), s.c2, e.y), d2, d3);
+                s.acc[0] = add_f32x2(s.acc[0], pack_f32x2(ex2(d0), ex2(d1)));
+                s.acc[1] = add_f32x2(s.acc[1], pack_f32x2(ex2(d2), ex2(d3)));
+            }
+        }
+    }
 }
 
 // PASS 1: blockIdx.y = head, .z = image, cluster index along x = query tile.
@@ -270,11 +347,11 @@ attn_mass(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CU
     } else {
         const int wg = (warp - 2) >> 2, q = warp & 3, row = q * 32 + lane;
         const uint32_t s_addr = tmem_base + ((uint32_t)(q * 32) << 16) + 128u * wg;
-        const float c = p.scale_log2e;
-        const uint64_t c2 = pack_f32x2(c, c);
         float* lse_s = (float*)(smem + L::kLseOff) + (warp - 2) * 2 * kAmTile;
-        float m2 = -1e30f, l = 0.f;                    // pass 1: running maximum (log2 domain) and sum
-        uint64_t acc[2] = {pack_f32x2(0.f, 0.f), pack_f32x2(0.f, 0.f)};      // pass 2: sums
+        AmRow s;
+        s.c = p.scale_log2e;
+        s.c2 = pack_f32x2(s.c, s.c);
+        s.reset();
         for (int i = wg; i < total; i += 2) {
             int valid = kAmTile;
             if (PASS == 1) {
@@ -294,60 +371,10 @@ attn_mass(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CU
             }
             if (!mbar_wait_warp(&s_full[wg], (uint32_t)(i >> 1) & 1u, abort_flag, p.status)) break;
             tc_fence_after();
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                uint32_t sv[64];
-                tmem_ld32(s_addr + h * 64, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
-                tmem_ld32(s_addr + h * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[32]));
-                tmem_ld_wait();
-                if (h == 1) {            // the tile now lives in registers: the tensor core may have the buffer
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&s_empty[wg]);
-                }
-                if (PASS == 1) {
-                    if (valid < (h + 1) * 64) {
-#pragma unroll
-                        for (int j = 0; j < 64; ++j)
-                            if (h * 64 + j >= valid) sv[j] = 0xff800000u;        // -inf: past the last key of the tile
-                    }
-                    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                    for (int j = 0; j < 64; ++j) mx[j & 3] = fmaxf(mx[j & 3], __uint_as_float(sv[j]));
-                    const float t2 = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c;
-                    const float m_new = fmaxf(m2, t2);
-                    const uint64_t nm2 = pack_f32x2(-m_new, -m_new);
-                    uint64_t part[2] = {pack_f32x2(0.f, 0.f), pack_f32x2(0.f, 0.f)};
-#pragma unroll
-                    for (int j = 0; j < 64; j += 2) {
-                        float d0, d1;
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), c2, nm2), d0, d1);
-                        part[(j >> 1) & 1] = add_f32x2(part[(j >> 1) & 1], pack_f32x2(ex2(d0), ex2(d1)));
-                    }
-                    float s0, s1;
-                    unpack_f32x2(add_f32x2(part[0], part[1]), s0, s1);
-                    l = l * ex2(m2 - m_new) + (s0 + s1);
-                    m2 = m_new;
-                } else {
-                    const ulonglong2* e2 = (const ulonglong2*)(lse_s + ((i >> 1) & 1) * kAmTile + h * 64);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const ulonglong2 e = e2[j];        // four -lse values, the same address in every lane
-                        float d0, d1, d2, d3;
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[4 * j]), __uint_as_float(sv[4 * j + 1])), c2, e.x), d0, d1);
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sv[4 * j + 2]), __uint_as_float(sv[4 * j + 3])), c2, e.y), d2, d3);
-                        acc[0] = add_f32x2(acc[0], pack_f32x2(ex2(d0), ex2(d1)));
-                        acc[1] = add_f32x2(acc[1], pack_f32x2(ex2(d2), ex2(d3)));
-                    }
-                }
-            }
+            am_tile<PASS>(s, s_addr, &s_empty[wg], lane, valid, lse_s + ((i >> 1) & 1) * kAmTile);
         }
-        float2 mine = make_float2(m2, l);
-        if (PASS == 2) {
-            float s0, s1;
-            unpack_f32x2(add_f32x2(acc[0], acc[1]), s0, s1);
-            mine = make_float2(s0 + s1, 0.f);
-        }
+        float2 mine = s.result<PASS>();
+        if (PASS == 2) mine = make_float2(mine.y, 0.f);
         ((float2*)(smem + L::kStatOff))[wg * kAmTile + row] = mine;
     }
     tc_fence_before();
@@ -379,6 +406,264 @@ attn_mass(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CU
     cluster_sync_all();              // nobody's shared memory goes while it is read
 }
 
+// The same for launches in which a CTA gets many tiles: the launch's tiles, in the order of their rows, are divided evenly over as
+// many CTAs as run at once. Rows that lie in the ranges of several CTAs are merged through memory by the CTA that finishes its part
+// last, in the order of the CTAs: reproducible bit for bit.
+// Where a CTA is in the launch's tiles. Pass 1: rows = (image, head, query tile), T = the image's key tiles. Pass 2: rows =
+// (image, key tile), T = query tiles of all heads.
+template <int PASS>
+struct AmWalk {
+    int b, item, t, T, items;
+    long row0;                   // first tile of the present row, counted over the launch
+    __device__ __forceinline__ static int tiles_of(const AmParams& p) { return (p.N + kAmTile - 1) / kAmTile; }
+    __device__ __forceinline__ static int old_keys(const AmParams& p, int b) { return PASS == 1 && p.kv_len ? min(max(p.kv_len[b], 0), p.Lmax) : 0; }
+    __device__ __forceinline__ static int row_tiles(const AmParams& p, int b)
+    {
+        return PASS == 1 ? tiles_of(p) + (old_keys(p, b) + kAmTile - 1) / kAmTile : tiles_of(p) * p.n_heads;
+    }
+    __device__ __forceinline__ static long total(const AmParams& p)
+    {
+        const long rows = PASS == 1 ? (long)tiles_of(p) * p.n_heads : tiles_of(p);
+        long n = 0;
+        for (int b = 0; b < p.B; ++b) n += rows * row_tiles(p, b);
+        return n;
+    }
+    __device__ __forceinline__ AmWalk(const AmParams& p, long at)
+    {
+        items = PASS == 1 ? tiles_of(p) * p.n_heads : tiles_of(p);
+        row0 = 0;
+        for (b = 0; b < p.B; ++b) {
+            T = row_tiles(p, b);
+            if (at < row0 + (long)items * T) break;
+            row0 += (long)items * T;
+        }
+        item = (int)((at - row0) / T);
+        row0 += (long)item * T;
+        t = (int)(at - row0);
+    }
+    __device__ __forceinline__ void next(const AmParams& p)
+    {
+        if (++t < T) return;
+        t = 0;
+        row0 += T;
+        if (++item < items) return;
+        item = 0;
+        if (++b < p.B) T = row_tiles(p, b);
+    }
+    __device__ __forceinline__ int head(const AmParams& p) const { return PASS == 1 ? item / tiles_of(p) : t / tiles_of(p); }
+    __device__ __forceinline__ int row_tile(const AmParams& p) const { return PASS == 1 ? item % tiles_of(p) : item; }
+    // does this tile need another A tile than the one before?
+    __device__ __forceinline__ bool new_a(const AmParams& p) const { return PASS == 1 ? t == 0 : t % tiles_of(p) == 0; }
+};
+__device__ __forceinline__ long am_start(long cta, long ctas, long total) { return cta * total / ctas; }
+__device__ __forceinline__ int am_owner(long tile, long ctas, long total) { return (int)(((tile + 1) * ctas - 1) / total); }
+
+template <int DH, int PASS>
+__global__ void __launch_bounds__(kAmThreads, DH == 64 ? 2 : 1)
+attn_mass_ranges(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
+          const __grid_constant__ CUtensorMap tmap_cache, const AmParams p)
+{
+    using namespace tc;
+    using L = AmSmem<DH>;
+    using Walk = AmWalk<PASS>;
+    constexpr int kStages = L::kStages;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t* a_full = (uint64_t*)(smem + L::kBarOff);     // 2
+    uint64_t* a_empty = a_full + 2;                        // 2
+    uint64_t* b_full = a_empty + 2;                        // kStages
+    uint64_t* b_empty = b_full + kStages;                  // kStages
+    uint64_t* s_full = b_empty + kStages;                  // 2
+    uint64_t* s_empty = s_full + 2;                        // 2, one arrival per warp of the warpgroup
+    uint32_t* tmem_slot = (uint32_t*)(s_empty + 2);
+    __shared__ int abort_flag_s, ticket_s;
+    volatile int* abort_flag = &abort_flag_s;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        abort_flag_s = 0;
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&a_full[i], 1);
+            mbar_init(&a_empty[i], 1);
+            mbar_init(&s_full[i], 1);
+            mbar_init(&s_empty[i], 4);
+        }
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(&b_full[i], 1);
+            mbar_init(&b_empty[i], 1);
+        }
+        fence_barrier_init();
+        prefetch_tmap(&tmap_q);
+        prefetch_tmap(&tmap_k);
+        if (PASS == 1) prefetch_tmap(&tmap_cache);
+    }
+    if (warp == 1) tmem_alloc(tmem_slot, 256);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    pdl_launch_dependents();
+    pdl_wait();
+    const long all = Walk::total(p), begin = am_start(blockIdx.x, gridDim.x, all);
+    const int total = (int)(am_start(blockIdx.x + 1, gridDim.x, all) - begin);
+
+    if (warp == 0) {
+        if (elect_one() && total > 0) {
+            bool ok = true;
+            int i = 0, groups = 0;
+            Walk w(p, begin);
+            for (; i < total && ok; ++i, w.next(p)) {
+                const int head = w.head(p);
+                if (i == 0 || w.new_a(p)) {
+                    const int g = groups & 1;
+                    if (groups >= 2) ok = mbar_wait(&a_empty[g], (uint32_t)((groups >> 1) - 1) & 1u, abort_flag, p.status);
+                    if (!ok) break;
+                    mbar_arrive_expect_tx(&a_full[g], L::kTileBytes);
+                    for (int sl = 0; sl < DH / 64; ++sl)
+                        tma_load_3d(smem + L::kAOff + g * L::kTileBytes + sl * kAmSlab, PASS == 1 ? &tmap_q : &tmap_k,
+                                    &a_full[g], head * DH + sl * 64, w.row_tile(p) * kAmTile, w.b);
+                    ++groups;
+                }
+                const int st = i % kStages;
+                if (i >= kStages) ok = mbar_wait(&b_empty[st], (uint32_t)((i / kStages) - 1) & 1u, abort_flag, p.status);
+                if (!ok) break;
+                const CUtensorMap* map = PASS == 1 ? &tmap_k : &tmap_q;
+                int tile = PASS == 1 ? w.t : w.t % Walk::tiles_of(p);
+                if (PASS == 1) {
+                    const int tiles_old = w.T - Walk::tiles_of(p);
+                    if (tile < tiles_old) map = &tmap_cache;
+                    else tile -= tiles_old;
+                }
+                mbar_arrive_expect_tx(&b_full[st], L::kTileBytes);
+                for (int sl = 0; sl < DH / 64; ++sl)
+                    tma_load_3d(smem + L::kBOff + st * L::kTileBytes + sl * kAmSlab, map, &b_full[st], head * DH + sl * 64,
+                                tile * kAmTile, w.b);
+            }
+            if (*abort_flag) {       // let the copies in flight land before shared memory is released
+                for (int g = max(0, groups - 2); g < groups; ++g) mbar_drain(&a_full[g & 1], (uint32_t)(g >> 1) & 1u);
+                for (int j = max(0, i - kStages); j < i; ++j) mbar_drain(&b_full[j % kStages], (uint32_t)(j / kStages) & 1u);
+            }
+        }
+    } else if (warp == 1) {
+        if (elect_one() && total > 0) {
+            constexpr uint32_t idesc = idesc_bf16_f32(kAmTile, kAmTile, 0);
+            const uint64_t a_desc = smem_desc_sw128(smem_u32(smem + L::kAOff), 16, 1024);
+            const uint64_t b_desc = smem_desc_sw128(smem_u32(smem + L::kBOff), 16, 1024);
+            bool ok = true;
+            int groups = 0;
+            Walk w(p, begin);
+            for (int i = 0; i < total && ok; ++i) {
+                if (i == 0 || w.new_a(p)) {
+                    ok = mbar_wait(&a_full[groups & 1], (uint32_t)(groups >> 1) & 1u, abort_flag, p.status);
+                    ++groups;
+                }
+                const int g = (groups - 1) & 1, st = i % kStages;
+                if (ok) ok = mbar_wait(&b_full[st], (uint32_t)(i / kStages) & 1u, abort_flag, p.status);
+                if (ok && i >= 2) ok = mbar_wait(&s_empty[i & 1], (uint32_t)((i >> 1) - 1) & 1u, abort_flag, p.status);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t ad = a_desc + (uint32_t)(g * (L::kTileBytes >> 4));
+                const uint64_t bd = b_desc + (uint32_t)(st * (L::kTileBytes >> 4));
+#pragma unroll
+                for (int kk = 0; kk < DH / 16; ++kk) {
+                    const uint32_t off = (kk >> 2) * (kAmSlab >> 4) + (kk & 3) * 2;
+                    mma_bf16_ss(tmem_base + 128u * (i & 1), ad + off, bd + off, idesc, kk ? 1u : 0u);
+                }
+                mma_commit(&s_full[i & 1]);
+                mma_commit(&b_empty[st]);
+                w.next(p);
+                if (i + 1 < total && w.new_a(p)) mma_commit(&a_empty[g]);
+            }
+        }
+    } else {
+        const int wg = (warp - 2) >> 2, q = warp & 3, row = q * 32 + lane;
+        const uint32_t s_addr = tmem_base + ((uint32_t)(q * 32) << 16) + 128u * wg;
+        float* lse_s = (float*)(smem + L::kLseOff) + (warp - 2) * 2 * kAmTile;
+        AmRow s;
+        s.c = p.scale_log2e;
+        s.c2 = pack_f32x2(s.c, s.c);
+        s.reset();
+        bool ok = true;                                // after a failed wait only the barriers are kept up: the status word says so
+        int ends = 0;                                  // rows finished so far, by this CTA's part of them
+        Walk w(p, begin);
+        for (int i = 0; i < total; ++i) {
+            if ((i & 1) == wg && ok) {
+                int valid = kAmTile;
+                if (PASS == 1) {
+                    const int tiles_old = w.T - Walk::tiles_of(p);
+                    valid = w.t < tiles_old ? Walk::old_keys(p, w.b) - w.t * kAmTile : p.N - (w.t - tiles_old) * kAmTile;
+                } else {
+                    // -lse of the tile's queries, a copy per warp (no barrier between warps); -inf past the last query
+                    const int q0 = (w.t % Walk::tiles_of(p)) * kAmTile;
+                    const float* src = p.lse + ((long)w.b * p.n_heads + w.head(p)) * p.N;
+                    float* dst = lse_s + ((i >> 1) & 1) * kAmTile;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int qi = q0 + j * 32 + lane;
+                        dst[j * 32 + lane] = qi < p.N ? -src[qi] : -INFINITY;
+                    }
+                    __syncwarp();
+                }
+                ok = mbar_wait_warp(&s_full[wg], (uint32_t)(i >> 1) & 1u, abort_flag, p.status);
+                tc_fence_after();
+                am_tile<PASS>(s, s_addr, &s_empty[wg], lane, valid, lse_s + ((i >> 1) & 1) * kAmTile);
+            }
+            if (w.t == w.T - 1 || i == total - 1) {
+                // the end of this CTA's part of the row: warpgroup 1 hands its half to warpgroup 0
+                float2* stat = (float2*)(smem + L::kStatOff) + (ends & 1) * 2 * kAmTile;
+                const float2 mine = s.result<PASS>();
+                s.reset();
+                ++ends;
+                if (wg == 1) stat[row] = mine;
+                asm volatile("bar.sync 1, 256;" ::: "memory");
+                if (wg == 0) {
+                    auto merge = [](float2 x, float2 y) {
+                        if (PASS == 2) return make_float2(0.f, x.y + y.y);
+                        const float m = fmaxf(x.x, y.x);
+                        return make_float2(m, x.y * exp2f(x.x - m) + y.y * exp2f(y.x - m));
+                    };
+                    float2 sum = merge(mine, stat[row]);
+                    const int first = am_owner(w.row0, gridDim.x, all), last = am_owner(w.row0 + w.T - 1, gridDim.x, all);
+                    bool write = true;
+                    if (first != last) {
+                        // a CTA's parts: of its first row, and of another that is its last
+                        auto slot = [&](int of) {
+                            return p.part + (of * 2 + (am_start(of, gridDim.x, all) < w.row0 ? 1 : 0)) * kAmTile + row;
+                        };
+                        __stcg(slot(blockIdx.x), sum);
+                        __threadfence();
+                        asm volatile("bar.sync 2, 128;" ::: "memory");
+                        if (threadIdx.x == 64) {
+                            const unsigned int drawn = atomicAdd(p.tickets + first, 1u);
+                            if ((int)drawn == last - first) p.tickets[first] = 0;       // ready for the next launch
+                            ticket_s = (int)drawn;
+                            __threadfence();
+                        }
+                        asm volatile("bar.sync 2, 128;" ::: "memory");
+                        write = ticket_s == last - first;                              // everybody else has published
+                        if (write) {
+                            sum = __ldcg(slot(first));
+                            for (int of = first + 1; of <= last; ++of) sum = merge(sum, __ldcg(slot(of)));
+                        }
+                    }
+                    const int at = w.row_tile(p) * kAmTile + row;
+                    if (write && at < p.N) {
+                        if (PASS == 1) p.lse[((long)w.b * p.n_heads + w.head(p)) * p.N + at] = sum.x + log2f(sum.y);
+                        else p.score[(long)w.b * p.N + at] = sum.y / ((float)p.n_heads * (float)p.N);
+                    }
+                }
+            }
+            w.next(p);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 256);
+    }
+}
+
 // Cluster size 1, 2, 4 or 8 for `items` rows of tiles of `steps` steps that can be split `ways` ways: the one
 // with the shortest schedule, a CTA's start-up and merge counted as two steps.
 int am_cluster(long items, long steps, int ways, int num_sms)
@@ -401,6 +686,8 @@ nova_status launch_mass(nova_ctx* ctx, const void* q, const void* k, const void*
     if (ctx->device >= 64 || !attr_done[ctx->device]) {
         NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attn_mass<DH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
         NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attn_mass<DH, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
+        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attn_mass_ranges<DH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
+        NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(attn_mass_ranges<DH, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
         if (ctx->device < 64) attr_done[ctx->device] = true;
     }
     CUtensorMap tq, tk, tcache;
@@ -413,9 +700,24 @@ nova_status launch_mass(nova_ctx* ctx, const void* q, const void* k, const void*
     AmParams p;
     p.kv_len = cached ? kv_len : nullptr; p.N = N; p.Lmax = Lmax; p.n_heads = n_heads;
     p.scale_log2e = (float)((1.0 / sqrt((double)DH)) * 1.4426950408889634);
-    p.lse = lse; p.score = score; p.status = ctx->dev_status;
+    p.lse = lse; p.score = score; p.status = ctx->dev_status; p.B = B;
+    p.tickets = ctx->dev_status + NOVA_STATUS_WORDS + NOVA_MEAN_MAX_SEGMENTS * 2;
+    p.part = (float2*)(p.tickets + NOVA_TICKETS);
     const int tiles = (N + kAmTile - 1) / kAmTile;
     const int steps1 = tiles + (cached ? (Lmax + kAmTile - 1) / kAmTile : 0);
+    // Ranges where a CTA gets at least so many tiles of the second pass; with fewer, merging rows through memory costs more
+    // than clusters do. us, clusters -> ranges, at tiles per CTA; head size 64: 2.6 33 -> 40, 5.1 56 -> 51, 6.5 70 -> 61, 8.6 78 -> 65,
+    // 13 104 -> 87, 27 180 -> 148; head size 128: 3.5 25 -> 31, 6.9 42 -> 44 and 46 -> 40, 13.8 78 -> 64, 73 287 -> 247.
+    const long slots = min((long)ctx->num_sms * (DH == 64 ? 2 : 1), (long)NOVA_TICKETS), tiles2 = (long)tiles * tiles * n_heads * B;
+    if (tiles2 >= (DH == 64 ? 5 : 8) * slots) {
+        {
+            nova_launch_scope scope(ctx, NOVA_K_SCORE, st);
+            NOVA_CUDA_CHECK(ctx, nova_launch_pdl(attn_mass_ranges<DH, 1>, dim3((unsigned)slots), dim3(kAmThreads), L::kTotal, st, 0, tq, tk, tcache, p));
+        }
+        nova_launch_scope scope(ctx, NOVA_K_SCORE, st);
+        NOVA_CUDA_CHECK(ctx, nova_launch_pdl(attn_mass_ranges<DH, 2>, dim3((unsigned)slots), dim3(kAmThreads), L::kTotal, st, 0, tq, tk, tcache, p));
+        return NOVA_OK;
+    }
     const int cs1 = am_cluster((long)tiles * n_heads * B, steps1, steps1, ctx->num_sms);
     const int cs2 = am_cluster((long)tiles * B, (long)n_heads * tiles, n_heads, ctx->num_sms);
     cudaLaunchConfig_t cfg;

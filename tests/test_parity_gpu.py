@@ -1530,6 +1530,15 @@ def test_score_attention_mass_matches_oracle(ctx, B, N, C, heads, Lmax, kv_lens)
     assert ctx.device_status() == 0
 
 
+@pytest.mark.parametrize("B,N,C,heads,Lmax,kv_lens", [
+    (2, 900, 896, 14, 1300, [300, 5]),        # head size 64
+    (2, 1000, 1280, 10, 1800, [0, 700]),      # head size 128
+])
+def test_score_attention_mass_rows_shared_by_ranges(ctx, B, N, C, heads, Lmax, kv_lens):
+    """Calls large enough for even ranges of tiles: images with different numbers of key tiles, ragged last tiles."""
+    test_score_attention_mass_matches_oracle(ctx, B, N, C, heads, Lmax, kv_lens)
+
+
 def test_score_bad_args(ctx):
     x = synth.activations(1, 16, 64, 1, DEV)
     s = torch.empty((1, 16), dtype=torch.float32, device=DEV)
