@@ -510,12 +510,13 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
     // The pruned rows depend on nothing that the block computes. With `beside` FC1 lets their kernel in as soon as it has
     // passed its wait, when everything up to LN2 has ended; FC1 itself neither writes what it reads nor reads what it
     // writes. It then runs in the registers and the memory bandwidth that FC1 leaves, one block per SM, which is worth it
-    // where FC1 takes longer: about 110 rows of 2048 a microsecond against 2 M F C / 1.3e15 s. Otherwise, and where the kept
-    // count is not known here, it follows the last GEMM. us after -> beside: a 20x20 scale of one image, 32 layers of 2048,
-    // 2923 -> 2681, a 32x32 scale of four, 30 layers of 1920, 8843 -> 8750, a 16-layer 256x256 generation 9070 -> 8840;
-    // a 64x64 scale of one image with 3072 pruned rows for 1024 kept 6674 -> 7087, and it stays behind.
+    // where FC1 takes well over the time of that: about 110 rows of 2048 a microsecond against 2 M F C / 1.3e15 s. Otherwise, and
+    // where the kept count is not known here, it follows the last GEMM. us after -> beside: a 20x20 scale of one image, 32 layers
+    // of 2048, 2923 -> 2681, a 32x32 scale of four, 30 layers of 1920, 8843 -> 8750, a 16-layer 256x256 generation 9070 -> 8840;
+    // with 3072 pruned rows for 1024 kept, 64x64 tokens, 6674 -> 7087, with 13107 for 3277 33.8 -> 34.4 ms. Above 4096 kept
+    // rows the GEMMs run at the power limit, and it makes no difference (8192: 39.7 ms either way).
     const long pruned = (long)s->B * s->N - M;
-    const bool beside = scatter && !m_on_device && pruned > 0 && pruned * 2048 < (long)M * F;
+    const bool beside = scatter && !m_on_device && pruned > 0 && M <= 4096 && pruned * 3072 < (long)M * F;
     auto restore = [&](bool wait_last) {
         return nova_restore_pruned_rows(ctx, x_in, scatter->prune_idx, cu_keep, scatter->cache_prev, scatter->hp, scatter->wp,
                                         scatter->h, scatter->w, C, s->B, M, m_on_device, scatter->x_out, scatter->cache_out, stream, wait_last);
