@@ -110,10 +110,13 @@ struct nova_launch_scope {
 // once all of its own CTAs have called pdl_launch_dependents or ended, so that launch, barrier and tensor-memory
 // set-up and the next kernel's first CTAs overlap its tail. The short kernels (LayerNorm, restore) call it first
 // thing, or the launch of the next would not be hidden (after their wait: a 16-layer generation 9540 -> 9730 us);
-// the GEMMs and the attention near their end. A kernel touches memory that earlier launches write only after
+// the GEMMs and the attention near their end (but FC1 behind its wait, where the restore works beside it). A kernel touches
+// memory that earlier launches write only after
 // pdl_wait, which returns when the launch before it has completed with all its writes visible; every CTA passes
-// it, also those with nothing to do, so that completion stays transitive. That goes for weights too: a kernel
-// may start while one two launches back, of the caller's, is still writing them. For the same reason these kernels
+// it, also those with nothing to do (or one for all of them: leave_to_other in gemm.cu), so that completion stays transitive.
+// That goes for weights too: a kernel may start while one two launches back, of the caller's, is still writing them. What three
+// kernels read before it (attention's table, a GEMM's device-side count, all of the restore beside FC1) is shown there to be
+// complete: the launch ahead lets this one in only after a wait of its own, or of one further ahead. For the same reason these kernels
 // read with ordinary loads only: ld.global.nc, also as the compiler makes it of a `const T* __restrict__` parameter, is
 // for memory that nobody writes while the kernel lives, and the wait does not order it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

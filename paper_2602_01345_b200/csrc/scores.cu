@@ -21,7 +21,7 @@ __device__ __forceinline__ void unpack2(uint32_t w, float& lo, float& hi)
 constexpr int kMseWarps = 8;
 
 __global__ void __launch_bounds__(kMseWarps * 32)
-score_mse_kernel(const uint4* __restrict__ x, const uint4* __restrict__ ref, int B, int hp, int wp, int h, int w,
+score_mse_kernel(const uint4* x, const uint4* ref, int B, int hp, int wp, int h, int w,
                  int vec_per_row, float* __restrict__ score)
 {
     const int lane = threadIdx.x & 31;
