@@ -32,19 +32,23 @@ struct LnModArgs {
 };
 
 // ---- LayerNorm ----------------------------------------------------------------------------
-// Two warps per row, and eight blocks of them per SM that go through the rows in turn, each loading its next row
-// before it works on the present one. The row (C <= 64 * 8 * VEC bf16) stays in registers between the mean, the
-// variance and the normalisation, so x is read once and out written once.
-// What bounds it: HBM and L2 at many rows; at few the chain list -> row -> two reductions -> store, so a thread
-// has little to do and all its loads go out first, gain and bias too. With one warp per row and eight rows per block the
-// code was four times as long and gain and bias were a load of their own at the end of the chain; back to back over warm
-// inputs, us: 300 rows x 2048 4.4 -> 2.4, 1024 x 2048 5.2 -> 3.3, 1600 x 2048 5.3 -> 4.2, 2252 x 1920 5.4 -> 4.7, 8192 x 2048
-// 12.5 -> 12.3 (5.5 TB/s), 256 x 1024 3.1 -> 2.3. With a block for each row 2.4, 3.7, 4.0, 5.0, 12.5 and 2.3, but a launch sized by
-// a bound paid for its empty blocks (1024 rows of 4096: 6.4, now 3.5). Six blocks per SM: 4.0, 4.5, 6.1, 15.9 from 1024 x 2048 on.
-// (Four warps per row: 3.0, 4.6, 4.6, 5.6, 14.9 and 2.0. The warps per row must not depend on the row count, which a
-// device-driven launch does not know, or the sums of the two forms would differ in their last bits.)
+// A row (C <= 64 * 8 * VEC bf16, or half of that with one warp) is the work of one or two warps, in persistent blocks of two
+// warps that go through the rows in turn. x is read once and out written once; in between the row stays in registers.
+// The sums of a row are made in an order that depends on its width alone, so that a token's result is the same to the last bit in any
+// launch: 32 partial sums, of the 128-bit pieces l, l + 32, l + 64, ..., the even and the odd features apart, the even added to
+// the odd ones, then a butterfly. One warp does that as packed pairs. Of two warps one has the row's even features and the other its odd
+// ones: they load alternate pieces, hand each other through shared memory the half that the other needs, and meet again for the
+// one addition per lane.
+// What bounds it: HBM and L2 at many rows, and instructions close behind; at few the chain list -> row -> two reductions -> store, so
+// a thread has little to do and all its loads go out first, gain and bias too. Two warps while all their rows run at once with some
+// room left for the next launch (7 of the 8 rows per SM: 1024 rows of 2048 in 4.0 us, with one warp 4.3; 1184 in 5.5 and 4.1), and
+// where a row is too wide for one warp's registers; else one, which saves the exchange. Back to back over warm inputs, us, with one
+// warp per row in blocks of eight rows that end with them -> this: 256 rows x 1024 2.5 -> 1.9, 300 x 2048 4.0 -> 2.8, 1600 x 2048
+// 4.9 -> 4.7, 2252 x 1920 4.9 -> 4.8, 8192 x 2048 11.4 -> 10.8 (6.2 TB/s), 2048 x 4096 13.5 -> 8.9, 2048 x 8192 43 -> 20. With two warps
+// that each add up their own pieces 1.9, 2.4, 5.4, 5.0, 10.4, 8.7 and 15, but other last bits.
 constexpr int kLnThreads = 64;
 constexpr int kLnBlocksPerSm = 8;
+constexpr int kLnOneVec = 8;           // widest row of one warp: 8 pieces per lane, C = 2048
 
 __device__ __forceinline__ uint4 ld_stream(const uint4* p)
 {
@@ -61,29 +65,59 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
-// Sum over the block's two warps, in warp order. Two slots in turn: all have read one when they meet at the other's barrier.
-__device__ __forceinline__ float row_sum(float v, float* slot)
+// A row's sum from its two warps' halves: lane by lane, then over the lanes. Two slots of 64 floats in turn: all have read one when
+// they meet at the other's barrier.
+__device__ __forceinline__ float row_sum(float half, float* slot)
 {
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = v;
+    slot[threadIdx.x] = half;
     __syncthreads();
-    return slot[0] + slot[1];
+    return warp_sum(half + slot[threadIdx.x ^ 32]);
 }
 
-template <int VEC, bool MAPS, bool MOD>
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float lo_f32(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float hi_f32(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+__device__ __forceinline__ uint64_t bf16x2_f32x2(uint32_t w) { return pack_f32x2(lo_f32(w), hi_f32(w)); }
+
+// VEC: 128-bit pieces per thread
+template <int VEC, int WARPS, bool MAPS, bool MOD>
 __global__ void __launch_bounds__(kLnThreads, kLnBlocksPerSm)
 layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps, int M, const int32_t* m_dev, int vec_per_row,
                uint4* __restrict__ out, const RowMapArgs maps, const LnModArgs mod)
 {
-    constexpr bool kAhead = VEC <= 4;      // wider rows have no registers for the next one, nor for gain and bias
-    __shared__ float part[4];
+    constexpr int T = 32 * WARPS, kRows = kLnThreads / T;      // threads of a row, rows of a block
+    // the next row, and gain and bias, are loaded ahead where there are registers for them
+    constexpr bool kAhead = VEC * WARPS <= 8, kGainAhead = WARPS == 2 && VEC <= 4;
+    __shared__ uint2 given[WARPS == 2 ? VEC * kLnThreads : 1];
+    __shared__ float part[2 * kLnThreads];
     pdl_launch_dependents();
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x & (T - 1);
     // Gain and bias come from HBM (each layer has its own): brought to L2 while the launch before this one ends. A
     // prefetch hands nothing to this kernel, so whoever still writes them does no harm. With few
     // rows the launch is a chain of latencies, of which this takes one off: a 16-layer 256x256 generation 9412 ->
     // 9316 us, a 20x20 scale of one image 3097 -> 3058.
-    for (int c = tid * 8; c < vec_per_row; c += kLnThreads * 8) {
+    for (int c = threadIdx.x * 8; c < vec_per_row; c += kLnThreads * 8) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(gamma + c));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(beta + c));
     }
@@ -107,27 +141,27 @@ layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps,
     auto load = [&](long src, uint4 (&d)[VEC]) {
 #pragma unroll
         for (int i = 0; i < VEC; ++i) {
-            const int c = i * kLnThreads + tid;
+            const int c = i * T + tid;
             d[i] = (c < vec_per_row) ? ld_stream(x + src * vec_per_row + c) : make_uint4(0, 0, 0, 0);
         }
     };
-    int r = blockIdx.x;
+    int r = blockIdx.x * kRows + threadIdx.x / T;
     if (r >= M) return;
     long src, src_next = 0;
     int img, img_next = 0;
     uint4 raw[VEC], next[VEC], g[VEC], bt[VEC];
     locate(r, src, img);
     load(src, raw);
-    if (kAhead) {
+    if (kGainAhead) {
 #pragma unroll
         for (int i = 0; i < VEC; ++i) {
-            const int c = i * kLnThreads + tid;
+            const int c = i * T + tid;
             if (c < vec_per_row) { g[i] = gamma[c]; bt[i] = beta[c]; }
         }
     }
     const float n = (float)(vec_per_row * 8);
     while (true) {
-        const int r_next = r + (int)gridDim.x;
+        const int r_next = r + (int)gridDim.x * kRows;
         if (r_next < M) {
             locate(r_next, src_next, img_next);
             if (kAhead) load(src_next, next);
@@ -143,38 +177,91 @@ layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps,
                 maps.kv_row[r] = img * maps.Lmax + len + (r - c0);
             }
         }
-        float sum0 = 0.f, sum1 = 0.f;
+        float mean, rstd;
+        uint2 f[WARPS == 2 ? 2 * VEC : 1];
+        const bool odd = WARPS == 2 && tid >= 32;
+        if constexpr (WARPS == 1) {
+            uint64_t sum = pack_f32x2(0.f, 0.f), sq = sum;
+            float even_f, odd_f;
 #pragma unroll
-        for (int i = 0; i < VEC; ++i) {
-            const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                sum0 += __uint_as_float(w[q] << 16);
-                sum1 += __uint_as_float(w[q] & 0xffff0000u);
-            }
-        }
-        const float mean = row_sum(sum0 + sum1, part) / n;
-        float sq0 = 0.f, sq1 = 0.f;
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) {
-            if (i * kLnThreads + tid < vec_per_row) {
+            for (int i = 0; i < VEC; ++i) {
                 const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float d0 = __uint_as_float(w[q] << 16) - mean, d1 = __uint_as_float(w[q] & 0xffff0000u) - mean;
-                    sq0 = fmaf(d0, d0, sq0);
-                    sq1 = fmaf(d1, d1, sq1);
+                for (int q = 0; q < 4; ++q) sum = add_f32x2(sum, bf16x2_f32x2(w[q]));
+            }
+            unpack_f32x2(sum, even_f, odd_f);
+            mean = warp_sum(even_f + odd_f) / n;
+            const uint64_t neg_mean = pack_f32x2(-mean, -mean);
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) {
+                if (i * T + tid < vec_per_row) {
+                    const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const uint64_t d = add_f32x2(bf16x2_f32x2(w[q]), neg_mean);
+                        sq = fma_f32x2(d, d, sq);
+                    }
                 }
             }
+            unpack_f32x2(sq, even_f, odd_f);
+            rstd = rsqrtf(warp_sum(even_f + odd_f) / n + eps);
+        } else {
+            // f: this warp's features of the whole row, two to a word
+            const uint32_t keep = odd ? 0x7632 : 0x5410, give = odd ? 0x5410 : 0x7632;
+#pragma unroll
+            for (int i = 0; i < VEC; ++i)
+                given[i * T + tid] = make_uint2(__byte_perm(raw[i].x, raw[i].y, give), __byte_perm(raw[i].z, raw[i].w, give));
+            __syncthreads();
+            float sum = 0.f, sq = 0.f;
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) {
+                const uint2 kept = make_uint2(__byte_perm(raw[i].x, raw[i].y, keep), __byte_perm(raw[i].z, raw[i].w, keep));
+                const uint2 got = given[i * T + (tid ^ 32)];
+                f[2 * i] = odd ? got : kept;
+                f[2 * i + 1] = odd ? kept : got;
+#pragma unroll
+                for (int j = 2 * i; j < 2 * i + 2; ++j) {
+                    sum += lo_f32(f[j].x);
+                    sum += hi_f32(f[j].x);
+                    sum += lo_f32(f[j].y);
+                    sum += hi_f32(f[j].y);
+                }
+            }
+            mean = row_sum(sum, part) / n;
+#pragma unroll
+            for (int j = 0; j < 2 * VEC; ++j) {
+                if (j * 32 + (tid & 31) < vec_per_row) {
+                    const float d0 = lo_f32(f[j].x) - mean, d1 = hi_f32(f[j].x) - mean, d2 = lo_f32(f[j].y) - mean, d3 = hi_f32(f[j].y) - mean;
+                    sq = fmaf(d0, d0, sq);
+                    sq = fmaf(d1, d1, sq);
+                    sq = fmaf(d2, d2, sq);
+                    sq = fmaf(d3, d3, sq);
+                }
+            }
+            rstd = rsqrtf(row_sum(sq, part + kLnThreads) / n + eps);
         }
-        const float rstd = rsqrtf(row_sum(sq0 + sq1, part + 2) / n + eps);
+        // (x - mean) * rstd = x * rstd + shift
         const float shift = -mean * rstd;
+        const uint64_t rstd2 = pack_f32x2(rstd, rstd), shift2 = pack_f32x2(shift, shift);
 #pragma unroll
         for (int i = 0; i < VEC; ++i) {
-            const int c = i * kLnThreads + tid;
+            const int c = i * T + tid;
             if (c < vec_per_row) {
-                if (!kAhead) { g[i] = gamma[c]; bt[i] = beta[c]; }
-                const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+                if (!kGainAhead) { g[i] = gamma[c]; bt[i] = beta[c]; }
+                uint64_t v[4];
+                if constexpr (WARPS == 1) {
+                    const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v[q] = bf16x2_f32x2(w[q]);
+                } else {
+                    // the piece from the two halves (the one that was given away is still in shared memory)
+                    const uint2 kept = odd ? f[2 * i + 1] : f[2 * i], gave = given[i * T + tid];
+                    const uint2 ev = odd ? gave : kept, od = odd ? kept : gave;
+                    v[0] = pack_f32x2(lo_f32(ev.x), lo_f32(od.x));
+                    v[1] = pack_f32x2(hi_f32(ev.x), hi_f32(od.x));
+                    v[2] = pack_f32x2(lo_f32(ev.y), lo_f32(od.y));
+                    v[3] = pack_f32x2(hi_f32(ev.y), hi_f32(od.y));
+                }
                 const uint32_t gw[4] = {g[i].x, g[i].y, g[i].z, g[i].w}, bw[4] = {bt[i].x, bt[i].y, bt[i].z, bt[i].w};
                 uint32_t o[4];
                 uint32_t sc[4] = {0, 0, 0, 0}, sh[4] = {0, 0, 0, 0};        // bf16 zeros: no modulation
@@ -182,14 +269,11 @@ layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps,
                 if (MOD && mod.shift) { const uint4 t = mod.shift[(long)img * vec_per_row + c]; sh[0] = t.x; sh[1] = t.y; sh[2] = t.z; sh[3] = t.w; }
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    // (x - mean) * rstd = x * rstd + shift
-                    const float n0 = fmaf(__uint_as_float(w[q] << 16), rstd, shift);
-                    const float n1 = fmaf(__uint_as_float(w[q] & 0xffff0000u), rstd, shift);
-                    float y0 = fmaf(n0, __uint_as_float(gw[q] << 16), __uint_as_float(bw[q] << 16));
-                    float y1 = fmaf(n1, __uint_as_float(gw[q] & 0xffff0000u), __uint_as_float(bw[q] & 0xffff0000u));
+                    float y0, y1;
+                    unpack_f32x2(fma_f32x2(fma_f32x2(v[q], rstd2, shift2), bf16x2_f32x2(gw[q]), bf16x2_f32x2(bw[q])), y0, y1);
                     if (MOD) {
-                        y0 = fmaf(y0, 1.f + __uint_as_float(sc[q] << 16), __uint_as_float(sh[q] << 16));
-                        y1 = fmaf(y1, 1.f + __uint_as_float(sc[q] & 0xffff0000u), __uint_as_float(sh[q] & 0xffff0000u));
+                        y0 = fmaf(y0, 1.f + lo_f32(sc[q]), lo_f32(sh[q]));
+                        y1 = fmaf(y1, 1.f + hi_f32(sc[q]), hi_f32(sh[q]));
                     }
                     __nv_bfloat162 t = __floats2bfloat162_rn(y0, y1);
                     o[q] = *reinterpret_cast<uint32_t*>(&t);
@@ -316,27 +400,32 @@ static nova_status launch_ln(nova_ctx* ctx, const __nv_bfloat16* x, const RowMap
 {
     if (M <= 0) return NOVA_OK;
     const int vec = C / 8;
-    const int per_lane = (vec + kLnThreads - 1) / kLnThreads;
-    const dim3 grid(min(M, ctx->num_sms * kLnBlocksPerSm)), block(kLnThreads);
+    const int fit = ctx->num_sms * kLnBlocksPerSm;
+    // (of a bound on a device-side count a quarter: a last scale keeps about that)
+    const bool one = (m_dev ? M / 4 : M) > fit - fit / 8 && vec <= 32 * kLnOneVec;
+    const dim3 grid(min(one ? (M + 1) / 2 : M, fit)), block(kLnThreads);
     RowMapArgs none;
     memset(&none, 0, sizeof(none));
     cudaError_t le = cudaSuccess;
     nova_launch_scope scope(ctx, NOVA_K_LAYERNORM, st);
-#define NOVA_LN_LAUNCH(V, MAPS, MOD, MAPARG)                                                                     \
-    le = nova_launch_pdl(layernorm_rows<V, MAPS, MOD>, grid, block, 0, st, 0, (const uint4*)x, (const uint4*)g, (const uint4*)b, eps, M, m_dev, vec, (uint4*)out, MAPARG, mod)
-#define NOVA_LN_CASE(V)                                                                                          \
+#define NOVA_LN_LAUNCH(V, W, MAPS, MOD, MAPARG)                                                                     \
+    le = nova_launch_pdl(layernorm_rows<V, W, MAPS, MOD>, grid, block, 0, st, 0, (const uint4*)x, (const uint4*)g, (const uint4*)b, eps, M, m_dev, vec, (uint4*)out, MAPARG, mod)
+#define NOVA_LN_CASE(V, W)                                                                                          \
     do {                                                                                                         \
-        if (maps && modulated) NOVA_LN_LAUNCH(V, true, true, *maps);                                             \
-        else if (maps) NOVA_LN_LAUNCH(V, true, false, *maps);                                                    \
-        else if (modulated) NOVA_LN_LAUNCH(V, false, true, none);                                                \
-        else NOVA_LN_LAUNCH(V, false, false, none);                                                              \
+        if (maps && modulated) NOVA_LN_LAUNCH(V, W, true, true, *maps);                                             \
+        else if (maps) NOVA_LN_LAUNCH(V, W, true, false, *maps);                                                    \
+        else if (modulated) NOVA_LN_LAUNCH(V, W, false, true, none);                                                \
+        else NOVA_LN_LAUNCH(V, W, false, false, none);                                                              \
     } while (0)
     const bool modulated = mod.scale || mod.shift;
-    if (per_lane <= 2) NOVA_LN_CASE(2);
-    else if (per_lane <= 3) NOVA_LN_CASE(3);
-    else if (per_lane <= 4) NOVA_LN_CASE(4);
-    else if (per_lane <= 8) NOVA_LN_CASE(8);
-    else if (per_lane <= 16) NOVA_LN_CASE(16);
+    if (one && vec <= 32 * 4) NOVA_LN_CASE(4, 1);
+    else if (one && vec <= 32 * 6) NOVA_LN_CASE(6, 1);
+    else if (one) NOVA_LN_CASE(kLnOneVec, 1);
+    else if (vec <= 64 * 2) NOVA_LN_CASE(2, 2);
+    else if (vec <= 64 * 3) NOVA_LN_CASE(3, 2);
+    else if (vec <= 64 * 4) NOVA_LN_CASE(4, 2);
+    else if (vec <= 64 * 8) NOVA_LN_CASE(8, 2);
+    else if (vec <= 64 * 16) NOVA_LN_CASE(16, 2);
     else return nova_fail(ctx, NOVA_ERR_SHAPE, "layernorm: C > 8192");
 #undef NOVA_LN_LAUNCH
 #undef NOVA_LN_CASE

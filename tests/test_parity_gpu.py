@@ -739,12 +739,57 @@ def test_block_gemm_tile_edges_host_and_device_count(ctx, C, heads, F, M):
 
 
 @pytest.mark.parametrize("C,heads,ks", [(64, 1, [3, 0]), (192, 3, [1, 2]), (576, 9, [5, 7]), (1088, 17, [2, 3]), (1600, 25, [3, 1]),
-                                        (2112, 33, [1, 2]), (128, 2, [700, 695])])
+                                        (2112, 33, [1, 2]), (128, 2, [700, 695]), (128, 2, [1300, 1295])])
 def test_block_layernorm_widths_and_rows_per_block(ctx, C, heads, ks):
     """LayerNorm's widths: one to five 128-bit pieces per thread, the last of them shared by only some threads, and more
-    rows than blocks, so that a block goes on to a second row (of the other image)."""
+    rows than warps that run at once, so that a block goes on to further rows (of the other image)."""
     N = max(max(ks), 8)
     _block_case(ctx, B=2, N=N, C=C, heads=heads, F=64, Lmax=N + 8, ks=ks, kv_lens=[5, 8], seed=C)
+
+
+def _layernorm_in_order(x, g, b, eps):
+    """LayerNorm of bf16 rows with its fp32 sums in the order that the kernel is to keep: 32 partial sums over the 8-feature
+    pieces l, l + 32, ..., the even features' added to the odd ones', then a butterfly. (Fused multiply-adds: in fp64, then
+    rounded; the reciprocal square root is CUDA's.)"""
+    M, C = x.shape
+    rows = -(-C // 256)
+    fma = lambda p, q, r: (p.astype(np.float64) * q + r).astype(np.float32)  # noqa: E731
+
+    def total(v, valid, fused):
+        acc = np.zeros((2, M, 32), np.float32)
+        for i in range(rows):
+            for j in range(8):
+                t = v[:, i, :, j]
+                acc[j & 1] = np.where(valid[i], fma(t, t, acc[j & 1]) if fused else acc[j & 1] + t, acc[j & 1])
+        t = acc[0] + acc[1]
+        for o in (16, 8, 4, 2, 1):
+            t = t + t[:, np.arange(32) ^ o]
+        return t[:, :1]
+
+    v = np.zeros((M, rows * 256), np.float32)
+    v[:, :C] = x
+    valid = (np.arange(rows * 256) < C).reshape(rows, 32, 8)[:, :, 0]
+    v = v.reshape(M, rows, 32, 8)
+    mean = total(v, valid, False) / np.float32(C)
+    var = total(v - mean[:, :, None, None], valid, True) / np.float32(C)
+    rstd = torch.rsqrt(torch.from_numpy(var + np.float32(eps)).to(DEV)).cpu().numpy()
+    return fma(fma(x, rstd, -mean * rstd), g, b)
+
+
+@pytest.mark.parametrize("C,heads,N", [(1024, 16, 1400), (1088, 17, 300), (1536, 12, 1400), (2048, 16, 300), (2048, 16, 1400), (4160, 65, 200)])
+def test_block_layernorm_order_of_sums(ctx, C, heads, N):
+    """LayerNorm to the last bit, with one and with two warps to a row: with an identity for the keys' projection the new cache rows
+    are its output."""
+    wt = synth.block_weights(C, 64, C, DEV)
+    wt["w_qkv"][C:2 * C] = torch.eye(C, dtype=torch.bfloat16, device=DEV)
+    wt["b_qkv"].zero_()
+    x = synth.activations(1, N, C, C + 1, DEV) + 2.0
+    keep_idx, _, cu, _ = gpu_select(ctx, torch.rand((1, N)).to(DEV), [N])
+    shape = nova.BlockShape(1, N, C, heads, 64, N, N)
+    k, v, kv_len = synth.kv_cache(1, N, 0, C, 5, DEV)
+    _run_block(ctx, shape, nova.BlockWeights(wt, 1e-6), x, keep_idx, cu, k, v, kv_len)
+    want = _layernorm_in_order(f32(x[0]), f32(wt["ln1_g"]), f32(wt["ln1_b"]), 1e-6)
+    assert torch.equal(k[0].cpu(), torch.from_numpy(want).to(torch.bfloat16))
 
 
 def test_block_without_append_leaves_kv_len(ctx):
