@@ -27,7 +27,7 @@
 #define NOVA_ATTN_TICKETS 96
 #define NOVA_MEAN_MAX_CTAS 192        // the accumulator's arrival count has 8 bits
 #define NOVA_MEAN_MAX_SEGMENTS 256
-#define NOVA_TICKETS 512              // of rows that several CTAs of the head or of the attention-mass kernel share, by CTA
+#define NOVA_TICKETS 1024             // of rows that several CTAs share: head, eight for each CTA pair (its reading warps), or attention mass, one for each CTA
 #define NOVA_STATUS_BYTES (NOVA_STATUS_WORDS * 4 + NOVA_MEAN_MAX_SEGMENTS * 8 + NOVA_TICKETS * 4)
 // Behind it: partial results of such rows. Head: [pair][first or last of its row blocks][m, s, u][256 rows] fp32; attention mass:
 // [CTA, up to two per SM][first or last of its rows][128 rows] float2.

@@ -513,7 +513,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     uint64_t* acc_full = empty_bar + STAGES;     // 2
     uint64_t* acc_empty = acc_full + 2;          // 2
     uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
-    __shared__ int abort_flag_s, head_ticket_s;
+    __shared__ int abort_flag_s;
     volatile int* abort_flag = &abort_flag_s;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -750,17 +750,18 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                         return p.head_part + (size_t)(of * 2 + which) * NOVA_HEAD_SLOT_FLOATS + rank * 128 + q * 32 + lane;
                     };
                     est.publish(slot(pair));
+                    // A ticket for each warp's 32 rows, not one for the block behind a barrier: a warp that gives up a wait leaves
+                    // the loop alone, and the others would stay at a barrier for good.
                     __threadfence();
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
-                    if (warp == 2 && lane == 0) {
-                        unsigned int* ticket = p.head_tickets + first * 2 + rank;
-                        const unsigned int drawn = atomicAdd(ticket, 1u);
+                    __syncwarp();
+                    unsigned int drawn = 0;
+                    if (lane == 0) {
+                        unsigned int* ticket = p.head_tickets + (first * 2 + rank) * 4 + q;
+                        drawn = atomicAdd(ticket, 1u);
                         if ((int)drawn == last - first) *ticket = 0;       // ready for the next launch
-                        head_ticket_s = (int)drawn;
                         __threadfence();
                     }
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
-                    mine = head_ticket_s == last - first;                 // everybody else has published
+                    mine = (int)__shfl_sync(0xffffffffu, drawn, 0) == last - first;      // everybody else has published
                     if (mine) {
                         for (int of = first; of <= last; ++of) est.merge(slot(of), of == first);      // in this order, whoever does it
                     }
@@ -804,7 +805,7 @@ nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
     const int tiles_m = (a.M + kPairBM - 1) / kPairBM, tiles_n = (a.N + BN - 1) / BN;
     const int tiles = tiles_m * tiles_n;
     constexpr bool entropy = (EPI == NOVA_EPI_ENTROPY);
-    const int all_pairs = min(ctx->num_sms / 2, NOVA_TICKETS / 2), block_pairs = min(tiles_m, all_pairs);
+    const int all_pairs = min(ctx->num_sms / 2, NOVA_TICKETS / 8), block_pairs = min(tiles_m, all_pairs);
     const bool ranges = entropy && 6 * ((tiles + all_pairs - 1) / all_pairs) <= 5 * ((tiles_m + block_pairs - 1) / block_pairs) * tiles_n;
     const int pairs = entropy && !ranges ? block_pairs : min(tiles, all_pairs);
     // a last partial wave that would occupy at most half of the pairs runs as half-width tiles

@@ -52,6 +52,17 @@ def test_workspace_bytes_host_side():
     assert nova.nova_block_workspace_bytes(bad_dh) == 0
 
 
+def test_gemm_warps_that_give_up_alone_share_no_barrier():
+    """In the GEMM for many tiles (and the head's entropy) each warp leaves its loop on its own when a bounded wait fails, so
+    the loops may not hold a barrier at which the others would stay: read from the source, as a wait that fails beside
+    one that does not cannot be arranged on a GPU without leaving it in an unknown state."""
+    text = open(os.path.join(ROOT, "paper_2602_01345_b200", "csrc", "gemm.cu")).read()
+    kernel = text[text.index("gemm_bf16_tn_pair(const"):text.index("nova_status launch_pair(")]
+    roles = re.sub(r"//[^\n]*", "", kernel[kernel.index("if (warp == 0) {"):kernel.rindex("__syncthreads();")])
+    assert "if (!ok) break;" in roles
+    assert not re.search(r"bar\.sync|barrier\.sync|__syncthreads|__barrier_sync|cluster_sync", roles)
+
+
 def _compare(p_or, p_lib, t, j, N, hs, hl):
     want = oracle.keep_ratios(p_or, t, j, N, hs, hl)
     got = nova.nova_keep_ratios(p_lib, t, j, N, torch.from_numpy(hs), torch.from_numpy(hl) if hl is not None else None)
