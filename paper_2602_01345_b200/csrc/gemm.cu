@@ -393,6 +393,15 @@ struct EntropyState {
         s2 = pack_f32x2(0.f, 0.f);
         u2 = s2;
     }
+    // Sums after a rise of their reference by -shift (log2 domain), f = 2^shift. A rise that leaves nothing of them leaves nothing of
+    // infinite ones either: below -1.5e9, where masks lie, the rounding of m2 is itself an exponent that can overflow.
+    // (A NaN stays one.)
+    static __device__ __forceinline__ void rescale(float& s, float& u, float shift, float f)
+    {
+        const bool gone = f == 0.f;
+        u = gone && u == u ? 0.f : (u + shift * s) * f;
+        s = gone && s == s ? 0.f : s * f;
+    }
     // 32 more logits of the row (fp32 accumulators plus bias)
     __device__ __forceinline__ void add_chunk(const uint32_t (&acc)[32], const __nv_bfloat16* bias)
     {
@@ -424,12 +433,9 @@ struct EntropyState {
             float s_lo, s_hi, u_lo, u_hi;
             unpack_f32x2(s2, s_lo, s_hi);
             unpack_f32x2(u2, u_lo, u_hi);
-            if (m == -INFINITY) { u_lo = u_hi = 0.f; }
-            else {
-                u_lo = (u_lo + shift * s_lo) * f;
-                u_hi = (u_hi + shift * s_hi) * f;
-            }
-            s2 = pack_f32x2(s_lo * f, s_hi * f);
+            rescale(s_lo, u_lo, shift, f);
+            rescale(s_hi, u_hi, shift, f);
+            s2 = pack_f32x2(s_lo, s_hi);
             u2 = pack_f32x2(u_lo, u_hi);
             m = cm;
             m2 = cm * kLog2e;
@@ -459,7 +465,8 @@ struct EntropyState {
     __device__ __forceinline__ void merge(const float* slot, bool first)
     {
         constexpr float kLog2e = 1.4426950408889634f;
-        const float m_p = __ldcg(slot), s_p = __ldcg(slot + 256), u_p = __ldcg(slot + 512);
+        const float m_p = __ldcg(slot);
+        float s_p = __ldcg(slot + 256), u_p = __ldcg(slot + 512);
         if (first) {
             m = m_p;
             s2 = pack_f32x2(s_p, 0.f);
@@ -469,9 +476,11 @@ struct EntropyState {
         float s, u, zero;
         unpack_f32x2(s2, s, zero);
         unpack_f32x2(u2, u, zero);
-        const float top = fmaxf(m, m_p), d = (m - top) * kLog2e, d_p = (m_p - top) * kLog2e, f = ex2_approx(d), f_p = ex2_approx(d_p);
-        u = (u + d * s) * f + (u_p + d_p * s_p) * f_p;
-        s = s * f + s_p * f_p;
+        const float top = fmaxf(m, m_p), d = (m - top) * kLog2e, d_p = (m_p - top) * kLog2e;
+        rescale(s, u, d, ex2_approx(d));
+        rescale(s_p, u_p, d_p, ex2_approx(d_p));
+        s += s_p;
+        u += u_p;
         m = top;
         s2 = pack_f32x2(s, 0.f);
         u2 = pack_f32x2(u, 0.f);

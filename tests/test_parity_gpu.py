@@ -240,6 +240,25 @@ def test_head_entropy_row_blocks_shared_by_cta_pairs(ctx, S, N, V):
     assert all(torch.equal(got[0], ent) for ent in got[1:])
 
 
+@pytest.mark.parametrize("N,V", [(130, 4096), (1000, 1024), (700, 2080), (17000, 1024)])
+@pytest.mark.parametrize("first,last", [(0.9, 1.0), (0.5, 1.0), (0.1, 0.8)])
+@pytest.mark.parametrize("mask", [-1e4, -1e9, -1e30, -1e38])
+def test_head_entropy_masked_codes(ctx, N, V, first, last, mask):
+    """Codes masked out by a bias far below the others, at the end and in the middle, in row blocks that CTA pairs share and (17000
+    rows) in whole ones: parts that hold nothing but masked codes, or begin with them, count for what is left, however low the mask."""
+    x, w = synth.activations(1, N, 64, 43, DEV), synth.randn_bf16((V, 64), 44, DEV, std=0.4)
+    keep = torch.ones((V,), dtype=torch.bool, device=DEV)
+    keep[int(first * V):int(last * V)] = False
+    bias = torch.zeros((V,), dtype=torch.bfloat16, device=DEV)
+    bias[~keep] = mask
+    ent = torch.full((1, N), float("nan"), dtype=torch.float32, device=DEV)
+    nova.nova_head_entropy(ctx, x, w, bias, ent, None)
+    assert ctx.device_status() == 0
+    rows = np.arange(0, N, max(1, N // 1000))
+    want, _ = oracle.head_entropy(f32(x)[:, rows], f32(w[keep]), None)
+    assert np.abs(ent.cpu().numpy()[:, rows] - want).max() <= ENT_TOL
+
+
 def test_head_entropy_full_size_sampled_rows(ctx):
     """Batch 4 at 64 x 64 tokens, width 2048, V = 4096 (the benchmark's launch): sampled rows."""
     rows = np.array([0, 127, 128, 255, 256, 4095, 4096, 8191, 12287, 12288, 16383])
