@@ -706,6 +706,8 @@ extern "C" nova_status nova_pruned_layer_forward(nova_ctx* ctx, const nova_block
     const bool on_dev = m_on_device != 0;
     if ((s->M < total || on_dev) && (!prune_idx || !cache_prev || hp < 1 || wp < 1))
         return nova_fail(ctx, NOVA_ERR_INVALID_ARG, "nova_pruned_layer_forward: pruned rows need prune_idx and cache_prev");
+    if (total > 0 && !nova_aligned16(cache_prev))       // the restore would refuse it too, with half of the layer done
+        return nova_fail(ctx, NOVA_ERR_ALIGNMENT, "nova_pruned_layer_forward: tensors must be 16-byte aligned");
     NOVA_DEVICE_GUARD(ctx, "nova_pruned_layer_forward");
     {   // debug mode: both lists are checked before the block's first kernel, so that a bad pruned list leaves no half-done layer
         const nova_status chk = nova_debug_check_lists(ctx, "nova_pruned_layer_forward", keep_idx, prune_idx, cu_keep,

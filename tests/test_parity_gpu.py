@@ -982,6 +982,29 @@ def test_whole_pruned_step_config1(ctx):
     assert ctx.device_status() == 0
 
 
+@pytest.mark.parametrize("C,heads,F,kept", [(1024, 16, 4096, 115), (128, 2, 256, 40)])     # restore beside FC1, and after FC2
+def test_layer_forward_refuses_misaligned_cache_before_any_launch(ctx, C, heads, F, kept):
+    from paper_2602_01345_b200 import pipeline
+    B, h, w, hp, wp, Lmax = 2, 16, 16, 5, 6, 300
+    N, M = h * w, 2 * kept
+    x = synth.activations(B, N, C, 91, DEV)
+    k, v, kv_len = synth.kv_cache(B, Lmax, 10, C, 92, DEV)
+    k0, v0 = k.clone(), v.clone()
+    keep_idx, prune_idx, cu, _ = gpu_select(ctx, torch.rand((B, N)).to(DEV), [kept, kept])
+    shape = nova.BlockShape(B, N, C, heads, F, Lmax, M)
+    ctx.ensure_workspace(shape)
+    cache_prev = torch.zeros(B * hp * wp * C + 8, dtype=torch.bfloat16, device=DEV)[1:1 + B * hp * wp * C].view(B, hp, wp, C)
+    x_out, cache_out = torch.full_like(x, 7.0), torch.full_like(x, 7.0)
+    launches = pipeline.launch_count(ctx)
+    with pytest.raises(nova.NovaError) as ei:
+        nova.nova_pruned_layer_forward(ctx, nova.BlockWeights(synth.block_weights(C, F, 93, DEV), 1e-6), None, shape, x, keep_idx,
+                                       prune_idx, cu, k, v, kv_len, True, cache_prev, h, w, x_out, cache_out)
+    assert ei.value.status == 3                          # NOVA_ERR_ALIGNMENT
+    assert pipeline.launch_count(ctx) == launches and ctx.device_status() == 0
+    assert torch.equal(k, k0) and torch.equal(v, v0) and kv_len.cpu().tolist() == [10, 10]
+    assert bool((x_out == 7.0).all()) and bool((cache_out == 7.0).all())
+
+
 def test_pipeline_literal_schedule_256_shape(ctx):
     """VAR-d16-shaped layers through the pipeline runner with the paper's schedule taken literally
     (no overrides): the scale history puts the inflection at scale 7, so scale 9 (13 x 13 tokens) is
