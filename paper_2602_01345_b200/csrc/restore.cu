@@ -123,9 +123,9 @@ restore_kernel(const uint4* x_in, const uint4* y_kept, const int32_t* keep_idx, 
             const int y1 = min(y0 + 1, hp - 1), x1 = min(x0 + 1, wp - 1);
             const float fy = sy - (float)y0, fx = sx - (float)x0;
             const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
-            const uint4* c_img = cache_prev + (long)b * hp * wp * vec_per_row;
-            const unsigned c00 = (unsigned)((y0 * wp + x0) * vec_per_row), c01 = (unsigned)((y0 * wp + x1) * vec_per_row);
-            const unsigned c10 = (unsigned)((y1 * wp + x0) * vec_per_row), c11 = (unsigned)((y1 * wp + x1) * vec_per_row);
+            const uint4* c_y0 = cache_prev + (((long)b * hp + y0) * wp + x0) * vec_per_row;      // (64-bit: a cache may be large)
+            const uint4* c_y1 = cache_prev + (((long)b * hp + y1) * wp + x0) * vec_per_row;
+            const int right = (x1 - x0) * vec_per_row;
             const long row = ((long)b * N + i) * vec_per_row;
             for (int v0 = lane; v0 < vec_per_row; v0 += 2 * row_threads) {
                 uint4 xv[2], c[2][4];
@@ -134,7 +134,7 @@ restore_kernel(const uint4* x_in, const uint4* y_kept, const int32_t* keep_idx, 
                     const int v = v0 + k * row_threads;
                     if (v < vec_per_row) {
                         xv[k] = ld_stream(x_in + row + v);
-                        c[k][0] = c_img[c00 + v]; c[k][1] = c_img[c01 + v]; c[k][2] = c_img[c10 + v]; c[k][3] = c_img[c11 + v];
+                        c[k][0] = c_y0[v]; c[k][1] = c_y0[v + right]; c[k][2] = c_y1[v]; c[k][3] = c_y1[v + right];
                     }
                 }
 #pragma unroll

@@ -982,6 +982,32 @@ def test_whole_pruned_step_config1(ctx):
     assert ctx.device_status() == 0
 
 
+def test_restore_from_a_cache_past_32_bit_offsets(ctx):
+    """A residual cache whose last rows lie more than 2^32 128-bit pieces (64 GiB) into the image."""
+    h, w, hp, wp, C = 64, 1, 2100, 2100, 8192
+    if torch.cuda.mem_get_info()[0] < (80 << 30):
+        pytest.skip("needs 80 GiB of free device memory")
+    cache_prev = torch.empty((1, hp, wp, C), dtype=torch.bfloat16, device=DEV)
+    sy, sx = 63.5 * hp / h - 0.5, 0.5 * wp / w - 0.5            # the last token's place in the map
+    y0, x0 = int(sy), int(sx)
+    assert (y0 * wp + x0) * (C // 8) > 2 ** 32
+    corners = synth.activations(2, 2, C, 95, DEV)
+    cache_prev[0, y0:y0 + 2, x0:x0 + 2] = corners
+    x = synth.activations(1, h * w, C, 96, DEV)
+    none = torch.empty((0,), dtype=torch.int32, device=DEV)
+    prune_idx, cu = torch.arange(h * w, dtype=torch.int32, device=DEV), torch.zeros(2, dtype=torch.int32, device=DEV)
+    x_out, cache_out = torch.empty_like(x), torch.empty_like(x)
+    nova.nova_restore_from_cache(ctx, x, x.new_empty((0, C)), none, prune_idx, cu, cache_prev, h, w, x_out, cache_out)
+    assert ctx.device_status() == 0
+    del cache_prev
+    torch.cuda.empty_cache()
+    fy, fx, c = sy - y0, sx - x0, f32(corners)
+    up = (1 - fy) * ((1 - fx) * c[0, 0] + fx * c[0, 1]) + fy * ((1 - fx) * c[1, 0] + fx * c[1, 1])
+    # sizes of 2100 leave the weights exact to about 2^-12 in fp32: within two bf16 units
+    assert np.abs(f32(cache_out)[0, -1] - up).max() <= 2.0 ** -6 * np.abs(up).max()
+    assert np.abs(f32(x_out)[0, -1] - (f32(x)[0, -1] + up)).max() <= 2.0 ** -6 * np.abs(f32(x_out)[0, -1]).max()
+
+
 @pytest.mark.parametrize("C,heads,F,kept", [(1024, 16, 4096, 115), (128, 2, 256, 40)])     # restore beside FC1, and after FC2
 def test_layer_forward_refuses_misaligned_cache_before_any_launch(ctx, C, heads, F, kept):
     from paper_2602_01345_b200 import pipeline
