@@ -413,7 +413,7 @@ attn_mass(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CU
 // (image, key tile), T = query tiles of all heads.
 template <int PASS>
 struct AmWalk {
-    int b, item, t, T, items;
+    int b = 0, item, t, T;
     long row0;                   // first tile of the present row, counted over the launch
     __device__ __forceinline__ static int tiles_of(const AmParams& p) { return (p.N + kAmTile - 1) / kAmTile; }
     __device__ __forceinline__ static int old_keys(const AmParams& p, int b) { return PASS == 1 && p.kv_len ? min(max(p.kv_len[b], 0), p.Lmax) : 0; }
@@ -421,22 +421,41 @@ struct AmWalk {
     {
         return PASS == 1 ? tiles_of(p) + (old_keys(p, b) + kAmTile - 1) / kAmTile : tiles_of(p) * p.n_heads;
     }
-    __device__ __forceinline__ static long total(const AmParams& p)
+    // The launch's tiles, and the place of one of them; by whole warps, 32 images at a time (with one after the other a launch of 60000
+    // images of 16 tokens took 11.2 ms, 3.0 of them for its tiles).
+    __device__ __forceinline__ long image_tiles(const AmParams& p, int b) const { return b < p.B ? (long)rows_of(p) * row_tiles(p, b) : 0; }
+    __device__ __forceinline__ explicit AmWalk(const AmParams&) {}
+    __device__ __forceinline__ static int rows_of(const AmParams& p) { return PASS == 1 ? tiles_of(p) * p.n_heads : tiles_of(p); }
+    __device__ __forceinline__ long total(const AmParams& p) const
     {
-        const long rows = PASS == 1 ? (long)tiles_of(p) * p.n_heads : tiles_of(p);
         long n = 0;
-        for (int b = 0; b < p.B; ++b) n += rows * row_tiles(p, b);
+        for (int b0 = threadIdx.x & 31; b0 < p.B; b0 += 32) n += image_tiles(p, b0);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
         return n;
     }
-    __device__ __forceinline__ AmWalk(const AmParams& p, long at)
+    __device__ __forceinline__ void find(const AmParams& p, long at)
     {
-        items = PASS == 1 ? tiles_of(p) * p.n_heads : tiles_of(p);
+        const int lane = threadIdx.x & 31;
         row0 = 0;
-        for (b = 0; b < p.B; ++b) {
-            T = row_tiles(p, b);
-            if (at < row0 + (long)items * T) break;
-            row0 += (long)items * T;
+        for (int b0 = 0; b0 < p.B; b0 += 32) {
+            const long mine = image_tiles(p, b0 + lane);
+            long incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const uint32_t past = __ballot_sync(0xffffffffu, at < row0 + incl);
+            if (past) {
+                const int at_lane = __ffs(past) - 1;
+                row0 += __shfl_sync(0xffffffffu, incl - mine, at_lane);
+                b = b0 + at_lane;
+                break;
+            }
+            row0 += __shfl_sync(0xffffffffu, incl, 31);
         }
+        T = row_tiles(p, b);
         item = (int)((at - row0) / T);
         row0 += (long)item * T;
         t = (int)(at - row0);
@@ -446,7 +465,7 @@ struct AmWalk {
         if (++t < T) return;
         t = 0;
         row0 += T;
-        if (++item < items) return;
+        if (++item < rows_of(p)) return;
         item = 0;
         if (++b < p.B) T = row_tiles(p, b);
     }
@@ -504,14 +523,15 @@ attn_mass_ranges(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
     const uint32_t tmem_base = *tmem_slot;
     pdl_launch_dependents();
     pdl_wait();
-    const long all = Walk::total(p), begin = am_start(blockIdx.x, gridDim.x, all);
+    Walk w(p);
+    const long all = w.total(p), begin = am_start(blockIdx.x, gridDim.x, all);
     const int total = (int)(am_start(blockIdx.x + 1, gridDim.x, all) - begin);
+    if (total > 0) w.find(p, begin);
 
     if (warp == 0) {
         if (elect_one() && total > 0) {
             bool ok = true;
             int i = 0, groups = 0;
-            Walk w(p, begin);
             for (; i < total && ok; ++i, w.next(p)) {
                 const int head = w.head(p);
                 if (i == 0 || w.new_a(p)) {
@@ -551,7 +571,6 @@ attn_mass_ranges(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
             const uint64_t b_desc = smem_desc_sw128(smem_u32(smem + L::kBOff), 16, 1024);
             bool ok = true;
             int groups = 0;
-            Walk w(p, begin);
             for (int i = 0; i < total && ok; ++i) {
                 if (i == 0 || w.new_a(p)) {
                     ok = mbar_wait(&a_full[groups & 1], (uint32_t)(groups >> 1) & 1u, abort_flag, p.status);
@@ -585,7 +604,6 @@ attn_mass_ranges(const __grid_constant__ CUtensorMap tmap_q, const __grid_consta
         s.reset();
         bool ok = true;                                // after a failed wait only the barriers are kept up: the status word says so
         int ends = 0;                                  // rows finished so far, by this CTA's part of them
-        Walk w(p, begin);
         for (int i = 0; i < total; ++i) {
             if ((i & 1) == wg && ok) {
                 int valid = kAmTile;
@@ -708,8 +726,12 @@ nova_status launch_mass(nova_ctx* ctx, const void* q, const void* k, const void*
     // Ranges where a CTA gets at least so many tiles of the second pass; with fewer, merging rows through memory costs more
     // than clusters do. us, clusters -> ranges, at tiles per CTA; head size 64: 2.6 33 -> 40, 5.1 56 -> 51, 6.5 70 -> 61, 8.6 78 -> 65,
     // 13 104 -> 87, 27 180 -> 148; head size 128: 3.5 25 -> 31, 6.9 42 -> 44 and 46 -> 40, 13.8 78 -> 64, 73 287 -> 247.
+    // At head size 64, where two CTAs share an SM and hide each other's start, clusters again with many rows of more than five key tiles:
+    // 16 images of 1024 tokens, 13 rows per CTA, 542 -> 559, 32 such 1039 -> 1125; 12 such, 10 rows, 434 -> 424; 256 images of 100
+    // tokens, 14 rows of three tiles, 139 -> 122. At 128 ranges throughout: 512 images of 256 tokens 1283 -> 905.
     const long slots = min((long)ctx->num_sms * (DH == 64 ? 2 : 1), (long)NOVA_TICKETS), tiles2 = (long)tiles * tiles * n_heads * B;
-    if (tiles2 >= (DH == 64 ? 5 : 8) * slots) {
+    const long rows1 = (long)tiles * n_heads * B;
+    if (tiles2 >= (DH == 64 ? 5 : 8) * slots && (DH == 128 || rows1 <= 10 * slots || steps1 <= 5)) {
         {
             nova_launch_scope scope(ctx, NOVA_K_SCORE, st);
             NOVA_CUDA_CHECK(ctx, nova_launch_pdl(attn_mass_ranges<DH, 1>, dim3((unsigned)slots), dim3(kAmThreads), L::kTotal, st, 0, tq, tk, tcache, p));

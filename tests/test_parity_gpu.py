@@ -1646,6 +1646,8 @@ def test_score_attention_mass_matches_oracle(ctx, B, N, C, heads, Lmax, kv_lens)
 @pytest.mark.parametrize("B,N,C,heads,Lmax,kv_lens", [
     (2, 900, 896, 14, 1300, [300, 5]),        # head size 64
     (2, 1000, 1280, 10, 1800, [0, 700]),      # head size 128
+    (100, 40, 1024, 16, 300, [37 * b % 261 for b in range(100)]),      # more images than a warp looks at in one go
+    (130, 30, 1280, 10, 200, [53 * b % 131 for b in range(130)]),
 ])
 def test_score_attention_mass_rows_shared_by_ranges(ctx, B, N, C, heads, Lmax, kv_lens):
     """Calls large enough for even ranges of tiles: images with different numbers of key tiles, ragged last tiles."""
