@@ -259,6 +259,21 @@ def test_head_entropy_masked_codes(ctx, N, V, first, last, mask):
     assert np.abs(ent.cpu().numpy()[:, rows] - want).max() <= ENT_TOL
 
 
+@pytest.mark.parametrize("V", [1024, 4096])
+def test_head_entropy_of_rows_alone_and_in_a_larger_call(ctx, V):
+    """Where a row's column tiles are divided follows from the number of rows: the same rows alone and among others agree within
+    the rounding of sums of V/2 terms (errors of 2^-24 each adding up like their square root, four times that), not to the last bit."""
+    x, w = synth.activations(1, 17000, 64, 45, DEV), synth.randn_bf16((V, 64), 46, DEV, std=0.4)
+    ents = {}
+    for rows in (256, 1000, 9000, 17000):          # ranges of three sizes, whole row blocks
+        ent = ents[rows] = torch.empty((1, rows), dtype=torch.float32, device=DEV)
+        nova.nova_head_entropy(ctx, x[:, :rows].contiguous(), w, None, ent, None)
+    assert ctx.device_status() == 0
+    bound = 4 * math.sqrt(V / 2) * 2.0 ** -24 * (1 + math.log(V))
+    for rows, ent in ents.items():
+        assert float((ent - ents[17000][:, :rows]).abs().max()) <= bound
+
+
 def test_head_entropy_full_size_sampled_rows(ctx):
     """Batch 4 at 64 x 64 tokens, width 2048, V = 4096 (the benchmark's launch): sampled rows."""
     rows = np.array([0, 127, 128, 255, 256, 4095, 4096, 8191, 12287, 12288, 16383])
@@ -980,6 +995,32 @@ def test_whole_pruned_step_config1(ctx):
     fx, _ = oracle.restore_from_cache(f32(x), wy, w_keep, w_prune, w_cu, f32(cache_prev), h, w)
     assert _rel_err(f32(x_out), fx) <= BLOCK_TOL
     assert ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("h,w,kept,F", [
+    (123, 100, 4096, 6400),       # 8204 pruned rows: one warp per row, eight rows to each
+    (100, 80, 3000, 6144),        # 5000: two warps per row, eight rows to each pair
+    (40, 25, 400, 6144),          # 600: a block per SM, two or three rows to each pair
+])
+def test_layer_forward_restore_beside_fc1(ctx, h, w, kept, F):
+    """The pruned rows restored beside FC1, in blocks that go through several rows, bit for bit as by the two calls."""
+    C, heads, hp, wp, Lmax = 128, 2, 11, 9, 64 + h * w
+    N = h * w
+    x = synth.activations(1, N, C, 97, DEV)
+    k_cache, v_cache, _ = synth.kv_cache(1, Lmax, 64, C, 98, DEV)
+    cache_prev = synth.residual_cache(1, hp, wp, C, 99, DEV)
+    keep_idx, prune_idx, cu, _ = gpu_select(ctx, torch.rand((1, N), generator=torch.Generator(device="cpu").manual_seed(h)).to(DEV), [kept])
+    shape = nova.BlockShape(1, N, C, heads, F, Lmax, kept)
+    ctx.ensure_workspace(shape)
+    bw = nova.BlockWeights(synth.block_weights(C, F, 100, DEV), 1e-6)
+    xa, ca, xb, cb = (torch.full_like(x, float("nan")) for _ in range(4))
+    y = torch.empty((kept, C), dtype=torch.bfloat16, device=DEV)
+    state = lambda: (k_cache.clone(), v_cache.clone(), torch.tensor([64], dtype=torch.int32, device=DEV))  # noqa: E731
+    nova.nova_pruned_block_forward(ctx, bw, shape, x, keep_idx, cu, *state(), True, y)
+    nova.nova_restore_from_cache(ctx, x, y, keep_idx, prune_idx, cu, cache_prev, h, w, xa, ca)
+    nova.nova_pruned_layer_forward(ctx, bw, None, shape, x, keep_idx, prune_idx, cu, *state(), True, cache_prev, h, w, xb, cb)
+    assert ctx.device_status() == 0
+    assert torch.equal(xa, xb) and torch.equal(ca, cb)
 
 
 def test_restore_from_a_cache_past_32_bit_offsets(ctx):
