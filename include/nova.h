@@ -62,9 +62,10 @@ typedef enum nova_dtype { NOVA_BF16 = 0, NOVA_F32 = 1 } nova_dtype;
 
 /* ---- context ------------------------------------------------------------------ */
 
-/* Creates a context bound to CUDA device `device`. Allocates about 3 KB of device memory for
- * the status word, tickets and the accumulators of the entropy means (the only allocation the
- * library ever makes). */
+/* Creates a context bound to CUDA device `device`. Allocates about 7 KB of device memory for the
+ * status word, tickets and the accumulators of the entropy means, and 4 KB per SM (0.6 MB on a
+ * B200) for partial results of rows that CTAs of nova_head_entropy or nova_score_attention_mass
+ * share (the only allocation the library ever makes). */
 nova_status nova_create(nova_ctx** out, int device);
 void        nova_destroy(nova_ctx* ctx);
 const char* nova_last_error(const nova_ctx* ctx);
@@ -160,6 +161,9 @@ nova_status nova_scale_entropy_layers(nova_ctx* ctx, const void* const* logits, 
  * b_head: device bf16 [V] or NULL.           ent: device f32 [S, N].   mean: device f32 [S] or NULL.
  * C must be a multiple of 64 and V of 32. A non-finite logit makes the row's entropy NaN and
  * records NOVA_ERR_NONFINITE in the device status word. S*N == 0 is a no-op.
+ * The order in which a row's V terms are added follows from S*N, V and the SM count: the same call
+ * gives the same bits every time, but a token's entropy can differ in its last bits between calls of
+ * different size (a batch of one and of four), and with it the order of tokens that all but tie.
  * Errors: bad sizes -> INVALID_ARG / SHAPE; misaligned pointer -> ALIGNMENT.
  */
 nova_status nova_head_entropy(nova_ctx* ctx, const void* x, const void* w_head, const void* b_head,
@@ -259,7 +263,8 @@ nova_status nova_select_topk_grouped_device(nova_ctx* ctx, const float* ent, int
  *   P[query, kv_len[b] + j]: the share of the scale's attention that lands on token j's key.
  *   q, k device bf16 [B, N, C]; k_cache device bf16 [B, Lmax, C] and kv_len device int32 [B], or both
  *   NULL (no prior keys); lse_scratch device f32 [B, n_heads, N] (scratch); score device f32 [B, N].
- *   Head size 64 or 128. Sums run in a fixed order: results are reproducible bit for bit.
+ *   Head size 64 or 128. Sums run in an order that follows from the sizes, the kv_len and the SM count: the
+ *   same call gives the same bits; calls of different size may differ in a score's last bits.
  * Errors: bad sizes -> INVALID_ARG / SHAPE; misaligned pointers -> ALIGNMENT. Empty inputs are no-ops.
  */
 nova_status nova_score_mse(nova_ctx* ctx, const void* x, const void* ref_prev, int B, int hp, int wp,

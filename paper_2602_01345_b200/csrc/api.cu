@@ -141,7 +141,8 @@ nova_status nova_device_status(nova_ctx* ctx, void* stream)
     unsigned int word = 0;
     NOVA_CUDA_CHECK(ctx, cudaMemcpyAsync(&word, ctx->dev_status, sizeof(word), cudaMemcpyDeviceToHost, st));
     NOVA_CUDA_CHECK(ctx, cudaStreamSynchronize(st));
-    // an aborted kernel may leave the entropy accumulators or attention tickets half way: clear everything
+    // an aborted kernel may leave half way what later ones rely on, the entropy accumulators or the tickets of the attention, the
+    // head and the attention mass: clear everything
     if (word) {
         NOVA_CUDA_CHECK(ctx, cudaMemsetAsync(ctx->dev_status, 0, NOVA_STATUS_BYTES, st));
         if (ctx->wait_limit_ns)     // the wait limit lives in the same block: put it back

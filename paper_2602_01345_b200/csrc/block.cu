@@ -599,11 +599,13 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
     // The pruned rows depend on nothing that the block computes. With `beside` FC1 lets their kernel in as soon as it has
     // passed its wait, when everything up to LN2 has ended; FC1 itself neither writes what it reads nor reads what it
     // writes. It then runs in the registers and the memory bandwidth that FC1 leaves, one block per SM, which is worth it
-    // where FC1 takes well over the time of that: about 110 rows of 2048 a microsecond against 2 M F C / 1.3e15 s. Otherwise, and
+    // where FC1 takes longer than that: about 110 rows of 2048 a microsecond against 2 M F C / 1.3e15 s, even at M F = 2885 pruned
+    // rows, and a few per cent more here. Otherwise, and
     // where the kept count is not known here, it follows the last GEMM. us after -> beside: a 20x20 scale of one image, 32 layers
     // of 2048, 2923 -> 2681, a 32x32 scale of four, 30 layers of 1920, 8843 -> 8750, a 16-layer 256x256 generation 9070 -> 8840;
-    // with 3072 pruned rows for 1024 kept, 64x64 tokens, 6674 -> 7087, with 13107 for 3277 33.8 -> 34.4 ms. Above 4096 kept
-    // rows the GEMMs run at the power limit, and it makes no difference (8192: 39.7 ms either way).
+    // with 3072 pruned rows for 1024 kept, 64x64 tokens (M F = 2731 pruned), 6674 -> 7087, with 13107 for 3277 (2048) 33.8 -> 34.4 ms; the
+    // first two have M F = 24600 and 9400 pruned. With 8192 kept rows, where the GEMMs run at the power limit, it makes no
+    // difference (39.7 ms either way); between that and the largest that was timed, 3277, the line at 4096 is a choice.
     const long pruned = (long)s->B * s->N - M;
     const bool beside = scatter && !m_on_device && pruned > 0 && M <= 4096 && pruned * 3072 < (long)M * F;
     auto restore = [&](bool wait_last) {

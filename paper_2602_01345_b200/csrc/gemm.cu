@@ -75,8 +75,8 @@ __device__ __forceinline__ int true_rows(const GemmParams& p)
 __device__ __forceinline__ bool count_known(const GemmParams& p) { return !p.m_dev || p.count_settled; }
 // The end of the kernel, of the two that are launched with a device-side count, that the problem does not belong to. One CTA
 // waits, so that the launch ends after the one before it; the others make room for the next launch at once. With all of
-// them waiting, and the count read only then, each such launch cost about 3 us; last 64x64 scale in a graph, three such
-// launches in each of 32 layers, 6867 -> 6788 us with the steps before.
+// them waiting, and the count read only then, the last 64x64 scale in a graph, three such launches in each of 32 layers, takes
+// 6786 us instead of 6722.
 __device__ __forceinline__ void leave_to_other(const GemmParams& p)
 {
     pdl_launch_dependents();
