@@ -41,11 +41,11 @@ struct LnModArgs {
 // one addition per lane.
 // What bounds it: HBM and L2 at many rows, and instructions close behind; at few the chain list -> row -> two reductions -> store, so
 // a thread has little to do and all its loads go out first, gain and bias too. Two warps while all their rows run at once with some
-// room left for the next launch (7 of the 8 rows per SM: 1024 rows of 2048 in 4.0 us, with one warp 4.3; 1184 in 5.5 and 4.1), and
+// room left for the next launch (7 of the 8 rows per SM: 1024 rows of 2048 in 3.6 us, with one warp 4.3; 1184 in 4.2 to 5.5 and 4.1 to 4.3), and
 // where a row is too wide for one warp's registers; else one, which saves the exchange. Back to back over warm inputs, us, with one
-// warp per row in blocks of eight rows that end with them -> this: 256 rows x 1024 2.5 -> 1.9, 300 x 2048 4.0 -> 2.8, 1600 x 2048
-// 4.9 -> 4.7, 2252 x 1920 4.9 -> 4.8, 8192 x 2048 11.4 -> 10.8 (6.2 TB/s), 2048 x 4096 13.5 -> 8.9, 2048 x 8192 43 -> 20. With two warps
-// that each add up their own pieces 1.9, 2.4, 5.4, 5.0, 10.4, 8.7 and 15, but other last bits.
+// warp per row in blocks of eight rows that end with them -> this: 256 rows x 1024 2.5 -> 1.8, 300 x 2048 4.0 -> 2.4, 1600 x 2048
+// 4.9 -> 4.7, 2252 x 1920 5.1 -> 4.9, 8192 x 2048 11.4 -> 10.7 (6.3 TB/s), 2048 x 4096 13.4 -> 8.1, 2048 x 8192 50 -> 20. With two warps
+// that each add up their own pieces 1.9, 2.3, 5.5, 5.0, 10.3, 7.8 and 15, but other last bits.
 constexpr int kLnThreads = 64;
 constexpr int kLnBlocksPerSm = 8;
 constexpr int kLnOneVec = 8;           // widest row of one warp: 8 pieces per lane, C = 2048
@@ -107,8 +107,10 @@ layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps,
                uint4* __restrict__ out, const RowMapArgs maps, const LnModArgs mod)
 {
     constexpr int T = 32 * WARPS, kRows = kLnThreads / T;      // threads of a row, rows of a block
-    // the next row, and gain and bias, are loaded ahead where there are registers for them
-    constexpr bool kAhead = VEC * WARPS <= 8, kGainAhead = WARPS == 2 && VEC <= 4;
+    // One warp loads its next row before it works on the present one. Two seldom have a second one (only with a bound on a device-side
+    // count): without the code for it 300 rows of 2048 take 2.4 us instead of 2.8, and 4096 rows 7.5 instead of 8.1.
+    // They load gain and bias early where there are registers for them.
+    constexpr bool kAhead = WARPS == 1, kGainAhead = WARPS == 2 && VEC <= 4;
     __shared__ uint2 given[WARPS == 2 ? VEC * kLnThreads : 1];
     __shared__ float part[2 * kLnThreads];
     pdl_launch_dependents();

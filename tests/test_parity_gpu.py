@@ -820,10 +820,12 @@ def test_block_layernorm_order_of_sums(ctx, C, heads, N):
     x = synth.activations(1, N, C, C + 1, DEV) + 2.0
     keep_idx, _, cu, _ = gpu_select(ctx, torch.rand((1, N)).to(DEV), [N])
     shape = nova.BlockShape(1, N, C, heads, 64, N, N)
-    k, v, kv_len = synth.kv_cache(1, N, 0, C, 5, DEV)
-    _run_block(ctx, shape, nova.BlockWeights(wt, 1e-6), x, keep_idx, cu, k, v, kv_len)
-    want = _layernorm_in_order(f32(x[0]), f32(wt["ln1_g"]), f32(wt["ln1_b"]), 1e-6)
-    assert torch.equal(k[0].cpu(), torch.from_numpy(want).to(torch.bfloat16))
+    ctx.ensure_workspace(shape)
+    want = torch.from_numpy(_layernorm_in_order(f32(x[0]), f32(wt["ln1_g"]), f32(wt["ln1_b"]), 1e-6)).to(torch.bfloat16)
+    for call in (nova.nova_pruned_block_forward, nova.nova_pruned_block_forward_device):     # (a bound: two warps, several rows to a block)
+        k, v, kv_len = synth.kv_cache(1, N, 0, C, 5, DEV)
+        call(ctx, nova.BlockWeights(wt, 1e-6), shape, x, keep_idx, cu, k, v, kv_len, True, torch.empty_like(x[0]))
+        assert torch.equal(k[0].cpu(), want)
 
 
 def test_block_without_append_leaves_kv_len(ctx):
