@@ -32,22 +32,28 @@ struct LnModArgs {
 };
 
 // ---- LayerNorm ----------------------------------------------------------------------------
-// A row (C <= 64 * 8 * VEC bf16, or half of that with one warp) is the work of one or two warps, in persistent blocks of two
-// warps that go through the rows in turn. x is read once and out written once; in between the row stays in registers.
+// A row (C <= 64 * 8 * VEC bf16, or half of that with one warp) is the work of one or two warps, in persistent blocks that go
+// through the rows in turn. x is read once and out written once; in between the row stays in registers.
 // The sums of a row are made in an order that depends on its width alone, so that a token's result is the same to the last bit in any
 // launch: 32 partial sums, of the 128-bit pieces l, l + 32, l + 64, ..., the even and the odd features apart, the even added to
 // the odd ones, then a butterfly. One warp does that as packed pairs. Of two warps one has the row's even features and the other its odd
 // ones: they load alternate pieces, hand each other through shared memory the half that the other needs, and meet again for the
 // one addition per lane.
 // What bounds it: HBM and L2 at many rows, and instructions close behind; at few the chain list -> row -> two reductions -> store, so
-// a thread has little to do and all its loads go out first, gain and bias too. Two warps while all their rows run at once with some
-// room left for the next launch (7 of the 8 rows per SM: 1024 rows of 2048 in 3.6 us, with one warp 4.3; 1184 in 4.2 to 5.5 and 4.1 to 4.3), and
-// where a row is too wide for one warp's registers; else one, which saves the exchange. Back to back over warm inputs, us, with one
-// warp per row in blocks of eight rows that end with them -> this: 256 rows x 1024 2.5 -> 1.8, 300 x 2048 4.0 -> 2.4, 1600 x 2048
-// 4.9 -> 4.7, 2252 x 1920 5.1 -> 4.9, 8192 x 2048 11.4 -> 10.7 (6.3 TB/s), 2048 x 4096 13.4 -> 8.1, 2048 x 8192 50 -> 20. With two warps
-// that each add up their own pieces 1.9, 2.3, 5.5, 5.0, 10.3, 7.8 and 15, but other last bits.
-constexpr int kLnThreads = 64;
+// a thread has little to do and all its loads go out first, gain and bias too. Two warps, in blocks of their own, while all their rows
+// run at once with some room left for the next launch (7 of the 8 rows per SM: 1024 rows of 2048 in 3.6 us, with one warp 4.3), and
+// where a row is too wide for one warp's registers; else one, which saves the exchange, eight rows to a block: two blocks per SM that load
+// their next row before they work on the present one, or three that do not where only those take all rows at once (3277 rows of 2048 over
+// inputs larger than L2 6.5 us instead of 7.8; with blocks of two rows 8.4).
+// us, one warp per row in blocks of eight rows that end with them -> this, back to back over warm inputs: 256 rows x 1024 2.5 -> 1.8,
+// 300 x 2048 4.0 -> 2.4, 1600 x 2048 4.9 -> 4.5, 2252 x 1920 5.1 -> 4.5, 4096 x 2048 8.6 -> 6.6, 8192 x 2048 11.4 -> 10.9, 2048 x 4096
+// 13.5 -> 8.2, 2048 x 8192 50 -> 20; over inputs larger than L2 2252 x 1920 5.8 -> 5.3, 4096 x 2048 10.1 -> 8.3, 8192 x 2048
+// 15.0 -> 13.6 (4.9 TB/s), 8192 x 1024 8.0 -> 7.8. With two warps that each add up their own pieces 1.9, 2.3, 4.4, 4.9, 6.7, 10.4, 7.8, 15 and
+// 5.9, 7.9, 13.3, 8.9, but other last bits.
+constexpr int kLnThreads = 64;         // two warps per row
 constexpr int kLnBlocksPerSm = 8;
+constexpr int kLnOneThreads = 256;     // one warp per row
+constexpr int kLnOneRows = kLnOneThreads / 32;
 constexpr int kLnOneVec = 8;           // widest row of one warp: 8 pieces per lane, C = 2048
 
 __device__ __forceinline__ uint4 ld_stream(const uint4* p)
@@ -100,17 +106,16 @@ __device__ __forceinline__ float lo_f32(uint32_t w) { return __uint_as_float(w <
 __device__ __forceinline__ float hi_f32(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 __device__ __forceinline__ uint64_t bf16x2_f32x2(uint32_t w) { return pack_f32x2(lo_f32(w), hi_f32(w)); }
 
-// VEC: 128-bit pieces per thread
-template <int VEC, int WARPS, bool MAPS, bool MOD>
-__global__ void __launch_bounds__(kLnThreads, kLnBlocksPerSm)
+// VEC: 128-bit pieces per thread. AHEAD: the next row is loaded before the present one is worked on. (Two warps seldom have a second
+// one, only with a bound on a device-side count: without the code for it 300 rows of 2048 take 2.4 us instead of 2.8, and 4096 rows
+// 7.5 instead of 8.1.)
+template <int VEC, int WARPS, bool AHEAD, bool MAPS, bool MOD>
+__global__ void __launch_bounds__(WARPS == 1 ? kLnOneThreads : kLnThreads, WARPS == 2 ? kLnBlocksPerSm : AHEAD ? 2 : 3)
 layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps, int M, const int32_t* m_dev, int vec_per_row,
                uint4* __restrict__ out, const RowMapArgs maps, const LnModArgs mod)
 {
-    constexpr int T = 32 * WARPS, kRows = kLnThreads / T;      // threads of a row, rows of a block
-    // One warp loads its next row before it works on the present one. Two seldom have a second one (only with a bound on a device-side
-    // count): without the code for it 300 rows of 2048 take 2.4 us instead of 2.8, and 4096 rows 7.5 instead of 8.1.
-    // They load gain and bias early where there are registers for them.
-    constexpr bool kAhead = WARPS == 1, kGainAhead = WARPS == 2 && VEC <= 4;
+    constexpr int T = 32 * WARPS, kRows = WARPS == 1 ? kLnOneRows : 1;      // threads of a row, rows of a block
+    constexpr bool kGainAhead = WARPS == 2 && VEC <= 4;      // gain and bias are loaded early where there are registers for them
     __shared__ uint2 given[WARPS == 2 ? VEC * kLnThreads : 1];
     __shared__ float part[2 * kLnThreads];
     pdl_launch_dependents();
@@ -119,7 +124,7 @@ layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps,
     // prefetch hands nothing to this kernel, so whoever still writes them does no harm. With few
     // rows the launch is a chain of latencies, of which this takes one off: a 16-layer 256x256 generation 9412 ->
     // 9316 us, a 20x20 scale of one image 3097 -> 3058.
-    for (int c = threadIdx.x * 8; c < vec_per_row; c += kLnThreads * 8) {
+    for (int c = threadIdx.x * 8; c < vec_per_row; c += T * kRows * 8) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(gamma + c));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(beta + c));
     }
@@ -147,7 +152,7 @@ layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps,
             d[i] = (c < vec_per_row) ? ld_stream(x + src * vec_per_row + c) : make_uint4(0, 0, 0, 0);
         }
     };
-    int r = blockIdx.x * kRows + threadIdx.x / T;
+    int r = blockIdx.x * kRows + (WARPS == 1 ? threadIdx.x / T : 0);
     if (r >= M) return;
     long src, src_next = 0;
     int img, img_next = 0;
@@ -166,7 +171,7 @@ layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps,
         const int r_next = r + (int)gridDim.x * kRows;
         if (r_next < M) {
             locate(r_next, src_next, img_next);
-            if (kAhead) load(src_next, next);
+            if (AHEAD) load(src_next, next);
         }
         if (MAPS && tid == 0) {
             const int c0 = maps.cu_keep[img], k_b = maps.cu_keep[img + 1] - c0, len = maps.kv_len[img];
@@ -287,7 +292,7 @@ layernorm_rows(const uint4* x, const uint4* gamma, const uint4* beta, float eps,
         r = r_next;
         src = src_next;
         img = img_next;
-        if (kAhead) {
+        if (AHEAD) {
 #pragma unroll
             for (int i = 0; i < VEC; ++i) raw[i] = next[i];
         } else {
@@ -405,29 +410,34 @@ static nova_status launch_ln(nova_ctx* ctx, const __nv_bfloat16* x, const RowMap
     const int fit = ctx->num_sms * kLnBlocksPerSm;
     // (of a bound on a device-side count a quarter: a last scale keeps about that)
     const bool one = (m_dev ? M / 4 : M) > fit - fit / 8 && vec <= 32 * kLnOneVec;
-    const dim3 grid(min(one ? (M + 1) / 2 : M, fit)), block(kLnThreads);
+    const int one_blocks = (M + kLnOneRows - 1) / kLnOneRows;
+    const bool ahead = m_dev || one_blocks <= 2 * ctx->num_sms || one_blocks > 3 * ctx->num_sms;
+    const dim3 grid(one ? min(one_blocks, (ahead ? 2 : 3) * ctx->num_sms) : min(M, fit)), block(one ? kLnOneThreads : kLnThreads);
     RowMapArgs none;
     memset(&none, 0, sizeof(none));
     cudaError_t le = cudaSuccess;
     nova_launch_scope scope(ctx, NOVA_K_LAYERNORM, st);
-#define NOVA_LN_LAUNCH(V, W, MAPS, MOD, MAPARG)                                                                     \
-    le = nova_launch_pdl(layernorm_rows<V, W, MAPS, MOD>, grid, block, 0, st, 0, (const uint4*)x, (const uint4*)g, (const uint4*)b, eps, M, m_dev, vec, (uint4*)out, MAPARG, mod)
-#define NOVA_LN_CASE(V, W)                                                                                          \
+#define NOVA_LN_LAUNCH(V, W, AHEAD, MAPS, MOD, MAPARG)                                                                     \
+    le = nova_launch_pdl(layernorm_rows<V, W, AHEAD, MAPS, MOD>, grid, block, 0, st, 0, (const uint4*)x, (const uint4*)g, (const uint4*)b, eps, M, m_dev, vec, (uint4*)out, MAPARG, mod)
+#define NOVA_LN_CASE(V, W, AHEAD)                                                                                          \
     do {                                                                                                         \
-        if (maps && modulated) NOVA_LN_LAUNCH(V, W, true, true, *maps);                                             \
-        else if (maps) NOVA_LN_LAUNCH(V, W, true, false, *maps);                                                    \
-        else if (modulated) NOVA_LN_LAUNCH(V, W, false, true, none);                                                \
-        else NOVA_LN_LAUNCH(V, W, false, false, none);                                                              \
+        if (maps && modulated) NOVA_LN_LAUNCH(V, W, AHEAD, true, true, *maps);                                             \
+        else if (maps) NOVA_LN_LAUNCH(V, W, AHEAD, true, false, *maps);                                                    \
+        else if (modulated) NOVA_LN_LAUNCH(V, W, AHEAD, false, true, none);                                                \
+        else NOVA_LN_LAUNCH(V, W, AHEAD, false, false, none);                                                              \
     } while (0)
     const bool modulated = mod.scale || mod.shift;
-    if (one && vec <= 32 * 4) NOVA_LN_CASE(4, 1);
-    else if (one && vec <= 32 * 6) NOVA_LN_CASE(6, 1);
-    else if (one) NOVA_LN_CASE(kLnOneVec, 1);
-    else if (vec <= 64 * 2) NOVA_LN_CASE(2, 2);
-    else if (vec <= 64 * 3) NOVA_LN_CASE(3, 2);
-    else if (vec <= 64 * 4) NOVA_LN_CASE(4, 2);
-    else if (vec <= 64 * 8) NOVA_LN_CASE(8, 2);
-    else if (vec <= 64 * 16) NOVA_LN_CASE(16, 2);
+    if (one && ahead && vec <= 32 * 4) NOVA_LN_CASE(4, 1, true);
+    else if (one && ahead && vec <= 32 * 6) NOVA_LN_CASE(6, 1, true);
+    else if (one && ahead) NOVA_LN_CASE(kLnOneVec, 1, true);
+    else if (one && vec <= 32 * 4) NOVA_LN_CASE(4, 1, false);
+    else if (one && vec <= 32 * 6) NOVA_LN_CASE(6, 1, false);
+    else if (one) NOVA_LN_CASE(kLnOneVec, 1, false);
+    else if (vec <= 64 * 2) NOVA_LN_CASE(2, 2, false);
+    else if (vec <= 64 * 3) NOVA_LN_CASE(3, 2, false);
+    else if (vec <= 64 * 4) NOVA_LN_CASE(4, 2, false);
+    else if (vec <= 64 * 8) NOVA_LN_CASE(8, 2, false);
+    else if (vec <= 64 * 16) NOVA_LN_CASE(16, 2, false);
     else return nova_fail(ctx, NOVA_ERR_SHAPE, "layernorm: C > 8192");
 #undef NOVA_LN_LAUNCH
 #undef NOVA_LN_CASE
