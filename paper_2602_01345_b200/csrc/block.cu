@@ -618,8 +618,11 @@ static nova_status block_forward(nova_ctx* ctx, const nova_block_weights* w, con
     // with 3072 pruned rows for 1024 kept, 64x64 tokens (M F = 2731 pruned), 6674 -> 7087, with 13107 for 3277 (2048) 33.8 -> 34.4 ms; the
     // first two have M F = 24600 and 9400 pruned. With 8192 kept rows, where the GEMMs run at the power limit, it makes no
     // difference (39.7 ms either way); between that and the largest that was timed, 3277, the line at 4096 is a choice.
+    // Not with event brackets around either of the two: events keep launches apart, and one block per SM alone is slow (a bracketed 64x64
+    // scale of one image, 2048 kept, 11.7 -> 12.4 ms).
     const long pruned = (long)s->B * s->N - M;
-    const bool beside = scatter && !m_on_device && pruned > 0 && M <= 4096 && pruned * 3072 < (long)M * F;
+    const bool apart = ctx->profiling && (ctx->prof_mask & (1ull << NOVA_K_GEMM_FC1 | 1ull << NOVA_K_RESTORE));
+    const bool beside = scatter && !m_on_device && !apart && pruned > 0 && M <= 4096 && pruned * 3072 < (long)M * F;
     auto restore = [&](bool wait_last) {
         return nova_restore_pruned_rows(ctx, x_in, scatter->prune_idx, cu_keep, scatter->cache_prev, scatter->hp, scatter->wp,
                                         scatter->h, scatter->w, C, s->B, M, m_on_device, scatter->x_out, scatter->cache_out, stream, wait_last);

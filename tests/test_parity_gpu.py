@@ -1006,6 +1006,7 @@ def test_whole_pruned_step_config1(ctx):
 ])
 def test_layer_forward_restore_beside_fc1(ctx, h, w, kept, F):
     """The pruned rows restored beside FC1, in blocks that go through several rows, bit for bit as by the two calls."""
+    from paper_2602_01345_b200 import pipeline
     C, heads, hp, wp, Lmax = 128, 2, 11, 9, 64 + h * w
     N = h * w
     x = synth.activations(1, N, C, 97, DEV)
@@ -1022,6 +1023,13 @@ def test_layer_forward_restore_beside_fc1(ctx, h, w, kept, F):
     nova.nova_restore_from_cache(ctx, x, y, keep_idx, prune_idx, cu, cache_prev, h, w, xa, ca)
     nova.nova_pruned_layer_forward(ctx, bw, None, shape, x, keep_idx, prune_idx, cu, *state(), True, cache_prev, h, w, xb, cb)
     assert ctx.device_status() == 0
+    assert torch.equal(xa, xb) and torch.equal(ca, cb)
+    # with event brackets around its launch it follows the last GEMM
+    xb.fill_(float("nan"))
+    cb.fill_(float("nan"))
+    pipeline.profile_begin(ctx)
+    nova.nova_pruned_layer_forward(ctx, bw, None, shape, x, keep_idx, prune_idx, cu, *state(), True, cache_prev, h, w, xb, cb)
+    assert pipeline.profile_end(ctx)["restore"][1] == 1
     assert torch.equal(xa, xb) and torch.equal(ca, cb)
 
 
