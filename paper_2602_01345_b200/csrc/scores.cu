@@ -422,13 +422,18 @@ struct AmWalk {
         return PASS == 1 ? tiles_of(p) + (old_keys(p, b) + kAmTile - 1) / kAmTile : tiles_of(p) * p.n_heads;
     }
     // The launch's tiles, and the place of one of them; by whole warps, 32 images at a time (with one after the other a launch of 60000
-    // images of 16 tokens took 11.2 ms, 3.0 of them for its tiles).
+    // images of 16 tokens took 11.2 ms, 3.0 of them for its tiles), or a few one after the other (two images: 0.7 us of a call of 106).
+    static constexpr int kFewImages = 4;
     __device__ __forceinline__ long image_tiles(const AmParams& p, int b) const { return b < p.B ? (long)rows_of(p) * row_tiles(p, b) : 0; }
     __device__ __forceinline__ explicit AmWalk(const AmParams&) {}
     __device__ __forceinline__ static int rows_of(const AmParams& p) { return PASS == 1 ? tiles_of(p) * p.n_heads : tiles_of(p); }
     __device__ __forceinline__ long total(const AmParams& p) const
     {
         long n = 0;
+        if (p.B <= kFewImages) {
+            for (int i = 0; i < p.B; ++i) n += image_tiles(p, i);
+            return n;
+        }
         for (int b0 = threadIdx.x & 31; b0 < p.B; b0 += 32) n += image_tiles(p, b0);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
@@ -438,7 +443,9 @@ struct AmWalk {
     {
         const int lane = threadIdx.x & 31;
         row0 = 0;
-        for (int b0 = 0; b0 < p.B; b0 += 32) {
+        if (p.B <= kFewImages) {
+            for (; b < p.B - 1 && at >= row0 + image_tiles(p, b); ++b) row0 += image_tiles(p, b);
+        } else for (int b0 = 0; b0 < p.B; b0 += 32) {
             const long mine = image_tiles(p, b0 + lane);
             long incl = mine;
 #pragma unroll
