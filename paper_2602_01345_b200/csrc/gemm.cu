@@ -134,8 +134,9 @@ struct EpiRows {
         }
     }
 };
-// What the epilogue reads of four features of those rows, fetched before the accumulator is ready.
-template <int EPI>
+// What the epilogue reads of four features of those rows, fetched before the accumulator is ready. DIFF: with a second output
+// (if there is none all the same, diff_out says so).
+template <int EPI, bool DIFF>
 struct EpiData {
     uint2 res[8], diff[8], gate;
     __device__ __forceinline__ void fetch(const GemmParams& p, const EpiRows<EPI>& r, int col)
@@ -143,7 +144,7 @@ struct EpiData {
         if (EPI != NOVA_EPI_BIAS_RES) return;
 #pragma unroll
         for (int i = 0; i < 8; ++i) res[i] = *(const uint2*)(p.res + (long)r.in[i] * p.N + col);
-        if (p.diff_out) {
+        if (DIFF && p.diff_out) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) diff[i] = *(const uint2*)(p.diff_in + (long)r.out[i] * p.N + col);
         }
@@ -152,9 +153,9 @@ struct EpiData {
 };
 // v = accumulators; + bias, then GELU / residual / QKV routing, rounded to bf16. Features col .. col + 3 of
 // rows row0 + STEP * (FROM + i) < row_end, four of the eight at a time (registers).
-template <int EPI, int STEP, int FROM>
+template <int EPI, int STEP, int FROM, bool DIFF>
 __device__ __forceinline__ void epi_store(const GemmParams& p, int row0, int row_end, const EpiRows<EPI>& r, int col, uint2 bias,
-                                          const EpiData<EPI>& d, float (&v)[4][4])
+                                          const EpiData<EPI, DIFF>& d, float (&v)[4][4])
 {
     float t[4];
     unpack_bf16x4(bias, t);
@@ -209,7 +210,7 @@ __device__ __forceinline__ void epi_store(const GemmParams& p, int row0, int row
 #pragma unroll
     for (int i = 0; i < 4; ++i)
         if (row0 + STEP * (FROM + i) < row_end) *(uint2*)(p.out + (long)r.out[FROM + i] * p.N + col) = y[i];
-    if (EPI == NOVA_EPI_BIAS_RES && p.diff_out) {
+    if (EPI == NOVA_EPI_BIAS_RES && DIFF && p.diff_out) {
         // second output: the stored (bf16-rounded) value minus diff_in's row, i.e. what a separate pass over
         // the stored output would compute
 #pragma unroll
@@ -508,7 +509,8 @@ struct EntropyState {
 //   empty[s]      each CTA's copy, signalled in both CTAs by the leader's tcgen05.commit
 //   acc_full[a]   each CTA's copy, same; a = accumulator buffer of tile parity
 //   acc_empty[a]  leader's copy: one arrival per epilogue warp of both CTAs (16)
-template <int BN, int STAGES, int EPI>
+// DIFF: the residual epilogue with a second output. Without one there are registers to fetch two chunks ahead.
+template <int BN, int STAGES, int EPI, bool DIFF>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                   const __grid_constant__ CUtensorMap tmap_w_half, const GemmParams p, const int span_host,
@@ -681,7 +683,9 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             } else {
                 // After the turn-round this lane holds features 4 * (lane % 8) .. + 3 of a chunk's 32, of rows
                 // row0 + lane / 8 + 4 i. What the epilogue reads of the first chunk is fetched before the accumulator is
-                // ready, of the next one while this one is worked on; in a pair's last tile all of it is brought to L2 before. With a residual the
+                // ready, of the next one while this one is worked on, with a residual alone of the one after that
+                // (K = 2048 leaves little time for it: by itself, 8192 rows x 2048 features 71.4 -> 68.2 us, 3277 rows 37.7 -> 34.6; whole calls,
+                // at the power limit, the same); in a pair's last tile all of it is brought to L2 before. With a residual the
                 // loop is not unrolled: a launch whose pairs have one tile each runs this code once. After the last MMA of
                 // 2252 rows x 1920 features, gated, it takes 6.4 us (7 before, unrolled and with the gate's row looked up and loaded
                 // in turn), 8.7 with a second output (13, its other operand loaded where it was used): latency of what is
@@ -690,7 +694,8 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 const int chunks = row0 < M ? min(n_chunks, (p.N - n0) / 32) : 0;
                 int col = n0 + c_first * 32 + (lane & 7) * 4;
                 EpiRows<EPI> er;
-                EpiData<EPI> ed;
+                constexpr bool kTwoAhead = EPI == NOVA_EPI_BIAS_RES && !DIFF;
+                EpiData<EPI, DIFF> ed, ed_next;
                 uint2 bias = make_uint2(0, 0);
                 const bool last_tile = pair_entry(local + 1, pair, num_pairs, num_tiles, group) < 0;
                 if (EPI == NOVA_EPI_BIAS_RES && last_tile && chunks > 0) {
@@ -704,6 +709,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                     er.template load<4>(p, rows0, M);
                     bias = *(const uint2*)(p.bias + col);
                     ed.fetch(p, er, col);
+                    if (kTwoAhead && c_first + 2 < chunks) ed_next.fetch(p, er, col + 64);
                 }
                 ok = mbar_wait_warp(&acc_full[a], (uint32_t)(local >> 1) & 1, abort_flag, p.status);
                 if (!ok) break;
@@ -715,12 +721,13 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 for (int c = 0; c < BN / 64; ++c, col += 64) {
                     const int ch = 2 * c + c_first;
                     if (ch >= chunks) break;
-                    EpiData<EPI> ed_next;
+                    EpiData<EPI, DIFF> ed_after;
                     uint2 bias_next = make_uint2(0, 0);
                     if (ch + 2 < chunks) {
                         bias_next = *(const uint2*)(p.bias + col + 64);
-                        ed_next.fetch(p, er, col + 64);
+                        if (!kTwoAhead) ed_next.fetch(p, er, col + 64);
                     }
+                    if (kTwoAhead && ch + 4 < chunks) ed_after.fetch(p, er, col + 128);
                     uint32_t acc[32];
                     tmem_ld32(t_addr + (uint32_t)(ch * 32), acc);
                     tmem_ld_wait();
@@ -740,10 +747,11 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                         }
                     };
                     take(0);
-                    epi_store<EPI, 4, 0>(p, rows0, M, er, col, bias, ed, v);
+                    epi_store<EPI, 4, 0, DIFF>(p, rows0, M, er, col, bias, ed, v);
                     take(4);
-                    epi_store<EPI, 4, 4>(p, rows0, M, er, col, bias, ed, v);
+                    epi_store<EPI, 4, 4, DIFF>(p, rows0, M, er, col, bias, ed, v);
                     ed = ed_next;
+                    if (kTwoAhead) ed_next = ed_after;
                     bias = bias_next;
                 }
             }
@@ -793,7 +801,7 @@ gemm_bf16_tn_pair(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     }
 }
 
-template <int BN, int STAGES, int EPI>
+template <int BN, int STAGES, int EPI, bool DIFF = false>
 nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
 {
     using L = PairSmem<BN, STAGES>;
@@ -804,7 +812,7 @@ nova_status launch_pair(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
     if (!make_tmap_bf16(ctx, &ta, a.A, 2, da, sa, 128) || !make_tmap_bf16(ctx, &tw, a.W, 2, dw, sw, BN / 2) ||
         !make_tmap_bf16(ctx, &tw_half, a.W, 2, dw, sw, BN / 4))
         return nova_fail(ctx, NOVA_ERR_CUDA, "gemm: cuTensorMapEncodeTiled failed");
-    auto kern = gemm_bf16_tn_pair<BN, STAGES, EPI>;
+    auto kern = gemm_bf16_tn_pair<BN, STAGES, EPI, DIFF>;
     static bool attr_done[64];
     if (ctx->device < 64 && !attr_done[ctx->device]) {
         NOVA_CUDA_CHECK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal));
@@ -931,7 +939,7 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
         const int col = f0 + lane * 4;
         const int first = t0 + part * share + warp - 2, t_end = min(t0 + (part + 1) * share, M);
         EpiRows<EPI> er;
-        EpiData<EPI> ed;
+        EpiData<EPI, true> ed;
         uint2 bias = make_uint2(0, 0);
         if (warp == 0) {
             if (active && elect_one()) {
@@ -1050,10 +1058,10 @@ gemm_bf16_split(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
                     }
                 };
                 take(0);
-                epi_store<EPI, 8, 0>(p, t, t_end, er, col, bias, ed, v);
+                epi_store<EPI, 8, 0, true>(p, t, t_end, er, col, bias, ed, v);
                 if (t + 32 < t_end) {
                     take(4);
-                    epi_store<EPI, 8, 4>(p, t, t_end, er, col, bias, ed, v);
+                    epi_store<EPI, 8, 4, true>(p, t, t_end, er, col, bias, ed, v);
                 }
                 if (t + 64 < t_end) {
                     er = er_next;
@@ -1135,6 +1143,7 @@ nova_status launch_gemm(nova_ctx* ctx, const nova_gemm_args& a, cudaStream_t st)
         const nova_status rs = launch_split<EPI>(ctx, a, plan, st);
         if (rs != NOVA_OK || plan.takes) return rs;
     }
+    if (EPI == NOVA_EPI_BIAS_RES && a.diff_out) return launch_pair<256, 6, EPI, EPI == NOVA_EPI_BIAS_RES>(ctx, a, st);
     return launch_pair<256, 6, EPI>(ctx, a, st);
 }
 
