@@ -9,9 +9,9 @@
 // What bounds it: HBM at many rows, the latency of list -> rows -> store at few. With one warp per row and one piece at
 // a time each piece waited for the one before it to be stored. Pruned rows alone, back to back over buffers larger than
 // L2, us before -> with two warps / with one: 100 rows of 2048 6.8 -> 3.6 / 3.9; 1640 x 1024 6.8 -> 4.8 / 5.0; 1844 x 1920
-// 10.5 -> 9.2 / 9.6; 3072 x 2048 12.7 -> 11.2 / 11.3; 4800 x 2048 16.4 -> 16.7 / 17.7; 6144 x 2048 22.5 -> 20.2 / 19.3; 8192 x 2048
-// 27.6 -> 27.2 / 27.5; 8192 x 1024 15.3 -> 15.7 / 15.2; 13108 x 2048 38.6 -> 37.4 / 36.5 (5.4 TB/s). (Over buffers that fit L2 one piece at a time
-// was the faster for 4800 to 8192 rows, 12.4 and 22.5 us against 13.4 and 24.1, with every row in flight at once.)
+// 10.5 -> 9.2 / 9.6; 3072 x 2048 12.7 -> 11.2 / 11.3; 4800 x 2048 16.4 -> 16.9 / 17.2; 6144 x 2048 22.5 -> 20.3 / 19.8; 8192 x 2048
+// 27.6 -> 27.7 / 27.1; 8192 x 1024 15.3 -> 16.5 / 15.4; 13108 x 2048 38.6 -> 37.4 with one (5.3 TB/s). (Over buffers that fit L2 one piece at a time
+// was the faster for 4800 to 8192 rows, 12.4 and 22.5 us against 13.5 and 23.9, with every row in flight at once.)
 #include "common.cuh"
 
 namespace {
@@ -19,8 +19,6 @@ namespace {
 constexpr int kThreads = 128;
 // Up to this many rows two warps share a row, above it one warp has it to itself (fewer index computations).
 constexpr long kWideRows = 5000;
-// Pruned rows alone: as many blocks as run at once go through them. (A block for every two rows of 8192: 34 us by itself instead of 31.)
-constexpr int kBlocksPerSm = 6;
 constexpr long kRowsBeside = 8;       // rows of a group of threads at most, in a launch that works beside another
 
 __device__ __forceinline__ uint4 ld_stream(const uint4* p)
@@ -49,7 +47,7 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi)
 // block.cu); it then works beside that one and waits only to end after it.
 // PRUNED_ONLY: the kept rows are written by the block's last epilogue; work items start at the first pruned entry.
 template <bool PRUNED_ONLY>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSm)
+__global__ void __launch_bounds__(kThreads, 6)
 restore_kernel(const uint4* x_in, const uint4* y_kept, const int32_t* keep_idx, const int32_t* prune_idx,
                const int32_t* cu_keep, const uint4* cache_prev,
                int hp, int wp, int h, int w, int vec_per_row, int row_threads, int B, int M, bool m_on_device, bool wait_last,
@@ -210,7 +208,8 @@ static nova_status restore(nova_ctx* ctx, const void* x_in, const void* y_kept,
     const int rows_per_block = kThreads / row_threads;
     long blocks = (items + rows_per_block - 1) / rows_per_block;
     // Beside another kernel one block per SM finds room: as many rows per block as that takes, up to kRowsBeside.
-    if (pruned_only && !wait_last) blocks = min(blocks, (long)ctx->num_sms * kBlocksPerSm);
+    // (Not as many blocks as run at once: by themselves 8192 rows take 31 us that way instead of 33, but the next layer's first kernel
+    // starts as blocks end, and a scale of 32 layers with 13107 pruned rows each took 33.2 ms instead of 33.0.)
     if (pruned_only && wait_last) blocks = max((blocks + kRowsBeside - 1) / kRowsBeside, min(blocks, (long)ctx->num_sms));
     nova_launch_scope scope(ctx, NOVA_K_RESTORE, (cudaStream_t)stream);
     NOVA_CUDA_CHECK(ctx, nova_launch_pdl(
